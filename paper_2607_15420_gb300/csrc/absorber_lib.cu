@@ -22,6 +22,7 @@
 #include "kernels_warp.cuh"
 #include "kernels_tc.cuh"
 #include "vec_kernels.cuh"
+#include "kernels_cond.cuh"
 #include "kernels_ldl.cuh"
 
 using namespace absorber;
@@ -338,6 +339,15 @@ cudaError_t upload_tables(int dev) {
         UP(g_lt, lt);
     }
 #undef UP
+    // the solve kernels' dynamic shared memory (per device, before any launch of them)
+    const int s64 = (int)cond_smem(sizeof(double)), s32 = (int)cond_smem(sizeof(float));
+    const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if ((e = cudaFuncSetAttribute(cond_solve_kernel<CP_FP64>, a, s64)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(cond_solve_kernel<CP_FP32>, a, s32)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(cond_solve_kernel<CP_MIXED>, a, s64)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(cond_direction_kernel<CP_FP64>, a, s64)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(cond_direction_kernel<CP_FP32>, a, s32)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(cond_direction_kernel<CP_MIXED>, a, s64)) != cudaSuccess) return e;
     g_uploaded[dev] = true;
     return cudaSuccess;
 }
@@ -424,10 +434,11 @@ struct abs_problem {
     double* jac = nullptr;       // nnzJ * ld
     double* hes = nullptr;       // nnzH * ld
     double* vec = nullptr;       // pool of primal-size vectors
-    void* LUp[2] = {nullptr, nullptr};   // factors per precision [ABS_PREC_FP64], [ABS_PREC_FP32]
-    void* Gp[2] = {nullptr, nullptr};
-    void* LU = nullptr;
-    void* G = nullptr;
+    // condensed factors per precision [ABS_PREC_FP64], [ABS_PREC_FP32] (kernels_cond.cuh)
+    void* cond[2] = {nullptr, nullptr};
+    // tensor-core FP32 factor: stage-block inverses, G blocks, row order
+    float* tcAI = nullptr;
+    float* tcG = nullptr;
     unsigned char* piv = nullptr;
     int* sing = nullptr;
     double* part = nullptr;      // per-thread partials [KMAX][N_STAGES][ld]
@@ -591,7 +602,6 @@ abs_status ensure_buffers(abs_problem* h) {
     CK(cudaMalloc(&h->hes, sizeof(double) * (size_t)h->nnzH * ld));
     CK(cudaMalloc(&h->vec, sizeof(double) * (size_t)vsize(h) * V_COUNT));
     CK(cudaMemset(h->vec, 0, sizeof(double) * (size_t)vsize(h) * V_COUNT));
-    CK(cudaMalloc(&h->piv, (size_t)N_STAGES * PIV_BYTES * ld));
     CK(cudaMalloc(&h->sing, sizeof(int) * (size_t)ld));
     CK(cudaMemset(h->sing, 0, sizeof(int) * (size_t)ld));
     CK(cudaMalloc(&h->part, sizeof(double) * (size_t)KMAX * N_STAGES * ld));
@@ -642,14 +652,17 @@ abs_status ensure_stream(abs_problem* h) {
     return ABS_OK;
 }
 
+// factor storage of a precision (FP32: with the tensor-core factor's own when it is selected)
 abs_status ensure_factor(abs_problem* h, int prec) {
-    if (!h->LUp[prec]) {
+    if (!h->cond[prec]) {
         const size_t es = prec == ABS_PREC_FP32 ? sizeof(float) : sizeof(double);
-        CK(cudaMalloc(&h->LUp[prec], es * (size_t)N_STAGES * NV * NV * h->ld));
-        CK(cudaMalloc(&h->Gp[prec], es * (size_t)N_STAGES * NV * NABV * h->ld));
+        CK(cudaMalloc(&h->cond[prec], es * (size_t)N_STAGES * CF_COUNT * h->ld));
     }
-    h->LU = h->LUp[prec];
-    h->G = h->Gp[prec];
+    if (prec == ABS_PREC_FP32 && h->factor_kernel == 1 && !h->tcAI) {
+        CK(cudaMalloc(&h->tcG, sizeof(float) * (size_t)N_STAGES * NV * NABV * h->ld));
+        CK(cudaMalloc(&h->piv, (size_t)N_STAGES * PIV_BYTES * h->ld));
+        CK(cudaMalloc(&h->tcAI, sizeof(float) * (size_t)N_STAGES * NV * NV * h->ld));
+    }
     return ABS_OK;
 }
 
@@ -722,8 +735,8 @@ double RED(const abs_problem* h, int k, int p) { return h->hmap[(size_t)k * h->N
 
 // ---- the KKT machinery (every active problem at once) ----------------------------------
 // factor precision of a KKT system: ABS_PREC_FP64, ABS_PREC_FP32, or mixed -- the FP32
-// stage-block inverses of most scenarios with FP64 LU factors of the scenarios escalated
-// in this iteration (esc flags)
+// factors of most scenarios with FP64 factors of the scenarios escalated in this iteration
+// (esc flags)
 constexpr int ABS_PREC_MIXED = 2;
 
 struct KKTSys {
@@ -735,12 +748,10 @@ struct KKTSys {
     // block LDL^T of every scenario block (FP64, dw = PS_DW, dc = PS_DC) instead of the
     // block LU of J_s
     bool ldl = false;
-    // set before kkt_factor_core: p = J^-1 rc is solved together with q = J^-1 b (one
-    // two-right-hand-side launch) and the first KKT solve with this rc reuses it
+    // set before kkt_factor_core: the factorization also solves p = J^-1 rc and (one design
+    // entry) forms the first solve's right-hand-side sums with this rz (q^T (rz - H p), q^T p;
+    // they do not depend on dw), so that the first KKT solve with them starts from both
     const double* pre_rc = nullptr;
-    // with pre_rc (one design entry): the Schur pass of kkt_factor_core also forms the
-    // right-hand-side sums of the first solve with this rz (q^T (rz - H p), q^T p and
-    // t = rz - H p; they do not depend on dw), so that solve skips its own Schur pass
     const double* pre_rz = nullptr;
     // device flag: when set, kkt_factor_core keeps the stored factors of J (those of the
     // least-squares multiplier estimate at the same point)
@@ -822,159 +833,199 @@ abs_status tuned_launch(abs_problem* h, int kind, int es, std::initializer_list<
     return launch(w);
 }
 
-// factor launch shape: W warps per block.  FP32: stage-block inverses and G by
-// Gauss-Jordan (factor_gj_kernel); FP64: LU factors, row order and G (factor_warp_kernel),
-// of the scenarios with mask[s] != 0 only when mask is given
-template <class T, int W>
-void factor_w(abs_problem* h, const double* jac, double pivtol, const int* mask, cudaStream_t st,
-              const int* skip) {
-    if constexpr (std::is_same<T, float>::value) {
-        if (h->factor_kernel == 1)
-            factor_gj_tc_kernel<W><<<gridw(h, W), 32 * W, 0, st>>>((int)h->S, h->ld, view(h), jac,
-                                                                   (float*)h->LUp[ABS_PREC_FP32], h->piv,
-                                                                   (float*)h->Gp[ABS_PREC_FP32], h->sing, pivtol);
-        else
-            factor_gj_kernel<W><<<gridw(h, W), 32 * W, 0, st>>>((int)h->S, h->ld, view(h), jac,
-                                                                (float*)h->LUp[ABS_PREC_FP32], h->piv,
-                                                                (float*)h->Gp[ABS_PREC_FP32], h->sing, pivtol,
-                                                                skip);
-    }
-    else if constexpr (factor_fits<T, W>())
-        factor_warp_kernel<T, W><<<gridw(h, W), 32 * W, 0, st>>>((int)h->S, h->ld, view(h), jac,
-                                                                (T*)h->LUp[ABS_PREC_FP64], h->piv,
-                                                                (T*)h->Gp[ABS_PREC_FP64], h->sing, pivtol, mask,
-                                                                skip);
+// the chain's launch shape in FP64.  A block of 32 scenarios over four warps keeps an SM's FP64
+// pipe busy; below a block per SM, 4 scenarios per one-warp block spread the same chains over
+// more SMs (measured at 500 scenarios: see chain_kernel)
+constexpr int CHAIN_WIDE_S = 32 * 152;
+
+template <class T, int SPB, int CG>
+abs_status chain_go(abs_problem* h, T* F, double pivtol, const int* mask, cudaStream_t st, const int* skip) {
+    chain_kernel<T, SPB, CG><<<(unsigned)((h->S + SPB - 1) / SPB), SPB * CG, chain_smem(sizeof(T), SPB, CG), st>>>(
+        (int)h->S, h->ld, view(h), F, h->sing, pivtol, mask, skip);
+    return launch_check(h, KD_FACTOR);
 }
 
-// skip (device flag, optional): when set at run time the launch leaves the stored factors
-// as they are (they are those of this Jacobian)
+// condensed factors of J_s (kernels_cond.cuh) in T, of the scenarios with mask[s] != 0 only when
+// mask is given.  skip (device flag, optional): when set at run time the launches leave the stored
+// factors as they are (they are those of this Jacobian).  The FP32 chain has one thread per
+// scenario: W warps per block.
 template <class T>
 abs_status factor_launch(abs_problem* h, const double* jac, double pivtol, cudaStream_t st,
                          const int* mask = nullptr, const int* skip = nullptr) {
+    constexpr bool f32 = std::is_same<T, float>::value;
+    T* F = (T*)h->cond[f32 ? ABS_PREC_FP32 : ABS_PREC_FP64];
     prof_begin(h, K_FACTOR, st);
-    auto go = [&](int w) {
-        switch (w) {
-            case 1: factor_w<T, 1>(h, jac, pivtol, mask, st, skip); break;
-            case 2: factor_w<T, 2>(h, jac, pivtol, mask, st, skip); break;
-            case 8: factor_w<T, 8>(h, jac, pivtol, mask, st, skip); break;
-            default: factor_w<T, 4>(h, jac, pivtol, mask, st, skip); break;
+    condense_kernel<T><<<dim3((unsigned)((h->S + 63) / 64), N_STAGES), 64, 0, st>>>((int)h->S, h->ld, view(h), jac, F,
+                                                                                    mask, skip);
+    abs_status r = launch_check(h, KD_FACTOR);
+    if (r != ABS_OK) return r;
+    if constexpr (f32) {
+        auto go = [&](int w) {
+            switch (w) {
+                case 1: return chain_go<float, 32, 1>(h, F, pivtol, mask, st, skip);
+                case 2: return chain_go<float, 64, 1>(h, F, pivtol, mask, st, skip);
+                case 8: return chain_go<float, 256, 1>(h, F, pivtol, mask, st, skip);
+                default: return chain_go<float, 128, 1>(h, F, pivtol, mask, st, skip);
+            }
+        };
+        if (h->factor_tile != 0) {
+            h->tile[TK_FACTOR] = h->factor_tile;
+            r = go(h->factor_tile);
+        } else {
+            r = tuned_launch(h, TK_FACTOR, sizeof(T), {1, 2, 4, 8}, WPB_F, go, st);
         }
-        return launch_check(h, KD_FACTOR);
-    };
-    abs_status r;
-    if (std::is_same<T, float>::value && h->factor_tile != 0) {
-        h->tile[TK_FACTOR] = h->factor_tile;
-        r = go(h->factor_tile);
-    } else if (std::is_same<T, float>::value)
-        r = tuned_launch(h, TK_FACTOR, h->factor_kernel == 1 ? 5 : (int)sizeof(T), {1, 2, 4, 8}, WPB_F, go, st);
-    else if (mask)
-        r = go(WPB_F);   // the escalation's masked factorization: the default shape
-    else
-        r = factor_fits<T, 8>() ? tuned_launch(h, TK_FACTOR, sizeof(T), {1, 2, 4, 8}, WPB_F, go, st)
-                                : tuned_launch(h, TK_FACTOR, sizeof(T), {1, 2, 4}, WPB_F, go, st);
+    } else {
+        r = h->S >= CHAIN_WIDE_S ? chain_go<double, 32, 4>(h, F, pivtol, mask, st, skip)
+                                 : chain_go<double, 4, 8>(h, F, pivtol, mask, st, skip);
+    }
     prof_end(h, st);
     return r;
 }
 
-template <class T, int NR_, int W>
-void solve_w(abs_problem* h, const double* jac, const double* x, const double* r0, const double* r1, double* o0,
-             double* o1, cudaStream_t st, int bsec) {
-    const int pi = std::is_same<T, float>::value ? ABS_PREC_FP32 : ABS_PREC_FP64;
-    solve_warp_kernel<T, NR_, W, std::is_same<T, float>::value><<<gridw(h, W), 32 * W, 0, st>>>(
-        h->P, (int)h->S, h->ld, view(h), jac, (const T*)h->LUp[pi], h->piv, (const T*)h->Gp[pi], x, r0, r1, o0, o1,
-        bsec);
+CondFac cond_fac(const abs_problem* h) {
+    return CondFac{(const float*)h->cond[ABS_PREC_FP32], (const double*)h->cond[ABS_PREC_FP64], h->esc};
 }
+int cond_prec(int prec) { return prec == ABS_PREC_MIXED ? CP_MIXED : (prec == ABS_PREC_FP32 ? CP_FP32 : CP_FP64); }
+dim3 gridc(const abs_problem* h) { return dim3((unsigned)((h->S + 31) / 32)); }
 
-// bsec: the design entry whose border column a null right-hand side stands for
-template <class T, int NR_>
-abs_status solve_launch(abs_problem* h, const double* jac, const double* x, const double* r0, const double* r1,
-                        double* o0, double* o1, cudaStream_t st, int bsec = 0) {
+// p = J^-1 rc with the condensed factors; planes: the Schur sums that go with it (cond_solve_kernel)
+abs_status solve_p(abs_problem* h, int prec, const KKTSys* K, const double* x, const double* rc, const double* rz,
+                   double* p, int planes, cudaStream_t st) {
     prof_begin(h, K_SOLVE, st);
-    auto go = [&](int w) {
-        switch (w) {
-            case 1: solve_w<T, NR_, 1>(h, jac, x, r0, r1, o0, o1, st, bsec); break;
-            case 2: solve_w<T, NR_, 2>(h, jac, x, r0, r1, o0, o1, st, bsec); break;
-            case 8: solve_w<T, NR_, 8>(h, jac, x, r0, r1, o0, o1, st, bsec); break;
-            default: solve_w<T, NR_, 4>(h, jac, x, r0, r1, o0, o1, st, bsec); break;
-        }
-        return launch_check(h, KD_SOLVE);
-    };
-    abs_status r = tuned_launch(h, NR_ == 1 ? TK_SOLVE1 : TK_SOLVE2, sizeof(T), {1, 2, 4, 8}, WPB_S, go, st);
-    prof_end(h, st);
-    return r;
-}
-
-// mixed factor precision (escalated scenarios FP64, the others FP32), default shape
-template <int NR_>
-abs_status solve_mixed(abs_problem* h, const double* jac, const double* x, const double* r0, const double* r1,
-                       double* o0, double* o1, cudaStream_t st, int bsec = 0) {
-    prof_begin(h, K_SOLVE, st);
-    solve_mixed_kernel<NR_, WPB_S><<<gridw(h, WPB_S), 32 * WPB_S, 0, st>>>(
-        h->P, (int)h->S, h->ld, view(h), jac, (const float*)h->LUp[ABS_PREC_FP32], (const double*)h->LUp[ABS_PREC_FP64],
-        h->piv, (const float*)h->Gp[ABS_PREC_FP32], (const double*)h->Gp[ABS_PREC_FP64], h->esc, x, r0, r1, o0, o1,
-        bsec);
+    const dim3 blk(32, N_STAGES);
+    const size_t sm = cond_smem(prec == ABS_PREC_FP32 ? sizeof(float) : sizeof(double));
+#define CS_GO(PR)                                                                                                  \
+    cond_solve_kernel<PR><<<gridc(h), blk, sm, st>>>(h->P, (int)h->S, h->ld, view(h), cond_fac(h), x, rc, rz,      \
+                                                     K ? K->sig : nullptr, K ? K->hes : nullptr, K && K->use_w,    \
+                                                     h->sing, p, h->part, planes)
+    switch (cond_prec(prec)) {
+        case CP_FP64: CS_GO(CP_FP64); break;
+        case CP_FP32: CS_GO(CP_FP32); break;
+        default: CS_GO(CP_MIXED); break;
+    }
+#undef CS_GO
     prof_end(h, st);
     return launch_check(h, KD_SOLVE);
 }
 
-abs_status solve_j(abs_problem* h, int prec, const double* jac, const double* x, const double* r0, double* o0,
-                   cudaStream_t st, int bsec = 0) {
-    if (prec == ABS_PREC_MIXED) return solve_mixed<1>(h, jac, x, r0, nullptr, o0, nullptr, st, bsec);
-    if (prec == ABS_PREC_FP32) return solve_launch<float, 1>(h, jac, x, r0, nullptr, o0, nullptr, st, bsec);
-    return solve_launch<double, 1>(h, jac, x, r0, nullptr, o0, nullptr, st, bsec);
+// the rest of a solve after solve_p (p in V_P, the design entries' steps in dz's slots): the
+// direction (dz, dl), or with az, al a correction added to it, and with res the KKT residual
+abs_status solve_direction(abs_problem* h, const KKTSys& K, const double* x, const double* rz, double* dz, double* dl,
+                           double* az, double* al, bool res, const double* rz0, const double* rc0, cudaStream_t st) {
+    prof_begin(h, K_SOLVE_T, st);
+    const dim3 blk(32, N_STAGES);
+    const size_t sm = cond_smem(K.prec == ABS_PREC_FP32 ? sizeof(float) : sizeof(double));
+#define CD_GO(PR)                                                                                                   \
+    cond_direction_kernel<PR><<<gridc(h), blk, sm, st>>>(h->P, (int)h->S, h->ld, view(h), cond_fac(h), K.jac, K.hes, \
+                                                         K.sig, K.use_w, x, V(h, V_P), rz, dz, dl, az, al, res, rz0, \
+                                                         rc0, V(h, V_RHOZ), V(h, V_RHOC), h->part)
+    switch (cond_prec(K.prec)) {
+        case CP_FP64: CD_GO(CP_FP64); break;
+        case CP_FP32: CD_GO(CP_FP32); break;
+        default: CD_GO(CP_MIXED); break;
+    }
+#undef CD_GO
+    prof_end(h, st);
+    return launch_check(h, KD_SOLVE_T);
 }
 
-// two right-hand sides in one launch (a null r means b = dc/dd)
-abs_status solve_j2(abs_problem* h, int prec, const double* jac, const double* x, const double* r0, const double* r1,
-                    double* o0, double* o1, cudaStream_t st) {
-    if (prec == ABS_PREC_MIXED) return solve_mixed<2>(h, jac, x, r0, r1, o0, o1, st);
-    if (prec == ABS_PREC_FP32) return solve_launch<float, 2>(h, jac, x, r0, r1, o0, o1, st);
-    return solve_launch<double, 2>(h, jac, x, r0, r1, o0, o1, st);
-}
-
-template <class T, int W>
-void solve_t_w(abs_problem* h, const double* jac, const double* g, double* out, cudaStream_t st) {
-    const int pi = std::is_same<T, float>::value ? ABS_PREC_FP32 : ABS_PREC_FP64;
-    solve_t_warp_kernel<T, W, std::is_same<T, float>::value><<<gridw(h, W), 32 * W, 0, st>>>(
-        (int)h->S, h->ld, view(h), jac, (const T*)h->LUp[pi], h->piv, (const T*)h->Gp[pi], g, out);
-}
-
-template <class T>
-abs_status solve_jt_t(abs_problem* h, const double* jac, const double* g, double* out, cudaStream_t st) {
+// ---- the tensor-core FP32 factor (options.factor_kernel = 1): stage-block inverses and their
+// block solves, W warps (scenarios) per block
+abs_status tc_factor(abs_problem* h, const double* jac, double pivtol, cudaStream_t st) {
+    prof_begin(h, K_FACTOR, st);
+#define TC_GO(W)                                                                                                     \
+    factor_gj_tc_kernel<W><<<gridw(h, W), 32 * W, 0, st>>>((int)h->S, h->ld, view(h), jac, h->tcAI, h->piv, h->tcG, \
+                                                           h->sing, pivtol)
     auto go = [&](int w) {
         switch (w) {
-            case 1: solve_t_w<T, 1>(h, jac, g, out, st); break;
-            case 2: solve_t_w<T, 2>(h, jac, g, out, st); break;
-            case 8: solve_t_w<T, 8>(h, jac, g, out, st); break;
-            default: solve_t_w<T, 4>(h, jac, g, out, st); break;
+            case 1: TC_GO(1); break;
+            case 2: TC_GO(2); break;
+            case 8: TC_GO(8); break;
+            default: TC_GO(4); break;
         }
-        return launch_check(h, KD_SOLVE_T);
+        return launch_check(h, KD_FACTOR);
     };
-    return tuned_launch(h, TK_SOLVE_T, sizeof(T), {1, 2, 4, 8}, WPB_S, go, st);
-}
-
-abs_status solve_jt(abs_problem* h, int prec, const double* jac, const double* g, double* out, cudaStream_t st) {
-    prof_begin(h, K_SOLVE_T, st);
+#undef TC_GO
     abs_status r;
-    if (prec == ABS_PREC_MIXED) {
-        solve_t_mixed_kernel<WPB_S><<<gridw(h, WPB_S), 32 * WPB_S, 0, st>>>(
-            (int)h->S, h->ld, view(h), jac, (const float*)h->LUp[ABS_PREC_FP32], (const double*)h->LUp[ABS_PREC_FP64],
-            h->piv, (const float*)h->Gp[ABS_PREC_FP32], (const double*)h->Gp[ABS_PREC_FP64], h->esc, g, out);
-        r = launch_check(h, KD_SOLVE_T);
+    if (h->factor_tile != 0) {
+        h->tile[TK_FACTOR] = h->factor_tile;
+        r = go(h->factor_tile);
     } else {
-        r = prec == ABS_PREC_FP32 ? solve_jt_t<float>(h, jac, g, out, st) : solve_jt_t<double>(h, jac, g, out, st);
+        r = tuned_launch(h, TK_FACTOR, 5, {1, 2, 4, 8}, WPB_F, go, st);
     }
     prof_end(h, st);
     return r;
 }
 
-// factor every active problem's J_s, q = J^-1 b (with p = J^-1 pre_rc when set) and the
-// Schur sums into h->red per problem: [0] A0 = sum q^T (W + Sigma) q, [1] Q2 = sum q^T q,
-// [4] the d-d Hessian entries, [5] singular stage blocks (fetch: also to the host, RED).
-// Mixed precision: FP64 factors of the escalated scenarios only (the others keep their
-// FP32 inverses).  x: primal vector whose d slots hold the problems' d.
+// J x = r with them (NR_ right-hand sides; a null one means b = dc/dtheta of design entry bsec)
+template <int NR_>
+abs_status tc_solve(abs_problem* h, const double* jac, const double* x, const double* r0, const double* r1, double* o0,
+                    double* o1, cudaStream_t st, int bsec = 0) {
+    prof_begin(h, K_SOLVE, st);
+#define TC_GO(W)                                                                                                  \
+    solve_warp_kernel<NR_, W><<<gridw(h, W), 32 * W, 0, st>>>(h->P, (int)h->S, h->ld, view(h), jac, h->tcAI, h->piv, \
+                                                              h->tcG, x, r0, r1, o0, o1, bsec)
+    auto go = [&](int w) {
+        switch (w) {
+            case 1: TC_GO(1); break;
+            case 2: TC_GO(2); break;
+            case 8: TC_GO(8); break;
+            default: TC_GO(4); break;
+        }
+        return launch_check(h, KD_SOLVE);
+    };
+#undef TC_GO
+    abs_status r = tuned_launch(h, NR_ == 1 ? TK_SOLVE1 : TK_SOLVE2, 4, {1, 2, 4, 8}, WPB_S, go, st);
+    prof_end(h, st);
+    return r;
+}
+
+// J^T v = g with them
+abs_status tc_solve_t(abs_problem* h, const double* jac, const double* g, double* out, cudaStream_t st) {
+    prof_begin(h, K_SOLVE_T, st);
+#define TC_GO(W)                                                                                             \
+    solve_t_warp_kernel<W><<<gridw(h, W), 32 * W, 0, st>>>((int)h->S, h->ld, view(h), jac, h->tcAI, h->piv, \
+                                                           h->tcG, g, out)
+    auto go = [&](int w) {
+        switch (w) {
+            case 1: TC_GO(1); break;
+            case 2: TC_GO(2); break;
+            case 8: TC_GO(8); break;
+            default: TC_GO(4); break;
+        }
+        return launch_check(h, KD_SOLVE_T);
+    };
+#undef TC_GO
+    abs_status r = tuned_launch(h, TK_SOLVE_T, 4, {1, 2, 4, 8}, WPB_S, go, st);
+    prof_end(h, st);
+    return r;
+}
+
+// the tensor-core factor serves plain FP32 systems; mixed ones take the condensed factors
+bool is_tc(const abs_problem* h, const KKTSys& K) { return K.prec == ABS_PREC_FP32 && h->factor_kernel == 1; }
+
+abs_status tc_schur(abs_problem* h, const KKTSys& K, const double* p, const double* rz, const int* sing, int terms,
+                    cudaStream_t st) {
+    double* hq = (terms & SCHUR_DD) ? V(h, V_HQ) : nullptr;
+    double* t = (terms & SCHUR_RHS) ? V(h, V_T) : nullptr;
+    if (h->P.nsec == 2)
+        schur_kernel<true><<<gridq(h), kThr, 0, st>>>((int)h->S, h->ld, view(h), K.hes, K.sig, K.use_w, p, V(h, V_Q),
+                                                       rz, sing, h->part, terms, hq, t, V(h, V_Q1),
+                                                       (terms & SCHUR_DD) ? V(h, V_HQ1) : nullptr);
+    else
+        schur_kernel<false><<<gridq(h), kThr, 0, st>>>((int)h->S, h->ld, view(h), K.hes, K.sig, K.use_w, p, V(h, V_Q),
+                                                        rz, sing, h->part, terms, hq, t);
+    return launch_check(h, KD_SCHUR);
+}
+
+// factor every active problem's J_s and form the Schur sums into h->red per problem: [0] A0 =
+// sum q^T (W + Sigma) q, [1] Q2 = sum q^T q, [4] the d-d Hessian entries, [5] singular stage blocks
+// (fetch: also to the host, RED); q = J^-1 b.  Mixed precision: FP64 factors of the escalated
+// scenarios only (the others keep their FP32 ones).  x: primal vector whose d slots hold the
+// problems' d.
 abs_status kkt_factor_core(abs_problem* h, const KKTSys& K, const double* x, cudaStream_t st, bool fetch) {
     abs_status r;
+    const bool two = h->P.nsec == 2;
     if (K.ldl) {
         // block LDL^T: the pivot inverses and the inertia counts ([2] positive, [3] negative,
         // [6] zero pivots, [5] scenarios with a zero pivot), then u = K_s^-1 [0; b] with
@@ -990,50 +1041,52 @@ abs_status kkt_factor_core(abs_problem* h, const KKTSys& K, const double* x, cud
         if ((r = launch_check(h, KD_SOLVE)) != ABS_OK) return r;
         return reduce(h, st, 7, make_ops({RSUM, RSUM, RSUM, RSUM, RSUM, RSUM, RSUM}), PS_ACT, fetch);
     }
+    // FP64: a pivot below 1e-14 of the core's largest entry marks the stage block singular; FP32:
+    // only (numerically) zero pivots do -- accuracy is guarded by the FP64 refinement instead, with
+    // FP64 escalation where it stalls
     if (K.prec == ABS_PREC_MIXED) {
         if ((r = ensure_factor(h, ABS_PREC_FP64)) != ABS_OK) return r;
-        if ((r = ensure_factor(h, ABS_PREC_FP32)) != ABS_OK) return r;
         r = factor_launch<double>(h, K.jac, 1e-14, st, h->esc);
     } else {
         if ((r = ensure_factor(h, K.prec)) != ABS_OK) return r;
-        // FP64: a pivot below 1e-14 of the block's largest entry marks the stage block
-        // singular; FP32: only (numerically) zero pivots do -- accuracy is guarded by the
-        // FP64 refinement instead, with FP64 escalation where it stalls
         if (K.prec == ABS_PREC_FP32) r = factor_launch<float>(h, K.jac, 1e-30, st, nullptr, K.skip);
         else r = factor_launch<double>(h, K.jac, 1e-14, st, nullptr, K.skip);
     }
     if (r != ABS_OK) return r;
-    r = K.pre_rc ? solve_j2(h, K.prec, K.jac, x, K.pre_rc, nullptr, V(h, V_P), V(h, V_Q), st)
-                 : solve_j(h, K.prec, K.jac, x, nullptr, V(h, V_Q), st);
+    if (is_tc(h, K)) {
+        if ((r = tc_factor(h, K.jac, 1e-30, st)) != ABS_OK) return r;
+        r = K.pre_rc ? tc_solve<2>(h, K.jac, x, K.pre_rc, nullptr, V(h, V_P), V(h, V_Q), st)
+                     : tc_solve<1>(h, K.jac, x, nullptr, nullptr, V(h, V_Q), nullptr, st);
+        if (r != ABS_OK) return r;
+        // a second design entry: q1 = J^-1 b1, b1 the border column of the second section
+        if (two && (r = tc_solve<1>(h, K.jac, x, nullptr, nullptr, V(h, V_Q1), nullptr, st, 1)) != ABS_OK) return r;
+        const bool rhs = K.pre_rc && K.pre_rz && !two;
+        r = tc_schur(h, K, rhs ? V(h, V_P) : nullptr, rhs ? K.pre_rz : nullptr, h->sing,
+                     SCHUR_DD | (rhs ? SCHUR_RHS : 0), st);
+    } else if (K.pre_rc && K.pre_rz && !two) {
+        r = solve_p(h, K.prec, &K, x, K.pre_rc, K.pre_rz, V(h, V_P), 2, st);
+    } else {
+        cond_schur_kernel<<<grid2(h), kThr, 0, st>>>(h->P, (int)h->S, h->ld, view(h), x, K.sig, K.hes, K.use_w, h->sing,
+                                                     h->part);
+        r = launch_check(h, KD_SCHUR);
+    }
     if (r != ABS_OK) return r;
-    // a second design entry: q1 = J^-1 b1, b1 the border column of the second section
-    const bool two = h->P.nsec == 2;
-    if (two && (r = solve_j(h, K.prec, K.jac, x, nullptr, V(h, V_Q1), st, 1)) != ABS_OK) return r;
-    if (two)
-        schur_kernel<true><<<gridq(h), kThr, 0, st>>>((int)h->S, h->ld, view(h), K.hes, K.sig, K.use_w, nullptr,
-                                                       V(h, V_Q), nullptr, h->sing, h->part, SCHUR_DD, V(h, V_HQ),
-                                                       nullptr, V(h, V_Q1), V(h, V_HQ1));
-    else if (K.pre_rc && K.pre_rz)
-        // the matrix sums and the first solve's right-hand-side sums in one pass: planes
-        // [0] q^T H q, [1] q^T q, [2] q^T (rz - H p), [3] q^T p, [4] d-d, [5] singular
-        schur_kernel<false><<<gridq(h), kThr, 0, st>>>((int)h->S, h->ld, view(h), K.hes, K.sig, K.use_w, V(h, V_P),
-                                                        V(h, V_Q), K.pre_rz, h->sing, h->part, SCHUR_DD | SCHUR_RHS,
-                                                        V(h, V_HQ), V(h, V_T));
-    else
-        schur_kernel<false><<<gridq(h), kThr, 0, st>>>((int)h->S, h->ld, view(h), K.hes, K.sig, K.use_w, nullptr,
-                                                        V(h, V_Q), nullptr, h->sing, h->part, SCHUR_DD, V(h, V_HQ),
-                                                        nullptr);
-    if ((r = launch_check(h, KD_SCHUR)) != ABS_OK) return r;
     if (two) return reduce(h, st, 9, make_ops({RSUM, RSUM, RSUM, RSUM, RSUM, RSUM, RSUM, RSUM, RSUM}), PS_ACT, fetch);
     return reduce(h, st, 6, make_ops({RSUM, RSUM, RSUM, RSUM, RSUM, RSUM}), PS_ACT, fetch);
 }
 
-// one Schur-reduced solve for every active problem: rz (z part), rc -> dz (d slots set),
-// dl.  PS_RD, PS_SD, PS_DW must be on the device.  No host round trip.  have_p: V_P
-// already holds J^-1 rc (solved with q in kkt_factor_core).
+// one Schur-reduced solve for every active problem: rz (z part), rc -> dz (d slots set), dl;
+// with az, al a correction added to that direction; with res the residual of the whole direction
+// against (rz0, rc0) into V_RHOZ, V_RHOC and the partials.  PS_RD, PS_SD, PS_DW must be on the
+// device.  No host round trip.  have_p: kkt_factor_core already solved p = J^-1 rc.
 abs_status kkt_solve_launches(abs_problem* h, const KKTSys& K, const double* x, const double* rz, const double* rc,
-                              double* dz, double* dl, cudaStream_t st, bool have_p = false) {
+                              double* dz, double* dl, cudaStream_t st, bool have_p = false, double* az = nullptr,
+                              double* al = nullptr, bool res = false, const double* rz0 = nullptr,
+                              const double* rc0 = nullptr) {
     abs_status r;
+    const int nsec = h->P.nsec;
+    const bool two = nsec == 2, tc = is_tc(h, K);
+    const double* dlast = dl;
     if (K.ldl) {
         // v = K_s^-1 [rz; rc] into dz, dl with [2] b^T v_l ([3] zero), dd, then x = v - u dd
         ldl_solve_kernel<<<(unsigned)h->S, 32, LDL_SOLVE_SMEM, st>>>((int)h->S, h->ld, view(h), K.jac, h->ldl_inv,
@@ -1045,33 +1098,45 @@ abs_status kkt_solve_launches(abs_problem* h, const KKTSys& K, const double* x, 
         if ((r = launch_check(h, KD_VEC)) != ABS_OK) return r;
         ldl_back_kernel<<<dim3((unsigned)((h->S + 127) / 128), N_STAGES), 128, 0, st>>>((int)h->S, h->ld, view(h),
                                                                                        V(h, V_Q), V(h, V_QL), dz, dl);
-        return launch_check(h, KD_DZ);
+        if ((r = launch_check(h, KD_DZ)) != ABS_OK) return r;
+    } else {
+        // kkt_factor_core formed this solve's sums with its p (h->red [2], [3])
+        const bool sums_ready = have_p && !two && K.pre_rc == rc && K.pre_rz == rz;
+        if (!sums_ready) {
+            if (tc) {
+                if (!have_p && (r = tc_solve<1>(h, K.jac, x, rc, nullptr, V(h, V_P), nullptr, st)) != ABS_OK) return r;
+                r = tc_schur(h, K, V(h, V_P), rz, nullptr, SCHUR_RHS, st);
+            } else {
+                r = solve_p(h, K.prec, &K, x, rc, rz, V(h, V_P), 1, st);
+            }
+            if (r != ABS_OK) return r;
+            if ((r = reduce(h, st, 4, make_ops({RSUM, RSUM, RSUM, RSUM}), PS_ACT, false)) != ABS_OK) return r;
+        }
+        finalize_dd_kernel<<<(unsigned)((h->NP + 127) / 128), 128, 0, st>>>(h->ld, view(h), h->red, dz, nsec);
+        if ((r = launch_check(h, KD_VEC)) != ABS_OK) return r;
+        if (!tc) return solve_direction(h, K, x, rz, dz, dl, az, al, res, rz0, rc0, st);
+        dz_fast_kernel<<<gride(h), kThr, 0, st>>>((int)h->S, h->ld, view(h), V(h, V_P), V(h, V_Q), V(h, V_T),
+                                                  V(h, V_HQ), dz, V(h, V_G), two ? V(h, V_Q1) : nullptr,
+                                                  two ? V(h, V_HQ1) : nullptr);
+        if ((r = launch_check(h, KD_DZ)) != ABS_OK) return r;
+        if ((r = tc_solve_t(h, K.jac, V(h, V_G), dl, st)) != ABS_OK) return r;
     }
-    if (!have_p && (r = solve_j(h, K.prec, K.jac, x, rc, V(h, V_P), st)) != ABS_OK) return r;
-    const bool two = h->P.nsec == 2;
-    // the Schur pass of kkt_factor_core already formed this solve's sums (h->red [2], [3])
-    const bool sums_ready = have_p && !two && K.pre_rc == rc && K.pre_rz == rz;
-    if (sums_ready) {
-        // nothing: t, hq and the reduced sums are in place
-    } else if (two)
-        schur_kernel<true><<<gridq(h), kThr, 0, st>>>((int)h->S, h->ld, view(h), K.hes, K.sig, K.use_w, V(h, V_P),
-                                                       V(h, V_Q), rz, nullptr, h->part, SCHUR_RHS, nullptr, V(h, V_T),
-                                                       V(h, V_Q1), nullptr);
+    if (az) {   // (ctl_refine adds the design entries' steps)
+        axpy2_kernel<<<gride(h), kThr, 0, st>>>((int)h->S, h->ld, view(h), dz, az, dl, al);
+        if ((r = launch_check(h, KD_VEC)) != ABS_OK) return r;
+    }
+    if (!res) return ABS_OK;
+    const double* zt = az ? az : dz;
+    const double* lt = al ? al : dl;
+    if (K.ldl)
+        kkt_residual_reg_kernel<<<dim3((unsigned)((h->S + 127) / 128), N_STAGES), 128, 0, st>>>(
+            (int)h->S, h->ld, view(h), K.jac, K.hes, K.sig, K.use_w, zt, lt, az ? dz : nullptr, rz0, rc0, V(h, V_RHOZ),
+            V(h, V_RHOC), h->part);
     else
-        schur_kernel<false><<<gridq(h), kThr, 0, st>>>((int)h->S, h->ld, view(h), K.hes, K.sig, K.use_w, V(h, V_P),
-                                                        V(h, V_Q), rz, nullptr, h->part, SCHUR_RHS, nullptr,
-                                                        V(h, V_T));
-    if (!sums_ready) {
-        if ((r = launch_check(h, KD_SCHUR)) != ABS_OK) return r;
-        if ((r = reduce(h, st, 4, make_ops({RSUM, RSUM, RSUM, RSUM}), PS_ACT, false)) != ABS_OK) return r;
-    }
-    finalize_dd_kernel<<<(unsigned)((h->NP + 127) / 128), 128, 0, st>>>(h->ld, view(h), h->red, dz, h->P.nsec);
-    if ((r = launch_check(h, KD_VEC)) != ABS_OK) return r;
-    dz_fast_kernel<<<gride(h), kThr, 0, st>>>((int)h->S, h->ld, view(h), V(h, V_P), V(h, V_Q), V(h, V_T),
-                                              V(h, V_HQ), dz, V(h, V_G), two ? V(h, V_Q1) : nullptr,
-                                              two ? V(h, V_HQ1) : nullptr);
-    if ((r = launch_check(h, KD_DZ)) != ABS_OK) return r;
-    return solve_jt(h, K.prec, K.jac, V(h, V_G), dl, st);
+        kkt_residual_kernel<<<gridq(h), kThr, 0, st>>>((int)h->S, h->ld, view(h), K.jac, V(h, V_G), dlast, zt, lt,
+                                                        az ? dz : nullptr, rz0, rc0, V(h, V_RHOZ), V(h, V_RHOC),
+                                                        h->part, nsec);
+    return launch_check(h, KD_RESIDUAL);
 }
 
 // the paper's layout (Section "Numerical results"): [d, z_1 .. z_S], z_s = per stage x
@@ -1291,10 +1356,9 @@ void absorber_destroy(abs_problem* h) {
     cudaFree(h->hes);
     cudaFree(h->vec);
     cudaFree(h->ldl_inv);
-    for (int k = 0; k < 2; ++k) {
-        cudaFree(h->LUp[k]);
-        cudaFree(h->Gp[k]);
-    }
+    for (int k = 0; k < 2; ++k) cudaFree(h->cond[k]);
+    cudaFree(h->tcAI);
+    cudaFree(h->tcG);
     cudaFree(h->piv);
     cudaFree(h->sing);
     cudaFree(h->part);
@@ -1489,7 +1553,7 @@ extern "C" abs_status abs_measure_fma_peak(int kind, double* gflops) {
 // ======================================================================================
 // For callers that cannot allocate device memory after start-up -- code running under
 // a fixed memory budget, inside another runtime's allocator, or between graph
-// captures -- this entry runs the FP64 stage-block LU, the Schur step on d and the
+// captures -- this entry runs the FP64 condensed factorization, the Schur step on d and the
 // block solves with every intermediate in one file-scope device array.  Nothing in the
 // array has to start at zero: every word a call reads was written earlier in that call
 // (the factor kernel writes every scenario's singular flag; every live (scenario,
@@ -1498,15 +1562,13 @@ namespace {
 
 constexpr int64_t NA_MAX_S = ABS_NOALLOC_MAX_SCENARIOS;    // scenarios per call, at most
 constexpr int64_t NA_LD = NA_MAX_S;                         // a multiple of 32
-constexpr size_t NA_LU = (size_t)N_STAGES * NV * NV * NA_LD;
-constexpr size_t NA_G = (size_t)N_STAGES * NV * NABV * NA_LD;
+constexpr size_t NA_FAC = (size_t)N_STAGES * CF_COUNT * NA_LD;
 constexpr size_t NA_VEC = (size_t)NSC * NA_LD + NA_LD;
 constexpr int NA_K = 6;                                     // Schur partial planes
 constexpr size_t NA_PART = (size_t)NA_K * N_STAGES * NA_LD;
-constexpr size_t NA_PIV = ((size_t)N_STAGES * PIV_BYTES * NA_LD + 7) / 8;   // bytes as doubles
 constexpr size_t NA_SING = (NA_LD + 1) / 2;                         // ints as doubles
 constexpr size_t NA_PS = PS_NFIELDS;                                // one problem's scalars
-constexpr size_t NA_TOTAL = NA_LU + NA_G + 3 * NA_VEC + NA_PART + NA_PIV + NA_SING + NA_PS;
+constexpr size_t NA_TOTAL = NA_FAC + NA_VEC + NA_PART + NA_SING + NA_PS;
 
 // the scratch: every device that loads the library holds it until the process exits
 static __device__ __align__(256) double g_noalloc_scratch[NA_TOTAL];
@@ -1544,21 +1606,15 @@ extern "C" abs_status kkt_newton_noalloc(const abs_params* p, int64_t S, int64_t
         CK(upload_tables(dev));
         g_na_base[dev] = ptr;
     }
-    double* LU = g_na_base[dev];
-    double* G = LU + NA_LU;
-    double* pv = G + NA_G;
-    double* qv = pv + NA_VEC;
-    double* gv = qv + NA_VEC;
-    double* part = gv + NA_VEC;
-    unsigned char* piv = (unsigned char*)(part + NA_PART);
-    int* sing = (int*)((double*)piv + NA_PIV);
+    double* F = g_na_base[dev];
+    double* pv = F + NA_FAC;
+    double* part = pv + NA_VEC;
+    int* sing = (int*)(part + NA_PART);
     double* psd = (double*)sing + NA_SING;
     // the problem's constants (derived fields as absorber_create computes them)
     Params P;
     if (!make_params(p, &P) || P.nsec != 1)
         return fail(nullptr, ABS_ERR_ARG, "kkt_newton_noalloc: scales must be positive, one section");
-    const dim3 g2((unsigned)((S + kThr - 1) / kThr), N_STAGES);
-    const dim3 gq((unsigned)((S + QS_SCEN - 1) / QS_SCEN), N_STAGES);
     const int64_t od = (int64_t)NSC * ld;
     cudaError_t e;
 #define NA_LAUNCHED()                                                                                  \
@@ -1571,15 +1627,17 @@ extern "C" abs_status kkt_newton_noalloc(const abs_params* p, int64_t S, int64_t
     g_na_host_ps[PS_DW] = delta_w;
     CK(cudaMemcpyAsync(psd, g_na_host_ps, sizeof(g_na_host_ps), cudaMemcpyHostToDevice, st));
     const BView bv{nullptr, psd, 1};
-    const dim3 gf((unsigned)((S + WPB_F - 1) / WPB_F)), gs((unsigned)((S + WPB_S - 1) / WPB_S));
-    factor_warp_kernel<double><<<gf, 32 * WPB_F, 0, st>>>((int)S, ld, bv, jac_vals, LU, piv, G, sing, 1e-14);
+    const dim3 gs((unsigned)((S + 31) / 32)), blk(32, N_STAGES);
+    const CondFac fac{nullptr, F, nullptr};
+    condense_kernel<double><<<dim3((unsigned)((S + 63) / 64), N_STAGES), 64, 0, st>>>((int)S, ld, bv, jac_vals, F,
+                                                                                      nullptr, nullptr);
     NA_LAUNCHED();
-    // p = J^-1 r_c, q = J^-1 b
-    solve_warp_kernel<double, 2><<<gs, 32 * WPB_S, 0, st>>>(P, (int)S, ld, bv, jac_vals, LU, piv, G, x, rhs_c, nullptr,
-                                                            pv, qv);
+    chain_kernel<double, 4, 8><<<(unsigned)((S + 3) / 4), 32, chain_smem(sizeof(double), 4, 8), st>>>(
+        (int)S, ld, bv, F, sing, 1e-14, nullptr, nullptr);
     NA_LAUNCHED();
-    schur_kernel<false><<<gq, kThr, 0, st>>>((int)S, ld, bv, hess_vals, sigma, true, pv, qv, rhs_x, sing, part,
-                                      SCHUR_DD | SCHUR_RHS, nullptr, nullptr);
+    // p = J^-1 r_c and the Schur sums
+    cond_solve_kernel<CP_FP64><<<gs, blk, cond_smem(sizeof(double)), st>>>(P, (int)S, ld, bv, fac, x, rhs_c, rhs_x, sigma,
+                                                                           hess_vals, true, sing, pv, part, 2);
     NA_LAUNCHED();
     double hx[2] = {0.0, 0.0};   // Sigma_dd and r_d
     const int64_t plane = (int64_t)N_STAGES * ld;
@@ -1603,9 +1661,9 @@ extern "C" abs_status kkt_newton_noalloc(const abs_params* p, int64_t S, int64_t
     const double beta = red[2] - delta_w * red[3];
     const double dd = (hx[1] - beta) / Sd;
     CK(cudaMemcpyAsync(sol_x + od, &dd, sizeof(double), cudaMemcpyHostToDevice, st));
-    dz_kernel<<<gq, kThr, 0, st>>>((int)S, ld, bv, hess_vals, sigma, true, pv, qv, rhs_x, sol_x, gv);
-    NA_LAUNCHED();
-    solve_t_warp_kernel<double><<<gs, 32 * WPB_S, 0, st>>>((int)S, ld, bv, jac_vals, LU, piv, G, gv, sol_c);
+    cond_direction_kernel<CP_FP64><<<gs, blk, cond_smem(sizeof(double)), st>>>(
+        P, (int)S, ld, bv, fac, jac_vals, hess_vals, sigma, true, x, pv, rhs_x, sol_x, sol_c, nullptr, nullptr, false,
+        nullptr, nullptr, nullptr, nullptr, nullptr);
     NA_LAUNCHED();
 #undef NA_LAUNCHED
     // dd lives on this stack frame until the copy above has completed

@@ -492,6 +492,7 @@ __global__ void __launch_bounds__(128) kkt_residual_reg_kernel(int S, int64_t ld
                                                                const double* __restrict__ sig, bool use_w,
                                                                const double* __restrict__ dz,
                                                                const double* __restrict__ dl,
+                                                               const double* __restrict__ cz,
                                                                const double* __restrict__ rz,
                                                                const double* __restrict__ rc, double* __restrict__ rhoz,
                                                                double* __restrict__ rhoc, double* part) {
@@ -501,7 +502,7 @@ __global__ void __launch_bounds__(128) kkt_residual_reg_kernel(int S, int64_t ld
     if (p < 0) return;
     const double dw = b.ps ? psv(b, PS_DW, p) : 0.0;
     const double dc = b.ps ? psv(b, PS_DC, p) : 0.0;
-    const double dd = dz[(int64_t)NSC * ld + p];
+    const double dd = dz[(int64_t)NSC * ld + p] + (cz ? cz[(int64_t)NSC * ld + p] : 0.0);
     double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     for (int j = 0; j < NV; ++j) {
         const int64_t oz = (int64_t)(NV * n + j) * ld + s, ol = (int64_t)(NR * n + j) * ld + s;

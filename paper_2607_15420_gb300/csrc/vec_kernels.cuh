@@ -227,34 +227,6 @@ __global__ void __launch_bounds__(128) schur_kernel(int S, int64_t ld, const BVi
     }
 }
 
-// dz = p - q dd ;  g = r - (W + Sigma + dw I) dz ;  dd, dw of the slot's problem.
-// QS threads per (scenario, stage); each writes its unknowns of dz, then (after the
-// block's writes) its entries of g, which read the whole stage's dz.
-__global__ void __launch_bounds__(128) dz_kernel(int S, int64_t ld, const BView b, const double* __restrict__ hes,
-                                                 const double* __restrict__ sig, bool use_w,
-                                                 const double* __restrict__ p, const double* __restrict__ q,
-                                                 const double* __restrict__ r, double* dz, double* __restrict__ g) {
-    const int gq = threadIdx.x >> 5;
-    const int s = blockIdx.x * QS_SCEN + (threadIdx.x & 31);
-    const int n = blockIdx.y;
-    const int pr = live_prob(b, s, S, PS_ACT);
-    const bool live = pr >= 0;
-    if (live) {
-        const double dd = dz[(int64_t)NSC * ld + pr];
-        for (int j = gq; j < NV; j += QS) {
-            const int64_t o = (int64_t)(NV * n + j) * ld + s;
-            dz[o] = p[o] - q[o] * dd;
-        }
-    }
-    __syncthreads();   // the block's dz entries are visible to all its threads below
-    if (!live) return;
-    const double dw = b.ps ? psv(b, PS_DW, pr) : 0.0;
-    for (int j = gq; j < NV; j += QS) {
-        const int64_t o = (int64_t)(NV * n + j) * ld + s;
-        g[o] = r[o] - hv_one(ld, hes, sig, dw, use_w, dz, s, n, j);
-    }
-}
-
 // dz = p - q dd and g = r - (H + dw I) dz from the Schur pass's vectors t = r - H p and
 // hq = H q (H = W + Sigma): g = t - dw p + dd (hq + dw q), no product with H; with a
 // second design entry also - q1 dd1 and + dd1 (hq1 + dw q1).  Elementwise.
@@ -287,12 +259,14 @@ __global__ void __launch_bounds__(128) dz_fast_kernel(int S, int64_t ld, const B
 // last correction), rho_z = g - J^T dl' (r' is r_z or the previous residual, so this is
 // r_z - H dz - J^T dl for the accumulated dz, dl without forming H dz again).
 // partials: [0] max|rho_z|, [1] max|rho_c|, [2] the stage's hydraulic dl, [3] max|r_z|,
-// [4] max|r_c|.  QS threads per (scenario, stage).
+// [4] max|r_c|.  cz (optional): a correction whose design entries are not in dz yet.  QS threads
+// per (scenario, stage).
 __global__ void __launch_bounds__(128) kkt_residual_kernel(int S, int64_t ld, const BView b,
                                                            const double* __restrict__ jac,
                                                            const double* __restrict__ g,
                                                            const double* __restrict__ dlast,
                                                            const double* __restrict__ dz, const double* __restrict__ dl,
+                                                           const double* __restrict__ cz,
                                                            const double* __restrict__ rz, const double* __restrict__ rc,
                                                            double* __restrict__ rhoz, double* __restrict__ rhoc,
                                                            double* part, int nsec = 1) {
@@ -305,7 +279,8 @@ __global__ void __launch_bounds__(128) kkt_residual_kernel(int S, int64_t ld, co
     const int sec = stage_sec(n, nsec);
     double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     if (live) {
-        const double dd = dz[(int64_t)NSC * ld + (int64_t)sec * b.NP + pr];   // the stage's section
+        const int64_t od = (int64_t)NSC * ld + (int64_t)sec * b.NP + pr;   // the stage's section
+        const double dd = dz[od] + (cz ? cz[od] : 0.0);
         bool bad = false;
         for (int j = gq; j < NV; j += QS) {
             const int64_t o = (int64_t)(NV * n + j) * ld + s;
@@ -591,15 +566,11 @@ __global__ void axpby_kernel(int S, int64_t ld, const BView b, int flag, int afi
     }
 }
 
-// y1 += x1 (per-scenario part and the problems' design slots) and y2 += x2 (per-scenario
-// part).  Elementwise.
+// y1 += x1 and y2 += x2 (per-scenario parts).  Elementwise.
 __global__ void __launch_bounds__(128) axpy2_kernel(int S, int64_t ld, const BView b, const double* __restrict__ x1,
                                                     double* __restrict__ y1, const double* __restrict__ x2,
-                                                    double* __restrict__ y2, int nsec = 1) {
+                                                    double* __restrict__ y2) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (blockIdx.y == 0 && s < b.NP && (!b.ps || psv(b, PS_ACT, s) != 0.0))
-        for (int k = 0; k < nsec; ++k)
-            y1[(int64_t)NSC * ld + (int64_t)k * b.NP + s] += x1[(int64_t)NSC * ld + (int64_t)k * b.NP + s];
     if (live_prob(b, s, S, PS_ACT) < 0) return;
     const int64_t o = (int64_t)blockIdx.y * ld + s;
     y1[o] += x1[o];
