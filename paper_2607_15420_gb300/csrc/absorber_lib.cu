@@ -339,15 +339,6 @@ cudaError_t upload_tables(int dev) {
         UP(g_lt, lt);
     }
 #undef UP
-    // the solve kernels' dynamic shared memory (per device, before any launch of them)
-    const int s64 = (int)cond_smem(sizeof(double)), s32 = (int)cond_smem(sizeof(float));
-    const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if ((e = cudaFuncSetAttribute(cond_solve_kernel<CP_FP64>, a, s64)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(cond_solve_kernel<CP_FP32>, a, s32)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(cond_solve_kernel<CP_MIXED>, a, s64)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(cond_direction_kernel<CP_FP64>, a, s64)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(cond_direction_kernel<CP_FP32>, a, s32)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(cond_direction_kernel<CP_MIXED>, a, s64)) != cudaSuccess) return e;
     g_uploaded[dev] = true;
     return cudaSuccess;
 }
@@ -833,10 +824,9 @@ abs_status tuned_launch(abs_problem* h, int kind, int es, std::initializer_list<
     return launch(w);
 }
 
-// the chain's launch shape in FP64.  A block of 32 scenarios over four warps keeps an SM's FP64
-// pipe busy; below a block per SM, 4 scenarios per one-warp block spread the same chains over
-// more SMs (measured at 500 scenarios: see chain_kernel)
-constexpr int CHAIN_WIDE_S = 32 * 152;
+// the FP64 chain's launch shape: one-warp blocks of 4 scenarios x 8 threads while they leave a
+// scheduler each (the shorter chain), of 8 x 4 above (fewer instructions per scenario)
+constexpr int CHAIN_WIDE_S = 4 * 4 * 152;
 
 template <class T, int SPB, int CG>
 abs_status chain_go(abs_problem* h, T* F, double pivtol, const int* mask, cudaStream_t st, const int* skip) {
@@ -847,8 +837,8 @@ abs_status chain_go(abs_problem* h, T* F, double pivtol, const int* mask, cudaSt
 
 // condensed factors of J_s (kernels_cond.cuh) in T, of the scenarios with mask[s] != 0 only when
 // mask is given.  skip (device flag, optional): when set at run time the launches leave the stored
-// factors as they are (they are those of this Jacobian).  The FP32 chain has one thread per
-// scenario: W warps per block.
+// factors as they are (they are those of this Jacobian).  The FP32 chain has four threads
+// per scenario: W warps per block.
 template <class T>
 abs_status factor_launch(abs_problem* h, const double* jac, double pivtol, cudaStream_t st,
                          const int* mask = nullptr, const int* skip = nullptr) {
@@ -862,10 +852,10 @@ abs_status factor_launch(abs_problem* h, const double* jac, double pivtol, cudaS
     if constexpr (f32) {
         auto go = [&](int w) {
             switch (w) {
-                case 1: return chain_go<float, 32, 1>(h, F, pivtol, mask, st, skip);
-                case 2: return chain_go<float, 64, 1>(h, F, pivtol, mask, st, skip);
-                case 8: return chain_go<float, 256, 1>(h, F, pivtol, mask, st, skip);
-                default: return chain_go<float, 128, 1>(h, F, pivtol, mask, st, skip);
+                case 1: return chain_go<float, 8, 4>(h, F, pivtol, mask, st, skip);
+                case 2: return chain_go<float, 16, 4>(h, F, pivtol, mask, st, skip);
+                case 8: return chain_go<float, 64, 4>(h, F, pivtol, mask, st, skip);
+                default: return chain_go<float, 32, 4>(h, F, pivtol, mask, st, skip);
             }
         };
         if (h->factor_tile != 0) {
@@ -875,7 +865,7 @@ abs_status factor_launch(abs_problem* h, const double* jac, double pivtol, cudaS
             r = tuned_launch(h, TK_FACTOR, sizeof(T), {1, 2, 4, 8}, WPB_F, go, st);
         }
     } else {
-        r = h->S >= CHAIN_WIDE_S ? chain_go<double, 32, 4>(h, F, pivtol, mask, st, skip)
+        r = h->S >= CHAIN_WIDE_S ? chain_go<double, 8, 4>(h, F, pivtol, mask, st, skip)
                                  : chain_go<double, 4, 8>(h, F, pivtol, mask, st, skip);
     }
     prof_end(h, st);
@@ -886,16 +876,15 @@ CondFac cond_fac(const abs_problem* h) {
     return CondFac{(const float*)h->cond[ABS_PREC_FP32], (const double*)h->cond[ABS_PREC_FP64], h->esc};
 }
 int cond_prec(int prec) { return prec == ABS_PREC_MIXED ? CP_MIXED : (prec == ABS_PREC_FP32 ? CP_FP32 : CP_FP64); }
-dim3 gridc(const abs_problem* h) { return dim3((unsigned)((h->S + 31) / 32)); }
+dim3 gridc(const abs_problem* h) { return dim3((unsigned)((h->S + CS_N - 1) / CS_N)); }
 
 // p = J^-1 rc with the condensed factors; planes: the Schur sums that go with it (cond_solve_kernel)
 abs_status solve_p(abs_problem* h, int prec, const KKTSys* K, const double* x, const double* rc, const double* rz,
                    double* p, int planes, cudaStream_t st) {
     prof_begin(h, K_SOLVE, st);
-    const dim3 blk(32, N_STAGES);
     const size_t sm = cond_smem(prec == ABS_PREC_FP32 ? sizeof(float) : sizeof(double));
 #define CS_GO(PR)                                                                                                  \
-    cond_solve_kernel<PR><<<gridc(h), blk, sm, st>>>(h->P, (int)h->S, h->ld, view(h), cond_fac(h), x, rc, rz,      \
+    cond_solve_kernel<PR><<<gridc(h), CS_T, sm, st>>>(h->P, (int)h->S, h->ld, view(h), cond_fac(h), x, rc, rz,      \
                                                      K ? K->sig : nullptr, K ? K->hes : nullptr, K && K->use_w,    \
                                                      h->sing, p, h->part, planes)
     switch (cond_prec(prec)) {
@@ -913,10 +902,9 @@ abs_status solve_p(abs_problem* h, int prec, const KKTSys* K, const double* x, c
 abs_status solve_direction(abs_problem* h, const KKTSys& K, const double* x, const double* rz, double* dz, double* dl,
                            double* az, double* al, bool res, const double* rz0, const double* rc0, cudaStream_t st) {
     prof_begin(h, K_SOLVE_T, st);
-    const dim3 blk(32, N_STAGES);
     const size_t sm = cond_smem(K.prec == ABS_PREC_FP32 ? sizeof(float) : sizeof(double));
 #define CD_GO(PR)                                                                                                   \
-    cond_direction_kernel<PR><<<gridc(h), blk, sm, st>>>(h->P, (int)h->S, h->ld, view(h), cond_fac(h), K.jac, K.hes, \
+    cond_direction_kernel<PR><<<gridc(h), CS_T, sm, st>>>(h->P, (int)h->S, h->ld, view(h), cond_fac(h), K.jac, K.hes, \
                                                          K.sig, K.use_w, x, V(h, V_P), rz, dz, dl, az, al, res, rz0, \
                                                          rc0, V(h, V_RHOZ), V(h, V_RHOC), h->part)
     switch (cond_prec(K.prec)) {
@@ -1627,7 +1615,7 @@ extern "C" abs_status kkt_newton_noalloc(const abs_params* p, int64_t S, int64_t
     g_na_host_ps[PS_DW] = delta_w;
     CK(cudaMemcpyAsync(psd, g_na_host_ps, sizeof(g_na_host_ps), cudaMemcpyHostToDevice, st));
     const BView bv{nullptr, psd, 1};
-    const dim3 gs((unsigned)((S + 31) / 32)), blk(32, N_STAGES);
+    const dim3 gs((unsigned)((S + CS_N - 1) / CS_N));
     const CondFac fac{nullptr, F, nullptr};
     condense_kernel<double><<<dim3((unsigned)((S + 63) / 64), N_STAGES), 64, 0, st>>>((int)S, ld, bv, jac_vals, F,
                                                                                       nullptr, nullptr);
@@ -1636,7 +1624,7 @@ extern "C" abs_status kkt_newton_noalloc(const abs_params* p, int64_t S, int64_t
         (int)S, ld, bv, F, sing, 1e-14, nullptr, nullptr);
     NA_LAUNCHED();
     // p = J^-1 r_c and the Schur sums
-    cond_solve_kernel<CP_FP64><<<gs, blk, cond_smem(sizeof(double)), st>>>(P, (int)S, ld, bv, fac, x, rhs_c, rhs_x, sigma,
+    cond_solve_kernel<CP_FP64><<<gs, CS_T, cond_smem(sizeof(double)), st>>>(P, (int)S, ld, bv, fac, x, rhs_c, rhs_x, sigma,
                                                                            hess_vals, true, sing, pv, part, 2);
     NA_LAUNCHED();
     double hx[2] = {0.0, 0.0};   // Sigma_dd and r_d
@@ -1661,7 +1649,7 @@ extern "C" abs_status kkt_newton_noalloc(const abs_params* p, int64_t S, int64_t
     const double beta = red[2] - delta_w * red[3];
     const double dd = (hx[1] - beta) / Sd;
     CK(cudaMemcpyAsync(sol_x + od, &dd, sizeof(double), cudaMemcpyHostToDevice, st));
-    cond_direction_kernel<CP_FP64><<<gs, blk, cond_smem(sizeof(double)), st>>>(
+    cond_direction_kernel<CP_FP64><<<gs, CS_T, cond_smem(sizeof(double)), st>>>(
         P, (int)S, ld, bv, fac, jac_vals, hess_vals, sigma, true, x, pv, rhs_x, sol_x, sol_c, nullptr, nullptr, false,
         nullptr, nullptr, nullptr, nullptr, nullptr);
     NA_LAUNCHED();

@@ -585,10 +585,9 @@ __host__ __device__ constexpr size_t chain_smem(size_t es, int spb, int cg) {
 // in-place Gauss-Jordan with partial pivoting, then K, D, T.  SPB scenarios per block, CG
 // threads per scenario, thread (scenario i, group g) at threadIdx.x = g SPB + i holding the
 // core's columns g, g + CG, ... in registers; a step's pivot column travels through shared
-// memory (one barrier per step, two buffers).  FP64: a multiply-add occupies one of an SM's
-// four schedulers for 64 cycles, so the columns of 32 scenarios are spread over four warps, and
-// for few scenarios over blocks on more SMs (chain_launch).  FP32 runs on latency: CG = 1, all
-// seven columns in one thread, no shared memory.
+// memory (one barrier per step, two buffers).  The chain is ten dependent inverses of seven
+// dependent steps: latency bounds it, FP64's (64 cycles per multiply-add and warp) most of all, so a
+// scenario's columns are spread over lanes and small blocks over all SMs.
 template <class T, int SPB, int CG>
 __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, const BView b, T* F, int* __restrict__ sing,
                                                          double pivtol, const int* __restrict__ mask,
@@ -679,19 +678,16 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
 #pragma unroll
                 for (int r = k + 1; r < NCORE; ++r) {
                     const unsigned v = core_key(c[r]);
-                    if (v > best) {
-                        best = v;
-                        p = r;
-                    }
+                    p = v > best ? r : p;
+                    best = max(v, best);
                 }
                 T pv = c[k];
 #pragma unroll
-                for (int r = k + 1; r < NCORE; ++r)
-                    if (p == r) {
-                        const T x = c[r];
-                        c[r] = pv;
-                        pv = x;
-                    }
+                for (int r = k + 1; r < NCORE; ++r) {
+                    const T x = c[r];
+                    c[r] = p == r ? pv : x;
+                    pv = p == r ? x : pv;
+                }
                 if (!((pv < T(0) ? -pv : pv) > tiny)) {   // too small, or NaN
                     bad = 1;
                     pv = (pv < T(0) ? T(-1) : T(1)) * (tiny > T(0) ? tiny : T(1));
@@ -718,26 +714,25 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
                     p = sR[(k & 1) * SPB + i];
                 }
             }
+            // rows k and p change places, row k scales by the pivot's reciprocal, the others subtract
+            // their multiple of it; the pivot column itself starts from the unit vector (one code
+            // path for all columns: no divergence inside a warp)
 #pragma unroll
             for (int c = 0; c < NCOL; ++c) {
-                if (own && c == k / CG) {
+                const bool unit = own && c == k / CG;
+                T u = a[c][k];
 #pragma unroll
-                    for (int r = 0; r < NCORE; ++r) a[c][r] = r == k ? piv : -fc[r] * piv;
-                } else {
-                    T u = a[c][k];
-#pragma unroll
-                    for (int r = k + 1; r < NCORE; ++r)
-                        if (p == r) {
-                            const T x = a[c][r];
-                            a[c][r] = u;
-                            u = x;
-                        }
-                    u *= piv;
-#pragma unroll
-                    for (int r = 0; r < NCORE; ++r)
-                        if (r != k) a[c][r] = cond_fma(-fc[r], u, a[c][r]);
-                    a[c][k] = u;
+                for (int r = k + 1; r < NCORE; ++r) {
+                    const T x = a[c][r];
+                    const bool h = p == r && !unit;
+                    a[c][r] = h ? u : x;
+                    u = h ? x : u;
                 }
+                u = (unit ? T(1) : u) * piv;
+#pragma unroll
+                for (int r = 0; r < NCORE; ++r)
+                    if (r != k) a[c][r] = cond_fma(-fc[r], u, unit ? T(0) : a[c][r]);
+                a[c][k] = u;
             }
             const unsigned x = ((orig >> (4 * k)) ^ (orig >> (4 * p))) & 15u;
             orig ^= (x << (4 * k)) | (x << (4 * p));
@@ -795,83 +790,110 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
 }
 
 // ---- block solves ----------------------------------------------------------------------------
-// The solve kernels: 32 scenarios (lanes) x 10 stages (warps) per block.  Neighbouring stages
-// exchange through shared memory, the two chains run on the block's first five warps, one
-// link quantity each.
-constexpr int CS_T = 32 * N_STAGES;
-constexpr int CS_LINK = NLINK * NLINK * 32;      // link map of a stage
-constexpr int CS_VEC = NLINK * 32;               // link quantities of a stage
-constexpr int CS_EX = 8 * 32;                    // exchanged values of a stage
+// The solve kernels: 6 scenarios x 10 stages on the 60 first threads of a two-warp block (scenario
+// fastest, so an access covers 48 consecutive bytes of an entry in FP64).  Neighbouring stages
+// exchange through shared memory; the chains run on the 30 first lanes of the first warp, a lane
+// per scenario and link quantity.  Small blocks because FP64 instructions bound these kernels and
+// 5000 scenarios are few: 834 blocks share out evenly over 152 SMs (32 scenarios x 10 stages per
+// block left five SMs with twice the others' work), and ten scenarios already use two SMs.
+constexpr int CS_N = 6;
+constexpr int CS_T = 64;
+constexpr int CS_LINK = NLINK * NLINK * CS_N;    // link map of a stage
+constexpr int CS_VEC = NLINK * CS_N;             // link quantities of a stage
+constexpr int CS_EX = 8 * CS_N;                  // exchanged values of a stage
+static_assert(CS_N * N_STAGES <= CS_T && CS_N * NLINK <= 32, "the block's threads and its chain lanes");
+
+// the thread's place: stage n, scenario slot i of the block, scenario s; the threads past the 60th
+// repeat places of the last stage (same values to the same shared memory, no global stores)
+struct CondPlace {
+    int n, i, s, pr;
+    int64_t o;       // a scenario of the problem arrays (s, or the last one past the end)
+    bool live;
+    __device__ __forceinline__ CondPlace(int S, const BView& b) {
+        const int t = threadIdx.x;
+        const bool slot = t < CS_N * N_STAGES;
+        n = slot ? t / CS_N : N_STAGES - 1;
+        i = slot ? t - n * CS_N : t - CS_N * N_STAGES;
+        s = blockIdx.x * CS_N + i;
+        pr = live_prob(b, s, S, PS_ACT);
+        live = slot && pr >= 0;
+        o = s < S ? s : S - 1;
+    }
+};
 __host__ __device__ constexpr size_t cond_smem(size_t es) {
     return es * (size_t)N_STAGES * (CS_LINK + 2 * CS_VEC + CS_EX);
 }
 
 // v_n += D_n v_prev along the column (UP: prev = n - 1, n = 1..8; else prev = n + 1, n = 8..1), the
-// maps d transposed with TR; warp i < 5 its quantity i.  The maps are in registers before the
-// first step.
+// maps d transposed with TR; the block's first warp, a lane per scenario and quantity.  The maps are
+// in registers before the first step.
 template <class T, bool TR, bool UP>
-__device__ __forceinline__ void link_chain(const T* d, T* v, int lane, int i) {
+__device__ __forceinline__ void link_chain(const T* d, T* v) {
+    if (threadIdx.x >= 32) return;
+    const int q = (int)threadIdx.x / CS_N, i = (int)threadIdx.x - q * CS_N;   // q = 5: idle
+    const int qq = q < NLINK ? q : 0;
     T m[8][NLINK];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         const int n = UP ? k + 1 : 8 - k;
 #pragma unroll
-        for (int j = 0; j < NLINK; ++j) m[k][j] = d[n * CS_LINK + (TR ? j * NLINK + i : i * NLINK + j) * 32 + lane];
+        for (int j = 0; j < NLINK; ++j) m[k][j] = d[n * CS_LINK + (TR ? j * NLINK + qq : qq * NLINK + j) * CS_N + i];
     }
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-        const int n = UP ? k + 1 : 8 - k, pn = UP ? n - 1 : n + 1;
-        T a = v[n * CS_VEC + i * 32 + lane], c = T(0);
-        a = cond_fma(m[k][0], v[pn * CS_VEC + lane], a);
-        c = m[k][1] * v[pn * CS_VEC + 32 + lane];
-        a = cond_fma(m[k][2], v[pn * CS_VEC + 64 + lane], a);
-        c = cond_fma(m[k][3], v[pn * CS_VEC + 96 + lane], c);
-        a = cond_fma(m[k][4], v[pn * CS_VEC + 128 + lane], a);
-        v[n * CS_VEC + i * 32 + lane] = a + c;
-        asm volatile("bar.sync 1, 160;" ::: "memory");   // the five chain warps
+        const int n = UP ? k + 1 : 8 - k;
+        const T* w = v + (UP ? n - 1 : n + 1) * CS_VEC + i;
+        T a = v[n * CS_VEC + qq * CS_N + i], c;
+        a = cond_fma(m[k][0], w[0], a);
+        c = m[k][1] * w[CS_N];
+        a = cond_fma(m[k][2], w[2 * CS_N], a);
+        c = cond_fma(m[k][3], w[3 * CS_N], c);
+        a = cond_fma(m[k][4], w[4 * CS_N], a);
+        if (q < NLINK) v[n * CS_VEC + q * CS_N + i] = a + c;
+        __syncwarp();
     }
 }
 
 template <class T>
 __device__ __forceinline__ void stage_links(const CondRef<const T>& f, int field, T* d, int n, int lane) {
 #pragma unroll
-    for (int e = 0; e < NLINK * NLINK; ++e) d[n * CS_LINK + e * 32 + lane] = f(field + e);
+    for (int e = 0; e < NLINK * NLINK; ++e) d[n * CS_LINK + e * CS_N + lane] = f(field + e);
 }
 
 // u = J^-1 r at the thread's (scenario, stage): every thread of the block takes part (its own
 // values are meaningless where the scenario's factors are not)
 template <class T>
-__device__ __forceinline__ void cond_solve_block(const T* __restrict__ F, int64_t ld, int s, int n, int lane,
+__device__ __forceinline__ void cond_solve_block(const T* __restrict__ F, int64_t ld, int64_t s, int n, int lane,
                                                  const T (&r)[NR], T* sm, T (&u)[NV]) {
     T* sd = sm;
     T* sg = sd + N_STAGES * CS_LINK;
     T* sl = sg + N_STAGES * CS_VEC;
     T* sx = sl + N_STAGES * CS_VEC;
-    const CondRef<const T> f = cond_ref(F, ld, n, (int64_t)s);
+    const CondRef<const T> f = cond_ref(F, ld, n, s);
     stage_links(f, CF_D, sd, n, lane);
     T rc[NCORE], rho[9], lo[4], go[4];
     cond_reduce(f, r, rc, rho, lo, go);
     T* x = sx + n * CS_EX + lane;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        x[32 * k] = lo[k];
-        x[32 * (4 + k)] = go[k];
+        x[CS_N * k] = lo[k];
+        x[CS_N * (4 + k)] = go[k];
     }
     __syncthreads();
     if (n + 1 < N_STAGES) {
         const T* xa = x + CS_EX;
         rc[1] += xa[0];
-        rc[2] += xa[32];
-        rc[3] += xa[64];
-        rc[6] += xa[96];
+        rc[2] += xa[CS_N];
+        rc[3] += xa[2 * CS_N];
+        rc[6] += xa[3 * CS_N];
     }
     if (n > 0) {
         const T* xb = x - CS_EX;
-        rc[1] += xb[128];
-        rc[2] += xb[128];
-        rc[3] += xb[160] - xb[128];
-        rc[4] += xb[192];
-        rc[6] += xb[224];
+        rc[1] += xb[4 * CS_N];
+        rc[2] += xb[4 * CS_N];
+        rc[3] += xb[5 * CS_N] - xb[4 * CS_N];
+        rc[4] += xb[6 * CS_N];
+        rc[6] += xb[7 * CS_N];
     }
     T t[NCORE];
     auto core = [&]() {
@@ -890,20 +912,20 @@ __device__ __forceinline__ void cond_solve_block(const T* __restrict__ F, int64_
 #pragma unroll
         for (int k = 0; k < 6; ++k)
             if (n_has(q, k)) a = cond_fma(f(CF_N + 6 * q + k), t[n_core(k)], a);
-        sg[n * CS_VEC + q * 32 + lane] = a;
+        sg[n * CS_VEC + q * CS_N + lane] = a;
     }
     __syncthreads();
-    if (n < NLINK) link_chain<T, false, true>(sd, sg, lane, n);
+    link_chain<T, false, true>(sd, sg);
     __syncthreads();
     stage_links(f, CF_T, sd, n, lane);
     if (n > 0) {
         const T* g = sg + (n - 1) * CS_VEC + lane;
         rc[1] += g[0];
         rc[2] += g[0];
-        rc[3] += g[32] - g[0];
-        rc[4] += g[64];
-        rc[5] += g[96];
-        rc[6] += g[128];
+        rc[3] += g[CS_N] - g[0];
+        rc[4] += g[2 * CS_N];
+        rc[5] += g[3 * CS_N];
+        rc[6] += g[4 * CS_N];
         core();
     }
 #pragma unroll
@@ -912,16 +934,16 @@ __device__ __forceinline__ void cond_solve_block(const T* __restrict__ F, int64_
 #pragma unroll
         for (int k = 0; k < 5; ++k)
             if (m_has(q, k)) a = cond_fma(f(CF_M + 5 * q + k), t[k], a);
-        sl[n * CS_VEC + q * 32 + lane] = a;
+        sl[n * CS_VEC + q * CS_N + lane] = a;
     }
     __syncthreads();
-    if (n < NLINK) link_chain<T, false, false>(sd, sl, lane, n);
+    link_chain<T, false, false>(sd, sl);
     __syncthreads();
     if (n + 1 < N_STAGES) {
         const T* l = sl + (n + 1) * CS_VEC + lane;
 #pragma unroll
         for (int k = 0; k < NLINK; ++k) {
-            const T lk = l[32 * k];
+            const T lk = l[CS_N * k];
 #pragma unroll
             for (int c = 0; c < NCORE; ++c) t[c] = cond_fma(f(CF_INV + NCORE * c + e_row(k)), lk, t[c]);
         }
@@ -929,48 +951,48 @@ __device__ __forceinline__ void cond_solve_block(const T* __restrict__ F, int64_
     T fl[6], fa[5], vb = T(0);
     cond_expand(f, t, rho, u, fl);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) x[32 * k] = fl[k];
+    for (int k = 0; k < 6; ++k) x[CS_N * k] = fl[k];
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 5; ++k) fa[k] = n + 1 < N_STAGES ? x[CS_EX + 32 * k] : T(0);
-    if (n > 0) vb = x[160 - CS_EX];
+    for (int k = 0; k < 5; ++k) fa[k] = n + 1 < N_STAGES ? x[CS_EX + CS_N * k] : T(0);
+    if (n > 0) vb = x[5 * CS_N - CS_EX];
     cond_extents(f, r, fl, fa, vb, u);
 }
 
 // v = J^-T g likewise
 template <class T>
-__device__ __forceinline__ void cond_solve_t_block(const T* __restrict__ F, int64_t ld, int s, int n, int lane,
+__device__ __forceinline__ void cond_solve_t_block(const T* __restrict__ F, int64_t ld, int64_t s, int n, int lane,
                                                    const T (&g)[NV], T* sm, T (&v)[NR]) {
     T* sd = sm;
     T* sg = sd + N_STAGES * CS_LINK;
     T* sl = sg + N_STAGES * CS_VEC;
     T* sx = sl + N_STAGES * CS_VEC;
-    const CondRef<const T> f = cond_ref(F, ld, n, (int64_t)s);
+    const CondRef<const T> f = cond_ref(F, ld, n, s);
     stage_links(f, CF_T, sd, n, lane);
     T* x = sx + n * CS_EX + lane;
 #pragma unroll
-    for (int k = 0; k < 5; ++k) x[32 * k] = g[LE + k];
+    for (int k = 0; k < 5; ++k) x[CS_N * k] = g[LE + k];
     __syncthreads();
     T eb[5], gc[NCORE], gam[9];
 #pragma unroll
-    for (int k = 0; k < 5; ++k) eb[k] = n > 0 ? x[32 * k - CS_EX] : T(0);
-    cond_reduce_t(f, g, n + 1 < N_STAGES ? x[128 + CS_EX] : T(0), eb, gc, gam);
+    for (int k = 0; k < 5; ++k) eb[k] = n > 0 ? x[CS_N * k - CS_EX] : T(0);
+    cond_reduce_t(f, g, n + 1 < N_STAGES ? x[4 * CS_N + CS_EX] : T(0), eb, gc, gam);
 #pragma unroll
     for (int k = 0; k < NLINK; ++k) {
         T a = f(CF_INV + e_row(k)) * gc[0];
 #pragma unroll
         for (int c = 1; c < NCORE; ++c) a = cond_fma(f(CF_INV + NCORE * c + e_row(k)), gc[c], a);
-        sg[n * CS_VEC + k * 32 + lane] = a;
+        sg[n * CS_VEC + k * CS_N + lane] = a;
     }
     __syncthreads();
-    if (n < NLINK) link_chain<T, true, true>(sd, sg, lane, n);
+    link_chain<T, true, true>(sd, sg);
     __syncthreads();
     stage_links(f, CF_D, sd, n, lane);
     if (n > 0) {
         const T* a = sg + (n - 1) * CS_VEC + lane;
 #pragma unroll
         for (int q = 0; q < NLINK; ++q) {
-            const T aq = a[32 * q];
+            const T aq = a[CS_N * q];
 #pragma unroll
             for (int k = 0; k < 5; ++k)
                 if (m_has(q, k)) gc[k] = cond_fma(f(CF_M + 5 * q + k), aq, gc[k]);
@@ -989,19 +1011,19 @@ __device__ __forceinline__ void cond_solve_t_block(const T* __restrict__ F, int6
     core();
     T* bl = sl + n * CS_VEC + lane;
     bl[0] = (w[1] + w[2]) - w[3];
-    bl[32] = w[3];
-    bl[64] = w[4];
-    bl[96] = w[5];
-    bl[128] = w[6];
+    bl[CS_N] = w[3];
+    bl[2 * CS_N] = w[4];
+    bl[3 * CS_N] = w[5];
+    bl[4 * CS_N] = w[6];
     __syncthreads();
-    if (n < NLINK) link_chain<T, true, false>(sd, sl, lane, n);
+    link_chain<T, true, false>(sd, sl);
     __syncthreads();
     T ba[4] = {T(0), T(0), T(0), T(0)};
     if (n + 1 < N_STAGES) {
         const T* bn = bl + CS_VEC;
 #pragma unroll
         for (int q = 0; q < NLINK; ++q) {
-            const T bq = bn[32 * q];
+            const T bq = bn[CS_N * q];
             if (q != 3) ba[q < 3 ? q : 3] = bq;
 #pragma unroll
             for (int k = 0; k < 6; ++k)
@@ -1010,14 +1032,14 @@ __device__ __forceinline__ void cond_solve_t_block(const T* __restrict__ F, int6
         core();
     }
     x[0] = w[1];
-    x[32] = w[2];
-    x[64] = w[3];
-    x[96] = w[6];
+    x[CS_N] = w[2];
+    x[2 * CS_N] = w[3];
+    x[3 * CS_N] = w[6];
     __syncthreads();
     T dl[4] = {w[1], w[2], w[3], w[6]};
     if (n > 0)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) dl[k] -= x[32 * k - CS_EX];
+        for (int k = 0; k < 4; ++k) dl[k] -= x[CS_N * k - CS_EX];
     const T dg[4] = {((w[1] + w[2]) - w[3]) - ba[0], w[3] - ba[1], w[4] - ba[2], w[6] - ba[3]};
     cond_expand_t(f, g, w, dl, dg, gam, v);
 }
@@ -1034,7 +1056,7 @@ __device__ __forceinline__ double slack_q(const Params& P, const double* x, int6
 // sections), [5] the singular flag, [2], [3] the given right-hand side's sums (or 0)
 __device__ __forceinline__ void store_schur(const Params& P, const double* __restrict__ sig,
                                             const double* __restrict__ hes, bool use_w, const int* __restrict__ sing,
-                                            double qs, double r2, double r3, double* part, int64_t ld, int s, int n) {
+                                            double qs, double r2, double r3, double* part, int64_t ld, int64_t s, int n) {
     const double a = qs * (sig[(int64_t)(NV * n + LS) * ld + s] * qs), q2 = qs * qs;
     const bool top = stage_sec(n, P.nsec) == 1;
     double w[9] = {top ? 0.0 : a, top ? 0.0 : q2, r2, r3, 0.0, 0.0, top ? a : 0.0, top ? q2 : 0.0, 0.0};
@@ -1045,10 +1067,10 @@ __device__ __forceinline__ void store_schur(const Params& P, const double* __res
         }
         if (sing) w[5] = (double)sing[s];
     }
-    if (P.nsec == 2) store_partials<9>(w, part, ld, s, n);
+    if (P.nsec == 2) store_partials<9>(w, part, ld, (int)s, n);
     else {
         const double w6[6] = {w[0], w[1], w[2], w[3], w[4], w[5]};
-        store_partials<6>(w6, part, ld, s, n);
+        store_partials<6>(w6, part, ld, (int)s, n);
     }
 }
 
@@ -1073,21 +1095,21 @@ enum { CP_FP64 = 0, CP_FP32 = 1, CP_MIXED = 2 };
 
 // o = J^-1 r (r, o doubles) in the factors' precision
 template <int PREC>
-__device__ __forceinline__ void cond_solve_prec(const CondFac& K, int64_t ld, int s, int n, int lane, bool live,
+__device__ __forceinline__ void cond_solve_prec(const CondFac& K, int64_t ld, const CondPlace& at,
                                                 const double (&r)[NR], unsigned char* sm, double (&o)[NV]) {
     if constexpr (PREC != CP_FP64) {
         float rf[NR], uf[NV];
 #pragma unroll
         for (int j = 0; j < NR; ++j) rf[j] = (float)r[j];
-        cond_solve_block<float>(K.f32, ld, s, n, lane, rf, (float*)sm, uf);
+        cond_solve_block<float>(K.f32, ld, at.o, at.n, at.i, rf, (float*)sm, uf);
 #pragma unroll
         for (int j = 0; j < NV; ++j) o[j] = (double)uf[j];
     }
     if constexpr (PREC != CP_FP32) {
-        const bool mine = PREC == CP_FP64 || (live && K.esc[s] != 0);
+        const bool mine = PREC == CP_FP64 || (at.live && K.esc[at.s] != 0);
         if (PREC == CP_FP64 || __syncthreads_or(mine)) {
             double u[NV];
-            cond_solve_block<double>(K.f64, ld, s, n, lane, r, (double*)sm, u);
+            cond_solve_block<double>(K.f64, ld, at.o, at.n, at.i, r, (double*)sm, u);
             if (mine)
 #pragma unroll
                 for (int j = 0; j < NV; ++j) o[j] = u[j];
@@ -1095,21 +1117,21 @@ __device__ __forceinline__ void cond_solve_prec(const CondFac& K, int64_t ld, in
     }
 }
 template <int PREC>
-__device__ __forceinline__ void cond_solve_t_prec(const CondFac& K, int64_t ld, int s, int n, int lane, bool live,
+__device__ __forceinline__ void cond_solve_t_prec(const CondFac& K, int64_t ld, const CondPlace& at,
                                                   const double (&g)[NV], unsigned char* sm, double (&o)[NR]) {
     if constexpr (PREC != CP_FP64) {
         float gf[NV], vf[NR];
 #pragma unroll
         for (int j = 0; j < NV; ++j) gf[j] = (float)g[j];
-        cond_solve_t_block<float>(K.f32, ld, s, n, lane, gf, (float*)sm, vf);
+        cond_solve_t_block<float>(K.f32, ld, at.o, at.n, at.i, gf, (float*)sm, vf);
 #pragma unroll
         for (int j = 0; j < NR; ++j) o[j] = (double)vf[j];
     }
     if constexpr (PREC != CP_FP32) {
-        const bool mine = PREC == CP_FP64 || (live && K.esc[s] != 0);
+        const bool mine = PREC == CP_FP64 || (at.live && K.esc[at.s] != 0);
         if (PREC == CP_FP64 || __syncthreads_or(mine)) {
             double v[NR];
-            cond_solve_t_block<double>(K.f64, ld, s, n, lane, g, (double*)sm, v);
+            cond_solve_t_block<double>(K.f64, ld, at.o, at.n, at.i, g, (double*)sm, v);
             if (mine)
 #pragma unroll
                 for (int j = 0; j < NR; ++j) o[j] = v[j];
@@ -1120,9 +1142,9 @@ __device__ __forceinline__ void cond_solve_t_prec(const CondFac& K, int64_t ld, 
 // p = J^-1 r_c, and with planes the Schur sums of the right-hand side (r_z, r_c): 1 -- planes [2]
 // q^T (r_z - H p), [3] q^T p of the first section, [0], [1] of the second; 2 (one section) -- the
 // factorization's sums with them (store_schur).  q has slack entries only, H none but Sigma
-// there: no product with H.  Grid ceil(S / 32), block (32, 10).
+// there: no product with H.  Grid ceil(S / CS_N), CS_T threads.
 template <int PREC>
-__global__ void __launch_bounds__(CS_T) cond_solve_kernel(const Params P, int S, int64_t ld, const BView b,
+__global__ void __launch_bounds__(CS_T, 6) cond_solve_kernel(const Params P, int S, int64_t ld, const BView b,
                                                           const CondFac K, const double* x,
                                                           const double* __restrict__ rc, const double* rz,
                                                           const double* __restrict__ sig,
@@ -1130,15 +1152,15 @@ __global__ void __launch_bounds__(CS_T) cond_solve_kernel(const Params P, int S,
                                                           const int* __restrict__ sing, double* __restrict__ po,
                                                           double* part, int planes) {
     extern __shared__ __align__(16) unsigned char cond_sm[];
-    const int lane = threadIdx.x, n = threadIdx.y;
-    const int s = blockIdx.x * 32 + lane;
-    const int pr = live_prob(b, s, S, PS_ACT);
-    const bool live = pr >= 0;
+    const CondPlace at(S, b);
+    const bool live = at.live;
+    const int n = at.n, pr = at.pr;
+    const int64_t s = at.o;
     if (!__syncthreads_or(live)) return;
     double r[NR], u[NV];
 #pragma unroll
     for (int j = 0; j < NR; ++j) r[j] = rc[(int64_t)(NR * n + j) * ld + s];
-    cond_solve_prec<PREC>(K, ld, s, n, lane, live, r, cond_sm, u);
+    cond_solve_prec<PREC>(K, ld, at, r, cond_sm, u);
     if (!live) return;
 #pragma unroll
     for (int j = 0; j < NV; ++j) po[(int64_t)(NV * n + j) * ld + s] = u[j];
@@ -1151,7 +1173,7 @@ __global__ void __launch_bounds__(CS_T) cond_solve_kernel(const Params P, int S,
         store_schur(P, sig, hes, use_w, sing, qs, a, c, part, ld, s, n);
     } else {
         const double w[4] = {sec ? a : 0.0, sec ? c : 0.0, sec ? 0.0 : a, sec ? 0.0 : c};
-        store_partials<4>(w, part, ld, s, n);
+        store_partials<4>(w, part, ld, (int)s, n);
     }
 }
 
@@ -1191,20 +1213,20 @@ __host__ __device__ constexpr bool hes_has(int i, int j) {
 // max|rc0| (two sections: [2] the first's, [5] the second's hydraulic dl).  A block holds its
 // scenarios' whole columns, so nothing leaves it between these steps: the right-hand side and the
 // step stay in registers, every Jacobian entry is read once for both products.  rho_z may be rz.
-// Grid ceil(S / 32), block (32, 10).
+// Grid ceil(S / CS_N), CS_T threads.
 template <int PREC>
-__global__ void __launch_bounds__(CS_T) cond_direction_kernel(
+__global__ void __launch_bounds__(CS_T, 6) cond_direction_kernel(
     const Params P, int S, int64_t ld, const BView b, const CondFac K, const double* __restrict__ jac,
     const double* __restrict__ hes, const double* __restrict__ sig, bool use_w, const double* x,
     const double* __restrict__ pv, const double* rz, double* dzo, double* dlo, double* az, double* al, bool res,
     const double* __restrict__ rz0, const double* __restrict__ rc0, double* rhoz, double* rhoc, double* part) {
     extern __shared__ __align__(16) unsigned char cond_sm[];
-    const int lane = threadIdx.x, n = threadIdx.y;
-    const int s = blockIdx.x * 32 + lane;
-    const int pr = live_prob(b, s, S, PS_ACT);
-    const bool live = pr >= 0;
+    const CondPlace at(S, b);
+    const bool live = at.live;
+    const int n = at.n, pr = at.pr;
+    const int64_t s = at.o;
     if (!__syncthreads_or(live)) return;
-    const int prc = live ? pr : 0;
+    const int prc = pr >= 0 ? pr : 0;
     const int sec = stage_sec(n, P.nsec);
     const int64_t od = (int64_t)NSC * ld + (int64_t)sec * b.NP + prc;
     const double dd = dzo[od], dw = b.ps ? psv(b, PS_DW, prc) : 0.0;
@@ -1230,7 +1252,7 @@ __global__ void __launch_bounds__(CS_T) cond_direction_kernel(
                 }
     }
     double dl[NR];
-    cond_solve_t_prec<PREC>(K, ld, s, n, lane, live, g, cond_sm, dl);
+    cond_solve_t_prec<PREC>(K, ld, at, g, cond_sm, dl);
     if (live) {
         double* zt = az ? az : dzo;
 #pragma unroll
@@ -1324,11 +1346,11 @@ __global__ void __launch_bounds__(CS_T) cond_direction_kernel(
     const double dlh = (al ? al : dlo)[(int64_t)(NR * n + R_H) * ld + s];
     if (P.nsec == 1) {
         const double w[5] = {key_double(k0), key_double(k1), dlh, key_double(k3), key_double(k4)};
-        store_partials<5>(w, part, ld, s, n);
+        store_partials<5>(w, part, ld, (int)s, n);
     } else {
         const double w[6] = {key_double(k0), key_double(k1), sec ? 0.0 : dlh, key_double(k3), key_double(k4),
                              sec ? dlh : 0.0};
-        store_partials<6>(w, part, ld, s, n);
+        store_partials<6>(w, part, ld, (int)s, n);
     }
 }
 
