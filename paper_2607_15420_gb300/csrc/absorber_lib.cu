@@ -338,6 +338,14 @@ cudaError_t upload_tables(int dev) {
         }
         UP(g_lt, lt);
     }
+    {
+        static LnEntry ln[LN_TAB];
+        for (int j = 0; j < LN_TAB; ++j) {
+            ln[j].inv = (double)(1.0L / (1.0L + ((long double)j + 0.5L) / LN_TAB));
+            ln[j].ln = (double)-logl((long double)ln[j].inv);
+        }
+        UP(g_ln, ln);
+    }
 #undef UP
     g_uploaded[dev] = true;
     return cudaSuccess;
@@ -533,9 +541,6 @@ abs_status fail(abs_problem* h, abs_status st, const std::string& msg) {
 int64_t vsize(const abs_problem* h) { return (int64_t)NSC * h->ld + (int64_t)h->P.nsec * h->ld; }
 double* V(abs_problem* h, int k) { return h->vec + (int64_t)k * vsize(h); }
 dim3 grid2(const abs_problem* h) { return dim3((unsigned)((h->S + kThr - 1) / kThr), N_STAGES); }
-// the trial evaluation (FP64-pipe-bound, limited by registers) in 32-thread blocks: the
-// blocks spread more evenly over the SMs (measured 7 % faster; the full evaluation is not)
-constexpr int EVAL_T = 32;
 dim3 geval(const abs_problem* h) { return dim3((unsigned)((h->S + EVAL_T - 1) / EVAL_T), N_STAGES); }
 // elementwise kernels: one thread per (entry, scenario)
 dim3 gride(const abs_problem* h) { return dim3((unsigned)((h->S + kThr - 1) / kThr), NSC); }
@@ -560,6 +565,36 @@ abs_status launch_check(abs_problem* h, int kind = KD_VEC, int weight = 1) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(h, ABS_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
     return ABS_OK;
+}
+
+// the evaluation at x: residuals c (with the partials part) and, when given, Jacobian and Hessian
+// values.  Up to EVAL_SPLIT_S scenarios the parts run on threads of their own (eval_split_kernel):
+// eight scenarios per SM are 2.5 warps of eval_kernel, where one thread's 64 cycles per instruction
+// and the three parts' larger sum meet.
+constexpr int EVAL_SPLIT_S = 8 * 152;
+abs_status eval_launch(abs_problem* h, const BView& b, const double* x, const double* lam, double* c, double* jac,
+                       double* hes, double* part, int kind, cudaStream_t st) {
+    const int S = (int)h->S;
+    dim3 g = geval(h);
+    if (h->S <= EVAL_SPLIT_S && jac) {
+        const int z0 = c || part ? 0 : 1;
+        g.z = (hes ? 3 : 2) - z0;
+        if (hes) eval_split_kernel<true><<<g, EVAL_T, 0, st>>>(h->P, S, h->ld, b, x, lam, h->feed, c, jac, hes, part, z0);
+        else eval_split_kernel<false><<<g, EVAL_T, 0, st>>>(h->P, S, h->ld, b, x, lam, h->feed, c, jac, hes, part, z0);
+    } else if (jac && hes) {
+        eval_kernel<true, true, true><<<g, EVAL_T, 0, st>>>(h->P, S, h->ld, b, false, x, nullptr, nullptr, lam, h->feed,
+                                                            c, jac, hes, part);
+    } else if (jac) {
+        eval_kernel<true, true, false><<<g, EVAL_T, 0, st>>>(h->P, S, h->ld, b, false, x, nullptr, nullptr, lam, h->feed,
+                                                             c, jac, nullptr, part);
+    } else if (hes) {
+        eval_kernel<true, false, true><<<g, EVAL_T, 0, st>>>(h->P, S, h->ld, b, false, x, nullptr, nullptr, lam, h->feed,
+                                                             c, nullptr, hes, part);
+    } else if (c || part) {
+        eval_kernel<true, false, false><<<g, EVAL_T, 0, st>>>(h->P, S, h->ld, b, false, x, nullptr, nullptr, lam,
+                                                              h->feed, c, nullptr, nullptr, part);
+    }
+    return launch_check(h, kind);
 }
 
 enum { K_EVAL = 0, K_EVAL_TRIAL = 1, K_FACTOR = 2, K_SOLVE = 3, K_SOLVE_T = 4 };
@@ -1201,6 +1236,8 @@ bool make_params(const abs_params* p, Params* P) {
         P->hL0[l] = p->hL_ref[l] + p->hL_dh[l];
     }
     for (int j = 0; j < 4; ++j) P->hV0[j] = p->hV_ref[j] + p->hV_dh[j];
+    for (int k = 0; k < 9; ++k)
+        for (int l = 0; l <= k; ++l) P->sxx[k * (k + 1) / 2 + l] = p->sx[k] * p->sx[l];
     P->Tlo_s = p->T_lo / p->sT;
     P->Thi_s = p->T_hi / p->sT;
     return p->n_sections >= 1 && p->n_sections <= KSEC;
@@ -1420,21 +1457,8 @@ abs_status eval_grad_jac_hess(abs_problem* h, const double* x, const double* lam
                               double* grad, double* c, double* jac_vals, double* hess_vals, abs_stream_t stream) {
     if (!h || !x || (hess_vals && !lambda)) return fail(h, ABS_ERR_ARG, "bad argument");
     cudaStream_t st = (cudaStream_t)stream;
-    const dim3 g = grid2(h);
     const BView b{h->pid, nullptr, h->NP};   // each scenario reads its own problem's d slot
-    if (jac_vals && hess_vals)
-        eval_kernel<true, true, true><<<g, kThr, 0, st>>>(h->P, (int)h->S, h->ld, b, false, x, nullptr, nullptr,
-                                                          lambda, h->feed, c, jac_vals, hess_vals, nullptr);
-    else if (jac_vals)
-        eval_kernel<true, true, false><<<g, kThr, 0, st>>>(h->P, (int)h->S, h->ld, b, false, x, nullptr, nullptr,
-                                                           lambda, h->feed, c, jac_vals, nullptr, nullptr);
-    else if (hess_vals)
-        eval_kernel<true, false, true><<<g, kThr, 0, st>>>(h->P, (int)h->S, h->ld, b, false, x, nullptr, nullptr,
-                                                           lambda, h->feed, c, nullptr, hess_vals, nullptr);
-    else if (c)
-        eval_kernel<true, false, false><<<g, kThr, 0, st>>>(h->P, (int)h->S, h->ld, b, false, x, nullptr, nullptr,
-                                                            lambda, h->feed, c, nullptr, nullptr, nullptr);
-    abs_status r = launch_check(h, KD_EVAL);
+    abs_status r = eval_launch(h, b, x, lambda, c, jac_vals, hess_vals, nullptr, KD_EVAL, st);
     if (r != ABS_OK) return r;
     // the objective sum_k w_k theta_k (w = 1, the single d, for one section)
     const int K = h->P.nsec;

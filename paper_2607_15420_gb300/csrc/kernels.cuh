@@ -212,11 +212,11 @@ __device__ inline void load_stage(const Params& P, int S, int64_t ld, const doub
 // the problems flagged PS_ACT; trial = true: at x + alpha_p dir of the problems flagged
 // PS_LSACT, dir = dxB where PS_SOC is set, else dxA.
 template <bool WR, bool WJ, bool WH>
-__global__ void __launch_bounds__(128) eval_kernel(const Params P, int S, int64_t ld, const BView b, bool trial,
-                                                   const double* __restrict__ x, const double* __restrict__ dxA,
-                                                   const double* __restrict__ dxB, const double* __restrict__ lam,
-                                                   const double* __restrict__ feed, double* c, double* jac,
-                                                   double* hes, double* part) {
+__device__ __forceinline__ void eval_body(const Params& P, int S, int64_t ld, const BView& b, bool trial,
+                                          const double* __restrict__ x, const double* __restrict__ dxA,
+                                          const double* __restrict__ dxB, const double* __restrict__ lam,
+                                          const double* __restrict__ feed, double* c, double* jac, double* hes,
+                                          double* part) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     const int n = blockIdx.y;
     const int p = live_prob(b, s, S, trial ? PS_LSACT : PS_ACT);
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(128) eval_kernel(const Params P, int S, int64_
             hes[(int64_t)(NHS * N_STAGES + k) * ld + s] = -P.u_max * M_PI * 0.5 * sl;
         }
     }
-    if (part) {
+    if (WR && part) {
         // sum of ln(slack) over the stage's 18 bounds as the logarithm of their product: the
         // product is carried as a mantissa in [1, 2) times a power of two (exponent read from
         // the bit pattern), so it neither overflows nor underflows; a slack that is not
@@ -292,10 +292,39 @@ __global__ void __launch_bounds__(128) eval_kernel(const Params P, int S, int64_
             if (has_lo(j)) take(in.q[j] - (j == LT ? P.Tlo_s : 0.0));
             if (has_hi(j)) take(P.Thi_s - in.q[j]);
         }
-        blog = bad ? NAN : log(m) + (double)e2 * 0.69314718055994530942;   // ln 2
+        blog = bad ? NAN : fma((double)e2, 0.69314718055994530942, ln_tab(m));   // ln 2
         const double v[3] = {em.asum, em.amax, blog};
         store_partials<3>(v, part, ld, s, n);
     }
+}
+
+// One thread per (scenario, stage), in 32-thread blocks: FP64 instructions bound it, and 1570 blocks
+// at 5000 scenarios share out evenly over 152 SMs.
+constexpr int EVAL_T = 32;
+template <bool WR, bool WJ, bool WH>
+__global__ void __launch_bounds__(EVAL_T) eval_kernel(const Params P, int S, int64_t ld, const BView b, bool trial,
+                                                      const double* __restrict__ x, const double* __restrict__ dxA,
+                                                      const double* __restrict__ dxB, const double* __restrict__ lam,
+                                                      const double* __restrict__ feed, double* c, double* jac,
+                                                      double* hes, double* part) {
+    eval_body<WR, WJ, WH>(P, S, ld, b, trial, x, dxA, dxB, lam, feed, c, jac, hes, part);
+}
+
+// The same with a thread per (scenario, stage) and part -- blockIdx.z + z0: 0 residuals, 1 Jacobian, 2
+// Hessian -- for sizes at which the threads of eval_kernel leave schedulers idle: a warp alone on its
+// scheduler issues an FP64 instruction per 64 cycles whatever else the SM does, so three shorter
+// threads finish sooner though together they compute a third more.  The parts' values are
+// eval_kernel's bit for bit (model.cuh: explicit fma).
+template <bool WH>
+__global__ void __launch_bounds__(EVAL_T) eval_split_kernel(const Params P, int S, int64_t ld, const BView b,
+                                                            const double* __restrict__ x,
+                                                            const double* __restrict__ lam,
+                                                            const double* __restrict__ feed, double* c, double* jac,
+                                                            double* hes, double* part, int z0) {
+    const int z = (int)blockIdx.z + z0;
+    if (z == 0) eval_body<true, false, false>(P, S, ld, b, false, x, nullptr, nullptr, lam, feed, c, jac, hes, part);
+    else if (z == 1) eval_body<false, true, false>(P, S, ld, b, false, x, nullptr, nullptr, lam, feed, c, jac, hes, part);
+    else if (WH) eval_body<false, false, true>(P, S, ld, b, false, x, nullptr, nullptr, lam, feed, c, jac, hes, part);
 }
 
 // ------------------------------------------------------------------------------------

@@ -88,7 +88,18 @@ struct Params {
     double hL0[9];   // hL_ref + hL_dh
     double hV0[4];
     double Tlo_s, Thi_s;   // T_lo / sT, T_hi / sT: the scaled temperature bounds
+    double sxx[45];        // sx_k sx_l, l <= k, at k (k + 1) / 2 + l
 };
+
+// The species of the apparent totals fall into five classes of equal membership (MEA, MEAH+ |
+// MEACOO- | HCO3-, CO3-- | OH-, H2O | CO2): Henry's derivatives are formed once per class.
+// c_t: totals the class counts in; c_a: 1 MEA, 2 H2O, 0 neither.
+__host__ __device__ constexpr int henry_cls(int k) {
+    constexpr int t[9] = {0, 0, -1, 1, 2, 3, 2, 4, 3};
+    return t[k];
+}
+__host__ __device__ constexpr int cls_t(int c) { return c == 1 || c == 2 ? 2 : 1; }
+__host__ __device__ constexpr int cls_a(int c) { return c < 2 ? 1 : (c < 4 ? 2 : 0); }
 
 constexpr int KSEC = 2;   // most column sections (design-vector entries)
 
@@ -124,12 +135,50 @@ struct StageLam {
 // Emitter concept:
 //   static constexpr bool want_res, want_jac, want_hes;
 //   void res(int r, double v); void jac(int r, int lv, double v); void hes(int i, int j, double v);
+//
+// FP64 instructions bound the evaluation on the device (one warp instruction per 19 cycles and
+// SM), so the terms are arranged for few of them: products by structural zeros and ones are left
+// out by hand (the compiler may not drop 0 x), Henry's second derivatives are formed per class of
+// species instead of per pair, one division serves several reciprocals.  Every product that is
+// added to something is an explicit fma, so a value comes out the same whichever of the three
+// parts (residuals, Jacobian, Hessian) an instance computes.
+#ifdef __CUDACC__
+// ln(x) for the residuals: x = 2^e m, m in [1, 2); 1 / c from a table at the centre c of m's
+// 128th, r = m / c - 1 (|r| < 2^-8, one fma), ln x = e ln 2 + ln c + (r - r^2 / 2 + ... + r^7 / 7)
+// (the table-driven method of Tang 1990): 11 FP64 instructions against about 30 of log(), errors
+// of a rounding of the larger terms.  Anything but a positive normal number goes to log().
+struct LnEntry {
+    double inv, ln;   // 1 / c rounded, -ln(inv)
+};
+constexpr int LN_TAB = 128;
+__device__ LnEntry g_ln[LN_TAB];
+#endif
+__host__ __device__ inline double ln_tab(double x) {
+#ifdef __CUDA_ARCH__
+    const int hi = __double2hiint(x);
+    if (!(hi >= 0x00100000 && hi < 0x7ff00000)) return log(x);
+    const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(x));
+    const LnEntry t = g_ln[(hi >> 13) & (LN_TAB - 1)];
+    const double e = (double)((hi >> 20) - 1023);
+    const double r = fma(m, t.inv, -1.0);
+    double q = fma(r, 1.0 / 7.0, -1.0 / 6.0);
+    q = fma(r, q, 0.2);
+    q = fma(r, q, -0.25);
+    q = fma(r, q, 1.0 / 3.0);
+    q = fma(r, q, -0.5);
+    return fma(e, 0.69314718055994530942, t.ln) + fma(r * r, q, r);
+#else
+    return log(x);
+#endif
+}
+
 #ifdef __CUDACC__
 #pragma nv_exec_check_disable
 #endif
 template <class E>
 __host__ __device__ inline void stage_eval(const Params& P, const StageIn& in, const StageLam* lam,
                                            E& e) {
+    constexpr bool WR = E::want_res, WJ = E::want_jac, WH = E::want_hes;
     const double sT = P.sT;
     double x[9], y[4];
 #pragma unroll
@@ -150,13 +199,9 @@ __host__ __device__ inline void stage_eval(const Params& P, const StageIn& in, c
     // of (9b) and T from one division: a = Tc Pr, b = tot T, r = 1 / (a b), then
     // 1/Tc = r b Pr, 1/Pr = r b Tc, 1/tot = r a T, 1/T = r a tot (all positive and O(1e-3
     // .. 1e3) at interior points)
-    double am = 0, ac = 0, aw = 0;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        am += app_m(k) * x[k];
-        ac += app_c(k) * x[k];
-        aw += app_w(k) * x[k];
-    }
+    const double am = x[0] + x[1] + x[3];
+    const double ac = x[3] + x[4] + x[6] + x[7];
+    const double aw = x[4] + x[5] + x[6] + x[8];
     const double tot = am + ac + aw;
     const double Tc = T + P.psat_c;
     const double ra = Tc * Pr, rb = tot * T;
@@ -164,49 +209,40 @@ __host__ __device__ inline void stage_eval(const Params& P, const StageIn& in, c
     const double rbr = r4 * rb, rar = r4 * ra;
     const double iTc = rbr * Pr, iPr = rbr * Tc, it = rar * T, invT = rar * tot;
 
-    // ---- enthalpies ---------------------------------------------------------------
+    // ---- enthalpies: h = h0 + dT (cpa + cpb / 2 dT), cp = cpa + cpb dT ----------------------
     const double dT = T - P.T_ref, dTa = Ta - P.T_ref, dTb = Tb - P.T_ref;
-    double hL[9], cpL[9], hLa[9], cpLa[9], hV[4], cpV[4], hVb[4], cpVb[4];
+    const double hdT = 0.5 * dT, hdTa = 0.5 * dTa, hdTb = 0.5 * dTb;
+    double hL[9], hV[4], hLa[9], hVb[4];
+    double HL = 0, HV = 0, CL = 0, CV = 0, HLa = 0, HVb = 0, CLa = 0, CVb = 0;
 #pragma unroll
     for (int l = 0; l < 9; ++l) {
-        cpL[l] = P.hL_cpa[l] + P.hL_cpb[l] * dT;
-        hL[l] = P.hL0[l] + dT * (P.hL_cpa[l] + 0.5 * P.hL_cpb[l] * dT);
-        cpLa[l] = P.hL_cpa[l] + P.hL_cpb[l] * dTa;
-        hLa[l] = P.hL0[l] + dTa * (P.hL_cpa[l] + 0.5 * P.hL_cpb[l] * dTa);
+        hL[l] = fma(dT, fma(P.hL_cpb[l], hdT, P.hL_cpa[l]), P.hL0[l]);
+        hLa[l] = fma(dTa, fma(P.hL_cpb[l], hdTa, P.hL_cpa[l]), P.hL0[l]);
+        HL = fma(x[l], hL[l], HL);
+        HLa = fma(xa[l], hLa[l], HLa);
+        if (WJ || WH) CL = fma(x[l], fma(P.hL_cpb[l], dT, P.hL_cpa[l]), CL);
+        if (WJ) CLa = fma(xa[l], fma(P.hL_cpb[l], dTa, P.hL_cpa[l]), CLa);
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        cpV[j] = P.hV_cpa[j] + P.hV_cpb[j] * dT;
-        hV[j] = P.hV0[j] + dT * (P.hV_cpa[j] + 0.5 * P.hV_cpb[j] * dT);
-        cpVb[j] = P.hV_cpa[j] + P.hV_cpb[j] * dTb;
-        hVb[j] = P.hV0[j] + dTb * (P.hV_cpa[j] + 0.5 * P.hV_cpb[j] * dTb);
-    }
-    double HL = 0, HV = 0, HLa = 0, HVb = 0, CL = 0, CV = 0, CLa = 0, CVb = 0;
-#pragma unroll
-    for (int l = 0; l < 9; ++l) {
-        HL += x[l] * hL[l];
-        CL += x[l] * cpL[l];
-        HLa += xa[l] * hLa[l];
-        CLa += xa[l] * cpLa[l];
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        HV += y[j] * hV[j];
-        CV += y[j] * cpV[j];
-        HVb += yb[j] * hVb[j];
-        CVb += yb[j] * cpVb[j];
+        hV[j] = fma(dT, fma(P.hV_cpb[j], hdT, P.hV_cpa[j]), P.hV0[j]);
+        hVb[j] = fma(dTb, fma(P.hV_cpb[j], hdTb, P.hV_cpa[j]), P.hV0[j]);
+        HV = fma(y[j], hV[j], HV);
+        HVb = fma(yb[j], hVb[j], HVb);
+        if (WJ || WH) CV = fma(y[j], fma(P.hV_cpb[j], dT, P.hV_cpa[j]), CV);
+        if (WJ) CVb = fma(yb[j], fma(P.hV_cpb[j], dTb, P.hV_cpa[j]), CVb);
     }
 
     // ---- (9a) water saturation pressure ---------------------------------------------
-    const double ps = exp(P.psat_a - P.psat_b * iTc);
+    const double ps = exp(fma(-P.psat_b, iTc, P.psat_a));
     const double bT2 = P.psat_b * iTc * iTc;
-    const double ps1 = ps * bT2;                                        // dPsat/dT
-    const double ps2 = ps * (bT2 * bT2 - 2.0 * P.psat_b * iTc * iTc * iTc);  // d2Psat/dT2
+    const double ps1 = ps * bT2;                                // dPsat/dT
+    const double ps2 = ps * fma(bT2, bT2, -2.0 * bT2 * iTc);    // d2Psat/dT2
     // reciprocals of the scaled liquid fractions (derivatives of their logarithms), all
     // nine from one division: prefix products p_c = q_0 ... q_c, r = 1 / p_8, then walking
     // back 1/q_c = r p_{c-1} and r <- r q_c (the fractions are positive and O(1))
     double iq[9];
-    if (E::want_jac || E::want_hes) {
+    if (WJ || WH) {
         double pre[9];
         pre[0] = in.q[LX];
 #pragma unroll
@@ -223,60 +259,73 @@ __host__ __device__ inline void stage_eval(const Params& P, const StageIn& in, c
         for (int c = 0; c < 9; ++c) iq[c] = 0.0;
     }
 
-    // ---- (9b) Henry coefficient --------------------------------------------------------
-    const double um = am * it, uw = aw * it;
-    const double g = P.henry_a + P.henry_b * invT + P.henry_m * um + P.henry_w * uw;
-    const double Hh = exp(g);
+    // ---- (9b) Henry coefficient: ln H = ha + hb / T + s, s = hm x_MEA^app + hw x_H2O^app; for a
+    // species of class c, ds/dx = (a_c - s t_c) / tot, a_c the class's hm, hw or 0 --------------
+    const double sh = fma(P.henry_m, am * it, P.henry_w * (aw * it));
+    const double Hh = exp(fma(P.henry_b, invT, P.henry_a) + sh);
     const double gT = -P.henry_b * invT * invT;
-    const double gTT = 2.0 * P.henry_b * invT * invT * invT;
-    double gk[9];   // dg/dx_k (physical x)
+    double gc[5];
 #pragma unroll
-    for (int k = 0; k < 9; ++k)
-        gk[k] = (P.henry_m * (app_m(k) - um * app_t(k)) + P.henry_w * (app_w(k) - uw * app_t(k))) * it;
+    for (int c = 0; c < 5; ++c) {
+        const double a = cls_a(c) == 1 ? P.henry_m : (cls_a(c) == 2 ? P.henry_w : 0.0);
+        const double ts = cls_t(c) == 2 ? 2.0 * sh : sh;
+        gc[c] = cls_a(c) ? (a - ts) * it : -ts * it;
+    }
     const double rhoH = P.rho_L * Hh;
     const double x7 = x[7];
 
     // ---- residuals ---------------------------------------------------------------------
-    if (E::want_res) {
+    if (WR) {
 #pragma unroll
         for (int c = 0; c < 11; ++c) {
             double r = 0.0;
-            if (c < 9) r += L * x[c] - La * xa[c];
-            if (c >= 7) r += V * y[c - 7] - Vb * yb[c - 7];
+            if (c < 9) r = fma(L, x[c], -La * xa[c]);
+            if (c >= 7) {
+                const double v = fma(V, y[c < 7 ? 0 : c - 7], -Vb * yb[c < 7 ? 0 : c - 7]);
+                r = c < 9 ? r + v : v;
+            }
 #pragma unroll
-            for (int k = 0; k < 5; ++k)
-                if (nu(c, k) != 0) r -= nu(c, k) * in.q[LE + k];
+            for (int k = 0; k < 5; ++k) {
+                if (nu(c, k) > 0) r -= in.q[LE + k];
+                if (nu(c, k) < 0) r += in.q[LE + k];
+            }
             e.res(c, r);
         }
-        e.res(R_VH, Pr * y[1] - x[8] * ps);
-        e.res(R_VC, Pr * y[0] - rhoH * x7);
+        e.res(R_VH, fma(Pr, y[1], -x[8] * ps));
+        e.res(R_VC, fma(Pr, y[0], -rhoH * x7));
         // sum_c nu_ck ln x_c as one logarithm per reaction: every nu is +-1, so it is
         // ln(prod over products of q_c / prod over reactants of q_c) + sum_c nu_ck ln sx_c
         // (the scaled fractions are O(1): the quotients stay far from over- and underflow)
-        const double lT = log(T);
+        const double lT = ln_tab(T);
         // the five quotients' denominators inverted together from one division (prefix
         // products, then back)
         double qn[5], qd[5], pre[5];
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
-            double num = 1.0, den = 1.0;
+            double num = 0.0, den = 0.0;
+            bool hn = false, hd = false;
 #pragma unroll
             for (int c = 0; c < 9; ++c) {
-                if (nu(c, k) > 0) num *= in.q[LX + c];
-                if (nu(c, k) < 0) den *= in.q[LX + c];
+                if (nu(c, k) > 0) {
+                    num = hn ? num * in.q[LX + c] : in.q[LX + c];
+                    hn = true;
+                }
+                if (nu(c, k) < 0) {
+                    den = hd ? den * in.q[LX + c] : in.q[LX + c];
+                    hd = true;
+                }
             }
             qn[k] = num;
             qd[k] = den;
-            pre[k] = k ? pre[k - 1] * den : den;
+            pre[k] = k ? pre[k ? k - 1 : 0] * den : den;
         }
         double rq = 1.0 / pre[4];
 #pragma unroll
         for (int k = 4; k >= 0; --k) {
-            const double rk = k ? rq * pre[k - 1] : rq;
+            const double rk = k ? rq * pre[k ? k - 1 : 0] : rq;
             if (k) rq *= qd[k];
-            const double r = -(P.KE_A[k] + P.KE_B[k] * invT + P.KE_C[k] * lT + P.KE_D[k] * T) + P.lnsxr[k] +
-                             log(qn[k] * rk);
-            e.res(R_RX + k, r);
+            const double lnK = fma(P.KE_D[k], T, fma(P.KE_C[k], lT, fma(P.KE_B[k], invT, P.KE_A[k])));
+            e.res(R_RX + k, (P.lnsxr[k] - lnK) + ln_tab(qn[k] * rk));
         }
         double sx_ = -1.0, sy_ = -1.0;
 #pragma unroll
@@ -285,29 +334,38 @@ __host__ __device__ inline void stage_eval(const Params& P, const StageIn& in, c
         for (int j = 0; j < 4; ++j) sy_ += y[j];
         e.res(R_SX, sx_);
         e.res(R_SY, sy_);
-        e.res(R_E, L * HL + V * HV - La * HLa - Vb * HVb);
-        e.res(R_H, V * P.R * T * iPr - P.u_max * M_PI * in.d * in.d * 0.25 + in.q[LS]);
+        e.res(R_E, fma(L, HL, -La * HLa) + fma(V, HV, -Vb * HVb));
+        e.res(R_H, fma(V, P.R * T * iPr, fma(-0.25 * M_PI * P.u_max, in.d * in.d, in.q[LS])));
     }
 
     // ---- Jacobian ----------------------------------------------------------------------
-    if (E::want_jac) {
+    if (WJ) {
+        const double nLa = -La, nVb = -Vb;
 #pragma unroll
         for (int c = 0; c < 11; ++c) {
             if (c < 9) {
-                e.jac(c, LX + c, L * P.sx[c]);
+                const double f = L * P.sx[c];
+                e.jac(c, LX + c, f);
                 e.jac(c, LL, x[c]);
+                e.jac(R_E, LX + c, f * hL[c]);
                 if (in.has_above) {
-                    e.jac(c, AX + c, -La * P.sx[c]);
+                    const double fa = nLa * P.sx[c];
+                    e.jac(c, AX + c, fa);
                     e.jac(c, AL, -xa[c]);
+                    e.jac(R_E, AX + c, fa * hLa[c]);
                 }
             }
             if (c >= 7) {
                 const int j = c - 7;
-                e.jac(c, LY + j, V * P.sy[j]);
+                const double f = V * P.sy[j];
+                e.jac(c, LY + j, f);
                 e.jac(c, LV, y[j]);
+                e.jac(R_E, LY + j, f * hV[j]);
                 if (in.has_below) {
-                    e.jac(c, BY + j, -Vb * P.sy[j]);
+                    const double fb = nVb * P.sy[j];
+                    e.jac(c, BY + j, fb);
                     e.jac(c, BV, -yb[j]);
+                    e.jac(R_E, BY + j, fb * hVb[j]);
                 }
             }
 #pragma unroll
@@ -319,18 +377,23 @@ __host__ __device__ inline void stage_eval(const Params& P, const StageIn& in, c
         e.jac(R_VH, LX + 8, -P.sx[8] * ps);
         e.jac(R_VH, LT, -x[8] * ps1 * sT);
         // (9b)
+        const double rx7 = -rhoH * x7;
         e.jac(R_VC, LY + 0, Pr * P.sy[0]);
+        double vc[5];
+#pragma unroll
+        for (int c = 0; c < 5; ++c) vc[c] = c == 4 ? fma(rx7, gc[c], -rhoH) : rx7 * gc[c];
 #pragma unroll
         for (int k = 0; k < 9; ++k)
-            if (in_henry(k)) e.jac(R_VC, LX + k, -rhoH * ((k == 7 ? 1.0 : 0.0) + x7 * gk[k]) * P.sx[k]);
-        e.jac(R_VC, LT, -rhoH * x7 * gT * sT);
+            if (in_henry(k)) e.jac(R_VC, LX + k, vc[henry_cls(k) < 0 ? 0 : henry_cls(k)] * P.sx[k]);
+        e.jac(R_VC, LT, rx7 * gT * sT);
         // (3a)
+        const double sTi = sT * invT;
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
 #pragma unroll
             for (int c = 0; c < 9; ++c)
-                if (nu(c, k) != 0) e.jac(R_RX + k, LX + c, nu(c, k) * iq[c]);
-            e.jac(R_RX + k, LT, -sT * (-P.KE_B[k] * invT * invT + P.KE_C[k] * invT + P.KE_D[k]));
+                if (nu(c, k) != 0) e.jac(R_RX + k, LX + c, nu(c, k) > 0 ? iq[c] : -iq[c]);
+            e.jac(R_RX + k, LT, fma(sTi, fma(P.KE_B[k], invT, -P.KE_C[k]), -sT * P.KE_D[k]));
         }
         // (4)
 #pragma unroll
@@ -338,110 +401,124 @@ __host__ __device__ inline void stage_eval(const Params& P, const StageIn& in, c
 #pragma unroll
         for (int j = 0; j < 4; ++j) e.jac(R_SY, LY + j, P.sy[j]);
         // (6)
-#pragma unroll
-        for (int l = 0; l < 9; ++l) e.jac(R_E, LX + l, L * P.sx[l] * hL[l]);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) e.jac(R_E, LY + j, V * P.sy[j] * hV[j]);
         e.jac(R_E, LL, HL);
         e.jac(R_E, LV, HV);
-        e.jac(R_E, LT, sT * (L * CL + V * CV));
+        e.jac(R_E, LT, sT * fma(L, CL, V * CV));
         if (in.has_above) {
-#pragma unroll
-            for (int l = 0; l < 9; ++l) e.jac(R_E, AX + l, -La * P.sx[l] * hLa[l]);
             e.jac(R_E, AL, -HLa);
-            e.jac(R_E, AT, -sT * La * CLa);
+            e.jac(R_E, AT, sT * nLa * CLa);
         }
         if (in.has_below) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) e.jac(R_E, BY + j, -Vb * P.sy[j] * hVb[j]);
             e.jac(R_E, BV, -HVb);
-            e.jac(R_E, BT, -sT * Vb * CVb);
+            e.jac(R_E, BT, sT * nVb * CVb);
         }
         // (10b)
         e.jac(R_H, LV, P.R * T * iPr);
-        e.jac(R_H, LT, V * P.R * sT * iPr);
+        e.jac(R_H, LT, V * (P.R * sT) * iPr);
         e.jac(R_H, LS, 1.0);
-        e.jac(R_H, LD_, -P.u_max * M_PI * in.d * 0.5);
+        e.jac(R_H, LD_, (-0.5 * M_PI * P.u_max) * in.d);
     }
 
     // ---- Lagrangian Hessian block of this stage's unknowns (lower triangle) ------------
     // Terms come from this stage's rows and from the neighbours' rows in which this
     // stage's streams appear: the stage below reads (L, x, T) of this stage as its
     // "from above" stream, the stage above reads (V, y, T) as its "from below" stream.
-    if (E::want_hes) {
+    if (WH) {
         const double* lo = lam->own;
         double muL[9], muV[4];
 #pragma unroll
-        for (int c = 0; c < 9; ++c) muL[c] = lo[c] - (in.has_below ? lam->below[c] : 0.0);
+        for (int c = 0; c < 9; ++c) muL[c] = in.has_below ? lo[c] - lam->below[c] : lo[c];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) muV[j] = lo[7 + j] - (in.has_above ? lam->above[j] : 0.0);
-        const double muEL = lo[R_E] - (in.has_below ? lam->below[9] : 0.0);
-        const double muEV = lo[R_E] - (in.has_above ? lam->above[4] : 0.0);
+        for (int j = 0; j < 4; ++j) muV[j] = in.has_above ? lo[7 + j] - lam->above[j] : lo[7 + j];
+        const double muEL = in.has_below ? lo[R_E] - lam->below[9] : lo[R_E];
+        const double muEV = in.has_above ? lo[R_E] - lam->above[4] : lo[R_E];
         const double lVH = lo[R_VH], lVC = lo[R_VC], lH = lo[R_H];
 
-        // Henry block over the species of the apparent totals (and the ln x diagonals)
+        // Henry block over the species of the apparent totals (and the ln x diagonals).  With g_k =
+        // (a_k - s t_k) / tot the second derivatives of H x7 / (H x7) are g_k g_l + dg_k/dx_l =
+        // ((a_k - p t_k)(a_l - p t_l) - t_k t_l) / tot^2, p = 1 + s: one value per pair of classes
+        const double c0 = -lVC * rhoH;
+        const double c7 = c0 * x7 * it * it, p1 = 1.0 + sh;
+        double bc[5], pc[15], g0[5];
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+            const double a = cls_a(c) == 1 ? P.henry_m : (cls_a(c) == 2 ? P.henry_w : 0.0);
+            const double tp = cls_t(c) == 2 ? 2.0 * p1 : p1;
+            bc[c] = cls_a(c) ? a - tp : -tp;
+            g0[c] = c0 * gc[c];
+        }
+#pragma unroll
+        for (int c = 0; c < 5; ++c)
+#pragma unroll
+            for (int d = 0; d <= c; ++d) {
+                double v = c7 * fma(bc[c], bc[d], -(double)(cls_t(c) * cls_t(d)));
+                if (c == 4) v += d == 4 ? 2.0 * g0[4] : g0[d];   // the factor x7 itself
+                pc[c * (c + 1) / 2 + d] = v;
+            }
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
 #pragma unroll
             for (int l = 0; l <= k; ++l) {
-                double v = 0.0;
-                bool present = false;
-                if (in_henry(k) && in_henry(l)) {
-                    const double gkl = (P.henry_m * (-app_m(k) * app_t(l) - app_m(l) * app_t(k) +
-                                                     2.0 * um * app_t(k) * app_t(l)) +
-                                        P.henry_w * (-app_w(k) * app_t(l) - app_w(l) * app_t(k) +
-                                                     2.0 * uw * app_t(k) * app_t(l))) * it * it;
-                    const double d2 = (k == 7 ? gk[l] : 0.0) + (l == 7 ? gk[k] : 0.0) +
-                                      x7 * (gk[k] * gk[l] + gkl);
-                    v += -lVC * rhoH * d2 * P.sx[k] * P.sx[l];
-                    present = true;
-                }
+                const bool henry = in_henry(k) && in_henry(l);
+                double a = 0.0;
+                bool any = false;
                 if (k == l) {
-                    double a = 0.0;
-                    bool any = false;
 #pragma unroll
-                    for (int r = 0; r < 5; ++r)
-                        if (nu(k, r) != 0) {
-                            a += lo[R_RX + r] * nu(k, r);
-                            any = true;
-                        }
-                    if (any) {
-                        v += -a * iq[k] * iq[k];
-                        present = true;
+                    for (int r = 0; r < 5; ++r) {
+                        if (nu(k, r) > 0) a = any ? a + lo[R_RX + r] : lo[R_RX + r];
+                        if (nu(k, r) < 0) a = any ? a - lo[R_RX + r] : -lo[R_RX + r];
+                        any = any || nu(k, r) != 0;
                     }
                 }
-                if (present) e.hes(LX + k, LX + l, v);
+                if (!henry && !any) continue;
+                double v = any ? -a * (iq[k] * iq[k]) : 0.0;
+                if (henry) {
+                    const int ck = henry_cls(k) < 0 ? 0 : henry_cls(k), cl = henry_cls(l) < 0 ? 0 : henry_cls(l);
+                    const int hi = ck > cl ? ck : cl, lw = ck > cl ? cl : ck;
+                    const double q = pc[hi * (hi + 1) / 2 + lw], w = P.sxx[k * (k + 1) / 2 + l];
+                    v = any ? fma(q, w, v) : q * w;
+                }
+                e.hes(LX + k, LX + l, v);
             }
         }
         // (L, x_l) and (V, y_j): bilinear flows in (1) and (6)
 #pragma unroll
-        for (int l = 0; l < 9; ++l) e.hes(LL, LX + l, P.sx[l] * (muL[l] + muEL * hL[l]));
+        for (int l = 0; l < 9; ++l) e.hes(LL, LX + l, P.sx[l] * fma(muEL, hL[l], muL[l]));
 #pragma unroll
-        for (int j = 0; j < 4; ++j) e.hes(LV, LY + j, P.sy[j] * (muV[j] + muEV * hV[j]));
+        for (int j = 0; j < 4; ++j) e.hes(LV, LY + j, P.sy[j] * fma(muEV, hV[j], muV[j]));
         // (T, x_l)
+        const double aL = sT * muEL * L, aV = sT * muEV * V;
+        const double hT = c0 * gT * sT, hT7 = hT * x7;
+        double tc[5];
+#pragma unroll
+        for (int c = 0; c < 5; ++c) tc[c] = c == 4 ? fma(hT7, gc[c], hT) : hT7 * gc[c];
 #pragma unroll
         for (int l = 0; l < 9; ++l) {
-            double v = sT * P.sx[l] * muEL * L * cpL[l];
-            if (l == 8) v += -lVH * P.sx[8] * ps1 * sT;
-            if (in_henry(l)) v += -lVC * rhoH * gT * ((l == 7 ? 1.0 : 0.0) + x7 * gk[l]) * P.sx[l] * sT;
-            e.hes(LT, LX + l, v);
+            const double cp = fma(P.hL_cpb[l], dT, P.hL_cpa[l]);
+            double v = in_henry(l) ? fma(aL, cp, tc[henry_cls(l) < 0 ? 0 : henry_cls(l)]) : aL * cp;
+            if (l == 8) v = fma(-lVH * sT, ps1, v);
+            e.hes(LT, LX + l, v * P.sx[l]);
         }
         // (T, y_j)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) e.hes(LT, LY + j, sT * P.sy[j] * muEV * V * cpV[j]);
+        for (int j = 0; j < 4; ++j)
+            e.hes(LT, LY + j, aV * fma(P.hV_cpb[j], dT, P.hV_cpa[j]) * P.sy[j]);
         e.hes(LT, LL, sT * muEL * CL);
-        e.hes(LT, LV, sT * muEV * CV + lH * P.R * sT * iPr);
+        e.hes(LT, LV, sT * fma(muEV, CV, lH * P.R * iPr));
         // (T, T)
         {
-            double dCL = 0.0, dCV = 0.0;
+            double dCL = 0.0, dCV = 0.0, rx = 0.0;
 #pragma unroll
-            for (int l = 0; l < 9; ++l) dCL += x[l] * P.hL_cpb[l];
+            for (int l = 0; l < 9; ++l) dCL = fma(x[l], P.hL_cpb[l], dCL);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) dCV += y[j] * P.hV_cpb[j];
-            double v = muEL * L * dCL + muEV * V * dCV - lVH * x[8] * ps2 - lVC * rhoH * x7 * (gT * gT + gTT);
+            for (int j = 0; j < 4; ++j) dCV = fma(y[j], P.hV_cpb[j], dCV);
+            const double i2 = invT * invT, ti = 2.0 * invT;
 #pragma unroll
-            for (int r = 0; r < 5; ++r)
-                v -= lo[R_RX + r] * (2.0 * P.KE_B[r] * invT * invT * invT - P.KE_C[r] * invT * invT);
+            for (int r = 0; r < 5; ++r) rx = fma(lo[R_RX + r], fma(P.KE_B[r], ti, -P.KE_C[r]), rx);
+            double v = fma(muEL * L, dCL, muEV * V * dCV);
+            v = fma(-lVH * x[8], ps2, v);
+            v = fma(c0 * x7, fma(gT, gT, 2.0 * P.henry_b * i2 * invT), v);
+            v = fma(-i2, rx, v);
             e.hes(LT, LT, sT * sT * v);
         }
     }
