@@ -933,15 +933,15 @@ abs_status solve_p(abs_problem* h, int prec, const KKTSys* K, const double* x, c
 }
 
 // the rest of a solve after solve_p (p in V_P, the design entries' steps in dz's slots): the
-// direction (dz, dl), or with az, al a correction added to it, and with res the KKT residual
+// direction (dz, dl), or with az, al a correction added to it; with res its g into V_G
 abs_status solve_direction(abs_problem* h, const KKTSys& K, const double* x, const double* rz, double* dz, double* dl,
-                           double* az, double* al, bool res, const double* rz0, const double* rc0, cudaStream_t st) {
+                           double* az, double* al, bool res, cudaStream_t st) {
     prof_begin(h, K_SOLVE_T, st);
     const size_t sm = cond_smem(K.prec == ABS_PREC_FP32 ? sizeof(float) : sizeof(double));
-#define CD_GO(PR)                                                                                                   \
-    cond_direction_kernel<PR><<<gridc(h), CS_T, sm, st>>>(h->P, (int)h->S, h->ld, view(h), cond_fac(h), K.jac, K.hes, \
-                                                         K.sig, K.use_w, x, V(h, V_P), rz, dz, dl, az, al, res, rz0, \
-                                                         rc0, V(h, V_RHOZ), V(h, V_RHOC), h->part)
+#define CD_GO(PR)                                                                                                  \
+    cond_direction_kernel<PR><<<gridc(h), CS_T, sm, st>>>(h->P, (int)h->S, h->ld, view(h), cond_fac(h), K.hes,     \
+                                                          K.sig, K.use_w, x, V(h, V_P), rz, dz, dl, az, al,        \
+                                                          res ? V(h, V_G) : nullptr)
     switch (cond_prec(K.prec)) {
         case CP_FP64: CD_GO(CP_FP64); break;
         case CP_FP32: CD_GO(CP_FP32); break;
@@ -1137,14 +1137,17 @@ abs_status kkt_solve_launches(abs_problem* h, const KKTSys& K, const double* x, 
         }
         finalize_dd_kernel<<<(unsigned)((h->NP + 127) / 128), 128, 0, st>>>(h->ld, view(h), h->red, dz, nsec);
         if ((r = launch_check(h, KD_VEC)) != ABS_OK) return r;
-        if (!tc) return solve_direction(h, K, x, rz, dz, dl, az, al, res, rz0, rc0, st);
-        dz_fast_kernel<<<gride(h), kThr, 0, st>>>((int)h->S, h->ld, view(h), V(h, V_P), V(h, V_Q), V(h, V_T),
-                                                  V(h, V_HQ), dz, V(h, V_G), two ? V(h, V_Q1) : nullptr,
-                                                  two ? V(h, V_HQ1) : nullptr);
-        if ((r = launch_check(h, KD_DZ)) != ABS_OK) return r;
-        if ((r = tc_solve_t(h, K.jac, V(h, V_G), dl, st)) != ABS_OK) return r;
+        if (!tc) {
+            if ((r = solve_direction(h, K, x, rz, dz, dl, az, al, res, st)) != ABS_OK) return r;
+        } else {
+            dz_fast_kernel<<<gride(h), kThr, 0, st>>>((int)h->S, h->ld, view(h), V(h, V_P), V(h, V_Q), V(h, V_T),
+                                                      V(h, V_HQ), dz, V(h, V_G), two ? V(h, V_Q1) : nullptr,
+                                                      two ? V(h, V_HQ1) : nullptr);
+            if ((r = launch_check(h, KD_DZ)) != ABS_OK) return r;
+            if ((r = tc_solve_t(h, K.jac, V(h, V_G), dl, st)) != ABS_OK) return r;
+        }
     }
-    if (az) {   // (ctl_refine adds the design entries' steps)
+    if (az && (K.ldl || tc)) {   // (ctl_refine adds the design entries' steps)
         axpy2_kernel<<<gride(h), kThr, 0, st>>>((int)h->S, h->ld, view(h), dz, az, dl, al);
         if ((r = launch_check(h, KD_VEC)) != ABS_OK) return r;
     }
@@ -1674,8 +1677,7 @@ extern "C" abs_status kkt_newton_noalloc(const abs_params* p, int64_t S, int64_t
     const double dd = (hx[1] - beta) / Sd;
     CK(cudaMemcpyAsync(sol_x + od, &dd, sizeof(double), cudaMemcpyHostToDevice, st));
     cond_direction_kernel<CP_FP64><<<gs, CS_T, cond_smem(sizeof(double)), st>>>(
-        P, (int)S, ld, bv, fac, jac_vals, hess_vals, sigma, true, x, pv, rhs_x, sol_x, sol_c, nullptr, nullptr, false,
-        nullptr, nullptr, nullptr, nullptr, nullptr);
+        P, (int)S, ld, bv, fac, hess_vals, sigma, true, x, pv, rhs_x, sol_x, sol_c, nullptr, nullptr, nullptr);
     NA_LAUNCHED();
 #undef NA_LAUNCHED
     // dd lives on this stack frame until the copy above has completed

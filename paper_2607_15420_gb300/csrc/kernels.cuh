@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "model.cuh"
 
 namespace absorber {
@@ -325,6 +327,130 @@ __global__ void __launch_bounds__(EVAL_T) eval_split_kernel(const Params P, int 
     if (z == 0) eval_body<true, false, false>(P, S, ld, b, false, x, nullptr, nullptr, lam, feed, c, jac, hes, part);
     else if (z == 1) eval_body<false, true, false>(P, S, ld, b, false, x, nullptr, nullptr, lam, feed, c, jac, hes, part);
     else if (WH) eval_body<false, false, true>(P, S, ld, b, false, x, nullptr, nullptr, lam, feed, c, jac, hes, part);
+}
+
+// the stage pattern at compile time: Jacobian entries of a stage's own unknowns, and Hessian entries
+// (lower triangle)
+__host__ __device__ constexpr bool own_has(int r, int c) {
+    if (r < 11) {
+        if (r < 9 && (c == r || c == LL)) return true;
+        if (r >= 7 && (c == LY + r - 7 || c == LV)) return true;
+        return c >= LE && c < LE + 5 && nu(r, c - LE) != 0;
+    }
+    if (r == R_VH) return c == LY + 1 || c == 8 || c == LT;
+    if (r == R_VC) return c == LY || c == LT || (c < 9 && in_henry(c));
+    if (r >= R_RX && r < R_RX + 5) return c == LT || (c < 9 && nu(c, r - R_RX) != 0);
+    if (r == R_SX) return c < 9;
+    if (r == R_SY) return c >= LY && c < LY + 4;
+    if (r == R_E) return c <= LT;
+    return c == LV || c == LT || c == LS;
+}
+// row r reads the stage above's unknown a (of the 11) / the stage below's b (of the 6)
+__host__ __device__ constexpr bool abv_has(int r, int a) { return r == R_E || (r < 9 && (a == r || a == 9)); }
+__host__ __device__ constexpr bool blw_has(int r, int b) {
+    return r == R_E || (r >= 7 && r < 11 && (b == r - 7 || b == 4));
+}
+__host__ __device__ constexpr bool hes_has(int i, int j) {
+    if (i < 9) return j <= i && ((in_henry(i) && in_henry(j)) || i == j);
+    if (i == LL) return j < 9;
+    if (i == LV) return j >= LY && j < LY + 4;
+    return i == LT && j <= LT;
+}
+
+// The products J v and J^T y of a stage shared out over four warps, with 150 entries each: rows and
+// unknowns grouped so that every warp has 70 to 80 of the 300 multiply-adds, all of it unrolled code
+// at fixed places (no tables, no loops).
+constexpr int NGRP = 4;
+__host__ __device__ constexpr int row_grp(int r) {
+    return r == R_E || r == R_VH || r == R_SY ? 0 : (r == R_SX || r == R_VC || r == 7 || r == 8 ? 1 : (r < 7 ? 2 : 3));
+}
+__host__ __device__ constexpr int col_grp(int j) {
+    return j == LL || j == LV ? 0 : (j < 5 ? 1 : (j < 9 || j == LE || j == LE + 1 ? 2 : 3));
+}
+
+// where a (scenario, stage)'s Jacobian entries lie: its own stage's and its neighbours' segments
+struct StageJac {
+    const double *own, *below, *above;   // segments of stage n, n - 1, n + 1 at the scenario
+    int t, tb, ta;                       // their stage types
+    int64_t ld;
+    __device__ __forceinline__ StageJac(const double* __restrict__ jac, int64_t ld_, int s, int n) : ld(ld_) {
+        t = stage_type(n);
+        tb = n > 0 ? stage_type(n - 1) : 0;
+        ta = n + 1 < N_STAGES ? stage_type(n + 1) : 0;
+        own = jac + (int64_t)c_segJ[n] * ld + s;
+        below = jac + (int64_t)c_segJ[n > 0 ? n - 1 : 0] * ld + s;
+        above = jac + (int64_t)c_segJ[n + 1 < N_STAGES ? n + 1 : 0] * ld + s;
+    }
+    __device__ __forceinline__ double at(int r, int lv) const { return own[(int64_t)c_slotJ[t][r][lv] * ld]; }
+    __device__ __forceinline__ double at_below(int r, int lv) const { return below[(int64_t)c_slotJ[tb][r][lv] * ld]; }
+    __device__ __forceinline__ double at_above(int r, int lv) const { return above[(int64_t)c_slotJ[ta][r][lv] * ld]; }
+};
+
+// f(0), f(1), ... f(N - 1) with compile-time arguments
+template <int I, int N, class F>
+__device__ __forceinline__ void static_for(const F& f) {
+    if constexpr (I < N) {
+        f(std::integral_constant<int, I>{});
+        static_for<I + 1, N>(f);
+    }
+}
+
+// a <- a + sgn (J^T y)_j for unknown j of stage n; y a row vector
+template <int SGN, int j>
+__device__ __forceinline__ double jt_col(const StageJac& J, const double* __restrict__ y, int s, int n, double a) {
+    const double* yn = y + (int64_t)(NR * n) * J.ld + s;
+    static_for<0, NR>([&](auto R) {
+        constexpr int r = decltype(R)::value;
+        if constexpr (own_has(r, j)) a = fma(SGN * J.at(r, j), yn[(int64_t)r * J.ld], a);
+    });
+    static_for<0, NABV>([&](auto K) {
+        constexpr int k = decltype(K)::value;
+        if constexpr (abv_var(k) == j) {
+            if (n > 0) {
+                const double* yb = yn - (int64_t)NR * J.ld;
+                static_for<0, NR>([&](auto R) {
+                    constexpr int r = decltype(R)::value;
+                    if constexpr (abv_has(r, k)) a = fma(SGN * J.at_below(r, AX + k), yb[(int64_t)r * J.ld], a);
+                });
+            }
+        }
+    });
+    static_for<0, NBLW>([&](auto K) {
+        constexpr int k = decltype(K)::value;
+        if constexpr (blw_var(k) == j) {
+            if (n + 1 < N_STAGES) {
+                const double* ya = yn + (int64_t)NR * J.ld;
+                static_for<0, NR>([&](auto R) {
+                    constexpr int r = decltype(R)::value;
+                    if constexpr (blw_has(r, k)) a = fma(SGN * J.at_above(r, BY + k), ya[(int64_t)r * J.ld], a);
+                });
+            }
+        }
+    });
+    return a;
+}
+
+// a <- a - (J v)_r for row r of stage n; v a primal vector, vd the step of its section's diameter
+template <int r>
+__device__ __forceinline__ double jv_row(const StageJac& J, const double* __restrict__ v, double vd, int s, int n,
+                                         double a) {
+    const double* vn = v + (int64_t)(NV * n) * J.ld + s;
+    static_for<0, NV>([&](auto C) {
+        constexpr int j = decltype(C)::value;
+        if constexpr (own_has(r, j)) a = fma(-J.at(r, j), vn[(int64_t)j * J.ld], a);
+    });
+    if (n + 1 < N_STAGES)
+        static_for<0, NABV>([&](auto K) {
+            constexpr int k = decltype(K)::value;
+            if constexpr (abv_has(r, k)) a = fma(-J.at(r, AX + k), vn[(int64_t)(NV + abv_var(k)) * J.ld], a);
+        });
+    if (n > 0)
+        static_for<0, NBLW>([&](auto K) {
+            constexpr int k = decltype(K)::value;
+            if constexpr (blw_has(r, k)) a = fma(-J.at(r, BY + k), vn[(int64_t)(blw_var(k) - NV) * J.ld], a);
+        });
+    if constexpr (r == R_H) a = fma(-J.own[(int64_t)c_dslot[J.t] * J.ld], vd, a);
+    return a;
 }
 
 // ------------------------------------------------------------------------------------

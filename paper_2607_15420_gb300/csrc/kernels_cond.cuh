@@ -1177,49 +1177,16 @@ __global__ void __launch_bounds__(CS_T, 6) cond_solve_kernel(const Params P, int
     }
 }
 
-// Jacobian entries of a stage's own unknowns, and Hessian entries (lower triangle)
-__host__ __device__ constexpr bool own_has(int r, int c) {
-    if (r < 11) {
-        if (r < 9 && (c == r || c == LL)) return true;
-        if (r >= 7 && (c == LY + r - 7 || c == LV)) return true;
-        return c >= LE && c < LE + 5 && nu(r, c - LE) != 0;
-    }
-    if (r == R_VH) return c == LY + 1 || c == 8 || c == LT;
-    if (r == R_VC) return c == LY || c == LT || (c < 9 && in_henry(c));
-    if (r >= R_RX && r < R_RX + 5) return c == LT || (c < 9 && nu(c, r - R_RX) != 0);
-    if (r == R_SX) return c < 9;
-    if (r == R_SY) return c >= LY && c < LY + 4;
-    if (r == R_E) return c <= LT;
-    return c == LV || c == LT || c == LS;
-}
-// row r reads the stage above's unknown a (of the 11) / the stage below's b (of the 6)
-__host__ __device__ constexpr bool abv_has(int r, int a) { return r == R_E || (r < 9 && (a == r || a == 9)); }
-__host__ __device__ constexpr bool blw_has(int r, int b) {
-    return r == R_E || (r >= 7 && r < 11 && (b == r - 7 || b == 4));
-}
-__host__ __device__ constexpr bool hes_has(int i, int j) {
-    if (i < 9) return j <= i && ((in_henry(i) && in_henry(j)) || i == j);
-    if (i == LL) return j < 9;
-    if (i == LV) return j >= LY && j < LY + 4;
-    return i == LT && j <= LT;
-}
-
 // One block-elimination solve after its J^-1 r_c (pv) and Schur step (the steps of the design
 // entries in dz's slots): dz = p - q dtheta, g = r_z - (W + Sigma + dw I) dz, dl = J^-T g.  With az,
-// al (a correction) they are added to that direction; with res, the residual of the whole
-// direction dz, dl against (rz0, rc0) follows: rho_c = rc0 - J dz - b dtheta, rho_z = g - J^T dl_last
-// (the last solve's right-hand side less its products, by linearity), and partials [0]
-// max|rho_z| (NaN if any row's is), [1] max|rho_c|, [2] the stage's hydraulic dl, [3] max|rz0|, [4]
-// max|rc0| (two sections: [2] the first's, [5] the second's hydraulic dl).  A block holds its
-// scenarios' whole columns, so nothing leaves it between these steps: the right-hand side and the
-// step stay in registers, every Jacobian entry is read once for both products.  rho_z may be rz.
-// Grid ceil(S / CS_N), CS_T threads.
+// al (a correction) they are added to that direction.  g0 (optional): g, for the residual.  Grid
+// ceil(S / CS_N), CS_T threads.
 template <int PREC>
 __global__ void __launch_bounds__(CS_T, 6) cond_direction_kernel(
-    const Params P, int S, int64_t ld, const BView b, const CondFac K, const double* __restrict__ jac,
-    const double* __restrict__ hes, const double* __restrict__ sig, bool use_w, const double* x,
-    const double* __restrict__ pv, const double* rz, double* dzo, double* dlo, double* az, double* al, bool res,
-    const double* __restrict__ rz0, const double* __restrict__ rc0, double* rhoz, double* rhoc, double* part) {
+    const Params P, int S, int64_t ld, const BView b, const CondFac K, const double* __restrict__ hes,
+    const double* __restrict__ sig, bool use_w, const double* x, const double* __restrict__ pv,
+    const double* __restrict__ rz, double* dzo, double* __restrict__ dlo, double* __restrict__ az,
+    double* __restrict__ al, double* __restrict__ g0) {
     extern __shared__ __align__(16) unsigned char cond_sm[];
     const CondPlace at(S, b);
     const bool live = at.live;
@@ -1228,129 +1195,47 @@ __global__ void __launch_bounds__(CS_T, 6) cond_direction_kernel(
     if (!__syncthreads_or(live)) return;
     const int prc = pr >= 0 ? pr : 0;
     const int sec = stage_sec(n, P.nsec);
-    const int64_t od = (int64_t)NSC * ld + (int64_t)sec * b.NP + prc;
-    const double dd = dzo[od], dw = b.ps ? psv(b, PS_DW, prc) : 0.0;
-    double dz[NV], g[NV];
+    const double dd = dzo[(int64_t)NSC * ld + (int64_t)sec * b.NP + prc], dw = b.ps ? psv(b, PS_DW, prc) : 0.0;
+    double g[NV];
+    {
+        double dz[NV];
 #pragma unroll
-    for (int j = 0; j < NV; ++j) dz[j] = pv[(int64_t)(NV * n + j) * ld + s];
-    dz[LS] = fma(-slack_q(P, x, ld, sec, b.NP, prc), dd, dz[LS]);
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-        const int64_t o = (int64_t)(NV * n + j) * ld + s;
-        g[j] = fma(-(sig[o] + dw), dz[j], rz[o]);
-    }
-    if (use_w) {
-        const double* h = hes + (int64_t)(NHS * n) * ld + s;
-#pragma unroll
-        for (int i = 0; i < NV; ++i)
-#pragma unroll
-            for (int j = 0; j <= i; ++j)
-                if (hes_has(i, j)) {
-                    const double v = h[(int64_t)c_slotH[i][j] * ld];
-                    g[i] = fma(-v, dz[j], g[i]);
-                    if (i != j) g[j] = fma(-v, dz[i], g[j]);
-                }
-    }
-    double dl[NR];
-    cond_solve_t_prec<PREC>(K, ld, at, g, cond_sm, dl);
-    if (live) {
-        double* zt = az ? az : dzo;
+        for (int j = 0; j < NV; ++j) dz[j] = pv[(int64_t)(NV * n + j) * ld + s];
+        dz[LS] = fma(-slack_q(P, x, ld, sec, b.NP, prc), dd, dz[LS]);
 #pragma unroll
         for (int j = 0; j < NV; ++j) {
             const int64_t o = (int64_t)(NV * n + j) * ld + s;
-            if (az) dz[j] += az[o];
-            zt[o] = dz[j];
-            dlo[o] = dl[j];
+            g[j] = fma(-(sig[o] + dw), dz[j], rz[o]);
         }
-        if (al)
+        if (use_w) {
+            const double* h = hes + (int64_t)(NHS * n) * ld + s;
 #pragma unroll
-            for (int j = 0; j < NR; ++j) al[(int64_t)(NR * n + j) * ld + s] += dl[j];
-    }
-    if (!res) return;
-    __syncthreads();   // the block's columns of dz and dl are visible
-    if (!live) return;
-    const double* zt = az ? az : dzo;
-    double c[NR];
+            for (int i = 0; i < NV; ++i)
 #pragma unroll
-    for (int r = 0; r < NR; ++r) c[r] = rc0[(int64_t)(NR * n + r) * ld + s];
-    unsigned long long k3 = 0, k4 = 0;
+                for (int j = 0; j <= i; ++j)
+                    if (hes_has(i, j)) {
+                        const double v = h[(int64_t)c_slotH[i][j] * ld];
+                        g[i] = fma(-v, dz[j], g[i]);
+                        if (i != j) g[j] = fma(-v, dz[i], g[j]);
+                    }
+        }
+        if (live)
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-        k4 = key_max(k4, mag_key(c[r]));
-        k3 = key_max(k3, mag_key(rz0[(int64_t)(NV * n + r) * ld + s]));
-    }
-    const int t = stage_type(n);
-    const double* jn = jac + (int64_t)c_segJ[n] * ld + s;
-    {
-        const double ddt = dd + (az ? az[od] : 0.0);
-        c[R_H] = fma(-jn[(int64_t)c_dslot[t] * ld], ddt, c[R_H]);
-    }
-#pragma unroll
-    for (int r = 0; r < NR; ++r)
-#pragma unroll
-        for (int q = 0; q < NV; ++q)
-            if (own_has(r, q)) {
-                const double v = jn[(int64_t)c_slotJ[t][r][q] * ld];
-                c[r] = fma(-v, dz[q], c[r]);
-                g[q] = fma(-v, dl[r], g[q]);
+            for (int j = 0; j < NV; ++j) {
+                const int64_t o = (int64_t)(NV * n + j) * ld + s;
+                if (az) az[o] += dz[j];
+                else dzo[o] = dz[j];
+                if (g0) g0[o] = g[j];
             }
-    if (n + 1 < N_STAGES) {
-        // this stage's rows on the stage above's unknowns; the stage above's rows on this stage's
-        double z[NABV], l[NR];
-#pragma unroll
-        for (int a = 0; a < NABV; ++a) z[a] = zt[(int64_t)(NV * (n + 1) + abv_var(a)) * ld + s];
-        const int ta = stage_type(n + 1);
-        const double* ja = jac + (int64_t)c_segJ[n + 1] * ld + s;
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            l[r] = 0.0;
-            if (r == R_E || (r >= 7 && r < 11)) l[r] = dlo[(int64_t)(NR * (n + 1) + r) * ld + s];
-#pragma unroll
-            for (int a = 0; a < NABV; ++a)
-                if (abv_has(r, a)) c[r] = fma(-jn[(int64_t)c_slotJ[t][r][AX + a] * ld], z[a], c[r]);
-#pragma unroll
-            for (int q = 0; q < NBLW; ++q)
-                if (blw_has(r, q))
-                    g[blw_var(q)] = fma(-ja[(int64_t)c_slotJ[ta][r][BY + q] * ld], l[r], g[blw_var(q)]);
-        }
     }
-    if (n > 0) {
-        double z[NBLW], l[NR];
+    double dl[NR];
+    cond_solve_t_prec<PREC>(K, ld, at, g, cond_sm, dl);
+    if (!live) return;
 #pragma unroll
-        for (int q = 0; q < NBLW; ++q) z[q] = zt[(int64_t)(NV * (n - 1) + blw_var(q)) * ld + s];
-        const int tb = stage_type(n - 1);
-        const double* jb = jac + (int64_t)c_segJ[n - 1] * ld + s;
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            l[r] = 0.0;
-            if (r == R_E || r < 9) l[r] = dlo[(int64_t)(NR * (n - 1) + r) * ld + s];
-#pragma unroll
-            for (int q = 0; q < NBLW; ++q)
-                if (blw_has(r, q)) c[r] = fma(-jn[(int64_t)c_slotJ[t][r][BY + q] * ld], z[q], c[r]);
-#pragma unroll
-            for (int a = 0; a < NABV; ++a)
-                if (abv_has(r, a))
-                    g[abv_var(a)] = fma(-jb[(int64_t)c_slotJ[tb][r][AX + a] * ld], l[r], g[abv_var(a)]);
-        }
-    }
-    unsigned long long k0 = 0, k1 = 0;
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-        const int64_t o = (int64_t)(NV * n + j) * ld + s;
-        k0 = key_max(k0, mag_key(g[j]));
-        k1 = key_max(k1, mag_key(c[j]));
-        rhoz[o] = g[j];
-        rhoc[o] = c[j];
-    }
-    if (k1 > 0x7ff0000000000000ull) k0 = k1;   // a NaN of the rows makes [0] NaN
-    const double dlh = (al ? al : dlo)[(int64_t)(NR * n + R_H) * ld + s];
-    if (P.nsec == 1) {
-        const double w[5] = {key_double(k0), key_double(k1), dlh, key_double(k3), key_double(k4)};
-        store_partials<5>(w, part, ld, (int)s, n);
-    } else {
-        const double w[6] = {key_double(k0), key_double(k1), sec ? 0.0 : dlh, key_double(k3), key_double(k4),
-                             sec ? dlh : 0.0};
-        store_partials<6>(w, part, ld, (int)s, n);
+    for (int j = 0; j < NR; ++j) {
+        const int64_t o = (int64_t)(NR * n + j) * ld + s;
+        dlo[o] = dl[j];
+        if (al) al[o] += dl[j];
     }
 }
 

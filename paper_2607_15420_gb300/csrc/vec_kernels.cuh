@@ -57,7 +57,40 @@ __device__ __forceinline__ void group_combine(double (&v)[K], double (*sm)[NC][3
 // [0] max |J^T l - zL + zU|, [1] sum |lambda|, [2] sum |zL| + |zU|, [3] max and [4] min
 // complementarity product over bounded unknowns, [5] the stage's hydraulic multiplier
 // (two sections: [5] for the first section's stages, [6] for the second's, each 0 on the
-// other's).  QS threads per (scenario, stage); grid (ceil(S / QS_SCEN), N_STAGES), 128 threads.
+// other's).  Warp = group of unknowns (col_grp), lane = scenario; grid (ceil(S / QS_SCEN),
+// N_STAGES), 128 threads.
+template <int G>
+__device__ __forceinline__ void dual_group(const Params& P, int64_t ld, const StageJac& J,
+                                           const double* __restrict__ lam, const double* __restrict__ x,
+                                           const double* __restrict__ zL, const double* __restrict__ zU,
+                                           double* __restrict__ jtl, int s, int n, double (&v)[6]) {
+    unsigned long long k0 = 0;   // max |J^T l - zL + zU| as an integer key (NaN survives)
+    static_for<0, NV>([&](auto C) {
+        constexpr int j = decltype(C)::value;
+        if constexpr (col_grp(j) == G) {
+            const int64_t o = (int64_t)(NV * n + j) * ld + s;
+            const double gj = jt_col<1, j>(J, lam, s, n, 0.0);
+            jtl[o] = gj;
+            const double zl = zL[o], zu = zU[o];
+            k0 = key_max(k0, mag_key(gj - zl + zu));
+            v[1] += fabs(lam[o]);
+            v[2] += fabs(zl) + fabs(zu);
+            const double xv = x[o];
+            if constexpr (has_lo(j)) {
+                const double cp = zl * (xv - lo_of(P, j));
+                v[3] = fmax(v[3], cp);
+                v[4] = fmin(v[4], cp);
+            }
+            if constexpr (has_hi(j)) {
+                const double cp = zu * (hi_of(P, j) - xv);
+                v[3] = fmax(v[3], cp);
+                v[4] = fmin(v[4], cp);
+            }
+        }
+    });
+    v[0] = key_double(k0);
+}
+
 __global__ void __launch_bounds__(128) dual_kernel(const Params P, int S, int64_t ld, const BView b,
                                                    const double* __restrict__ jac, const double* __restrict__ lam,
                                                    const double* __restrict__ x, const double* __restrict__ zL,
@@ -70,29 +103,13 @@ __global__ void __launch_bounds__(128) dual_kernel(const Params P, int S, int64_
     const bool live = live_prob(b, s, S, PS_ACT) >= 0;
     double v[6] = {0.0, 0.0, 0.0, -INFINITY, INFINITY, 0.0};
     if (live) {
-        unsigned long long k0 = 0;   // max |J^T l - zL + zU| as an integer key (NaN survives)
-#pragma unroll 1
-        for (int j = q; j < NV; j += QS) {
-            const int64_t o = (int64_t)(NV * n + j) * ld + s;
-            const double gj = jt_one(ld, jac, lam, s, n, j);
-            jtl[o] = gj;
-            const double zl = zL[o], zu = zU[o];
-            k0 = key_max(k0, mag_key(gj - zl + zu));
-            v[1] += fabs(lam[o]);
-            v[2] += fabs(zl) + fabs(zu);
-            const double xv = x[o];
-            if (has_lo(j)) {
-                const double cp = zl * (xv - lo_of(P, j));
-                v[3] = fmax(v[3], cp);
-                v[4] = fmin(v[4], cp);
-            }
-            if (has_hi(j)) {
-                const double cp = zu * (hi_of(P, j) - xv);
-                v[3] = fmax(v[3], cp);
-                v[4] = fmin(v[4], cp);
-            }
+        const StageJac J(jac, ld, s, n);
+        switch (q) {
+            case 0: dual_group<0>(P, ld, J, lam, x, zL, zU, jtl, s, n, v); break;
+            case 1: dual_group<1>(P, ld, J, lam, x, zL, zU, jtl, s, n, v); break;
+            case 2: dual_group<2>(P, ld, J, lam, x, zL, zU, jtl, s, n, v); break;
+            default: dual_group<3>(P, ld, J, lam, x, zL, zU, jtl, s, n, v); break;
         }
-        v[0] = key_double(k0);
     }
     constexpr int ops[5] = {RMAX, RSUM, RSUM, RMAX, RMIN};
     group_combine<6, 5>(v, sm, ops);
@@ -258,9 +275,44 @@ __global__ void __launch_bounds__(128) dz_fast_kernel(int S, int64_t ld, const B
 // r' - H dz' (its right-hand side r' and solution dz', dl' -- the first solve, or the
 // last correction), rho_z = g - J^T dl' (r' is r_z or the previous residual, so this is
 // r_z - H dz - J^T dl for the accumulated dz, dl without forming H dz again).
-// partials: [0] max|rho_z|, [1] max|rho_c|, [2] the stage's hydraulic dl, [3] max|r_z|,
-// [4] max|r_c|.  cz (optional): a correction whose design entries are not in dz yet.  QS threads
-// per (scenario, stage).
+// partials: [0] max|rho_z| (NaN if any of the rows' is), [1] max|rho_c|, [2] the stage's hydraulic
+// dl, [3] max|r_z|, [4] max|r_c|.  cz (optional): a correction whose design entries are not in dz
+// yet.  Warp = group of rows and unknowns (row_grp, col_grp), lane = scenario.
+template <int G>
+__device__ __forceinline__ void residual_group(int64_t ld, const StageJac& J, const double* __restrict__ g,
+                                               const double* __restrict__ dlast, const double* __restrict__ dz,
+                                               double dd, const double* __restrict__ rz, const double* __restrict__ rc,
+                                               double* __restrict__ rhoz, double* __restrict__ rhoc, int s, int n,
+                                               double (&v)[5]) {
+    unsigned long long k0 = 0, k1 = 0, k3 = 0, k4 = 0;   // maxima of magnitudes as integer keys
+    static_for<0, NV>([&](auto C) {
+        constexpr int j = decltype(C)::value;
+        if constexpr (col_grp(j) == G) {
+            const int64_t o = (int64_t)(NV * n + j) * ld + s;
+            const double a = jt_col<-1, j>(J, dlast, s, n, g[o]);
+            rhoz[o] = a;
+            k0 = key_max(k0, mag_key(a));
+            k3 = key_max(k3, mag_key(rz[o]));
+        }
+    });
+    static_for<0, NR>([&](auto R) {
+        constexpr int r = decltype(R)::value;
+        if constexpr (row_grp(r) == G) {
+            const int64_t o = (int64_t)(NR * n + r) * ld + s;
+            const double r0 = rc[o];
+            const double c = jv_row<r>(J, dz, dd, s, n, r0);
+            rhoc[o] = c;
+            k1 = key_max(k1, mag_key(c));
+            k4 = key_max(k4, mag_key(r0));
+        }
+    });
+    if (k1 > 0x7ff0000000000000ull) k0 = k1;   // NaN
+    v[0] = key_double(k0);
+    v[1] = key_double(k1);
+    v[3] = key_double(k3);
+    v[4] = key_double(k4);
+}
+
 __global__ void __launch_bounds__(128) kkt_residual_kernel(int S, int64_t ld, const BView b,
                                                            const double* __restrict__ jac,
                                                            const double* __restrict__ g,
@@ -281,20 +333,13 @@ __global__ void __launch_bounds__(128) kkt_residual_kernel(int S, int64_t ld, co
     if (live) {
         const int64_t od = (int64_t)NSC * ld + (int64_t)sec * b.NP + pr;   // the stage's section
         const double dd = dz[od] + (cz ? cz[od] : 0.0);
-        bool bad = false;
-        for (int j = gq; j < NV; j += QS) {
-            const int64_t o = (int64_t)(NV * n + j) * ld + s;
-            const double a = g[o] - jt_one(ld, jac, dlast, s, n, j);
-            const double c = rc[o] - jv_one(ld, jac, dz, dd, s, n, j);
-            rhoz[o] = a;
-            rhoc[o] = c;
-            v[0] = fmax(v[0], fabs(a));
-            v[1] = fmax(v[1], fabs(c));
-            v[3] = fmax(v[3], fabs(rz[o]));
-            v[4] = fmax(v[4], fabs(rc[o]));
-            bad = bad || a != a || c != c;
+        const StageJac J(jac, ld, s, n);
+        switch (gq) {
+            case 0: residual_group<0>(ld, J, g, dlast, dz, dd, rz, rc, rhoz, rhoc, s, n, v); break;
+            case 1: residual_group<1>(ld, J, g, dlast, dz, dd, rz, rc, rhoz, rhoc, s, n, v); break;
+            case 2: residual_group<2>(ld, J, g, dlast, dz, dd, rz, rc, rhoz, rhoc, s, n, v); break;
+            default: residual_group<3>(ld, J, g, dlast, dz, dd, rz, rc, rhoz, rhoc, s, n, v); break;
         }
-        if (bad) v[0] = NAN;   // fmax skips a NaN: any NaN of the rows makes [0] NaN
     }
     constexpr int ops[5] = {RMAX, RMAX, RSUM, RMAX, RMAX};   // [2] is set below
     group_combine<5, 5>(v, sm, ops);
