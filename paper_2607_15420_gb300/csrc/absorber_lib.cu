@@ -466,7 +466,7 @@ struct abs_problem {
         double d = 0.0, dw = 0.0, dc = 0.0, Kdd = 0.0, A0 = 0.0, Q2 = 0.0, Sd = 0.0;
         bool ldl = false;            // factored by the block LDL^T (kernels_ldl.cuh)
     } fac;
-    double* ldl_inv = nullptr;       // [S][N_STAGES][44][44] inverses of the block LDL^T pivot blocks
+    double* ldl_inv = nullptr;       // [S][N_STAGES][990] inverses of the block LDL^T pivot blocks, packed
     Prof prof;
     int autotune = 1;                // tile autotuner on (options.autotune)
     int factor_tile = 0;             // forced FP32 factor shape (options.factor_tile; 0: none)
@@ -692,12 +692,10 @@ abs_status ensure_factor(abs_problem* h, int prec) {
     return ABS_OK;
 }
 
-// the block LDL^T's inverses (allocated on first use) and its kernels' shared memory
+// the block LDL^T's inverses (allocated on first use)
 abs_status ensure_ldl(abs_problem* h) {
     if (!h->ldl_inv) {
         CK(cudaMalloc(&h->ldl_inv, sizeof(double) * (size_t)LDL_BLOCK * N_STAGES * h->S));
-        CK(cudaFuncSetAttribute(ldl_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)LDL_FACTOR_SMEM));
     }
     return ABS_OK;
 }
@@ -1054,10 +1052,10 @@ abs_status kkt_factor_core(abs_problem* h, const KKTSys& K, const double* x, cud
         // [6] zero pivots, [5] scenarios with a zero pivot), then u = K_s^-1 [0; b] with
         // [0] A0 = -sum b^T u_l (so that S_d = K_dd + dw + A0), [1] 0, [4] the d-d entries
         if ((r = ensure_ldl(h)) != ABS_OK) return r;
-        ldl_factor_kernel<<<(unsigned)h->S, 32, LDL_FACTOR_SMEM, st>>>((int)h->S, h->ld, view(h), K.jac, K.hes, K.sig,
+        ldl_factor_kernel<<<(unsigned)h->S, LDL_T, 0, st>>>((int)h->S, h->ld, view(h), K.jac, K.hes, K.sig,
                                                                        K.use_w, h->ldl_inv, h->part);
         if ((r = launch_check(h, KD_FACTOR)) != ABS_OK) return r;
-        ldl_solve_kernel<<<(unsigned)h->S, 32, LDL_SOLVE_SMEM, st>>>((int)h->S, h->ld, view(h), K.jac, h->ldl_inv,
+        ldl_solve_kernel<<<(unsigned)h->S, LDL_T, 0, st>>>((int)h->S, h->ld, view(h), K.jac, h->ldl_inv,
                                                                      nullptr, nullptr, true, V(h, V_Q), V(h, V_QL),
                                                                      h->part, 0, -1.0, true,
                                                                      K.use_w ? K.hes : nullptr);
@@ -1112,7 +1110,7 @@ abs_status kkt_solve_launches(abs_problem* h, const KKTSys& K, const double* x, 
     const double* dlast = dl;
     if (K.ldl) {
         // v = K_s^-1 [rz; rc] into dz, dl with [2] b^T v_l ([3] zero), dd, then x = v - u dd
-        ldl_solve_kernel<<<(unsigned)h->S, 32, LDL_SOLVE_SMEM, st>>>((int)h->S, h->ld, view(h), K.jac, h->ldl_inv,
+        ldl_solve_kernel<<<(unsigned)h->S, LDL_T, 0, st>>>((int)h->S, h->ld, view(h), K.jac, h->ldl_inv,
                                                                      rz, rc, false, dz, dl, h->part, 2, 1.0, false,
                                                                      nullptr);
         if ((r = launch_check(h, KD_SOLVE)) != ABS_OK) return r;
@@ -1155,7 +1153,7 @@ abs_status kkt_solve_launches(abs_problem* h, const KKTSys& K, const double* x, 
     const double* zt = az ? az : dz;
     const double* lt = al ? al : dl;
     if (K.ldl)
-        kkt_residual_reg_kernel<<<dim3((unsigned)((h->S + 127) / 128), N_STAGES), 128, 0, st>>>(
+        kkt_residual_reg_kernel<<<gridq(h), kThr, 0, st>>>(
             (int)h->S, h->ld, view(h), K.jac, K.hes, K.sig, K.use_w, zt, lt, az ? dz : nullptr, rz0, rc0, V(h, V_RHOZ),
             V(h, V_RHOC), h->part);
     else

@@ -456,59 +456,6 @@ __device__ __forceinline__ double jv_row(const StageJac& J, const double* __rest
 // ------------------------------------------------------------------------------------
 // sparse products with the stage-structured Jacobian / Hessian
 // ------------------------------------------------------------------------------------
-// (J^T y)_j for unknown j of stage n: rows of stage n (own entries), of stage n-1 (their
-// stream-from-above entries) and of stage n+1 (stream-from-below), in a fixed order
-__device__ __forceinline__ double jt_one(int64_t ld, const double* __restrict__ jac, const double* __restrict__ y, int s,
-                                int n, int j) {
-    const int t = stage_type(n);
-    const int base = c_segJ[n];
-    double a = 0.0;
-    for (int k = c_ownCp[t][j]; k < c_ownCp[t][j + 1]; ++k) {
-        const Ent e = c_ownC[t][k];
-        a += jac[(int64_t)(base + e.slot) * ld + s] * y[(int64_t)(NR * n + e.r) * ld + s];
-    }
-    if (n > 0) {
-        const int tb = stage_type(n - 1), bb = c_segJ[n - 1];
-        for (int k = c_abvCp[tb][j]; k < c_abvCp[tb][j + 1]; ++k) {
-            const Ent e = c_abvC[tb][k];
-            a += jac[(int64_t)(bb + e.slot) * ld + s] * y[(int64_t)(NR * (n - 1) + e.r) * ld + s];
-        }
-    }
-    if (n + 1 < N_STAGES) {
-        const int ta = stage_type(n + 1), ba = c_segJ[n + 1];
-        for (int k = c_blwCp[ta][j]; k < c_blwCp[ta][j + 1]; ++k) {
-            const Ent e = c_blwC[ta][k];
-            a += jac[(int64_t)(ba + e.slot) * ld + s] * y[(int64_t)(NR * (n + 1) + e.r) * ld + s];
-        }
-    }
-    return a;
-}
-
-// (J v)_r for row r of stage n; v a primal vector, vd the step of the stage's section
-// diameter (the hydraulic row's d column)
-__device__ __forceinline__ double jv_one(int64_t ld, const double* __restrict__ jac, const double* __restrict__ v, double vd,
-                                int s, int n, int r) {
-    const int t = stage_type(n);
-    const int base = c_segJ[n];
-    double a = 0.0;
-    for (int k = c_ownRp[t][r]; k < c_ownRp[t][r + 1]; ++k) {
-        const Ent e = c_own[t][k];
-        a += jac[(int64_t)(base + e.slot) * ld + s] * v[(int64_t)(NV * n + e.c) * ld + s];
-    }
-    if (n + 1 < N_STAGES)
-        for (int k = c_abvRp[t][r]; k < c_abvRp[t][r + 1]; ++k) {
-            const Ent e = c_abv[t][k];
-            a += jac[(int64_t)(base + e.slot) * ld + s] * v[(int64_t)(NV * (n + 1) + abv_var(e.c)) * ld + s];
-        }
-    if (n > 0)
-        for (int k = c_blwRp[t][r]; k < c_blwRp[t][r + 1]; ++k) {
-            const Ent e = c_blw[t][k];
-            a += jac[(int64_t)(base + e.slot) * ld + s] * v[(int64_t)(NV * (n - 1) + blw_var(e.c)) * ld + s];
-        }
-    if (r == R_H) a += jac[(int64_t)(base + c_dslot[t]) * ld + s] * vd;
-    return a;
-}
-
 // ((W + Sigma + dw I) v)_j for unknown j of stage n (W block diagonal by stage);
 // use_w = false gives (Sigma + dw I) v
 __device__ __forceinline__ double hv_one(int64_t ld, const double* __restrict__ hes, const double* __restrict__ sig,
