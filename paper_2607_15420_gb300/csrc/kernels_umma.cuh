@@ -1,22 +1,12 @@
-// kernels_umma.cuh -- the warm-start network's forward products on the fifth-generation
-// tensor cores (tcgen05, kind::f16), accumulators in tensor memory.
+// kernels_umma.cuh -- tcgen05 (fifth-generation tensor core) building blocks of the warm-start
+// network's forward pass (network_forward_kernel, mlp_lib.cu): kind::f16 MMAs on shared-memory
+// operands in the no-swizzle K-major core-matrix layout, FP32 accumulators in tensor memory,
+// mbarriers, bulk copies.
 //
-// C[m][n] = sum_k A[m][k] W[n][k] for the layers with K a multiple of 64 (the 256-wide
-// ones): A FP32 row-major [M][K] (the previous layer's activations), W bfloat16 row-major
-// [N][K] (the layer's rounded weights), FP32 accumulation.  An MMA takes both operands in
-// one type, so each FP32 activation enters as the sum of three bfloat16 terms
-// a = h + m + l (h the rounding of a, m of a - h, l of a - h - m: 24 significand bits),
-// and the three products with the bfloat16 weight are exact in the FP32 accumulator: the
-// layer's product at FP32 accuracy from three MMAs per K step.
-//
-// Block: 256 threads; tile 128 rows x 64 columns; K in chunks of 64 staged in shared
-// memory by the threads (FP32 loads, the split, 8-byte stores) in the no-swizzle K-major
-// layout of 8-row x 16-byte core matrices, each half-warp filling whole core matrices (no
-// bank conflicts).  One thread issues the chunk's 12 MMAs (4 K steps x 3 terms) and
-// commits them to an mbarrier; every thread waits on it (bounded) before the chunk's
-// shared memory is refilled.  The accumulator (128 lanes x 64 FP32 columns of tensor
-// memory) is read back by tcgen05.ld -- warp w its lanes 32 (w % 4) + 0..31 = its rows,
-// columns 32 (w / 4) + 0..31 -- for the fused epilogue.
+// An MMA takes both operands in one type and the weights are bfloat16, so each FP32 activation
+// enters as the sum of three bfloat16 terms a = h + m + l (h the rounding of a, m of a - h, l of
+// a - h - m: 24 significand bits); the three products with a bfloat16 weight are exact in the FP32
+// accumulator: a layer's product at FP32 accuracy from three MMAs per K step.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -24,19 +14,13 @@
 
 namespace umma {
 
-constexpr int TM = 128, TN = 64, KC = 64, T = 256;
-constexpr int A_PLANE = TM * KC * 2;              // one bfloat16 term of the A chunk: 16 KB
-constexpr int B_BYTES = TN * KC * 2;              // the W chunk: 8 KB
-// dynamic shared memory: the chunk (56 KB) + 1 KB alignment slack; at most three blocks
-// per SM, 192 of the 512 tensor-memory columns
-constexpr int SMEM = 3 * A_PLANE + B_BYTES + 1024;
-// core-matrix strides (bytes): A [kc][16 row groups], B [kc][8 row groups]; adjacent
-// core matrices along K ("leading") and along M / N ("stride")
-constexpr uint32_t A_LBO = (TM / 8) * 128, A_SBO = 128, B_LBO = (TN / 8) * 128, B_SBO = 128;
-constexpr long long WAIT_LIMIT = 1ll << 22;      // mbarrier polls before a wait gives up
-static_assert(TM == 128 && TN % 16 == 0 && TN >= 32 && TN <= 256 && (TN & (TN - 1)) == 0,
-              "an M = 128 MMA shape; tensor-memory columns a power of two >= 32");
-static_assert((TM * KC / 4) % T == 0 && (TN * KC / 8) % T == 0 && (TN / 2) % 16 == 0, "staging and epilogue split");
+constexpr int TM = 64, TN = 64, TK = 256;         // a block's rows; a weight chunk's columns; inputs
+constexpr int TILE_BYTES = TM * TK * 2;           // one bfloat16 term of the activations; a weight chunk
+// core matrices are 8 rows x 16 bytes; 8 row groups per 8-column K block: strides in bytes between core
+// matrices adjacent along K ("leading") and along M / N ("stride")
+constexpr uint32_t LBO = (TM / 8) * 128, SBO = 128;
+constexpr long long WAIT_LIMIT = 1ll << 22;       // mbarrier polls before a wait gives up
+static_assert(TM == TN, "activations and weight chunks share one layout");
 
 // instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A and B bfloat16 (bits 7-9,
 // 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at bit 17, M >> 4 at bit 24
@@ -100,25 +84,38 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, long l
     return false;
 }
 
-// 16 consecutive accumulator columns of this thread's lane (32x32b shape: lane = row)
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
+__device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint32_t mbar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
+}
+// bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) to shared memory; its
+// arrival completes on mbar
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+        "r"(bytes), "r"(mbar)
         : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// byte offset of element (r, k) of a K-major chunk in core-matrix layout with `groups`
-// 8-row groups per 8-column K block
-__device__ __forceinline__ uint32_t core_off(int r, int k, int groups) {
-    return (uint32_t)((((k >> 3) * groups + (r >> 3)) << 7) + ((r & 7) << 4) + ((k & 7) << 1));
+// 16 accumulator columns of 16 rows over the warp (16x256b shape): thread t gets, for i < 2, columns 8 i
+// + 2 (t % 4) + {0, 1} of row t / 4 in v[4 i + {0, 1}] and of row t / 4 + 8 in v[4 i + {2, 3}].  An M = 64
+// accumulator keeps rows 16 w .. 16 w + 15 in the first 16 lanes of the 32 that warp w (mod 4) reads.
+__device__ __forceinline__ void tmem_ld_16x16(uint32_t taddr, float (&v)[8]) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// byte offset of element (r, k) of a 64-row tile in core-matrix layout
+__device__ __forceinline__ uint32_t core_off(int r, int k) {
+    return (uint32_t)((((k >> 3) * (TM / 8) + (r >> 3)) << 7) + ((r & 7) << 4) + ((k & 7) << 1));
 }
 
 __device__ __forceinline__ uint32_t pack2(__nv_bfloat16 a, __nv_bfloat16 b) {

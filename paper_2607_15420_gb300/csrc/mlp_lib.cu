@@ -18,7 +18,6 @@
 #include <cstdint>
 #include <cstring>
 #include <string>
-#include <type_traits>
 #include <vector>
 
 #include "absorber.h"
@@ -29,12 +28,13 @@ namespace {
 constexpr int NIN = ABS_MLP_IN, NH = ABS_MLP_HIDDEN, NOUT = ABS_MLP_OUT;
 constexpr int64_t NPAR = ABS_MLP_PARAMS;
 // layer l: fan-in, fan-out, offsets of W_l ([out][in], row-major) and b_l in the flat vector
-constexpr int L_IN[4] = {NIN, NH, NH, NH};
-constexpr int L_OUT[4] = {NH, NH, NH, NOUT};
-constexpr int64_t OFF_W[4] = {0, NIN * NH + NH, NIN * NH + NH + NH * NH + NH,
-                              NIN * NH + NH + 2 * (NH * NH + NH)};
-constexpr int64_t OFF_B[4] = {OFF_W[0] + NIN * NH, OFF_W[1] + NH * NH, OFF_W[2] + NH * NH, OFF_W[3] + NH * NOUT};
-static_assert(OFF_B[3] + NOUT == NPAR, "parameter layout");
+__host__ __device__ constexpr int l_in(int l) { return l == 0 ? NIN : NH; }
+__host__ __device__ constexpr int l_out(int l) { return l == 3 ? NOUT : NH; }
+__host__ __device__ constexpr int64_t off_w(int l) { return l == 0 ? 0 : off_w(l - 1) + l_in(l - 1) * l_out(l - 1) + l_out(l - 1); }
+__host__ __device__ constexpr int64_t off_b(int l) { return off_w(l) + l_in(l) * l_out(l); }
+static_assert(off_b(3) + NOUT == NPAR, "parameter layout");
+static_assert(off_w(1) % 4 == 0 && off_w(2) % 4 == 0 && off_w(3) % 4 == 0 && NH % 4 == 0 && NOUT % 4 == 0,
+              "four consecutive weights of layers 2-4 are read and written together");
 
 constexpr int CHUNK_ROWS = 8192;   // inference rows per pass (bounds the activation workspace)
 
@@ -46,6 +46,7 @@ struct abs_mlp {
     int dev = 0;
     float* theta = nullptr;          // FP32 master parameters [NPAR]
     __nv_bfloat16* wb = nullptr;     // bfloat16 copies at the same offsets (weights only are read)
+    __nv_bfloat16* wt = nullptr;     // W2..W4's again as 64 x 256 tiles in the tensor cores' layout
     float* grad = nullptr;           // [NPAR]
     float* m = nullptr;              // Adam moments [NPAR]
     float* v = nullptr;
@@ -103,28 +104,39 @@ __device__ __forceinline__ float gelu_prime_f(float x) {
     return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
 }
 
-__device__ __forceinline__ float ld_el(const float* p, int64_t i) { return p[i]; }
-__device__ __forceinline__ float ld_el(const __nv_bfloat16* p, int64_t i) { return __bfloat162float(p[i]); }
+// the 64-output tiles of W2, W3 (four each) and W4 (seven, the last one padded with zeros)
+constexpr int NCHUNK = 4 + 4 + 7;
+constexpr int CHUNK_ELS = umma::TILE_BYTES / 2;
+// where weight i of the flat parameters lies in wt (-1: W1 or a bias)
+__device__ __forceinline__ int tile_index(int64_t i) {
+#pragma unroll
+    for (int l = 1; l < 4; ++l) {
+        const int64_t e = i - off_w(l);
+        if (e >= 0 && e < (int64_t)l_out(l) * NH) {
+            const int o = (int)(e / NH), k = (int)(e % NH);
+            return ((l - 1) * 4 + o / umma::TN) * CHUNK_ELS + (int)(umma::core_off(o % umma::TN, k) >> 1);
+        }
+    }
+    return -1;
+}
 
-enum { EPI_STORE = 0, EPI_BIAS_GELU = 1, EPI_BIAS = 2, EPI_GELU_GRAD = 3, EPI_DENORM = 4 };
+enum { EPI_BIAS_GELU = 1, EPI_BIAS = 2, EPI_DENORM = 4 };
 
 constexpr int BM = 64, BN = 64, BK = 16, GT = 256;
 
-// C[m][n] = sum_k A(m, k) B(k, n) with A(m, k) = A[m sam + k sak] and
-// B(k, n) = B[k sbk + n sbn]; 64x64 tile per block, 4x4 outputs per thread, K in steps
-// of 16 staged in shared memory.  Epilogues:
-//   EPI_STORE      C = acc
+// C[m][n] = sum_k A[m][k] W[n][k] on the CUDA cores (the first layer, and every layer with the tensor
+// cores switched off): A FP32 [M][K], W bfloat16 [N][K]; 64x64 tile per block, 4x4 outputs per
+// thread, K in steps of 16 staged in shared memory.  Epilogues:
 //   EPI_BIAS_GELU  Z = acc + bias[n] (stored), C = gelu(Z)
 //   EPI_BIAS       C = acc + bias[n]
-//   EPI_GELU_GRAD  C = acc * gelu'(aux[m][n])
 //   EPI_DENORM     C = (acc + bias[n]) * scale[n] + shift[n]
-// Row-major C, Z and aux with leading dimension ldc = N.
-template <class TB, int EPI>
-__global__ void __launch_bounds__(GT) gemm_kernel(int M, int N, int K, const float* __restrict__ A, int64_t sam,
-                                                  int64_t sak, const TB* __restrict__ B, int64_t sbk, int64_t sbn,
-                                                  const float* __restrict__ bias, const float* __restrict__ aux,
-                                                  float* __restrict__ Z, float* __restrict__ C,
-                                                  const float* __restrict__ scale, const float* __restrict__ shift) {
+// Row-major C and Z with leading dimension N.
+template <int EPI>
+__global__ void __launch_bounds__(GT) gemm_kernel(int M, int N, int K, const float* __restrict__ A,
+                                                  const __nv_bfloat16* __restrict__ W,
+                                                  const float* __restrict__ bias, float* __restrict__ Z,
+                                                  float* __restrict__ C, const float* __restrict__ scale,
+                                                  const float* __restrict__ shift) {
     __shared__ __align__(16) float As[BK][BM + 4];
     __shared__ __align__(16) float Bs[BK][BN + 4];
     const int tid = threadIdx.x;
@@ -135,35 +147,18 @@ __global__ void __launch_bounds__(GT) gemm_kernel(int M, int N, int K, const flo
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
-    const bool a_kfast = sak == 1, b_nfast = sbn == 1;
     for (int k0 = 0; k0 < K; k0 += BK) {
 #pragma unroll
         for (int r = 0; r < (BM * BK) / GT; ++r) {
-            const int e = tid + r * GT;
-            int mm, kk;
-            if (a_kfast) {
-                mm = e / BK;
-                kk = e % BK;
-            } else {
-                kk = e / BM;
-                mm = e % BM;
-            }
+            const int e = tid + r * GT, mm = e / BK, kk = e % BK;
             const int gm = m0 + mm, gk = k0 + kk;
-            As[kk][mm] = (gm < M && gk < K) ? A[(int64_t)gm * sam + (int64_t)gk * sak] : 0.0f;
+            As[kk][mm] = (gm < M && gk < K) ? A[(int64_t)gm * K + gk] : 0.0f;
         }
 #pragma unroll
         for (int r = 0; r < (BN * BK) / GT; ++r) {
-            const int e = tid + r * GT;
-            int nn, kk;
-            if (b_nfast) {
-                kk = e / BN;
-                nn = e % BN;
-            } else {
-                nn = e / BK;
-                kk = e % BK;
-            }
+            const int e = tid + r * GT, nn = e / BK, kk = e % BK;
             const int gn = n0 + nn, gk = k0 + kk;
-            Bs[kk][nn] = (gn < N && gk < K) ? ld_el(B, (int64_t)gk * sbk + (int64_t)gn * sbn) : 0.0f;
+            Bs[kk][nn] = (gn < N && gk < K) ? __bfloat162float(W[(int64_t)gn * K + gk]) : 0.0f;
         }
         __syncthreads();
 #pragma unroll
@@ -188,198 +183,277 @@ __global__ void __launch_bounds__(GT) gemm_kernel(int M, int N, int K, const flo
             const int gn = n0 + tc * 4 + j;
             if (gn >= N) continue;
             const int64_t o = (int64_t)gm * N + gn;
-            float vv = acc[i][j];
+            float vv = acc[i][j] + bias[gn];
             if (EPI == EPI_BIAS_GELU) {
-                vv += bias[gn];
                 Z[o] = vv;
                 vv = gelu_f(vv);
-            } else if (EPI == EPI_BIAS) {
-                vv += bias[gn];
-            } else if (EPI == EPI_GELU_GRAD) {
-                vv *= gelu_prime_f(aux[o]);
             } else if (EPI == EPI_DENORM) {
-                vv = (vv + bias[gn]) * scale[gn] + shift[gn];
+                vv = vv * scale[gn] + shift[gn];
             }
             C[o] = vv;
         }
     }
 }
 
-// The forward products on the tensor cores (kernels_umma.cuh): A FP32 [M][K] row-major, W
-// bfloat16 [N][K] row-major, K a multiple of 64; epilogues EPI_BIAS_GELU, EPI_BIAS,
-// EPI_DENORM as gemm_kernel's.  Grid (ceil(N / 64), ceil(M / 128)), 128 threads,
-// umma::SMEM bytes of dynamic shared memory.  fault: set when a wait for the MMAs gave up
-// (the block then frees its tensor memory and leaves its outputs unwritten).  idle (the
-// self-test of that path): no MMA and no commit are issued, so the first wait runs out
-// after wait_limit polls.
 template <int EPI>
-__global__ void __launch_bounds__(umma::T) gemm_tc_kernel(int M, int N, int K, const float* __restrict__ A,
-                                                          const __nv_bfloat16* __restrict__ W,
-                                                          const float* __restrict__ bias, float* __restrict__ Z,
-                                                          float* __restrict__ C, const float* __restrict__ scale,
-                                                          const float* __restrict__ shift, int* __restrict__ fault,
-                                                          int idle, long long wait_limit) {
+abs_status gemm(abs_mlp* net, cudaStream_t st, int M, int N, int K, const float* A, const __nv_bfloat16* W, float* C,
+                const float* bias, float* Z = nullptr, const float* scale = nullptr, const float* shift = nullptr) {
+    if (M <= 0 || N <= 0) return ABS_OK;
+    const dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM));
+    gemm_kernel<EPI><<<grid, GT, 0, st>>>(M, N, K, A, W, bias, Z, C, scale, shift);
+    return mlaunch(net);
+}
+
+// The whole forward pass of 64 rows per block, the products of layers 2-4 on the tensor cores
+// (kernels_umma.cuh).  The activations stay on chip: their three bfloat16 terms in shared memory
+// (96 KB), the weights streaming past them in 15 chunks of 64 outputs (32 KB each, bulk copies of the
+// tiled weights wt into a ring of three), the accumulators in two tensor-memory buffers of 64
+// columns.  Warps 0-15: the layers' biases and GELU and the split into terms, a 16-row x 16-column piece
+// of every chunk each, while the next chunk's MMAs run; a layer's activations are kept in registers until
+// its last MMA has read the previous ones.  Warp 16: one thread loads the chunks and issues the 48
+// MMAs of each (16 K steps x 3 terms).  Biases, scales and W1 wait in shared memory: with four warps per
+// scheduler and no global loads between a chunk's sums and its activations, the arithmetic of GELU and
+// split, about 36 instructions per activation, bounds the pass.
+// TRAIN: also a0, the pre-activations z and activations a of the layers, and normalised outputs;
+// otherwise outputs de-normalised.  vec: Y allows 8-byte stores.  Every wait is bounded (wait_limit
+// polls); when one gives up the block sets fault and leaves, its outputs unwritten.  idle (the
+// self-test of that path): no MMA is issued.
+constexpr int FWD_E = 512, FWD_T = FWD_E + 32;
+// constants in shared memory (floats): biases of layers 1-4, output shift and scale, W1
+constexpr int FC_B = 0, FC_OUT = 3 * NH + NOUT, FC_W1 = FC_OUT + 2 * NOUT, FC_COUNT = FC_W1 + NIN * NH;
+constexpr int FWD_SMEM = 6 * umma::TILE_BYTES + 4 * FC_COUNT + 1024;
+static_assert(FWD_SMEM <= 227 * 1024, "shared memory of a block");
+struct FwdTrain {
+    float *a0, *z[3], *a[3];
+};
+template <bool TRAIN>
+__global__ void __launch_bounds__(FWD_T, 1) network_forward_kernel(int M, const float* __restrict__ X,
+                                                                   const float* __restrict__ norm,
+                                                                   const float* __restrict__ theta,
+                                                                   const __nv_bfloat16* __restrict__ wb,
+                                                                   const __nv_bfloat16* __restrict__ wt,
+                                                                   float* __restrict__ Y, const FwdTrain tr, bool vec,
+                                                                   int* __restrict__ fault, int idle,
+                                                                   long long wait_limit) {
     using namespace umma;
     extern __shared__ unsigned char tc_smem[];
-    __shared__ __align__(8) uint64_t mbar;
+    __shared__ __align__(8) uint64_t bars[3 + 2 + 2 + 1];
     __shared__ uint32_t tbase;
     unsigned char* sm = (unsigned char*)(((uintptr_t)tc_smem + 1023) & ~(uintptr_t)1023);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-    const uint32_t sa = smem_u32(sm), sb = sa + 3 * A_PLANE, mb = smem_u32(&mbar);
+    const int m0 = blockIdx.x * TM;
+    const uint32_t sa = smem_u32(sm), sw = sa + 3 * TILE_BYTES;
+    const uint32_t wfull = smem_u32(&bars[0]), mdone = smem_u32(&bars[3]), tfree = smem_u32(&bars[5]),
+                   aready = smem_u32(&bars[7]);
     if (warp == 0) {
-        tmem_alloc(smem_u32(&tbase), TN);
+        tmem_alloc(smem_u32(&tbase), 2 * TN);
         tmem_relinquish();
     }
-    if (tid == 0) mbar_init(mb, 1);
+    if (tid == 0) {
+        for (int i = 0; i < 3; ++i) mbar_init(wfull + 8 * i, 1);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(mdone + 8 * i, 1);
+            mbar_init(tfree + 8 * i, FWD_E);
+        }
+        mbar_init(aready, FWD_E);
+    }
+    float* fc = reinterpret_cast<float*>(sm + 6 * TILE_BYTES);
+    for (int i = tid; i < FC_COUNT; i += FWD_T) {
+        float f;
+        if (i < FC_OUT) f = theta[i < 3 * NH ? (i < NH ? off_b(0) + i : (i < 2 * NH ? off_b(1) + i - NH : off_b(2) + i - 2 * NH))
+                                             : off_b(3) + i - 3 * NH];
+        else if (i < FC_W1) f = norm[2 * NIN + i - FC_OUT];
+        else f = __bfloat162float(wb[off_w(0) + i - FC_W1]);
+        fc[i] = f;
+    }
     fence_before();
     __syncthreads();
     fence_after();
     const uint32_t tmem = tbase;
     bool ok = true;
-    for (int c = 0; c < K / KC; ++c) {
-        const int k0 = c * KC;
-        // A chunk: 128 x 64 FP32 as float4, W chunk: 64 x 64 bfloat16 as 16-byte rows of core
-        // matrices; every load in flight before the first store.  Float4 e of the A chunk
-        // fills half a row of core matrix cm = e / 16 (row group cm / 8, K block cm % 8) and
-        // W's row v of core matrix v / 8 (row group (v / 8) / 8, K block (v / 8) % 8): a
-        // half-warp's stores cover whole 128-byte core matrices.  A is split into its three
-        // bfloat16 terms (8-byte stores into the three term planes)
-        constexpr int NA = (TM * KC / 4) / T, NB = (TN * KC / 8) / T;
-        float4 av[NA];
-        uint4 wv[NB];
-#pragma unroll
-        for (int i = 0; i < NA; ++i) {
-            const int e = i * T + tid, cm = e >> 4, q = e & 15;
-            const int r = ((cm >> 3) << 3) + (q >> 1), k = ((cm & 7) << 3) + ((q & 1) << 2);
-            av[i] = m0 + r < M ? *reinterpret_cast<const float4*>(A + (int64_t)(m0 + r) * K + k0 + k)
-                               : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int i = 0; i < NB; ++i) {
-            const int v = i * T + tid, cm = v >> 3;
-            const int n = ((cm >> 3) << 3) + (v & 7), k = (cm & 7) << 3;
-            wv[i] = n0 + n < N ? *reinterpret_cast<const uint4*>(W + (int64_t)(n0 + n) * K + k0 + k)
-                               : make_uint4(0u, 0u, 0u, 0u);
-        }
-#pragma unroll
-        for (int i = 0; i < NA; ++i) {
-            const int e = i * T + tid, cm = e >> 4, q = e & 15;
-            const int r = ((cm >> 3) << 3) + (q >> 1), k = ((cm & 7) << 3) + ((q & 1) << 2);
-            const float a4[4] = {av[i].x, av[i].y, av[i].z, av[i].w};
-            __nv_bfloat16 t[3][4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const __nv_bfloat16 h = __float2bfloat16_rn(a4[j]);
-                const float r1 = a4[j] - __bfloat162float(h);
-                const __nv_bfloat16 m = __float2bfloat16_rn(r1);
-                t[0][j] = h;
-                t[1][j] = m;
-                t[2][j] = __float2bfloat16_rn(r1 - __bfloat162float(m));
-            }
-            const uint32_t o = core_off(r, k, TM / 8);
-#pragma unroll
-            for (int p = 0; p < 3; ++p)
-                *reinterpret_cast<uint2*>(sm + p * A_PLANE + o) = make_uint2(pack2(t[p][0], t[p][1]), pack2(t[p][2], t[p][3]));
-        }
-#pragma unroll
-        for (int i = 0; i < NB; ++i) {
-            const int v = i * T + tid, cm = v >> 3;
-            const int n = ((cm >> 3) << 3) + (v & 7), k = (cm & 7) << 3;
-            *reinterpret_cast<uint4*>(sm + 3 * A_PLANE + core_off(n, k, TN / 8)) = wv[i];
-        }
-        fence_smem_async();
-        __syncthreads();
-        if (tid == 0 && !idle) {
-            fence_after();
-#pragma unroll
-            for (int s = 0; s < KC / 16; ++s)
-#pragma unroll
-                for (int p = 0; p < 3; ++p)
-                    mma(tmem, desc(sa + p * A_PLANE + s * 2 * (TM / 8) * 128, A_LBO, A_SBO),
-                        desc(sb + s * 2 * (TN / 8) * 128, B_LBO, B_SBO), IDESC, (c | s | p) != 0);
-            commit(mb);
-        }
-        // the chunk's MMAs are done before its shared memory is refilled
-        ok = __syncthreads_and(ok && mbar_wait(mb, (uint32_t)(c & 1), wait_limit));
-        if (!ok) break;
-        fence_after();
-    }
-    if (ok) {
-        // accumulator rows + bias into a padded shared tile over the A planes (the MMAs are
-        // done): warp w its lanes (rows) 32 (w % 4) + 0..31, columns TN / 2 (w / 4) + ...
-        // Then rows written with the lanes along the columns (coalesced), the epilogue's
-        // nonlinearity on the way
-        constexpr int LDS = TN + 1;
-        float* tile = reinterpret_cast<float*>(sm);
-        const int q4 = warp & 3, ch = warp >> 2;
-        const int r = q4 * 32 + lane;
-#pragma unroll
-        for (int cb = ch * (TN / 2); cb < (ch + 1) * (TN / 2); cb += 16) {
-            float v[16];
-            tmem_ld16(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)cb, v);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int gn = n0 + cb + j;
-                tile[r * LDS + cb + j] = v[j] + (gn < N ? bias[gn] : 0.0f);
-            }
-        }
-        __syncthreads();
-        for (int rr = warp; rr < TM; rr += T / 32) {
-            const int row = m0 + rr;
-            if (row >= M) break;   // warp-uniform
-#pragma unroll
-            for (int h = 0; h < TN / 32; ++h) {
-                const int c = lane + 32 * h, gn = n0 + c;
-                if (gn >= N) continue;
-                const int64_t o = (int64_t)row * N + gn;
-                float vv = tile[rr * LDS + c];
-                if (EPI == EPI_BIAS_GELU) {
-                    Z[o] = vv;
-                    vv = gelu_f(vv);
-                } else if (EPI == EPI_DENORM) {
-                    vv = vv * scale[gn] + shift[gn];
+    if (warp == FWD_E / 32) {
+        if (lane == 0) {
+            int loaded = 0, taken = 0;   // chunks asked for / arrived
+            auto load = [&]() {
+                const uint32_t bar = wfull + 8 * (loaded % 3);
+                mbar_expect(bar, TILE_BYTES);
+                bulk_load(sw + (loaded % 3) * TILE_BYTES, wt + (int64_t)loaded * CHUNK_ELS, TILE_BYTES, bar);
+                ++loaded;
+            };
+            for (int i = 0; i < 3; ++i) load();
+            for (int q = 0; q < NCHUNK && ok; ++q) {
+                // a layer's first chunk: the activations of the layer before are in shared memory
+                const int layer = q < 8 ? q >> 2 : 2;
+                if (q == 0 || q == 4 || q == 8) ok = mbar_wait(aready, (uint32_t)(layer & 1), wait_limit);
+                if (ok) ok = mbar_wait(wfull + 8 * (q % 3), (uint32_t)((q / 3) & 1), wait_limit);
+                if (ok) taken = q + 1;
+                if (ok && q >= 2) ok = mbar_wait(tfree + 8 * (q & 1), (uint32_t)(((q >> 1) - 1) & 1), wait_limit);
+                if (!ok || idle) {
+                    ok = false;
+                    break;
                 }
-                C[o] = vv;
+                fence_after();
+                const uint32_t acc = tmem + (uint32_t)((q & 1) * TN), w = sw + (q % 3) * TILE_BYTES;
+                for (int s = 0; s < TK / 16; ++s)
+#pragma unroll
+                    for (int p = 0; p < 3; ++p)
+                        mma(acc, desc(sa + p * TILE_BYTES + s * 2 * LBO, LBO, SBO), desc(w + s * 2 * LBO, LBO, SBO), IDESC,
+                            (s | p) != 0);
+                commit(mdone + 8 * (q & 1));
+                // the chunk before is done with: its buffer takes the chunk after the next
+                if (q >= 1 && loaded < NCHUNK) {
+                    ok = mbar_wait(mdone + 8 * ((q - 1) & 1), (uint32_t)(((q - 1) >> 1) & 1), wait_limit);
+                    if (ok) load();
+                }
+            }
+            // copies still in flight land before the block leaves
+            for (int i = taken; i < loaded; ++i) mbar_wait(wfull + 8 * (i % 3), (uint32_t)((i / 3) & 1), WAIT_LIMIT);
+        }
+    } else {
+        const int sp = warp & 3, ch = warp >> 2;
+        const int r0 = 16 * sp + (lane >> 2), c0 = 16 * ch + 2 * (lane & 3);   // rows r0, r0 + 8; columns c0 + 8 i + {0, 1}
+        const int row[2] = {m0 + r0, m0 + r0 + 8};
+        const uint32_t tlane = tmem + ((uint32_t)(32 * sp) << 16) + (uint32_t)(16 * ch);
+        float v[32];   // a layer's activations: chunk c's in v[8 c ..], as tmem_ld_16x16 lays them out
+        // bias and GELU of chunk c (v: sums), stored for the backward pass when training
+        auto gelu_chunk = [&](int c, const float* bias, float* z, float* a) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int col = 64 * c + c0 + 8 * i;
+                const float2 bb = make_float2(bias[col], bias[col + 1]);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float& x0 = v[8 * c + 4 * i + 2 * h];
+                    float& x1 = v[8 * c + 4 * i + 2 * h + 1];
+                    x0 += bb.x;
+                    x1 += bb.y;
+                    const int64_t o = (int64_t)row[h] * NH + col;
+                    if (TRAIN && row[h] < M) *reinterpret_cast<float2*>(z + o) = make_float2(x0, x1);
+                    x0 = gelu_f(x0);
+                    x1 = gelu_f(x1);
+                    if (TRAIN && row[h] < M) *reinterpret_cast<float2*>(a + o) = make_float2(x0, x1);
+                }
+            }
+        };
+        // the layer's activations split into their three terms, to shared memory
+        auto put = [&]() {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint32_t o = core_off(r0 + 8 * h, 64 * c + c0 + 8 * i);
+                        float e0 = v[8 * c + 4 * i + 2 * h], e1 = v[8 * c + 4 * i + 2 * h + 1];
+#pragma unroll
+                        for (int p = 0; p < 3; ++p) {
+                            const __nv_bfloat16 t0 = __float2bfloat16_rn(e0), t1 = __float2bfloat16_rn(e1);
+                            *reinterpret_cast<uint32_t*>(sm + p * TILE_BYTES + o) = pack2(t0, t1);
+                            e0 -= __bfloat162float(t0);
+                            e1 -= __bfloat162float(t1);
+                        }
+                    }
+            fence_smem_async();
+            mbar_arrive(aready);
+        };
+        // layer 1: three inputs, on the CUDA cores
+        float x[2][3];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                x[h][k] = row[h] < M ? (X[(int64_t)row[h] * NIN + k] - norm[k]) / norm[NIN + k] : 0.0f;
+                if (TRAIN && ch == 0 && (lane & 3) == 0 && row[h] < M) tr.a0[(int64_t)row[h] * NIN + k] = x[h][k];
+            }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const float* w = fc + FC_W1 + (64 * c + c0 + 8 * i + j) * NIN;
+                    const float w0 = w[0], w1 = w[1], w2 = w[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        v[8 * c + 4 * i + 2 * h + j] = fmaf(x[h][2], w2, fmaf(x[h][1], w1, x[h][0] * w0));
+                }
+            gelu_chunk(c, fc + FC_B, tr.z[0], tr.a[0]);
+        }
+        put();
+        int q = 0;
+        auto take = [&](float (&t)[8]) {   // chunk q's sums
+            ok = ok && mbar_wait(mdone + 8 * (q & 1), (uint32_t)((q >> 1) & 1), wait_limit);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) return;
+            fence_after();
+            tmem_ld_16x16(tlane + (uint32_t)((q & 1) * TN), t);
+            fence_before();
+            mbar_arrive(tfree + 8 * (q & 1));
+            ++q;
+        };
+#pragma unroll
+        for (int l = 1; l < 3; ++l) {
+            if (!ok) break;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                if (!ok) break;
+                float t[8];
+                take(t);
+                if (!ok) break;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[8 * c + i] = t[i];
+                gelu_chunk(c, fc + FC_B + l * NH, tr.z[l], tr.a[l]);
+            }
+            if (ok) put();   // the layer's last MMA is done: its inputs may go
+        }
+        for (int c = 0; c < 7 && ok; ++c) {
+            float t[8];
+            take(t);
+            if (!ok) break;
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int col = 64 * c + c0 + 8 * i;
+                if (col >= NOUT) continue;   // (NOUT is even)
+                const float* bb = fc + FC_B + 3 * NH + col;
+                const float* nn = fc + FC_OUT + col;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (row[h] >= M) continue;
+                    float y0 = t[4 * i + 2 * h] + bb[0], y1 = t[4 * i + 2 * h + 1] + bb[1];
+                    if (!TRAIN) {
+                        y0 = y0 * nn[NOUT] + nn[0];
+                        y1 = y1 * nn[NOUT + 1] + nn[1];
+                    }
+                    float* dst = Y + (int64_t)row[h] * NOUT + col;
+                    if (vec) *reinterpret_cast<float2*>(dst) = make_float2(y0, y1);
+                    else {
+                        dst[0] = y0;
+                        dst[1] = y1;
+                    }
+                }
             }
         }
     }
     fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, TN);
+    ok = __syncthreads_and(ok);
+    if (warp == 0) tmem_dealloc(tmem, 2 * TN);
     if (!ok && tid == 0) atomicExch(fault, 1);
 }
 
-template <int EPI>
-abs_status gemm_tc(abs_mlp* net, cudaStream_t st, int M, int N, int K, const float* A, const __nv_bfloat16* W,
-                   float* C, const float* bias, float* Z, const float* scale, const float* shift,
-                   bool idle = false) {
-    static bool attr = false;
-    if (!attr) {
-        MCK(cudaFuncSetAttribute(gemm_tc_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, umma::SMEM));
-        attr = true;
+template <bool TRAIN>
+abs_status network_forward(abs_mlp* net, cudaStream_t st, const float* X, int64_t n, float* Y, bool idle = false) {
+    MCK(cudaFuncSetAttribute(network_forward_kernel<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, FWD_SMEM));
+    FwdTrain tr{};
+    if (TRAIN) {
+        tr.a0 = net->a0;
+        for (int l = 0; l < 3; ++l) {
+            tr.z[l] = net->z[l];
+            tr.a[l] = net->a[l];
+        }
     }
-    const dim3 grid((unsigned)((N + umma::TN - 1) / umma::TN), (unsigned)((M + umma::TM - 1) / umma::TM));
-    gemm_tc_kernel<EPI><<<grid, umma::T, umma::SMEM, st>>>(M, N, K, A, W, bias, Z, C, scale, shift, net->dfault,
-                                                           idle ? 1 : 0, idle ? 1024ll : umma::WAIT_LIMIT);
-    return mlaunch(net);
-}
-
-template <class TB, int EPI>
-abs_status gemm(abs_mlp* net, cudaStream_t st, int M, int N, int K, const float* A, int64_t sam, int64_t sak,
-                const TB* B, int64_t sbk, int64_t sbn, float* C, const float* bias = nullptr,
-                const float* aux = nullptr, float* Z = nullptr, const float* scale = nullptr,
-                const float* shift = nullptr) {
-    if (M <= 0 || N <= 0) return ABS_OK;
-    if constexpr (std::is_same<TB, __nv_bfloat16>::value &&
-                  (EPI == EPI_BIAS_GELU || EPI == EPI_BIAS || EPI == EPI_DENORM)) {
-        // a forward product of a 256-input layer: A [M][K], W [N][K] row-major, aligned
-        if (net->tc && K % umma::KC == 0 && sak == 1 && sam == K && sbk == 1 && sbn == K &&
-            ((uintptr_t)A & 15) == 0 && ((uintptr_t)B & 15) == 0)
-            return gemm_tc<EPI>(net, st, M, N, K, A, B, C, bias, Z, scale, shift);
-    }
-    const dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM));
-    gemm_kernel<TB, EPI><<<grid, GT, 0, st>>>(M, N, K, A, sam, sak, B, sbk, sbn, bias, aux, Z, C, scale, shift);
+    network_forward_kernel<TRAIN><<<(unsigned)((n + umma::TM - 1) / umma::TM), FWD_T, FWD_SMEM, st>>>(
+        (int)n, X, net->norm, net->theta, net->wb, net->wt, Y, tr, ((uintptr_t)Y & 7) == 0, net->dfault, idle ? 1 : 0,
+        idle ? 1024ll : umma::WAIT_LIMIT);
     return mlaunch(net);
 }
 
@@ -429,23 +503,173 @@ __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restr
     if (threadIdx.x == 0) *out = (accumulate ? *out : 0.0) + scale * sh[0];
 }
 
-// db[o] = sum over rows of dz[row][o]  (one thread per column, rows in order)
-__global__ void colsum_kernel(int rows, int cols, const float* __restrict__ dz, float* __restrict__ db) {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= cols) return;
-    float a = 0.0f;
-    for (int r = 0; r < rows; ++r) a += dz[(int64_t)r * cols + o];
-    db[o] = a;
+// One layer of the backward pass in one launch: dW[o][i] = sum_r D[r][o] A[r][i], db[o] = sum_r
+// D[r][o] and, in the remaining blocks, Dn[r][i] = (sum_o D[r][o] W[o][i]) gelu'(z[r][i]);
+// D [n][O], A and z [n][I], W bfloat16 [O][I]; O and I multiples of 4, rows 16-byte aligned.  The
+// products are independent: the first blocks take the 32 x 32 tiles of dW (those of the first column
+// also db), the others the tiles of Dn.  A minibatch has few tiles for 152 SMs and a tile's
+// sum is one chain of latencies, so the tiles are small and two groups of 128 threads share a tile's sum
+// (even and odd steps of 32 terms, added at the end), each with the next step's global loads in
+// flight while the current one is multiplied, 2 x 4 outputs per thread.
+constexpr int BT = 32, BT_G = 128;
+constexpr int BT_SA = BT + 2, BT_SB = BT + 4;   // shared row strides: two-way conflicts at most on A's transposed stores
+__global__ void __launch_bounds__(2 * BT_G) layer_backward_kernel(int n, int O, int I, const float* __restrict__ D,
+                                                                  const float* __restrict__ A,
+                                                                  const __nv_bfloat16* __restrict__ W,
+                                                                  const float* __restrict__ z, float* __restrict__ dW,
+                                                                  float* __restrict__ db, float* __restrict__ Dn) {
+    __shared__ __align__(16) float As[2][2][BT][BT_SA];   // [group][buffer][k][m]
+    __shared__ __align__(16) float Bs[2][2][BT][BT_SB];   // [group][buffer][k][n]
+    const int grp = threadIdx.x / BT_G, tid = threadIdx.x % BT_G;
+    const int tn = (I + BT - 1) / BT;
+    const int tw = ((O + BT - 1) / BT) * tn;
+    const bool isw = (int)blockIdx.x < tw;
+    const int tile = isw ? blockIdx.x : blockIdx.x - tw;
+    const int m0 = (tile / tn) * BT, n0 = (tile % tn) * BT;
+    const int M = isw ? O : n, K = isw ? n : O;
+    // four consecutive entries of rows hi and hi + 16 of a step's two tiles; D is read along its rows in
+    // both products: D[k][m] for dW (hi = k, lo = m), D[m][k] for Dn (hi = m, lo = k)
+    const int hi = tid >> 3, lo = (tid & 7) * 4;
+    float4 ra[2], rb[2];
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int h = hi + 16 * q;
+            const int kr = isw ? k0 + h : m0 + h, kc = isw ? m0 + lo : k0 + lo;   // D's row and column
+            ra[q] = (kr < n && kc < O) ? *reinterpret_cast<const float4*>(D + (int64_t)kr * O + kc) : zero;
+            rb[q] = zero;
+            if (k0 + h < K && n0 + lo < I) {
+                const int64_t e = (int64_t)(k0 + h) * I + n0 + lo;
+                if (isw) {
+                    rb[q] = *reinterpret_cast<const float4*>(A + e);
+                } else {
+                    const uint2 w = *reinterpret_cast<const uint2*>(W + e);   // four bfloat16
+                    rb[q] = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u),
+                                        __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
+                }
+            }
+        }
+    };
+    auto store = [&](int b) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int h = hi + 16 * q;
+            if (isw) {
+                *reinterpret_cast<float2*>(&As[grp][b][h][lo]) = make_float2(ra[q].x, ra[q].y);
+                *reinterpret_cast<float2*>(&As[grp][b][h][lo + 2]) = make_float2(ra[q].z, ra[q].w);
+            } else {
+                As[grp][b][lo][h] = ra[q].x;
+                As[grp][b][lo + 1][h] = ra[q].y;
+                As[grp][b][lo + 2][h] = ra[q].z;
+                As[grp][b][lo + 3][h] = ra[q].w;
+            }
+            *reinterpret_cast<float4*>(&Bs[grp][b][h][lo]) = rb[q];
+        }
+    };
+    const int tr = (tid >> 3) * 2, tc = (tid & 7) * 4;   // this thread's 2 rows and 4 columns
+    float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    float colsum = 0.0f;
+    const bool sums = isw && n0 == 0 && tid < BT;
+    load(grp * BT);
+    int b = 0;
+    for (int k0 = grp * BT; k0 < K; k0 += 2 * BT, b ^= 1) {
+        store(b);
+        // one barrier of the group per step: the other buffer is free once all passed the last
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "r"(BT_G) : "memory");
+        if (k0 + 2 * BT < K) load(k0 + 2 * BT);
+#pragma unroll
+        for (int k = 0; k < BT; ++k) {
+            const float2 av = *reinterpret_cast<const float2*>(&As[grp][b][k][tr]);
+            const float4 bv = *reinterpret_cast<const float4*>(&Bs[grp][b][k][tc]);
+            const float br[4] = {bv.x, bv.y, bv.z, bv.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                acc[0][j] = fmaf(av.x, br[j], acc[0][j]);
+                acc[1][j] = fmaf(av.y, br[j], acc[1][j]);
+            }
+        }
+        if (sums)
+#pragma unroll
+            for (int k = 0; k < BT; ++k) colsum += As[grp][b][k][tid];
+    }
+    __syncthreads();
+    // the second group's sums, through its own tiles
+    float* ex = &Bs[1][0][0][0];
+    static_assert(2 * BT * BT_SB >= 9 * BT_G, "exchange fits");
+    if (grp == 1) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) ex[e * BT_G + tid] = acc[e >> 2][e & 3];
+        if (tid < BT) ex[8 * BT_G + tid] = colsum;
+    }
+    __syncthreads();
+    if (grp == 1) return;
+    if (sums && m0 + tid < O) db[m0 + tid] = colsum + ex[8 * BT_G + tid];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int m = m0 + tr + i;
+        if (m >= M || n0 + tc >= I) continue;
+        float o4[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) o4[j] = acc[i][j] + ex[(4 * i + j) * BT_G + tid];
+        const int64_t o = (int64_t)m * I + n0 + tc;
+        if (!isw) {
+            const float4 zz = *reinterpret_cast<const float4*>(z + o);
+            o4[0] *= gelu_prime_f(zz.x);
+            o4[1] *= gelu_prime_f(zz.y);
+            o4[2] *= gelu_prime_f(zz.z);
+            o4[3] *= gelu_prime_f(zz.w);
+        }
+        *reinterpret_cast<float4*>((isw ? dW : Dn) + o) = make_float4(o4[0], o4[1], o4[2], o4[3]);
+    }
 }
 
-__global__ void to_bf16_kernel(int64_t n, const float* __restrict__ src, __nv_bfloat16* __restrict__ dst) {
+// the first layer's: dW[o][k] = sum_r D[r][o] a0[r][k] (three inputs), db[o] = sum_r D[r][o].  32 outputs
+// per block on the lanes, the rows dealt to 32 warps, their sums added in warp order.
+__global__ void __launch_bounds__(1024) first_backward_kernel(int n, const float* __restrict__ D,
+                                                              const float* __restrict__ a0, float* __restrict__ dW,
+                                                              float* __restrict__ db) {
+    __shared__ float sm[4][32][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, o = blockIdx.x * 32 + lane;
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int r = w; r < n; r += 32) {
+        const float d = D[(int64_t)r * NH + o];
+#pragma unroll
+        for (int k = 0; k < NIN; ++k) s[k] = fmaf(d, a0[(int64_t)r * NIN + k], s[k]);
+        s[3] += d;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) sm[k][w][lane] = s[k];
+    __syncthreads();
+    if (w >= 4) return;
+    float t = 0.0f;
+    for (int q = 0; q < 32; ++q) t += sm[w][q][lane];
+    if (w < NIN) dW[(int64_t)o * NIN + w] = t;
+    else db[o] = t;
+}
+
+// the rounded parameters, and the weights of layers 2-4 again in tiles
+__device__ __forceinline__ void put_bf16(int64_t i, float v, __nv_bfloat16* wb, __nv_bfloat16* wt) {
+    const __nv_bfloat16 h = __float2bfloat16_rn(v);
+    wb[i] = h;
+    const int t = tile_index(i);
+    if (t >= 0) wt[t] = h;
+}
+
+// (and the last tile's padding rows: zero)
+__global__ void to_bf16_kernel(int64_t n, const float* __restrict__ src, __nv_bfloat16* __restrict__ wb,
+                               __nv_bfloat16* __restrict__ wt) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) dst[i] = __float2bfloat16_rn(src[i]);
+    if (i < n) put_bf16(i, src[i], wb, wt);
+    constexpr int PAD = NOUT % umma::TN;   // rows of the last tile in use
+    if (i < (umma::TN - PAD) * NH)
+        wt[(NCHUNK - 1) * CHUNK_ELS + (umma::core_off(PAD + (int)(i / NH), (int)(i % NH)) >> 1)] = __float2bfloat16_rn(0.0f);
 }
 
 __global__ void adam_kernel(int64_t n, float* __restrict__ th, const float* __restrict__ g, float* __restrict__ m,
                             float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2,
-                            __nv_bfloat16* __restrict__ wb) {
+                            __nv_bfloat16* __restrict__ wb, __nv_bfloat16* __restrict__ wt) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float gi = g[i];
@@ -455,7 +679,7 @@ __global__ void adam_kernel(int64_t n, float* __restrict__ th, const float* __re
     v[i] = vi;
     const float t = th[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
     th[i] = t;
-    wb[i] = __float2bfloat16_rn(t);
+    put_bf16(i, t, wb, wt);
 }
 
 __global__ void gather_rows_kernel(int64_t rows, int cols, const int* __restrict__ idx, const float* __restrict__ src,
@@ -537,23 +761,21 @@ abs_status ensure_cap(abs_mlp* net, int64_t rows) {
 // forward pass of rows X [n][3] (raw); train: normalised outputs in net->yh and the
 // layer values kept for backward; else raw outputs into Yout
 abs_status forward_rows(abs_mlp* net, const float* X, int64_t n, bool train, float* Yout, cudaStream_t st) {
+    if (net->tc) return train ? network_forward<true>(net, st, X, n, net->yh) : network_forward<false>(net, st, X, n, Yout);
     abs_status r;
     normalize_kernel<<<grid1(n * NIN), 256, 0, st>>>(n, X, net->norm, net->a0);
     if ((r = mlaunch(net)) != ABS_OK) return r;
     const float* prev = net->a0;
     for (int l = 0; l < 3; ++l) {
-        const int in = L_IN[l];
-        if ((r = gemm<__nv_bfloat16, EPI_BIAS_GELU>(net, st, (int)n, NH, in, prev, in, 1, net->wb + OFF_W[l], 1, in,
-                                                    net->a[l], net->theta + OFF_B[l], nullptr, net->z[l])) != ABS_OK)
+        if ((r = gemm<EPI_BIAS_GELU>(net, st, (int)n, NH, l_in(l), prev, net->wb + off_w(l), net->a[l],
+                                     net->theta + off_b(l), net->z[l])) != ABS_OK)
             return r;
         prev = net->a[l];
     }
     if (train)
-        return gemm<__nv_bfloat16, EPI_BIAS>(net, st, (int)n, NOUT, NH, prev, NH, 1, net->wb + OFF_W[3], 1, NH,
-                                            net->yh, net->theta + OFF_B[3]);
-    return gemm<__nv_bfloat16, EPI_DENORM>(net, st, (int)n, NOUT, NH, prev, NH, 1, net->wb + OFF_W[3], 1, NH, Yout,
-                                          net->theta + OFF_B[3], nullptr, nullptr, net->norm + 2 * NIN + NOUT,
-                                          net->norm + 2 * NIN);
+        return gemm<EPI_BIAS>(net, st, (int)n, NOUT, NH, prev, net->wb + off_w(3), net->yh, net->theta + off_b(3));
+    return gemm<EPI_DENORM>(net, st, (int)n, NOUT, NH, prev, net->wb + off_w(3), Yout, net->theta + off_b(3), nullptr,
+                            net->norm + 2 * NIN + NOUT, net->norm + 2 * NIN);
 }
 
 // loss and gradient of the rows last passed through forward_rows(train) against raw
@@ -567,27 +789,22 @@ abs_status backward_rows(abs_mlp* net, const float* Y, int64_t n, double* loss_d
     if ((r = mlaunch(net)) != ABS_OK) return r;
     sum_partials_kernel<<<1, 256, 0, st>>>(net->lpart, nb, scale / (2.0 * (double)nel), acc, loss_dev);
     if ((r = mlaunch(net)) != ABS_OK) return r;
-    // layer 4: dW4 = g^T a3, db4 = colsum g, da3 = g W4
+    // layer l: dW_l = dcur^T a_{l-1}, db_l = colsum dcur, dz_{l-1} = (dcur W_l) * gelu'(z_{l-1}); dcur
+    // and the result alternate buffers
     const float* dcur = net->g;
     int ocur = NOUT;
-    for (int l = 3; l >= 0; --l) {
-        const int in = L_IN[l];
-        const float* aprev = l > 0 ? net->a[l - 1] : net->a0;
-        if ((r = gemm<float, EPI_STORE>(net, st, ocur, in, (int)n, dcur, 1, ocur, aprev, in, 1,
-                                        net->grad + OFF_W[l])) != ABS_OK)
-            return r;
-        colsum_kernel<<<grid1(ocur, 128), 128, 0, st>>>((int)n, ocur, dcur, net->grad + OFF_B[l]);
-        if ((r = mlaunch(net)) != ABS_OK) return r;
-        if (l == 0) break;
-        // dz_{l-1} = (dcur W_l) * gelu'(z_{l-1}); dcur and the result alternate buffers
+    for (int l = 3; l > 0; --l) {
         float* dst = (dcur == net->dz) ? net->da : net->dz;
-        if ((r = gemm<__nv_bfloat16, EPI_GELU_GRAD>(net, st, (int)n, in, ocur, dcur, ocur, 1, net->wb + OFF_W[l], in,
-                                                    1, dst, nullptr, net->z[l - 1])) != ABS_OK)
-            return r;
+        const int64_t ti = NH / BT, tiles = ((ocur + BT - 1) / BT + (n + BT - 1) / BT) * ti;
+        layer_backward_kernel<<<(unsigned)tiles, 2 * BT_G, 0, st>>>((int)n, ocur, NH, dcur, net->a[l - 1],
+                                                                   net->wb + off_w(l), net->z[l - 1],
+                                                                   net->grad + off_w(l), net->grad + off_b(l), dst);
+        if ((r = mlaunch(net)) != ABS_OK) return r;
         dcur = dst;
-        ocur = in;
+        ocur = NH;
     }
-    return ABS_OK;
+    first_backward_kernel<<<NH / 32, 1024, 0, st>>>((int)n, dcur, net->a0, net->grad + off_w(0), net->grad + off_b(0));
+    return mlaunch(net);
 }
 
 uint64_t splitmix64(uint64_t& s) {
@@ -632,12 +849,15 @@ abs_status abs_mlp_create(uint64_t seed, abs_mlp** out) {
         }                                                                                             \
     } while (0)
     MCK2(cudaGetDevice(&net->dev));
-    MCK2(cudaMalloc(&net->theta, sizeof(float) * NPAR));
-    MCK2(cudaMalloc(&net->wb, sizeof(__nv_bfloat16) * NPAR));
-    MCK2(cudaMalloc(&net->grad, sizeof(float) * NPAR));
-    MCK2(cudaMalloc(&net->m, sizeof(float) * NPAR));
-    MCK2(cudaMalloc(&net->v, sizeof(float) * NPAR));
-    MCK2(cudaMalloc(&net->norm, sizeof(float) * (2 * NIN + 2 * NOUT)));
+    // one allocation: theta, grad, m, v, norm (floats), then wb, wt (bfloat16); every part 256-byte aligned
+    constexpr size_t PF = (NPAR + 63) / 64 * 64, PN = (2 * NIN + 2 * NOUT + 63) / 64 * 64, PB = (NPAR + 127) / 128 * 128;
+    MCK2(cudaMalloc(&net->theta, sizeof(float) * (4 * PF + PN) + sizeof(__nv_bfloat16) * (PB + NCHUNK * CHUNK_ELS)));
+    net->grad = net->theta + PF;
+    net->m = net->grad + PF;
+    net->v = net->m + PF;
+    net->norm = net->v + PF;
+    net->wb = reinterpret_cast<__nv_bfloat16*>(net->norm + PN);
+    net->wt = net->wb + PB;
     MCK2(cudaHostAlloc(&net->hfault, sizeof(int), cudaHostAllocMapped));
     *net->hfault = 0;
     MCK2(cudaHostGetDevicePointer(&net->dfault, net->hfault, 0));
@@ -646,10 +866,10 @@ abs_status abs_mlp_create(uint64_t seed, abs_mlp** out) {
     std::vector<float> th(NPAR, 0.0f);
     uint64_t s = seed;
     for (int l = 0; l < 4; ++l) {
-        const double lim = std::sqrt(6.0 / (double)(L_IN[l] + L_OUT[l]));
-        for (int64_t i = 0; i < (int64_t)L_IN[l] * L_OUT[l]; ++i) {
+        const double lim = std::sqrt(6.0 / (double)(l_in(l) + l_out(l)));
+        for (int64_t i = 0; i < (int64_t)l_in(l) * l_out(l); ++i) {
             const double u = (double)(splitmix64(s) >> 11) * (1.0 / 9007199254740992.0);
-            th[OFF_W[l] + i] = (float)((2.0 * u - 1.0) * lim);
+            th[off_w(l) + i] = (float)((2.0 * u - 1.0) * lim);
         }
     }
     for (int i = 0; i < NIN; ++i) {
@@ -669,12 +889,7 @@ abs_status abs_mlp_create(uint64_t seed, abs_mlp** out) {
 void abs_mlp_destroy(abs_mlp* net) {
     if (!net) return;
     if (net->hfault) cudaFreeHost(net->hfault);
-    cudaFree(net->theta);
-    cudaFree(net->wb);
-    cudaFree(net->grad);
-    cudaFree(net->m);
-    cudaFree(net->v);
-    cudaFree(net->norm);
+    cudaFree(net->theta);   // with grad, m, v, norm, wb, wt
     cudaFree(net->a0);
     for (int l = 0; l < 3; ++l) {
         cudaFree(net->z[l]);
@@ -695,10 +910,9 @@ void abs_mlp_destroy(abs_mlp* net) {
 abs_status abs_mlp_set_params(abs_mlp* net, const float* params) {
     if (!net || !params) return mfail(net, ABS_ERR_ARG, "bad argument");
     MCK(cudaMemcpy(net->theta, params, sizeof(float) * NPAR, cudaMemcpyHostToDevice));
-    MCK(cudaMemset(net->m, 0, sizeof(float) * NPAR));
-    MCK(cudaMemset(net->v, 0, sizeof(float) * NPAR));
+    MCK(cudaMemset(net->m, 0, (size_t)((char*)(net->v + NPAR) - (char*)net->m)));   // both moments
     net->step = 0;
-    to_bf16_kernel<<<grid1(NPAR), 256>>>(NPAR, net->theta, net->wb);
+    to_bf16_kernel<<<grid1(NPAR), 256>>>(NPAR, net->theta, net->wb, net->wt);
     abs_status r = mlaunch(net);
     if (r != ABS_OK) return r;
     MCK(cudaDeviceSynchronize());
@@ -765,10 +979,9 @@ abs_status abs_mlp_selftest_wait(abs_mlp* net, abs_stream_t stream) {
     cudaStream_t st = (cudaStream_t)stream;
     abs_status r;
     if ((r = ensure_cap(net, umma::TM)) != ABS_OK) return r;
-    // one 128 x 256 x 256 product with its MMAs withheld, on the activation workspace
-    if ((r = gemm_tc<EPI_BIAS_GELU>(net, st, umma::TM, NH, NH, net->a[0], net->wb + OFF_W[1], net->a[1],
-                                     net->theta + OFF_B[1], net->z[1], nullptr, nullptr, true)) != ABS_OK)
-        return r;
+    // one block's forward pass with its MMAs withheld, on the activation workspace
+    MCK(cudaMemsetAsync(net->xb, 0, sizeof(float) * umma::TM * NIN, st));
+    if ((r = network_forward<true>(net, st, net->xb, umma::TM, net->yh, true)) != ABS_OK) return r;
     MCK(cudaStreamSynchronize(st));
     const bool expired = abs_mlp_device_fault(net) != 0;
     *(volatile int*)net->hfault = 0;
@@ -781,9 +994,13 @@ abs_status abs_mlp_forward(abs_mlp* net, const float* X, int64_t n, float* Y, ab
     if (abs_mlp_device_fault(net)) return mfail(net, ABS_ERR_TIMEOUT, "a tensor-core product gave up waiting");
     cudaStream_t st = (cudaStream_t)stream;
     abs_status r;
-    for (int64_t r0 = 0; r0 < n; r0 += CHUNK_ROWS) {
-        const int64_t rows = std::min<int64_t>(CHUNK_ROWS, n - r0);
-        if ((r = ensure_cap(net, rows)) != ABS_OK) return r;
+    if (n == 0) return ABS_OK;
+    // the tensor-core pass keeps its activations on chip: no workspace, any number of rows (in pieces a
+    // launch's row index holds)
+    const int64_t piece = net->tc ? (int64_t)1 << 30 : CHUNK_ROWS;
+    for (int64_t r0 = 0; r0 < n; r0 += piece) {
+        const int64_t rows = std::min<int64_t>(piece, n - r0);
+        if (!net->tc && (r = ensure_cap(net, rows)) != ABS_OK) return r;
         if ((r = forward_rows(net, X + r0 * NIN, rows, false, Y + r0 * NOUT, st)) != ABS_OK) return r;
     }
     return ABS_OK;
@@ -878,7 +1095,7 @@ abs_status abs_mlp_train(abs_mlp* net, const float* X, const float* Y, int64_t n
             const double c2 = 1.0 - std::pow(o.beta2, (double)net->step);
             adam_kernel<<<grid1(NPAR), 256, 0, st>>>(NPAR, net->theta, net->grad, net->m, net->v, (float)lr,
                                                      (float)o.beta1, (float)o.beta2, (float)o.eps, (float)c1,
-                                                     (float)c2, net->wb);
+                                                     (float)c2, net->wb, net->wt);
             if ((r = mlaunch(net)) != ABS_OK) return r;
         }
         MCK(cudaStreamSynchronize(st));
