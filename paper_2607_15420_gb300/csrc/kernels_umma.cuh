@@ -1,7 +1,7 @@
 // kernels_umma.cuh -- tcgen05 (fifth-generation tensor core) building blocks of the warm-start
 // network's forward pass (network_forward_kernel, mlp_lib.cu): kind::f16 MMAs on shared-memory
-// operands in the no-swizzle K-major core-matrix layout, FP32 accumulators in tensor memory,
-// mbarriers, bulk copies.
+// operands in the no-swizzle core-matrix layouts, FP32 accumulators in tensor memory, mbarriers, bulk
+// copies.
 //
 // An MMA takes both operands in one type and the weights are bfloat16, so each FP32 activation
 // enters as the sum of three bfloat16 terms a = h + m + l (h the rounding of a, m of a - h, l of
@@ -14,17 +14,24 @@
 
 namespace umma {
 
-constexpr int TM = 64, TN = 64, TK = 256;         // a block's rows; a weight chunk's columns; inputs
-constexpr int TILE_BYTES = TM * TK * 2;           // one bfloat16 term of the activations; a weight chunk
-// core matrices are 8 rows x 16 bytes; 8 row groups per 8-column K block: strides in bytes between core
-// matrices adjacent along K ("leading") and along M / N ("stride")
-constexpr uint32_t LBO = (TM / 8) * 128, SBO = 128;
+// A layer's products are formed transposed, outputs as the MMA's 128 rows and samples as its 64
+// columns: M = 128 runs at twice the rate of M = 64, 64 samples per block leave few SMs idle at 5000
+// samples, and an accumulator lane is an output, so its bias is one register.
+constexpr int TR = 64, TK = 256;                  // samples of a block; a layer's inputs
+constexpr int TO = 128, KC = 128;                 // outputs and inputs of a weight chunk
+constexpr int TILE_BYTES = TR * TK * 2;           // one bfloat16 term of the activations; a weight chunk
+static_assert(TO * KC * 2 == TILE_BYTES, "a chunk takes a tile's room");
+// Core matrices are 128 bytes.  Weights are K-major: 8 outputs x 8 inputs, an output's 8 inputs in 16
+// bytes.  Activations are sample-major: 8 inputs x 8 samples, an input's 8 samples in 16 bytes (what a
+// lane that holds one output for many samples stores at once).  Both: core matrices adjacent along
+// outputs / samples 128 bytes apart ("stride"), along the inputs after them ("leading").
+constexpr uint32_t SBO = 128, W_LBO = (TO / 8) * 128, X_LBO = (TR / 8) * 128;
 constexpr long long WAIT_LIMIT = 1ll << 22;       // mbarrier polls before a wait gives up
-static_assert(TM == TN, "activations and weight chunks share one layout");
 
 // instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A and B bfloat16 (bits 7-9,
-// 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at bit 17, M >> 4 at bit 24
-constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+// 10-12 = 1), A K-major (bit 15 = 0), B N-major (bit 16 = 1), N >> 3 at bit 17, M >> 4 at bit 24
+constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(TR >> 3) << 17) |
+                           ((uint32_t)(TO >> 4) << 24);
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -34,6 +41,8 @@ __device__ __forceinline__ uint64_t desc(uint32_t saddr, uint32_t lbo, uint32_t 
     return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo & 0x3FFFFu) >> 4) << 16) |
            ((uint64_t)((sbo & 0x3FFFFu) >> 4) << 32) | (1ull << 46);
 }
+
+__device__ __forceinline__ uint64_t desc_at(uint32_t lo, uint32_t hi) { return ((uint64_t)hi << 32) | lo; }
 
 __device__ __forceinline__ void tmem_alloc(uint32_t dst, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"(ncols)
@@ -99,27 +108,34 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
         : "memory");
 }
 
-// 16 accumulator columns of 16 rows over the warp (16x256b shape): thread t gets, for i < 2, columns 8 i
-// + 2 (t % 4) + {0, 1} of row t / 4 in v[4 i + {0, 1}] and of row t / 4 + 8 in v[4 i + {2, 3}].  An M = 64
-// accumulator keeps rows 16 w .. 16 w + 15 in the first 16 lanes of the 32 that warp w (mod 4) reads.
-__device__ __forceinline__ void tmem_ld_16x16(uint32_t taddr, float (&v)[8]) {
-    uint32_t r[8];
-    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr)
-                 : "memory");
+// 16 consecutive accumulator columns of this thread's lane (32x32b shape: lane = row)
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// byte offset of element (r, k) of a 64-row tile in core-matrix layout
-__device__ __forceinline__ uint32_t core_off(int r, int k) {
-    return (uint32_t)((((k >> 3) * (TM / 8) + (r >> 3)) << 7) + ((r & 7) << 4) + ((k & 7) << 1));
+// byte offset of weight (output o, input k) in a chunk; of activation (input k, sample r) in a tile
+__host__ __device__ constexpr uint32_t w_off(int o, int k) {
+    return (uint32_t)((((k >> 3) * (TO / 8) + (o >> 3)) << 7) + ((o & 7) << 4) + ((k & 7) << 1));
+}
+__host__ __device__ constexpr uint32_t x_off(int k, int r) {
+    return (uint32_t)((((k >> 3) * (TR / 8) + (r >> 3)) << 7) + ((k & 7) << 4) + ((r & 7) << 1));
 }
 
-__device__ __forceinline__ uint32_t pack2(__nv_bfloat16 a, __nv_bfloat16 b) {
-    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+// two values rounded to bfloat16, the first in the low half
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+    return r;
 }
 
 }  // namespace umma

@@ -104,18 +104,21 @@ __device__ __forceinline__ float gelu_prime_f(float x) {
     return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
 }
 
-// the 64-output tiles of W2, W3 (four each) and W4 (seven, the last one padded with zeros)
-constexpr int NCHUNK = 4 + 4 + 7;
+// the chunks of W2, W3 (two groups of 128 outputs each) and W4 (four groups, the outputs past the
+// 440th zero), each group in two halves of its inputs
+constexpr int NGROUP = 2 + 2 + 4, NCHUNK = 2 * NGROUP;
 constexpr int CHUNK_ELS = umma::TILE_BYTES / 2;
+// element (output o, input k) of layer l = 1, 2, 3 in wt
+__device__ __forceinline__ int tile_element(int l, int o, int k) {
+    const int g = (l - 1) * 2 + o / umma::TO;
+    return (2 * g + k / umma::KC) * CHUNK_ELS + (int)(umma::w_off(o % umma::TO, k % umma::KC) >> 1);
+}
 // where weight i of the flat parameters lies in wt (-1: W1 or a bias)
 __device__ __forceinline__ int tile_index(int64_t i) {
 #pragma unroll
     for (int l = 1; l < 4; ++l) {
         const int64_t e = i - off_w(l);
-        if (e >= 0 && e < (int64_t)l_out(l) * NH) {
-            const int o = (int)(e / NH), k = (int)(e % NH);
-            return ((l - 1) * 4 + o / umma::TN) * CHUNK_ELS + (int)(umma::core_off(o % umma::TN, k) >> 1);
-        }
+        if (e >= 0 && e < (int64_t)l_out(l) * NH) return tile_element(l, (int)(e / NH), (int)(e % NH));
     }
     return -1;
 }
@@ -204,23 +207,24 @@ abs_status gemm(abs_mlp* net, cudaStream_t st, int M, int N, int K, const float*
     return mlaunch(net);
 }
 
-// The whole forward pass of 64 rows per block, the products of layers 2-4 on the tensor cores
+// The whole forward pass of 64 samples per block, the products of layers 2-4 on the tensor cores
 // (kernels_umma.cuh).  The activations stay on chip: their three bfloat16 terms in shared memory
-// (96 KB), the weights streaming past them in 15 chunks of 64 outputs (32 KB each, bulk copies of the
-// tiled weights wt into a ring of three), the accumulators in two tensor-memory buffers of 64
-// columns.  Warps 0-15: the layers' biases and GELU and the split into terms, a 16-row x 16-column piece
-// of every chunk each, while the next chunk's MMAs run; a layer's activations are kept in registers until
-// its last MMA has read the previous ones.  Warp 16: one thread loads the chunks and issues the 48
-// MMAs of each (16 K steps x 3 terms).  Biases, scales and W1 wait in shared memory: with four warps per
-// scheduler and no global loads between a chunk's sums and its activations, the arithmetic of GELU and
-// split, about 36 instructions per activation, bounds the pass.
+// (96 KB), the weights streaming past them in 16 chunks of 128 outputs x 128 inputs (32 KB each, bulk
+// copies of the tiled weights wt into a ring of three), the accumulators in two tensor-memory buffers of
+// 64 columns, one per group of 128 outputs.  Warps 0-15: the layers' biases and GELU and the split into
+// terms, 32 outputs x 16 samples of every group each, while the next group's MMAs run; a layer's
+// activations are kept in registers until its last MMA has read the previous ones.  Warp 16: one
+// thread loads the chunks and issues the 24 MMAs of each (8 K steps x 3 terms).  Biases, scales and W1
+// wait in shared memory.
+// Every wait is bounded (wait_limit polls); when one gives up the block sets fault and leaves, its
+// outputs unwritten.  idle (the self-test of that path): no MMA is issued.
 // TRAIN: also a0, the pre-activations z and activations a of the layers, and normalised outputs;
-// otherwise outputs de-normalised.  vec: Y allows 8-byte stores.  Every wait is bounded (wait_limit
-// polls); when one gives up the block sets fault and leaves, its outputs unwritten.  idle (the
-// self-test of that path): no MMA is issued.
+// otherwise outputs de-normalised.
 constexpr int FWD_E = 512, FWD_T = FWD_E + 32;
-// constants in shared memory (floats): biases of layers 1-4, output shift and scale, W1
-constexpr int FC_B = 0, FC_OUT = 3 * NH + NOUT, FC_W1 = FC_OUT + 2 * NOUT, FC_COUNT = FC_W1 + NIN * NH;
+// constants in shared memory (floats): biases of layers 1-4, output shift and scale, W1, the block's
+// normalised inputs
+constexpr int FC_B = 0, FC_OUT = 3 * NH + NOUT, FC_W1 = FC_OUT + 2 * NOUT, FC_X = FC_W1 + NIN * NH,
+              FC_COUNT = FC_X + NIN * umma::TR;
 constexpr int FWD_SMEM = 6 * umma::TILE_BYTES + 4 * FC_COUNT + 1024;
 static_assert(FWD_SMEM <= 227 * 1024, "shared memory of a block");
 struct FwdTrain {
@@ -232,25 +236,28 @@ __global__ void __launch_bounds__(FWD_T, 1) network_forward_kernel(int M, const 
                                                                    const float* __restrict__ theta,
                                                                    const __nv_bfloat16* __restrict__ wb,
                                                                    const __nv_bfloat16* __restrict__ wt,
-                                                                   float* __restrict__ Y, const FwdTrain tr, bool vec,
+                                                                   float* __restrict__ Y, const FwdTrain tr,
                                                                    int* __restrict__ fault, int idle,
                                                                    long long wait_limit) {
     using namespace umma;
     extern __shared__ unsigned char tc_smem[];
-    __shared__ __align__(8) uint64_t bars[3 + 2 + 2 + 1];
+    __shared__ __align__(8) uint64_t bars[3 + 3 + 2 + 2 + 1];
     __shared__ uint32_t tbase;
     unsigned char* sm = (unsigned char*)(((uintptr_t)tc_smem + 1023) & ~(uintptr_t)1023);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * TM;
-    const uint32_t sa = smem_u32(sm), sw = sa + 3 * TILE_BYTES;
-    const uint32_t wfull = smem_u32(&bars[0]), mdone = smem_u32(&bars[3]), tfree = smem_u32(&bars[5]),
-                   aready = smem_u32(&bars[7]);
+    const int m0 = blockIdx.x * TR;
+    const uint32_t sx = smem_u32(sm), sw = sx + 3 * TILE_BYTES;
+    const uint32_t wfull = smem_u32(&bars[0]), wfree = smem_u32(&bars[3]), mdone = smem_u32(&bars[6]),
+                   tfree = smem_u32(&bars[8]), aready = smem_u32(&bars[10]);
     if (warp == 0) {
-        tmem_alloc(smem_u32(&tbase), 2 * TN);
+        tmem_alloc(smem_u32(&tbase), 2 * TR);
         tmem_relinquish();
     }
     if (tid == 0) {
-        for (int i = 0; i < 3; ++i) mbar_init(wfull + 8 * i, 1);
+        for (int i = 0; i < 3; ++i) {
+            mbar_init(wfull + 8 * i, 1);
+            mbar_init(wfree + 8 * i, 1);
+        }
         for (int i = 0; i < 2; ++i) {
             mbar_init(mdone + 8 * i, 1);
             mbar_init(tfree + 8 * i, FWD_E);
@@ -260,10 +267,21 @@ __global__ void __launch_bounds__(FWD_T, 1) network_forward_kernel(int M, const 
     float* fc = reinterpret_cast<float*>(sm + 6 * TILE_BYTES);
     for (int i = tid; i < FC_COUNT; i += FWD_T) {
         float f;
-        if (i < FC_OUT) f = theta[i < 3 * NH ? (i < NH ? off_b(0) + i : (i < 2 * NH ? off_b(1) + i - NH : off_b(2) + i - 2 * NH))
-                                             : off_b(3) + i - 3 * NH];
-        else if (i < FC_W1) f = norm[2 * NIN + i - FC_OUT];
-        else f = __bfloat162float(wb[off_w(0) + i - FC_W1]);
+        if (i < FC_OUT) {
+            f = theta[i < 3 * NH ? (i < NH ? off_b(0) + i : (i < 2 * NH ? off_b(1) + i - NH : off_b(2) + i - 2 * NH))
+                                 : off_b(3) + i - 3 * NH];
+        } else if (i < FC_W1) {
+            f = norm[2 * NIN + i - FC_OUT];
+        } else if (i < FC_X) {
+            f = __bfloat162float(wb[off_w(0) + i - FC_W1]);
+        } else {
+            const int e = i - FC_X, r = e / NIN, k = e % NIN;
+            f = 0.0f;
+            if (m0 + r < M) {
+                f = (X[(int64_t)(m0 + r) * NIN + k] - norm[k]) / norm[NIN + k];
+                if (TRAIN) tr.a0[(int64_t)(m0 + r) * NIN + k] = f;
+            }
+        }
         fc[i] = f;
     }
     fence_before();
@@ -274,6 +292,8 @@ __global__ void __launch_bounds__(FWD_T, 1) network_forward_kernel(int M, const 
     if (warp == FWD_E / 32) {
         if (lane == 0) {
             int loaded = 0, taken = 0;   // chunks asked for / arrived
+            const uint64_t dx = desc(sx, X_LBO, SBO), dw = desc(sw, W_LBO, SBO);
+            const uint32_t xlo = (uint32_t)dx, xhi = (uint32_t)(dx >> 32), wlo = (uint32_t)dw, whi = (uint32_t)(dw >> 32);
             auto load = [&]() {
                 const uint32_t bar = wfull + 8 * (loaded % 3);
                 mbar_expect(bar, TILE_BYTES);
@@ -281,112 +301,109 @@ __global__ void __launch_bounds__(FWD_T, 1) network_forward_kernel(int M, const 
                 ++loaded;
             };
             for (int i = 0; i < 3; ++i) load();
-            for (int q = 0; q < NCHUNK && ok; ++q) {
-                // a layer's first chunk: the activations of the layer before are in shared memory
-                const int layer = q < 8 ? q >> 2 : 2;
-                if (q == 0 || q == 4 || q == 8) ok = mbar_wait(aready, (uint32_t)(layer & 1), wait_limit);
-                if (ok) ok = mbar_wait(wfull + 8 * (q % 3), (uint32_t)((q / 3) & 1), wait_limit);
-                if (ok) taken = q + 1;
-                if (ok && q >= 2) ok = mbar_wait(tfree + 8 * (q & 1), (uint32_t)(((q >> 1) - 1) & 1), wait_limit);
-                if (!ok || idle) {
-                    ok = false;
-                    break;
-                }
-                fence_after();
-                const uint32_t acc = tmem + (uint32_t)((q & 1) * TN), w = sw + (q % 3) * TILE_BYTES;
-                for (int s = 0; s < TK / 16; ++s)
+            for (int g = 0; g < NGROUP && ok; ++g) {
+                // a layer's first group: the activations of the layer before are in shared memory
+                if (g == 0 || g == 2 || g == 4) ok = mbar_wait(aready, (uint32_t)((g >> 1) & 1), wait_limit);
+                if (ok && g >= 2) ok = mbar_wait(tfree + 8 * (g & 1), (uint32_t)(((g >> 1) - 1) & 1), wait_limit);
+                for (int kc = 0; kc < 2 && ok; ++kc) {
+                    const int c = 2 * g + kc;
+                    ok = mbar_wait(wfull + 8 * (c % 3), (uint32_t)((c / 3) & 1), wait_limit);
+                    if (ok) taken = c + 1;
+                    if (!ok || idle) {
+                        ok = false;
+                        break;
+                    }
+                    fence_after();
+                    // descriptors differ in the start address alone (its 14 bits hold every address of
+                    // the block): one add per operand
+                    const uint32_t acc = tmem + (uint32_t)((g & 1) * TR);
+                    const uint32_t w = wlo + (uint32_t)((c % 3) * (TILE_BYTES >> 4));
+                    const uint32_t x = xlo + (uint32_t)((kc * (KC / 8) * (int)X_LBO) >> 4);
 #pragma unroll
-                    for (int p = 0; p < 3; ++p)
-                        mma(acc, desc(sa + p * TILE_BYTES + s * 2 * LBO, LBO, SBO), desc(w + s * 2 * LBO, LBO, SBO), IDESC,
-                            (s | p) != 0);
-                commit(mdone + 8 * (q & 1));
-                // the chunk before is done with: its buffer takes the chunk after the next
-                if (q >= 1 && loaded < NCHUNK) {
-                    ok = mbar_wait(mdone + 8 * ((q - 1) & 1), (uint32_t)(((q - 1) >> 1) & 1), wait_limit);
-                    if (ok) load();
+                    for (int s = 0; s < KC / 16; ++s)
+#pragma unroll
+                        for (int p = 0; p < 3; ++p)
+                            mma(acc, desc_at(w + (uint32_t)((s * 2 * (int)W_LBO) >> 4), whi),
+                                desc_at(x + (uint32_t)((p * TILE_BYTES + s * 2 * (int)X_LBO) >> 4), xhi), IDESC,
+                                (kc | s | p) != 0);
+                    commit(wfree + 8 * (c % 3));
+                    // the chunk before is done with: its buffer takes the chunk after the next
+                    if (c >= 1 && loaded < NCHUNK) {
+                        ok = mbar_wait(wfree + 8 * ((c - 1) % 3), (uint32_t)(((c - 1) / 3) & 1), wait_limit);
+                        if (ok) load();
+                    }
                 }
+                if (ok) commit(mdone + 8 * (g & 1));
             }
             // copies still in flight land before the block leaves
             for (int i = taken; i < loaded; ++i) mbar_wait(wfull + 8 * (i % 3), (uint32_t)((i / 3) & 1), WAIT_LIMIT);
         }
     } else {
-        const int sp = warp & 3, ch = warp >> 2;
-        const int r0 = 16 * sp + (lane >> 2), c0 = 16 * ch + 2 * (lane & 3);   // rows r0, r0 + 8; columns c0 + 8 i + {0, 1}
-        const int row[2] = {m0 + r0, m0 + r0 + 8};
-        const uint32_t tlane = tmem + ((uint32_t)(32 * sp) << 16) + (uint32_t)(16 * ch);
-        float v[32];   // a layer's activations: chunk c's in v[8 c ..], as tmem_ld_16x16 lays them out
-        // bias and GELU of chunk c (v: sums), stored for the backward pass when training
-        auto gelu_chunk = [&](int c, const float* bias, float* z, float* a) {
+        // this thread: output f of every group, samples r0 .. r0 + 15 of the block
+        const int f = 32 * (warp & 3) + lane, r0 = 16 * (warp >> 2);
+        const int left = M - (m0 + r0);   // samples of them that exist
+        const uint32_t tlane = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)r0;
+        float v[2][16];   // a layer's activations of the thread's two outputs
+        // bias and GELU of group c's sums, stored for the backward pass when training
+        auto gelu_group = [&](int c, const float* bias, float* z, float* a) {
+            const int o = TO * c + f;
+            const float bb = bias[o];
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int col = 64 * c + c0 + 8 * i;
-                const float2 bb = make_float2(bias[col], bias[col + 1]);
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    float& x0 = v[8 * c + 4 * i + 2 * h];
-                    float& x1 = v[8 * c + 4 * i + 2 * h + 1];
-                    x0 += bb.x;
-                    x1 += bb.y;
-                    const int64_t o = (int64_t)row[h] * NH + col;
-                    if (TRAIN && row[h] < M) *reinterpret_cast<float2*>(z + o) = make_float2(x0, x1);
-                    x0 = gelu_f(x0);
-                    x1 = gelu_f(x1);
-                    if (TRAIN && row[h] < M) *reinterpret_cast<float2*>(a + o) = make_float2(x0, x1);
+            for (int i = 0; i < 16; ++i) {
+                const float zz = v[c][i] + bb;
+                v[c][i] = gelu_f(zz);
+                if (TRAIN && i < left) {
+                    const int64_t e = (int64_t)(m0 + r0 + i) * NH + o;
+                    z[e] = zz;
+                    a[e] = v[c][i];
                 }
             }
         };
-        // the layer's activations split into their three terms, to shared memory
+        // the layer's activations split into their three terms, to shared memory: 8 samples at once
         auto put = [&]() {
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
+            for (int c = 0; c < 2; ++c)
 #pragma unroll
-                for (int i = 0; i < 2; ++i)
+                for (int h = 0; h < 2; ++h) {
+                    float e[8];
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const uint32_t o = core_off(r0 + 8 * h, 64 * c + c0 + 8 * i);
-                        float e0 = v[8 * c + 4 * i + 2 * h], e1 = v[8 * c + 4 * i + 2 * h + 1];
+                    for (int i = 0; i < 8; ++i) e[i] = v[c][8 * h + i];
+                    const uint32_t o = x_off(TO * c + f, r0 + 8 * h);
 #pragma unroll
-                        for (int p = 0; p < 3; ++p) {
-                            const __nv_bfloat16 t0 = __float2bfloat16_rn(e0), t1 = __float2bfloat16_rn(e1);
-                            *reinterpret_cast<uint32_t*>(sm + p * TILE_BYTES + o) = pack2(t0, t1);
-                            e0 -= __bfloat162float(t0);
-                            e1 -= __bfloat162float(t1);
+                    for (int p = 0; p < 3; ++p) {
+                        uint32_t t[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            t[i] = pack2(e[2 * i], e[2 * i + 1]);
+                            e[2 * i] -= __uint_as_float(t[i] << 16);
+                            e[2 * i + 1] -= __uint_as_float(t[i] & 0xffff0000u);
                         }
+                        *reinterpret_cast<uint4*>(sm + p * TILE_BYTES + o) = make_uint4(t[0], t[1], t[2], t[3]);
                     }
+                }
             fence_smem_async();
             mbar_arrive(aready);
         };
         // layer 1: three inputs, on the CUDA cores
-        float x[2][3];
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+        for (int c = 0; c < 2; ++c) {
+            const float* w = fc + FC_W1 + (TO * c + f) * NIN;
+            const float w0 = w[0], w1 = w[1], w2 = w[2];
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                x[h][k] = row[h] < M ? (X[(int64_t)row[h] * NIN + k] - norm[k]) / norm[NIN + k] : 0.0f;
-                if (TRAIN && ch == 0 && (lane & 3) == 0 && row[h] < M) tr.a0[(int64_t)row[h] * NIN + k] = x[h][k];
+            for (int i = 0; i < 16; ++i) {
+                const float* x = fc + FC_X + (r0 + i) * NIN;
+                v[c][i] = fmaf(x[2], w2, fmaf(x[1], w1, x[0] * w0));
             }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    const float* w = fc + FC_W1 + (64 * c + c0 + 8 * i + j) * NIN;
-                    const float w0 = w[0], w1 = w[1], w2 = w[2];
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-                        v[8 * c + 4 * i + 2 * h + j] = fmaf(x[h][2], w2, fmaf(x[h][1], w1, x[h][0] * w0));
-                }
-            gelu_chunk(c, fc + FC_B, tr.z[0], tr.a[0]);
+            gelu_group(c, fc + FC_B, tr.z[0], tr.a[0]);
         }
         put();
         int q = 0;
-        auto take = [&](float (&t)[8]) {   // chunk q's sums
+        auto take = [&](float (&t)[16]) {   // group q's sums
             ok = ok && mbar_wait(mdone + 8 * (q & 1), (uint32_t)((q >> 1) & 1), wait_limit);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) return;
             fence_after();
-            tmem_ld_16x16(tlane + (uint32_t)((q & 1) * TN), t);
+            tmem_ld16(tlane + (uint32_t)((q & 1) * TR), t);
             fence_before();
             mbar_arrive(tfree + 8 * (q & 1));
             ++q;
@@ -395,48 +412,31 @@ __global__ void __launch_bounds__(FWD_T, 1) network_forward_kernel(int M, const 
         for (int l = 1; l < 3; ++l) {
             if (!ok) break;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < 2; ++c) {
                 if (!ok) break;
-                float t[8];
-                take(t);
+                take(v[c]);
                 if (!ok) break;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) v[8 * c + i] = t[i];
-                gelu_chunk(c, fc + FC_B + l * NH, tr.z[l], tr.a[l]);
+                gelu_group(c, fc + FC_B + l * NH, tr.z[l], tr.a[l]);
             }
             if (ok) put();   // the layer's last MMA is done: its inputs may go
         }
-        for (int c = 0; c < 7 && ok; ++c) {
-            float t[8];
+        for (int c = 0; c < 4 && ok; ++c) {
+            float t[16];
             take(t);
-            if (!ok) break;
+            const int o = TO * c + f;
+            if (!ok || o >= NOUT) continue;
+            const float bb = fc[FC_B + 3 * NH + o], sh = fc[FC_OUT + o], sc = fc[FC_OUT + NOUT + o];
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int col = 64 * c + c0 + 8 * i;
-                if (col >= NOUT) continue;   // (NOUT is even)
-                const float* bb = fc + FC_B + 3 * NH + col;
-                const float* nn = fc + FC_OUT + col;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    if (row[h] >= M) continue;
-                    float y0 = t[4 * i + 2 * h] + bb[0], y1 = t[4 * i + 2 * h + 1] + bb[1];
-                    if (!TRAIN) {
-                        y0 = y0 * nn[NOUT] + nn[0];
-                        y1 = y1 * nn[NOUT + 1] + nn[1];
-                    }
-                    float* dst = Y + (int64_t)row[h] * NOUT + col;
-                    if (vec) *reinterpret_cast<float2*>(dst) = make_float2(y0, y1);
-                    else {
-                        dst[0] = y0;
-                        dst[1] = y1;
-                    }
-                }
+            for (int i = 0; i < 16; ++i) {
+                float y = t[i] + bb;
+                if (!TRAIN) y = y * sc + sh;
+                if (i < left) Y[(int64_t)(m0 + r0 + i) * NOUT + o] = y;
             }
         }
     }
     fence_before();
     ok = __syncthreads_and(ok);
-    if (warp == 0) tmem_dealloc(tmem, 2 * TN);
+    if (warp == 0) tmem_dealloc(tmem, 2 * TR);
     if (!ok && tid == 0) atomicExch(fault, 1);
 }
 
@@ -451,8 +451,8 @@ abs_status network_forward(abs_mlp* net, cudaStream_t st, const float* X, int64_
             tr.a[l] = net->a[l];
         }
     }
-    network_forward_kernel<TRAIN><<<(unsigned)((n + umma::TM - 1) / umma::TM), FWD_T, FWD_SMEM, st>>>(
-        (int)n, X, net->norm, net->theta, net->wb, net->wt, Y, tr, ((uintptr_t)Y & 7) == 0, net->dfault, idle ? 1 : 0,
+    network_forward_kernel<TRAIN><<<(unsigned)((n + umma::TR - 1) / umma::TR), FWD_T, FWD_SMEM, st>>>(
+        (int)n, X, net->norm, net->theta, net->wb, net->wt, Y, tr, net->dfault, idle ? 1 : 0,
         idle ? 1024ll : umma::WAIT_LIMIT);
     return mlaunch(net);
 }
@@ -657,14 +657,13 @@ __device__ __forceinline__ void put_bf16(int64_t i, float v, __nv_bfloat16* wb, 
     if (t >= 0) wt[t] = h;
 }
 
-// (and the last tile's padding rows: zero)
+// (and zeros for W4's outputs past the last)
 __global__ void to_bf16_kernel(int64_t n, const float* __restrict__ src, __nv_bfloat16* __restrict__ wb,
                                __nv_bfloat16* __restrict__ wt) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) put_bf16(i, src[i], wb, wt);
-    constexpr int PAD = NOUT % umma::TN;   // rows of the last tile in use
-    if (i < (umma::TN - PAD) * NH)
-        wt[(NCHUNK - 1) * CHUNK_ELS + (umma::core_off(PAD + (int)(i / NH), (int)(i % NH)) >> 1)] = __float2bfloat16_rn(0.0f);
+    constexpr int END = 4 * umma::TO;   // outputs the groups of W4 hold
+    if (i < (END - NOUT) * NH) wt[tile_element(3, NOUT + (int)(i / NH), (int)(i % NH))] = __float2bfloat16_rn(0.0f);
 }
 
 __global__ void adam_kernel(int64_t n, float* __restrict__ th, const float* __restrict__ g, float* __restrict__ m,
@@ -978,10 +977,10 @@ abs_status abs_mlp_selftest_wait(abs_mlp* net, abs_stream_t stream) {
     if (abs_mlp_device_fault(net)) return mfail(net, ABS_ERR_TIMEOUT, "a tensor-core product gave up waiting");
     cudaStream_t st = (cudaStream_t)stream;
     abs_status r;
-    if ((r = ensure_cap(net, umma::TM)) != ABS_OK) return r;
+    if ((r = ensure_cap(net, umma::TR)) != ABS_OK) return r;
     // one block's forward pass with its MMAs withheld, on the activation workspace
-    MCK(cudaMemsetAsync(net->xb, 0, sizeof(float) * umma::TM * NIN, st));
-    if ((r = network_forward<true>(net, st, net->xb, umma::TM, net->yh, true)) != ABS_OK) return r;
+    MCK(cudaMemsetAsync(net->xb, 0, sizeof(float) * umma::TR * NIN, st));
+    if ((r = network_forward<true>(net, st, net->xb, umma::TR, net->yh, true)) != ABS_OK) return r;
     MCK(cudaStreamSynchronize(st));
     const bool expired = abs_mlp_device_fault(net) != 0;
     *(volatile int*)net->hfault = 0;
