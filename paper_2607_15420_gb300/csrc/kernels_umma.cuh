@@ -6,7 +6,10 @@
 // An MMA takes both operands in one type and the weights are bfloat16, so each FP32 activation
 // enters as the sum of three bfloat16 terms a = h + m + l (h the rounding of a, m of a - h, l of
 // a - h - m: 24 significand bits); the three products with a bfloat16 weight are exact in the FP32
-// accumulator: a layer's product at FP32 accuracy from three MMAs per K step.
+// accumulator.  The three terms of 64 samples stand side by side as 192 columns of one MMA, so a weight
+// is read from shared memory once for all three: 24 MMAs of 64 columns took 1.6-2.1 k cycles per chunk of
+// weights whatever their M, and 8 of 192 columns brought 5000 samples from 30.8 to 26.6 us.  An output's
+// three sums are added as they leave tensor memory.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -14,23 +17,25 @@
 
 namespace umma {
 
-// A layer's products are formed transposed, outputs as the MMA's 128 rows and samples as its 64
-// columns: M = 128 runs at twice the rate of M = 64, 64 samples per block leave few SMs idle at 5000
-// samples, and an accumulator lane is an output, so its bias is one register.
+// A layer's products are formed transposed, outputs as the MMA's 128 rows and samples as its
+// columns: 64 samples per block leave few SMs idle at 5000 samples, an accumulator lane is an output, so
+// its bias is one register, and a lane stores eight samples of a term at once (samples as rows: 43 us).
 constexpr int TR = 64, TK = 256;                  // samples of a block; a layer's inputs
 constexpr int TO = 128, KC = 128;                 // outputs and inputs of a weight chunk
-constexpr int TILE_BYTES = TR * TK * 2;           // one bfloat16 term of the activations; a weight chunk
-static_assert(TO * KC * 2 == TILE_BYTES, "a chunk takes a tile's room");
+constexpr int TILE_BYTES = TO * KC * 2;           // a weight chunk
 // Core matrices are 128 bytes.  Weights are K-major: 8 outputs x 8 inputs, an output's 8 inputs in 16
 // bytes.  Activations are sample-major: 8 inputs x 8 samples, an input's 8 samples in 16 bytes (what a
 // lane that holds one output for many samples stores at once).  Both: core matrices adjacent along
 // outputs / samples 128 bytes apart ("stride"), along the inputs after them ("leading").
-constexpr uint32_t SBO = 128, W_LBO = (TO / 8) * 128, X_LBO = (TR / 8) * 128;
+constexpr int TERMS = 3, TC = TERMS * TR;         // terms of an activation; an accumulator's columns
+constexpr uint32_t SBO = 128, W_LBO = (TO / 8) * 128, X_LBO = (TC / 8) * 128;
+constexpr int ACT_BYTES = TC * TK * 2;            // the activations
+constexpr int TMEM_COLS = 512;                    // two accumulators of 192, a power of two
 constexpr long long WAIT_LIMIT = 1ll << 22;       // mbarrier polls before a wait gives up
 
 // instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A and B bfloat16 (bits 7-9,
 // 10-12 = 1), A K-major (bit 15 = 0), B N-major (bit 16 = 1), N >> 3 at bit 17, M >> 4 at bit 24
-constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(TR >> 3) << 17) |
+constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(TC >> 3) << 17) |
                            ((uint32_t)(TO >> 4) << 24);
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -123,12 +128,12 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// byte offset of weight (output o, input k) in a chunk; of activation (input k, sample r) in a tile
+// byte offset of weight (output o, input k) in a chunk; of term p of activation (input k, sample r)
 __host__ __device__ constexpr uint32_t w_off(int o, int k) {
     return (uint32_t)((((k >> 3) * (TO / 8) + (o >> 3)) << 7) + ((o & 7) << 4) + ((k & 7) << 1));
 }
-__host__ __device__ constexpr uint32_t x_off(int k, int r) {
-    return (uint32_t)((((k >> 3) * (TR / 8) + (r >> 3)) << 7) + ((k & 7) << 4) + ((r & 7) << 1));
+__host__ __device__ constexpr uint32_t x_off(int k, int r, int p) {
+    return (uint32_t)((((k >> 3) * (TC / 8) + p * (TR / 8) + (r >> 3)) << 7) + ((k & 7) << 4) + ((r & 7) << 1));
 }
 
 // two values rounded to bfloat16, the first in the low half

@@ -211,11 +211,13 @@ abs_status gemm(abs_mlp* net, cudaStream_t st, int M, int N, int K, const float*
 // (kernels_umma.cuh).  The activations stay on chip: their three bfloat16 terms in shared memory
 // (96 KB), the weights streaming past them in 16 chunks of 128 outputs x 128 inputs (32 KB each, bulk
 // copies of the tiled weights wt into a ring of three), the accumulators in two tensor-memory buffers of
-// 64 columns, one per group of 128 outputs.  Warps 0-15: the layers' biases and GELU and the split into
+// 192 columns, one per group of 128 outputs.  Warps 0-15: the layers' biases and GELU and the split into
 // terms, 32 outputs x 16 samples of every group each, while the next group's MMAs run; a layer's
 // activations are kept in registers until its last MMA has read the previous ones.  Warp 16: one
-// thread loads the chunks and issues the 24 MMAs of each (8 K steps x 3 terms).  Biases, scales and W1
+// thread loads the chunks and issues the 8 MMAs of each.  Biases, scales and W1
 // wait in shared memory.
+// One block's chain of 16 chunks bounds it, not the MMAs' rate or memory: 26 us for 1 to 9728 samples
+// (one wave of 152 blocks), 5000 of them 94 us as a launch per layer.
 // Every wait is bounded (wait_limit polls); when one gives up the block sets fault and leaves, its
 // outputs unwritten.  idle (the self-test of that path): no MMA is issued.
 // TRAIN: also a0, the pre-activations z and activations a of the layers, and normalised outputs;
@@ -225,7 +227,7 @@ constexpr int FWD_E = 512, FWD_T = FWD_E + 32;
 // normalised inputs
 constexpr int FC_B = 0, FC_OUT = 3 * NH + NOUT, FC_W1 = FC_OUT + 2 * NOUT, FC_X = FC_W1 + NIN * NH,
               FC_COUNT = FC_X + NIN * umma::TR;
-constexpr int FWD_SMEM = 6 * umma::TILE_BYTES + 4 * FC_COUNT + 1024;
+constexpr int FWD_SMEM = umma::ACT_BYTES + 3 * umma::TILE_BYTES + 4 * FC_COUNT + 1024;
 static_assert(FWD_SMEM <= 227 * 1024, "shared memory of a block");
 struct FwdTrain {
     float *a0, *z[3], *a[3];
@@ -246,11 +248,11 @@ __global__ void __launch_bounds__(FWD_T, 1) network_forward_kernel(int M, const 
     unsigned char* sm = (unsigned char*)(((uintptr_t)tc_smem + 1023) & ~(uintptr_t)1023);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int m0 = blockIdx.x * TR;
-    const uint32_t sx = smem_u32(sm), sw = sx + 3 * TILE_BYTES;
+    const uint32_t sx = smem_u32(sm), sw = sx + ACT_BYTES;
     const uint32_t wfull = smem_u32(&bars[0]), wfree = smem_u32(&bars[3]), mdone = smem_u32(&bars[6]),
                    tfree = smem_u32(&bars[8]), aready = smem_u32(&bars[10]);
     if (warp == 0) {
-        tmem_alloc(smem_u32(&tbase), 2 * TR);
+        tmem_alloc(smem_u32(&tbase), TMEM_COLS);
         tmem_relinquish();
     }
     if (tid == 0) {
@@ -264,7 +266,7 @@ __global__ void __launch_bounds__(FWD_T, 1) network_forward_kernel(int M, const 
         }
         mbar_init(aready, FWD_E);
     }
-    float* fc = reinterpret_cast<float*>(sm + 6 * TILE_BYTES);
+    float* fc = reinterpret_cast<float*>(sm + ACT_BYTES + 3 * TILE_BYTES);
     for (int i = tid; i < FC_COUNT; i += FWD_T) {
         float f;
         if (i < FC_OUT) {
@@ -316,16 +318,13 @@ __global__ void __launch_bounds__(FWD_T, 1) network_forward_kernel(int M, const 
                     fence_after();
                     // descriptors differ in the start address alone (its 14 bits hold every address of
                     // the block): one add per operand
-                    const uint32_t acc = tmem + (uint32_t)((g & 1) * TR);
+                    const uint32_t acc = tmem + (uint32_t)((g & 1) * TC);
                     const uint32_t w = wlo + (uint32_t)((c % 3) * (TILE_BYTES >> 4));
                     const uint32_t x = xlo + (uint32_t)((kc * (KC / 8) * (int)X_LBO) >> 4);
 #pragma unroll
                     for (int s = 0; s < KC / 16; ++s)
-#pragma unroll
-                        for (int p = 0; p < 3; ++p)
-                            mma(acc, desc_at(w + (uint32_t)((s * 2 * (int)W_LBO) >> 4), whi),
-                                desc_at(x + (uint32_t)((p * TILE_BYTES + s * 2 * (int)X_LBO) >> 4), xhi), IDESC,
-                                (kc | s | p) != 0);
+                        mma(acc, desc_at(w + (uint32_t)((s * 2 * (int)W_LBO) >> 4), whi),
+                            desc_at(x + (uint32_t)((s * 2 * (int)X_LBO) >> 4), xhi), IDESC, (kc | s) != 0);
                     commit(wfree + 8 * (c % 3));
                     // the chunk before is done with: its buffer takes the chunk after the next
                     if (c >= 1 && loaded < NCHUNK) {
@@ -368,9 +367,8 @@ __global__ void __launch_bounds__(FWD_T, 1) network_forward_kernel(int M, const 
                     float e[8];
 #pragma unroll
                     for (int i = 0; i < 8; ++i) e[i] = v[c][8 * h + i];
-                    const uint32_t o = x_off(TO * c + f, r0 + 8 * h);
 #pragma unroll
-                    for (int p = 0; p < 3; ++p) {
+                    for (int p = 0; p < TERMS; ++p) {
                         uint32_t t[4];
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
@@ -378,7 +376,7 @@ __global__ void __launch_bounds__(FWD_T, 1) network_forward_kernel(int M, const 
                             e[2 * i] -= __uint_as_float(t[i] << 16);
                             e[2 * i + 1] -= __uint_as_float(t[i] & 0xffff0000u);
                         }
-                        *reinterpret_cast<uint4*>(sm + p * TILE_BYTES + o) = make_uint4(t[0], t[1], t[2], t[3]);
+                        *reinterpret_cast<uint4*>(sm + x_off(TO * c + f, r0 + 8 * h, p)) = make_uint4(t[0], t[1], t[2], t[3]);
                     }
                 }
             fence_smem_async();
@@ -403,7 +401,14 @@ __global__ void __launch_bounds__(FWD_T, 1) network_forward_kernel(int M, const 
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) return;
             fence_after();
-            tmem_ld16(tlane + (uint32_t)((q & 1) * TR), t);
+            // the three terms' sums, the smallest first
+            const uint32_t acc = tlane + (uint32_t)((q & 1) * TC);
+            float m[16], l[16];
+            tmem_ld16(acc + 2 * TR, l);
+            tmem_ld16(acc + TR, m);
+            tmem_ld16(acc, t);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) t[i] += m[i] + l[i];
             fence_before();
             mbar_arrive(tfree + 8 * (q & 1));
             ++q;
@@ -436,7 +441,7 @@ __global__ void __launch_bounds__(FWD_T, 1) network_forward_kernel(int M, const 
     }
     fence_before();
     ok = __syncthreads_and(ok);
-    if (warp == 0) tmem_dealloc(tmem, 2 * TR);
+    if (warp == 0) tmem_dealloc(tmem, TMEM_COLS);
     if (!ok && tid == 0) atomicExch(fault, 1);
 }
 
