@@ -567,34 +567,50 @@ abs_status launch_check(abs_problem* h, int kind = KD_VEC, int weight = 1) {
     return ABS_OK;
 }
 
-// the evaluation at x: residuals c (with the partials part) and, when given, Jacobian and Hessian
-// values.  Up to EVAL_SPLIT_S scenarios the parts run on threads of their own (eval_split_kernel):
-// eight scenarios per SM are 2.5 warps of eval_kernel, where one thread's 64 cycles per instruction
-// and the three parts' larger sum meet.
-constexpr int EVAL_SPLIT_S = 8 * 152;
+// the evaluation that A asks for: residuals c and, with part, their partials; Jacobian and Hessian values
+// where given.  Up to EVAL_SPLIT_S scenarios in parts on warps of their own (eval_split_kernel): with 21
+// blocks of 32 scenarios (x 10 stages x 3 kinds) an SM holds four blocks.  Parts / one thread, us: 33
+// scenarios with Jacobian and Hessian 13.0 / 41.5, residuals 10.9 / 18.7; 672 scenarios Hessian 35 / 41,
+// Jacobian 21 / 28, residuals 14.8 / 18.9; 800 scenarios Hessian 36 / 41, but Jacobian 35 / 29; 1216
+// Hessian 56 / 41.
+constexpr int EVAL_SPLIT_S = 21 * 32;
+template <bool PSUM>
+void eval_dispatch(abs_problem* h, const EvalArgs& A, cudaStream_t st) {
+    dim3 g = geval(h);
+    const bool res = A.c || A.part;
+    if (h->S <= EVAL_SPLIT_S) {
+        int what = 0;
+        g.z = 0;
+        if (res) what |= 0 << (4 * g.z++);
+        if (A.jac) what |= 1 << (4 * g.z++);
+        if (A.hes) what |= 2 << (4 * g.z++);
+        if (g.z) eval_split_kernel<PSUM><<<g, dim3(EVAL_T, EVAL_PARTS), 0, st>>>(h->P, A, what);
+    } else if (A.jac && A.hes) {
+        eval_kernel<true, true, true, PSUM><<<g, EVAL_T, 0, st>>>(h->P, A);
+    } else if (A.jac) {
+        eval_kernel<true, true, false, PSUM><<<g, EVAL_T, 0, st>>>(h->P, A);
+    } else if (A.hes) {
+        eval_kernel<true, false, true, PSUM><<<g, EVAL_T, 0, st>>>(h->P, A);
+    } else if (res) {
+        eval_kernel<true, false, false, PSUM><<<g, EVAL_T, 0, st>>>(h->P, A);
+    }
+}
+void eval_any(abs_problem* h, const EvalArgs& A, cudaStream_t st) {
+    if (A.part) eval_dispatch<true>(h, A, st);
+    else eval_dispatch<false>(h, A, st);
+}
+
 abs_status eval_launch(abs_problem* h, const BView& b, const double* x, const double* lam, double* c, double* jac,
                        double* hes, double* part, int kind, cudaStream_t st) {
-    const int S = (int)h->S;
-    dim3 g = geval(h);
-    if (h->S <= EVAL_SPLIT_S && jac) {
-        const int z0 = c || part ? 0 : 1;
-        g.z = (hes ? 3 : 2) - z0;
-        if (hes) eval_split_kernel<true><<<g, EVAL_T, 0, st>>>(h->P, S, h->ld, b, x, lam, h->feed, c, jac, hes, part, z0);
-        else eval_split_kernel<false><<<g, EVAL_T, 0, st>>>(h->P, S, h->ld, b, x, lam, h->feed, c, jac, hes, part, z0);
-    } else if (jac && hes) {
-        eval_kernel<true, true, true><<<g, EVAL_T, 0, st>>>(h->P, S, h->ld, b, false, x, nullptr, nullptr, lam, h->feed,
-                                                            c, jac, hes, part);
-    } else if (jac) {
-        eval_kernel<true, true, false><<<g, EVAL_T, 0, st>>>(h->P, S, h->ld, b, false, x, nullptr, nullptr, lam, h->feed,
-                                                             c, jac, nullptr, part);
-    } else if (hes) {
-        eval_kernel<true, false, true><<<g, EVAL_T, 0, st>>>(h->P, S, h->ld, b, false, x, nullptr, nullptr, lam, h->feed,
-                                                             c, nullptr, hes, part);
-    } else if (c || part) {
-        eval_kernel<true, false, false><<<g, EVAL_T, 0, st>>>(h->P, S, h->ld, b, false, x, nullptr, nullptr, lam,
-                                                              h->feed, c, nullptr, nullptr, part);
-    }
+    eval_any(h, EvalArgs{(int)h->S, h->ld, b, false, x, nullptr, nullptr, lam, h->feed, c, jac, hes, part}, st);
     return launch_check(h, kind);
+}
+
+// residuals and partials at the trial points of the problems in the line search
+abs_status eval_trial_launch(abs_problem* h, const BView& b, const double* x, const double* dxA, const double* dxB,
+                             double* c, double* part, cudaStream_t st) {
+    eval_any(h, EvalArgs{(int)h->S, h->ld, b, true, x, dxA, dxB, nullptr, h->feed, c, nullptr, nullptr, part}, st);
+    return launch_check(h, KD_EVAL_TRIAL);
 }
 
 enum { K_EVAL = 0, K_EVAL_TRIAL = 1, K_FACTOR = 2, K_SOLVE = 3, K_SOLVE_T = 4 };

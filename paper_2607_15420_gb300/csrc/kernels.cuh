@@ -141,7 +141,23 @@ __device__ inline void store_partials(const double (&v)[K], double* part, int64_
 // A1 + A2: residuals, Jacobian and Lagrangian Hessian values, one thread per
 // (scenario, stage); grid (ceil(S / blockDim), N_STAGES).
 // ------------------------------------------------------------------------------------
-template <bool WR, bool WJ, bool WH>
+// The evaluation's values in parts of similar length, for threads that compute one part each (PART >= 0):
+// four of the residuals, four of the Jacobian, four of the Hessian; PART < 0: everything asked for.  What a
+// part leaves out is known at compile time, so the compiler drops what only that needs.
+constexpr int EVAL_PARTS = 4;
+constexpr int PART_LOG = 3;   // the part of the residuals that also sums the barrier's logarithms
+__host__ __device__ constexpr int res_part(int r) {
+    return r < 11 || r == R_SX || r == R_SY ? 0 : (r >= R_RX && r < R_RX + 5 ? 1 : (r == R_E ? 2 : 3));
+}
+__host__ __device__ constexpr int jac_part(int r, int lv) {
+    return r < 11 || (r >= R_RX && r < R_RX + 5) ? 0 : (r == R_E ? (lv < NV ? 1 : 2) : 3);
+}
+__host__ __device__ constexpr int hes_part(int i, int j) {
+    return i < 7 ? 0 : (i < LT ? 1 : (j < 9 ? 2 : 3));
+}
+
+// PSUM: also the partials |c| summed and maximal (as a key, off the FP64 pipe)
+template <bool WR, bool WJ, bool WH, bool PSUM, int PART>
 struct DevEmit {
     static constexpr bool want_res = WR, want_jac = WJ, want_hes = WH;
     double* cv;
@@ -149,17 +165,22 @@ struct DevEmit {
     double* hv;
     int64_t ld;
     int s, n, t;
-    double asum, amax;
-    __device__ void res(int r, double v) {
+    double asum;
+    unsigned long long amax;
+    __device__ __forceinline__ void res(int r, double v) {
+        if (PART >= 0 && res_part(r) != PART) return;
         if (cv) cv[(int64_t)(NR * n + r) * ld + s] = v;
-        const double a = fabs(v);
-        asum += a;
-        amax = (a > amax || a != a) ? a : amax;
+        if (PSUM) {
+            asum += fabs(v);
+            amax = key_max(amax, mag_key(v));
+        }
     }
-    __device__ void jac(int r, int lv, double v) {
+    __device__ __forceinline__ void jac(int r, int lv, double v) {
+        if (PART >= 0 && jac_part(r, lv) != PART) return;
         jv[(int64_t)(c_segJ[n] + c_slotJ[t][r][lv]) * ld + s] = v;
     }
-    __device__ void hes(int i, int j, double v) {
+    __device__ __forceinline__ void hes(int i, int j, double v) {
+        if (PART >= 0 && hes_part(i, j) != PART) return;
         hv[(int64_t)(NHS * n + c_slotH[i][j]) * ld + s] = v;
     }
 };
@@ -182,13 +203,13 @@ __device__ inline void load_stage(const Params& P, int S, int64_t ld, const doub
             const int64_t o = (int64_t)(NV * (n + 1) + abv_var(a)) * ld + s;
             double v = x[o];
             if (dx) v += alpha * dx[o];
-            in.qa[a] = v;
+            in.qa[a] = a < 9 ? P.sx[a] * v : (a == 9 ? v : P.sT * v);
         }
     } else {
 #pragma unroll
-        for (int l = 0; l < 9; ++l) in.qa[l] = feed[(int64_t)(F_XIN + l) * ld + s] / P.sx[l];
+        for (int l = 0; l < 9; ++l) in.qa[l] = feed[(int64_t)(F_XIN + l) * ld + s];
         in.qa[9] = feed[(int64_t)F_LIN * ld + s];
-        in.qa[10] = feed[(int64_t)F_TIN * ld + s] / P.sT;
+        in.qa[10] = feed[(int64_t)F_TIN * ld + s];
     }
     if (in.has_below) {
 #pragma unroll
@@ -196,54 +217,59 @@ __device__ inline void load_stage(const Params& P, int S, int64_t ld, const doub
             const int64_t o = (int64_t)(NV * (n - 1) + blw_var(b)) * ld + s;
             double v = x[o];
             if (dx) v += alpha * dx[o];
-            in.qb[b] = v;
+            in.qb[b] = b < 4 ? P.sy[b] * v : (b == 4 ? v : P.sT * v);
         }
     } else {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) in.qb[j] = feed[(int64_t)(F_Y0 + j) * ld + s] / P.sy[j];
+        for (int j = 0; j < 4; ++j) in.qb[j] = feed[(int64_t)(F_Y0 + j) * ld + s];
         in.qb[4] = feed[(int64_t)F_V0 * ld + s];
-        in.qb[5] = feed[(int64_t)F_T0 * ld + s] / P.sT;
+        in.qb[5] = feed[(int64_t)F_T0 * ld + s];
     }
     const int64_t od = (int64_t)NSC * ld + (int64_t)stage_sec(n, P.nsec) * NP + p;   // its section's diameter
     in.d = x[od] + (dx ? alpha * dx[od] : 0.0);
     in.P = stage_pres(P, feed[(int64_t)F_P * ld + s], n);
 }
 
-// partials (if part non-null): [0] |c| summed over the stage's rows, [1] their max,
-// [2] sum of the barrier logs of the stage unknowns.  trial = false: evaluation at x of
-// the problems flagged PS_ACT; trial = true: at x + alpha_p dir of the problems flagged
-// PS_LSACT, dir = dxB where PS_SOC is set, else dxA.
-template <bool WR, bool WJ, bool WH>
-__device__ __forceinline__ void eval_body(const Params& P, int S, int64_t ld, const BView& b, bool trial,
-                                          const double* __restrict__ x, const double* __restrict__ dxA,
-                                          const double* __restrict__ dxB, const double* __restrict__ lam,
-                                          const double* __restrict__ feed, double* c, double* jac, double* hes,
-                                          double* part) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n = blockIdx.y;
-    const int p = live_prob(b, s, S, trial ? PS_LSACT : PS_ACT);
-    if (p < 0) return;
-    DevEmit<WR, WJ, WH> em;
-    em.cv = c;
-    em.jv = jac;
-    em.hv = hes;
+// The evaluation's argument list: at x (trial = false: the problems flagged PS_ACT) or at x + alpha_p dir
+// (trial = true: those flagged PS_LSACT; dir = dxB where PS_SOC is set, else dxA).
+struct EvalArgs {
+    int S;
+    int64_t ld;
+    BView b;
+    bool trial;
+    const double *x, *dxA, *dxB, *lam, *feed;
+    double *c, *jac, *hes;
+    double* part;
+};
+
+// what scenario slot s and stage n ask for; false: the slot takes no part.  PSUM: v = |c| summed over the
+// part's rows, their max, the sum of the barrier logs of the stage unknowns.
+template <bool WR, bool WJ, bool WH, bool PSUM, int PART>
+__device__ __forceinline__ bool eval_body(const Params& P, const EvalArgs& A, int s, int n, double (&v)[3]) {
+    const int64_t ld = A.ld;
+    const int p = live_prob(A.b, s, A.S, A.trial ? PS_LSACT : PS_ACT);
+    if (p < 0) return false;
+    DevEmit<WR, WJ, WH, PSUM, PART> em;
+    em.cv = A.c;
+    em.jv = A.jac;
+    em.hv = A.hes;
     em.ld = ld;
     em.s = s;
     em.n = n;
     em.t = stage_type(n);
     em.asum = 0.0;
-    em.amax = 0.0;
-    double blog = 0.0;
+    em.amax = 0;
     StageIn in;
     const double* dx = nullptr;
     double alpha = 0.0;
-    if (trial) {
-        dx = (b.ps && psv(b, PS_SOC, p) != 0.0) ? dxB : dxA;
-        alpha = psv(b, PS_ALPHA, p);
+    if (A.trial) {
+        dx = (A.b.ps && psv(A.b, PS_SOC, p) != 0.0) ? A.dxB : A.dxA;
+        alpha = psv(A.b, PS_ALPHA, p);
     }
-    load_stage(P, S, ld, x, dx, alpha, feed, s, n, p, b.NP, in);
+    load_stage(P, A.S, ld, A.x, dx, alpha, A.feed, s, n, p, A.b.NP, in);
     StageLam L;
     if (WH) {
+        const double* lam = A.lam;
 #pragma unroll
         for (int r = 0; r < NR; ++r) L.own[r] = lam[(int64_t)(NR * n + r) * ld + s];
         if (n > 0) {
@@ -258,18 +284,23 @@ __device__ __forceinline__ void eval_body(const Params& P, int S, int64_t ld, co
         }
     }
     stage_eval(P, in, WH ? &L : nullptr, em);
-    if (WH && n == 0) {
+    if (WH && n == 0 && (PART < 0 || PART == EVAL_PARTS - 1)) {
         // the scenario's share of d-d: -u_max pi / 2 * sum_n lambda_hydraulic, one entry per
         // section (its stages' rows)
         for (int k = 0; k < P.nsec; ++k) {
             double sl = 0.0;
 #pragma unroll
             for (int m = 0; m < N_STAGES; ++m)
-                if (stage_sec(m, P.nsec) == k) sl += lam[(int64_t)(NR * m + R_H) * ld + s];
-            hes[(int64_t)(NHS * N_STAGES + k) * ld + s] = -P.u_max * M_PI * 0.5 * sl;
+                if (stage_sec(m, P.nsec) == k) sl += A.lam[(int64_t)(NR * m + R_H) * ld + s];
+            A.hes[(int64_t)(NHS * N_STAGES + k) * ld + s] = -P.u_max * M_PI * 0.5 * sl;
         }
     }
-    if (WR && part) {
+    if (PSUM) {
+        v[0] = em.asum;
+        v[1] = key_double(em.amax);
+        v[2] = 0.0;
+    }
+    if (PSUM && (PART < 0 || PART == PART_LOG)) {
         // sum of ln(slack) over the stage's 18 bounds as the logarithm of their product: the
         // product is carried as a mantissa in [1, 2) times a power of two (exponent read from
         // the bit pattern), so it neither overflows nor underflows; a slack that is not
@@ -278,7 +309,8 @@ __device__ __forceinline__ void eval_body(const Params& P, int S, int64_t ld, co
         long long e2 = 0;
         bool bad = false;
         auto take = [&](double sl) {
-            bad = bad || !(sl > 0.0) || !(sl < INFINITY);
+            // positive and finite: a bit pattern in [1, that of +inf)
+            bad = bad || (unsigned long long)__double_as_longlong(sl) - 1ull >= (0x7ffull << 52) - 1ull;
             m *= sl;
             const unsigned long long bits = (unsigned long long)__double_as_longlong(m);
             const int ex = (int)((bits >> 52) & 0x7ffull);
@@ -294,39 +326,68 @@ __device__ __forceinline__ void eval_body(const Params& P, int S, int64_t ld, co
             if (has_lo(j)) take(in.q[j] - (j == LT ? P.Tlo_s : 0.0));
             if (has_hi(j)) take(P.Thi_s - in.q[j]);
         }
-        blog = bad ? NAN : fma((double)e2, 0.69314718055994530942, ln_tab(m));   // ln 2
-        const double v[3] = {em.asum, em.amax, blog};
-        store_partials<3>(v, part, ld, s, n);
+        v[2] = bad ? NAN : fma((double)e2, 0.69314718055994530942, ln_tab(m));   // ln 2
     }
+    return true;
 }
 
-// One thread per (scenario, stage), in 32-thread blocks: FP64 instructions bound it, and 1570 blocks
-// at 5000 scenarios share out evenly over 152 SMs.
+// One thread per (scenario, stage), in 32-thread blocks: FP64 instructions bound it (5000 scenarios, all
+// values: 121 us; residuals only 45 us), and 1570 blocks at 5000 scenarios share
+// out evenly over 152 SMs.
 constexpr int EVAL_T = 32;
-template <bool WR, bool WJ, bool WH>
-__global__ void __launch_bounds__(EVAL_T) eval_kernel(const Params P, int S, int64_t ld, const BView b, bool trial,
-                                                      const double* __restrict__ x, const double* __restrict__ dxA,
-                                                      const double* __restrict__ dxB, const double* __restrict__ lam,
-                                                      const double* __restrict__ feed, double* c, double* jac,
-                                                      double* hes, double* part) {
-    eval_body<WR, WJ, WH>(P, S, ld, b, trial, x, dxA, dxB, lam, feed, c, jac, hes, part);
+template <bool WR, bool WJ, bool WH, bool PSUM>
+__global__ void __launch_bounds__(EVAL_T) eval_kernel(const Params P, const EvalArgs A) {
+    const int s = blockIdx.x * EVAL_T + threadIdx.x, n = blockIdx.y;
+    double v[3];
+    if (eval_body<WR, WJ, WH, PSUM, -1>(P, A, s, n, v) && PSUM) store_partials<3>(v, A.part, A.ld, s, n);
 }
 
-// The same with a thread per (scenario, stage) and part -- blockIdx.z + z0: 0 residuals, 1 Jacobian, 2
-// Hessian -- for sizes at which the threads of eval_kernel leave schedulers idle: a warp alone on its
-// scheduler issues an FP64 instruction per 64 cycles whatever else the SM does, so three shorter
-// threads finish sooner though together they compute a third more.  The parts' values are
-// eval_kernel's bit for bit (model.cuh: explicit fma).
-template <bool WH>
-__global__ void __launch_bounds__(EVAL_T) eval_split_kernel(const Params P, int S, int64_t ld, const BView b,
-                                                            const double* __restrict__ x,
-                                                            const double* __restrict__ lam,
-                                                            const double* __restrict__ feed, double* c, double* jac,
-                                                            double* hes, double* part, int z0) {
-    const int z = (int)blockIdx.z + z0;
-    if (z == 0) eval_body<true, false, false>(P, S, ld, b, false, x, nullptr, nullptr, lam, feed, c, jac, hes, part);
-    else if (z == 1) eval_body<false, true, false>(P, S, ld, b, false, x, nullptr, nullptr, lam, feed, c, jac, hes, part);
-    else if (WH) eval_body<false, false, true>(P, S, ld, b, false, x, nullptr, nullptr, lam, feed, c, jac, hes, part);
+// the part of a warp of eval_split_kernel
+template <bool WR, bool WJ, bool WH, bool PSUM>
+__device__ __forceinline__ bool eval_part(const Params& P, const EvalArgs& A, int part, int s, int n, double (&v)[3]) {
+    if (part == 0) return eval_body<WR, WJ, WH, PSUM, 0>(P, A, s, n, v);
+    if (part == 1) return eval_body<WR, WJ, WH, PSUM, 1>(P, A, s, n, v);
+    if (part == 2) return eval_body<WR, WJ, WH, PSUM, 2>(P, A, s, n, v);
+    return eval_body<WR, WJ, WH, PSUM, 3>(P, A, s, n, v);
+}
+
+// The same by four warps per 32 (scenario, stage) pairs, each a part, in blocks of their own for the
+// residuals, the Jacobian and the Hessian -- what: 0, 1, 2, a digit per blockIdx.z -- for sizes at which
+// the threads of eval_kernel leave schedulers idle: a warp alone on its scheduler issues an FP64
+// instruction per 64 cycles whatever else the SM does, so twelve short threads finish sooner though
+// together they compute more.  Values agree with eval_kernel's to rounding (the compiler contracts sums
+// differently).
+template <bool PSUM>
+__global__ void __launch_bounds__(EVAL_PARTS * EVAL_T) eval_split_kernel(const Params P, const EvalArgs A, int what) {
+    __shared__ double sh[3][EVAL_PARTS][EVAL_T];
+    const int lane = threadIdx.x, part = threadIdx.y;
+    const int s = blockIdx.x * EVAL_T + lane, n = blockIdx.y;
+    const int kind = (what >> (4 * blockIdx.z)) & 15;
+    double v[3];
+    if (kind == 1) {
+        eval_part<false, true, false, false>(P, A, part, s, n, v);
+    } else if (kind == 2) {
+        eval_part<false, false, true, false>(P, A, part, s, n, v);
+    } else {
+        const bool live = eval_part<true, false, false, PSUM>(P, A, part, s, n, v);
+        if (PSUM) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) sh[k][part][lane] = live ? v[k] : 0.0;
+            __syncthreads();
+            if (part == 0 && live) {
+                unsigned long long mx = 0;
+                v[0] = 0.0;
+#pragma unroll
+                for (int q = 0; q < EVAL_PARTS; ++q) {
+                    v[0] += sh[0][q][lane];
+                    mx = key_max(mx, mag_key(sh[1][q][lane]));
+                }
+                v[1] = key_double(mx);
+                v[2] = sh[2][PART_LOG][lane];
+                store_partials<3>(v, A.part, A.ld, s, n);
+            }
+        }
+    }
 }
 
 // the stage pattern at compile time: Jacobian entries of a stage's own unknowns, and Hessian entries

@@ -120,8 +120,8 @@ __host__ __device__ inline double stage_pres(const Params& P, double Pt, int n) 
 
 struct StageIn {
     double q[NV];     // own scaled unknowns
-    double qa[11];    // from above: xt[9], L, Tt  (the lean feed, scaled, on the top stage)
-    double qb[6];     // from below: yt[4], V, Tt  (the flue gas, scaled, on stage 0)
+    double qa[11];    // from above, in physical units: x[9], L, T  (the lean feed on the top stage)
+    double qb[6];     // from below: y[4], V, T  (the flue gas on stage 0)
     double d, P;
     bool has_above, has_below;   // neighbour stage exists (its values are unknowns)
 };
@@ -139,9 +139,8 @@ struct StageLam {
 // FP64 instructions bound the evaluation on the device (one warp instruction per 19 cycles and
 // SM), so the terms are arranged for few of them: products by structural zeros and ones are left
 // out by hand (the compiler may not drop 0 x), Henry's second derivatives are formed per class of
-// species instead of per pair, one division serves several reciprocals.  Every product that is
-// added to something is an explicit fma, so a value comes out the same whichever of the three
-// parts (residuals, Jacobian, Hessian) an instance computes.
+// species instead of per pair, one division serves several reciprocals.  Every loop unrolls, so
+// an emitter that keeps only some rows or entries leaves out what only the others need.
 #ifdef __CUDACC__
 // ln(x) for the residuals: x = 2^e m, m in [1, 2); 1 / c from a table at the centre c of m's
 // 128th, r = m / c - 1 (|r| < 2^-8, one fma), ln x = e ln 2 + ln c + (r - r^2 / 2 + ... + r^7 / 7)
@@ -188,11 +187,11 @@ __host__ __device__ inline void stage_eval(const Params& P, const StageIn& in, c
     const double L = in.q[LL], V = in.q[LV], T = sT * in.q[LT];
     double xa[9], yb[4];
 #pragma unroll
-    for (int l = 0; l < 9; ++l) xa[l] = P.sx[l] * in.qa[l];
+    for (int l = 0; l < 9; ++l) xa[l] = in.qa[l];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) yb[j] = P.sy[j] * in.qb[j];
-    const double La = in.qa[9], Ta = sT * in.qa[10];
-    const double Vb = in.qb[4], Tb = sT * in.qb[5];
+    for (int j = 0; j < 4; ++j) yb[j] = in.qb[j];
+    const double La = in.qa[9], Ta = in.qa[10];
+    const double Vb = in.qb[4], Tb = in.qb[5];
     const double Pr = in.P;
 
     // ---- reciprocals of T + C (Antoine), the stage pressure, the apparent-fraction total
