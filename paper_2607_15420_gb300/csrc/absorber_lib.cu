@@ -448,7 +448,7 @@ struct abs_problem {
     int* rcnt = nullptr;         // [NP] chunk arrivals of the running reduction (zero between launches)
     double* red = nullptr;       // [KMAX][NP]
     double* hred = nullptr;      // pinned [KMAX + 2][NP] staging for scalar copies
-    double* hmap = nullptr;      // pinned, device-mapped [RED_KMAX + 1][NP]: fetched reductions
+    double* hmap = nullptr;      // pinned, device-mapped [RED_HOUT][NP]: fetched reductions
     double* hmap_dev = nullptr;  // (the reduction kernel writes them straight to host memory)
     double* ps = nullptr;        // device per-problem scalars [PS_NFIELDS][NP]
     double* hps = nullptr;       // host values of ps
@@ -672,7 +672,7 @@ abs_status ensure_buffers(abs_problem* h) {
     CK(cudaMemset(h->rcnt, 0, sizeof(int) * (size_t)h->NP));
     CK(cudaMalloc(&h->red, sizeof(double) * (size_t)KMAX * h->NP));
     CK(cudaMallocHost(&h->hred, sizeof(double) * (size_t)(KMAX + 2) * h->NP));
-    CK(cudaHostAlloc(&h->hmap, sizeof(double) * (size_t)(RED_KMAX + 1) * h->NP, cudaHostAllocMapped));
+    CK(cudaHostAlloc(&h->hmap, sizeof(double) * (size_t)RED_HOUT * h->NP, cudaHostAllocMapped));
     CK(cudaHostGetDevicePointer(&h->hmap_dev, h->hmap, 0));
     CK(cudaMalloc(&h->ps, sizeof(double) * (size_t)PS_NFIELDS * h->NP));
     h->hps = new double[(size_t)PS_NFIELDS * h->NP]();
@@ -749,17 +749,16 @@ RedOps make_ops(std::initializer_list<int> l) {
 }
 
 // combine the K partial planes per problem (device result in h->red[k][p]); with fetch,
-// the reduction kernel also writes them (and the problems' d slots of `dslots`, if given)
+// the reduction kernel also writes them (and the entries of d0 and d1, one per problem, if given)
 // to mapped host memory, read after one stream synchronization (no copy round trip)
 abs_status reduce(abs_problem* h, cudaStream_t st, int K, const RedOps& ops, int flag, bool fetch,
-                  const double* dslots = nullptr) {
+                  const double* d0 = nullptr, const double* d1 = nullptr) {
     double* hout = fetch ? h->hmap_dev : nullptr;
-    const double* ds = fetch ? dslots : nullptr;
     switch (K) {
 #define RK(k)                                                                                                      \
     case k:                                                                                                        \
         reduce_kernel<k><<<(unsigned)h->nchunk, RED_T, 0, st>>>(h->part, h->ld, ops, h->chunks, h->nchunk, h->pchunk, \
-                                                                 h->ps, h->NP, flag, h->cred, h->rcnt, h->red, hout, ds); \
+                                                                 h->ps, h->NP, flag, h->cred, h->rcnt, h->red, hout, d0, d1); \
         break;
         RK(1) RK(2) RK(3) RK(4) RK(5) RK(6) RK(7) RK(8) RK(9) RK(10)
 #undef RK

@@ -122,14 +122,6 @@ __device__ __forceinline__ unsigned long long key_max(unsigned long long a, unsi
 }
 __device__ __forceinline__ double key_double(unsigned long long k) { return __longlong_as_double((long long)k); }
 
-__device__ inline double red_id(int op) { return op == RSUM ? 0.0 : (op == RMAX ? -INFINITY : INFINITY); }
-
-__device__ inline double red_op(int op, double a, double b) {
-    if (op == RSUM) return a + b;
-    if (op == RMAX) return (b > a || b != b) ? b : a;
-    return (b < a || b != b) ? b : a;
-}
-
 template <int K>
 __device__ inline void store_partials(const double (&v)[K], double* part, int64_t ld, int s, int n) {
     const int64_t plane = (int64_t)N_STAGES * ld;

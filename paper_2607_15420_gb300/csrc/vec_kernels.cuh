@@ -639,123 +639,148 @@ __global__ void max_abs_kernel(int S, int64_t ld, const BView b, const double* _
 // chunk c covers elements [i0, i1) of problem p (element i: stage i / S_p, slot off_p +
 // i % S_p); one block per chunk, fixed-order tree; out[k * nchunk + c]
 constexpr int RED_T = 128;                  // threads per chunk block
-constexpr int RED_PER = 2;                  // elements per thread and plane
-constexpr int RED_CHUNK = RED_T * RED_PER;  // elements per chunk
+constexpr int RED_PER = 8;                  // elements per lane and plane, their loads issued together
+constexpr int RED_CHUNK = 32 * RED_PER;     // elements per chunk
 constexpr int RED_KMAX = 12;
-constexpr int RED_TAIL = 8;                 // chunk rounds whose loads the last block issues together
+constexpr int RED_HOUT = RED_KMAX + 2;      // rows of the host's copy: the planes, two d slots
 
-__device__ inline double warp_red(int op, double a) {
-    // xor tree: every lane ends with the same value (each pair is combined in both orders
-    // by commutative operations), in a fixed order
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a = red_op(op, a, __shfl_xor_sync(0xffffffffu, a, o));
-    return a;
+// Maxima and minima run on integer keys that order like the values (an FP64 comparison costs a warp 64
+// cycles, an integer one a few): the bits with a negative value's magnitude inverted, a NaN above
+// everything, all complemented for a minimum, so that both are maxima of keys.
+__device__ __forceinline__ long long red_key(int op, double a) {
+    const long long b = __double_as_longlong(a);
+    if ((b & 0x7fffffffffffffffll) > (0x7ffll << 52)) return 0x7fffffffffffffffll;
+    const long long k = b ^ ((b >> 63) & 0x7fffffffffffffffll);
+    return op == RMAX ? k : ~k;
 }
+__device__ __forceinline__ double red_val(int op, long long k) {
+    if (k == 0x7fffffffffffffffll) return NAN;
+    if (op != RMAX) k = ~k;
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+}
+__device__ __forceinline__ long long key_max(long long a, long long b) { return a > b ? a : b; }
 
-// One block per chunk of a problem's (stage, slot) elements: every plane k < K reduced in
-// a fixed order (RED_PER elements per thread, xor trees within warps, warps in order) into
-// cout[k][c].  The problem's chunk block that finishes last (a per-problem arrival
-// counter; no block waits for another) then combines the problem's chunk results, chunk c
-// on lane (c - c0) % 32 in increasing c, then an xor tree, into out[k][p] (and hout[k][p]
-// with hout[RED_KMAX][p] = dslots[p], when the host fetches them) and re-arms the
-// counter.  Every combination order depends on the problem's own size only.  All of a
-// thread's loads are issued before the first combination (one memory latency per block
-// instead of one per plane).
+// a lane's running combination of a plane: the sum in v or the key in k
+struct RedAcc {
+    double v;
+    long long k;
+    __device__ __forceinline__ explicit RedAcc(int op)
+        : v(0.0), k(red_key(op, op == RMAX ? -INFINITY : INFINITY)) {}
+    __device__ __forceinline__ void take(int op, const double (&t)[RED_PER], const bool (&ok)[RED_PER]) {
+        if (op == RSUM) {
+#pragma unroll
+            for (int i = 0; i < RED_PER; ++i)
+                if (ok[i]) v += t[i];
+        } else {
+#pragma unroll
+            for (int i = 0; i < RED_PER; ++i)
+                if (ok[i]) k = key_max(k, red_key(op, t[i]));
+        }
+    }
+    // over the warp's lanes by an xor tree: every lane ends with the same value, in a fixed order
+    __device__ __forceinline__ double warp(int op) {
+        if (op == RSUM) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            return v;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) k = key_max(k, __shfl_xor_sync(0xffffffffu, k, o));
+        return red_val(op, k);
+    }
+};
+
+// One block per chunk of 256 of a problem's (stage, slot) elements; plane k on warp k % 4, element
+// i0 + lane + 32 t on lane `lane` in increasing t, then an xor tree, into cout[k][c].  The problem's chunk
+// block that finishes last (a per-problem arrival counter; no block waits for another) then combines the
+// problem's chunk results in the same manner into out[k][p] (and hout[k][p], when the host fetches them)
+// and re-arms the counter; a problem of one chunk is done at once.  hout's last rows take the problem's
+// entries of d0 and d1, if given.  Every combination order depends on the problem's own size only.
+// Latencies bound it, a chain of a load, eight combinations and five exchanges per plane and phase: so few
+// FP64 instructions and little code, and a plane's loads together.  Five planes of 5000 scenarios:
+// 14.7 -> 9.4 us, of 10 scenarios 10.7 -> 5.0 us against planes spread over the whole block with
+// FP64 comparisons.
 template <int K>
 __global__ void __launch_bounds__(RED_T) reduce_kernel(const double* __restrict__ part, int64_t ld,
                                                        const RedOps ops, const int* __restrict__ ch, int nchunk,
                                                        const int* __restrict__ pchunk, const double* __restrict__ ps,
                                                        int NP, int flag, double* cout, int* cnt,
                                                        double* __restrict__ out, double* __restrict__ hout,
-                                                       const double* __restrict__ dslots) {
+                                                       const double* __restrict__ d0, const double* __restrict__ d1) {
     static_assert(K >= 1 && K <= RED_KMAX, "planes per reduction");
-    __shared__ double sm[RED_T / 32][K];
+    constexpr int NW = RED_T / 32;
+    constexpr int KW = (K + NW - 1) / NW;   // planes per warp
     __shared__ int last;
     const int c = blockIdx.x;
     const int p = ch[5 * c + 0], off = ch[5 * c + 1], Sp = ch[5 * c + 2], i0 = ch[5 * c + 3], i1 = ch[5 * c + 4];
+    const int c0 = pchunk[p], nc = pchunk[p + 1] - c0;
     const bool live = !ps || ps[(int64_t)flag * NP + p] != 0.0;
     const int64_t plane = (int64_t)N_STAGES * ld;
-    int64_t idx[RED_PER];
-    bool ok[RED_PER];
-#pragma unroll
-    for (int t = 0; t < RED_PER; ++t) {
-        const int i = i0 + (int)threadIdx.x + RED_T * t;
-        ok[t] = live && i < i1;
-        idx[t] = ok[t] ? (int64_t)(i / Sp) * ld + off + i % Sp : 0;
-    }
-    double v[K][RED_PER];
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-#pragma unroll
-        for (int t = 0; t < RED_PER; ++t) v[k][t] = ok[t] ? part[(int64_t)k * plane + idx[t]] : 0.0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto done = [&](int k, double a) {
+        out[(int64_t)k * NP + p] = a;
+        if (hout) hout[(int64_t)k * NP + p] = a;
+    };
+    {
+        int64_t idx[RED_PER];
+        bool ok[RED_PER];
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const int op = ops.op[k];
-        double a = red_id(op);
-#pragma unroll
-        for (int t = 0; t < RED_PER; ++t)
-            if (ok[t]) a = red_op(op, a, v[k][t]);
-        a = warp_red(op, a);
-        if (lane == 0) sm[warp][k] = a;
-    }
-    __syncthreads();
-    if ((int)threadIdx.x < K) {
-        const int k = threadIdx.x, op = ops.op[k];
-        double a = red_id(op);
-#pragma unroll
-        for (int w = 0; w < RED_T / 32; ++w) a = red_op(op, a, sm[w][k]);
-        cout[(int64_t)k * nchunk + c] = a;
-    }
-    const int c0 = pchunk[p], c1 = pchunk[p + 1];
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(&cnt[p], 1) == c1 - c0 - 1;
-    __syncthreads();
-    if (!last) return;
-    if (threadIdx.x == 0) cnt[p] = 0;
-    __threadfence();
-    // the problem's chunk results: plane k on warp k % 4, chunk c0 + lane + 32 i on lane
-    // `lane` in increasing i (L2 reads: other blocks wrote them).  The loads of RED_TAIL
-    // rounds of all the warp's planes are issued before the first combination: one L2
-    // latency per RED_TAIL rounds instead of one per round and plane
-    constexpr int NW = RED_T / 32;
-    constexpr int KW = (K + NW - 1) / NW;   // planes per warp
-    int opk[KW];
-    double acc[KW];
-#pragma unroll
-    for (int u = 0; u < KW; ++u) {
-        const int k = warp + NW * u;
-        opk[u] = k < K ? ops.op[k] : RSUM;
-        acc[u] = red_id(opk[u]);
-    }
-    const int nc = c1 - c0;
-    for (int base = 0; base < nc; base += 32 * RED_TAIL) {
-        double t[KW][RED_TAIL];
+        for (int t = 0; t < RED_PER; ++t) {
+            const int i = i0 + lane + 32 * t;
+            ok[t] = live && i < i1;
+            idx[t] = ok[t] ? (int64_t)(i / Sp) * ld + off + i % Sp : 0;
+        }
+        double v[KW][RED_PER];
 #pragma unroll
         for (int u = 0; u < KW; ++u)
 #pragma unroll
-            for (int i = 0; i < RED_TAIL; ++i) {
-                const int k = warp + NW * u, cc = base + lane + 32 * i;
-                t[u][i] = (k < K && cc < nc) ? __ldcg(&cout[(int64_t)k * nchunk + c0 + cc]) : 0.0;
+            for (int t = 0; t < RED_PER; ++t)
+                v[u][t] = (ok[t] && warp + NW * u < K) ? part[(int64_t)(warp + NW * u) * plane + idx[t]] : 0.0;
+#pragma unroll
+        for (int u = 0; u < KW; ++u) {
+            const int k = warp + NW * u;
+            if (k >= K) continue;   // warp-uniform
+            const int op = ops.op[k];
+            RedAcc acc(op);
+            acc.take(op, v[u], ok);
+            const double a = acc.warp(op);
+            if (lane == 0) {
+                if (nc == 1) done(k, a);
+                else cout[(int64_t)k * nchunk + c] = a;
             }
-#pragma unroll
-        for (int u = 0; u < KW; ++u)
-#pragma unroll
-            for (int i = 0; i < RED_TAIL; ++i)
-                if (base + lane + 32 * i < nc) acc[u] = red_op(opk[u], acc[u], t[u][i]);
-    }
-#pragma unroll
-    for (int u = 0; u < KW; ++u) {
-        const int k = warp + NW * u;
-        if (k >= K) continue;   // warp-uniform
-        const double a = warp_red(opk[u], acc[u]);
-        if (lane == 0) {
-            out[(int64_t)k * NP + p] = a;
-            if (hout) hout[(int64_t)k * NP + p] = a;
         }
     }
-    if (hout && dslots && threadIdx.x == 0) hout[(int64_t)RED_KMAX * NP + p] = dslots[p];
+    if (nc > 1) {
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(&cnt[p], 1) == nc - 1;
+        __syncthreads();
+        if (!last) return;
+        if (threadIdx.x == 0) cnt[p] = 0;
+        __threadfence();
+#pragma unroll 1
+        for (int k = warp; k < K; k += NW) {
+            const int op = ops.op[k];
+            RedAcc acc(op);
+            for (int base = 0; base < nc; base += 32 * RED_PER) {
+                double t[RED_PER];
+                bool ok[RED_PER];
+#pragma unroll
+                for (int i = 0; i < RED_PER; ++i) {   // L2 reads: other blocks wrote them
+                    const int cc = base + lane + 32 * i;
+                    ok[i] = cc < nc;
+                    t[i] = ok[i] ? __ldcg(&cout[(int64_t)k * nchunk + c0 + cc]) : 0.0;
+                }
+                acc.take(op, t, ok);
+            }
+            const double a = acc.warp(op);
+            if (lane == 0) done(k, a);
+        }
+    }
+    if (hout && threadIdx.x == 0) {
+        if (d0) hout[(int64_t)RED_KMAX * NP + p] = d0[p];
+        if (d1) hout[(int64_t)(RED_KMAX + 1) * NP + p] = d1[p];
+    }
 }
 
 // dd_p = (r_d - (beta - dw qp)) / S_d from the Schur sums red[2][p], red[3][p]; into the
