@@ -1059,7 +1059,10 @@ abs_status tc_schur(abs_problem* h, const KKTSys& K, const double* p, const doub
 // (fetch: also to the host, RED); q = J^-1 b.  Mixed precision: FP64 factors of the escalated
 // scenarios only (the others keep their FP32 ones).  x: primal vector whose d slots hold the
 // problems' d.
-abs_status kkt_factor_core(abs_problem* h, const KKTSys& K, const double* x, cudaStream_t st, bool fetch) {
+// fetch: the sums also to the host, with the entries of d0 and d1 (one per problem), after one
+// synchronization
+abs_status kkt_factor_core(abs_problem* h, const KKTSys& K, const double* x, cudaStream_t st, bool fetch,
+                           const double* d0 = nullptr, const double* d1 = nullptr) {
     abs_status r;
     const bool two = h->P.nsec == 2;
     if (K.ldl) {
@@ -1075,7 +1078,7 @@ abs_status kkt_factor_core(abs_problem* h, const KKTSys& K, const double* x, cud
                                                                      h->part, 0, -1.0, true,
                                                                      K.use_w ? K.hes : nullptr);
         if ((r = launch_check(h, KD_SOLVE)) != ABS_OK) return r;
-        return reduce(h, st, 7, make_ops({RSUM, RSUM, RSUM, RSUM, RSUM, RSUM, RSUM}), PS_ACT, fetch);
+        return reduce(h, st, 7, make_ops({RSUM, RSUM, RSUM, RSUM, RSUM, RSUM, RSUM}), PS_ACT, fetch, d0, d1);
     }
     // FP64: a pivot below 1e-14 of the core's largest entry marks the stage block singular; FP32:
     // only (numerically) zero pivots do -- accuracy is guarded by the FP64 refinement instead, with
@@ -1107,8 +1110,9 @@ abs_status kkt_factor_core(abs_problem* h, const KKTSys& K, const double* x, cud
         r = launch_check(h, KD_SCHUR);
     }
     if (r != ABS_OK) return r;
-    if (two) return reduce(h, st, 9, make_ops({RSUM, RSUM, RSUM, RSUM, RSUM, RSUM, RSUM, RSUM, RSUM}), PS_ACT, fetch);
-    return reduce(h, st, 6, make_ops({RSUM, RSUM, RSUM, RSUM, RSUM, RSUM}), PS_ACT, fetch);
+    if (two)
+        return reduce(h, st, 9, make_ops({RSUM, RSUM, RSUM, RSUM, RSUM, RSUM, RSUM, RSUM, RSUM}), PS_ACT, fetch, d0, d1);
+    return reduce(h, st, 6, make_ops({RSUM, RSUM, RSUM, RSUM, RSUM, RSUM}), PS_ACT, fetch, d0, d1);
 }
 
 // one Schur-reduced solve for every active problem: rz (z part), rc -> dz (d slots set), dl;
