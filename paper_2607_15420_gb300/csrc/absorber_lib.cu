@@ -750,15 +750,16 @@ RedOps make_ops(std::initializer_list<int> l) {
 
 // combine the K partial planes per problem (device result in h->red[k][p]); with fetch,
 // the reduction kernel also writes them (and the entries of d0 and d1, one per problem, if given)
-// to mapped host memory, read after one stream synchronization (no copy round trip)
+// to mapped host memory, read after one stream synchronization (no copy round trip); with dz
+// the planes are a solve's Schur sums and the design entries' steps go to dz's slots
 abs_status reduce(abs_problem* h, cudaStream_t st, int K, const RedOps& ops, int flag, bool fetch,
-                  const double* d0 = nullptr, const double* d1 = nullptr) {
+                  const double* d0 = nullptr, const double* d1 = nullptr, double* dz = nullptr) {
     double* hout = fetch ? h->hmap_dev : nullptr;
     switch (K) {
 #define RK(k)                                                                                                      \
     case k:                                                                                                        \
         reduce_kernel<k><<<(unsigned)h->nchunk, RED_T, 0, st>>>(h->part, h->ld, ops, h->chunks, h->nchunk, h->pchunk, \
-                                                                 h->ps, h->NP, flag, h->cred, h->rcnt, h->red, hout, d0, d1); \
+                                                                 h->ps, h->NP, flag, h->cred, h->rcnt, h->red, hout, d0, d1, dz, h->P.nsec); \
         break;
         RK(1) RK(2) RK(3) RK(4) RK(5) RK(6) RK(7) RK(8) RK(9) RK(10)
 #undef RK
@@ -768,6 +769,11 @@ abs_status reduce(abs_problem* h, cudaStream_t st, int K, const RedOps& ops, int
     if (r != ABS_OK) return r;
     if (!fetch) return ABS_OK;
     return sync(h, st);
+}
+
+// the Schur sums of a solve's right-hand side and its design steps, into dz's slots
+abs_status solve_sums(abs_problem* h, double* dz, cudaStream_t st) {
+    return reduce(h, st, 4, make_ops({RSUM, RSUM, RSUM, RSUM}), PS_ACT, false, nullptr, nullptr, dz);
 }
 
 double RED(const abs_problem* h, int k, int p) { return h->hmap[(size_t)k * h->NP + p]; }
@@ -1133,9 +1139,7 @@ abs_status kkt_solve_launches(abs_problem* h, const KKTSys& K, const double* x, 
                                                                      rz, rc, false, dz, dl, h->part, 2, 1.0, false,
                                                                      nullptr);
         if ((r = launch_check(h, KD_SOLVE)) != ABS_OK) return r;
-        if ((r = reduce(h, st, 4, make_ops({RSUM, RSUM, RSUM, RSUM}), PS_ACT, false)) != ABS_OK) return r;
-        finalize_dd_kernel<<<(unsigned)((h->NP + 127) / 128), 128, 0, st>>>(h->ld, view(h), h->red, dz);
-        if ((r = launch_check(h, KD_VEC)) != ABS_OK) return r;
+        if ((r = solve_sums(h, dz, st)) != ABS_OK) return r;
         ldl_back_kernel<<<dim3((unsigned)((h->S + 127) / 128), N_STAGES), 128, 0, st>>>((int)h->S, h->ld, view(h),
                                                                                        V(h, V_Q), V(h, V_QL), dz, dl);
         if ((r = launch_check(h, KD_DZ)) != ABS_OK) return r;
@@ -1150,10 +1154,11 @@ abs_status kkt_solve_launches(abs_problem* h, const KKTSys& K, const double* x, 
                 r = solve_p(h, K.prec, &K, x, rc, rz, V(h, V_P), 1, st);
             }
             if (r != ABS_OK) return r;
-            if ((r = reduce(h, st, 4, make_ops({RSUM, RSUM, RSUM, RSUM}), PS_ACT, false)) != ABS_OK) return r;
+            if ((r = solve_sums(h, dz, st)) != ABS_OK) return r;
+        } else {
+            finalize_dd_kernel<<<(unsigned)((h->NP + 127) / 128), 128, 0, st>>>(h->ld, view(h), h->red, dz, nsec);
+            if ((r = launch_check(h, KD_VEC)) != ABS_OK) return r;
         }
-        finalize_dd_kernel<<<(unsigned)((h->NP + 127) / 128), 128, 0, st>>>(h->ld, view(h), h->red, dz, nsec);
-        if ((r = launch_check(h, KD_VEC)) != ABS_OK) return r;
         if (!tc) {
             if ((r = solve_direction(h, K, x, rz, dz, dl, az, al, res, st)) != ABS_OK) return r;
         } else {

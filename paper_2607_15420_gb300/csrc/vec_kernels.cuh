@@ -635,6 +635,26 @@ __global__ void max_abs_kernel(int S, int64_t ld, const BView b, const double* _
     store_partials<1>(m, part, ld, s, n);
 }
 
+// dd_p = (r_d - (beta - dw qp)) / S_d from the Schur sums red[2][p], red[3][p]; into the
+// problem's d slot of dz
+__device__ inline void finalize_dd(int64_t ld, const BView& b, const double* red, double* dz, int nsec, int p) {
+    const double beta = red[2 * (int64_t)b.NP + p], qp = red[3 * (int64_t)b.NP + p];
+    const double dw = psv(b, PS_DW, p);
+    if (nsec == 1) {
+        dz[(int64_t)NSC * ld + p] = (psv(b, PS_RD, p) - (beta - dw * qp)) / psv(b, PS_SD, p);
+        return;
+    }
+    // two design entries: S_theta [dd0; dd1] = r_theta - (beta - dw qp), S_theta symmetric
+    // positive definite (Algorithm IC), solved by its LDL^T
+    const double beta1 = red[0 * (int64_t)b.NP + p], qp1 = red[1 * (int64_t)b.NP + p];
+    const double r0 = psv(b, PS_RD, p) - (beta - dw * qp), r1 = psv(b, PS_RD1, p) - (beta1 - dw * qp1);
+    const double s00 = psv(b, PS_SD, p), s01 = psv(b, PS_SD01, p), s11 = psv(b, PS_SD11, p);
+    const double l = s01 / s00, e = s11 - l * s01;
+    const double dd1 = (r1 - l * r0) / e;
+    dz[(int64_t)NSC * ld + p] = (r0 - s01 * dd1) / s00;
+    dz[(int64_t)NSC * ld + b.NP + p] = dd1;
+}
+
 // ---- reductions per problem ---------------------------------------------------------
 // chunk c covers elements [i0, i1) of problem p (element i: stage i / S_p, slot off_p +
 // i % S_p); one block per chunk, fixed-order tree; out[k * nchunk + c]
@@ -695,7 +715,8 @@ struct RedAcc {
 // block that finishes last (a per-problem arrival counter; no block waits for another) then combines the
 // problem's chunk results in the same manner into out[k][p] (and hout[k][p], when the host fetches them)
 // and re-arms the counter; a problem of one chunk is done at once.  hout's last rows take the problem's
-// entries of d0 and d1, if given.  Every combination order depends on the problem's own size only.
+// entries of d0 and d1, if given; with dz the sums are a solve's and the problem's design steps follow
+// from them (finalize_dd: 2.9 us and a launch's gap as a kernel of its own).  Every combination order depends on the problem's own size only.
 // Latencies bound it, a chain of a load, eight combinations and five exchanges per plane and phase: so few
 // FP64 instructions and little code, and a plane's loads together.  Five planes of 5000 scenarios:
 // 14.7 -> 9.4 us, of 10 scenarios 10.7 -> 5.0 us against planes spread over the whole block with
@@ -705,8 +726,9 @@ __global__ void __launch_bounds__(RED_T) reduce_kernel(const double* __restrict_
                                                        const RedOps ops, const int* __restrict__ ch, int nchunk,
                                                        const int* __restrict__ pchunk, const double* __restrict__ ps,
                                                        int NP, int flag, double* cout, int* cnt,
-                                                       double* __restrict__ out, double* __restrict__ hout,
-                                                       const double* __restrict__ d0, const double* __restrict__ d1) {
+                                                       double* out, double* __restrict__ hout,
+                                                       const double* __restrict__ d0, const double* __restrict__ d1,
+                                                       double* dz, int nsec) {
     static_assert(K >= 1 && K <= RED_KMAX, "planes per reduction");
     constexpr int NW = RED_T / 32;
     constexpr int KW = (K + NW - 1) / NW;   // planes per warp
@@ -781,29 +803,16 @@ __global__ void __launch_bounds__(RED_T) reduce_kernel(const double* __restrict_
         if (d0) hout[(int64_t)RED_KMAX * NP + p] = d0[p];
         if (d1) hout[(int64_t)(RED_KMAX + 1) * NP + p] = d1[p];
     }
+    if (dz && live) {
+        __syncthreads();
+        if (threadIdx.x == 0) finalize_dd(ld, BView{nullptr, ps, NP}, out, dz, nsec, p);
+    }
 }
 
-// dd_p = (r_d - (beta - dw qp)) / S_d from the Schur sums red[2][p], red[3][p]; into the
-// problem's d slot of dz
 __global__ void finalize_dd_kernel(int64_t ld, const BView b, const double* __restrict__ red, double* __restrict__ dz,
                                    int nsec = 1) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= b.NP || psv(b, PS_ACT, p) == 0.0) return;
-    const double beta = red[2 * (int64_t)b.NP + p], qp = red[3 * (int64_t)b.NP + p];
-    const double dw = psv(b, PS_DW, p);
-    if (nsec == 1) {
-        dz[(int64_t)NSC * ld + p] = (psv(b, PS_RD, p) - (beta - dw * qp)) / psv(b, PS_SD, p);
-        return;
-    }
-    // two design entries: S_theta [dd0; dd1] = r_theta - (beta - dw qp), S_theta symmetric
-    // positive definite (Algorithm IC), solved by its LDL^T
-    const double beta1 = red[0 * (int64_t)b.NP + p], qp1 = red[1 * (int64_t)b.NP + p];
-    const double r0 = psv(b, PS_RD, p) - (beta - dw * qp), r1 = psv(b, PS_RD1, p) - (beta1 - dw * qp1);
-    const double s00 = psv(b, PS_SD, p), s01 = psv(b, PS_SD01, p), s11 = psv(b, PS_SD11, p);
-    const double l = s01 / s00, e = s11 - l * s01;
-    const double dd1 = (r1 - l * r0) / e;
-    dz[(int64_t)NSC * ld + p] = (r0 - s01 * dd1) / s00;
-    dz[(int64_t)NSC * ld + b.NP + p] = dd1;
+    if (p < b.NP && psv(b, PS_ACT, p) != 0.0) finalize_dd(ld, b, red, dz, nsec, p);
 }
 
 }  // namespace absorber
