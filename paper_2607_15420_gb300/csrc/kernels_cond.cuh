@@ -576,6 +576,13 @@ __device__ __forceinline__ unsigned core_key(float a) { return __float_as_uint(a
 __device__ __forceinline__ double core_mag(unsigned k, double) { return __hiloint2double((int)k, 0); }
 __device__ __forceinline__ float core_mag(unsigned k, float) { return __uint_as_float(k); }
 
+// |a| > tiny >= 0, false for NaN; FP64 on the integer pipe (the order of the bits)
+__device__ __forceinline__ bool core_above(double a, double tiny) {
+    const long long m = __double_as_longlong(a) & 0x7fffffffffffffffll;
+    return m > __double_as_longlong(tiny) && m <= (0x7ffll << 52);
+}
+__device__ __forceinline__ bool core_above(float a, float tiny) { return fabsf(a) > tiny; }
+
 __host__ __device__ constexpr size_t chain_smem(size_t es, int spb, int cg) {
     // N At^-1 (7 x 5); CG > 1: two pivot-column buffers (7 + reciprocal), pivot rows, column maxima
     return (size_t)spb * (35 * es + (cg > 1 ? 16 * es + (2 + 2 * cg) * sizeof(int) : 0));
@@ -605,6 +612,22 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
     if (CG == 1 ? !live : !__syncthreads_or(live)) return;
     int bad = 0;
     T kc[5][5];   // K of the stage below
+    // the thread's columns of a stage's M and N (CG > 1): loaded a stage ahead, so that the elimination
+    // does not start with a wait for memory
+    T cm[NCOL][5], ce[NCOL][5];
+    auto columns = [&](int n) {
+        const CondRef<T> f = cond_ref(F, ld, n, (int64_t)s);
+#pragma unroll
+        for (int c = 0; c < NCOL; ++c) {
+            const int j = g + CG * c;
+#pragma unroll
+            for (int k = 0; k < 5; ++k) {
+                cm[c][k] = j < 5 ? f(CF_M + 5 * k + (j < 5 ? j : 0)) : T(0);
+                ce[c][k] = (j < NCORE && j != 4) ? f(CF_N + 6 * k + (j < 4 ? j : (j < NCORE ? j - 1 : 0))) : T(0);
+            }
+        }
+    };
+    if constexpr (CG > 1) columns(0);
 #pragma unroll 1
     for (int n = 0; n < N_STAGES; ++n) {
         const CondRef<T> f = cond_ref(F, ld, n, (int64_t)s);
@@ -635,11 +658,10 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
                     e[k] = c < 4 ? N[k][c < 4 ? c : 0] : (c == 5 ? N[k][4] : (c == 6 ? N[k][5] : T(0)));
                 }
             } else {
-                // the thread's column by address: cached loads of values just read
 #pragma unroll
                 for (int k = 0; k < 5; ++k) {
-                    m[k] = j < 5 ? f(CF_M + 5 * k + (j < 5 ? j : 0)) : T(0);
-                    e[k] = (j < NCORE && j != 4) ? f(CF_N + 6 * k + (j < 4 ? j : (j < NCORE ? j - 1 : 0))) : T(0);
+                    m[k] = cm[c][k];
+                    e[k] = ce[c][k];
                 }
             }
             if (n > 0) {
@@ -665,6 +687,8 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
 #pragma unroll
             for (int q = 0; q < CG; ++q) km = max(km, sK[((n & 1) * CG + q) * SPB + i]);
         }
+        if constexpr (CG > 1)
+            if (n + 1 < N_STAGES) columns(n + 1);
         const T tiny = (T)pivtol * core_mag(km, T(0));
         unsigned orig = 0x6543210u;   // nibble k: the row now at position k
 #pragma unroll
@@ -688,7 +712,7 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
                     c[r] = p == r ? pv : x;
                     pv = p == r ? x : pv;
                 }
-                if (!((pv < T(0) ? -pv : pv) > tiny)) {   // too small, or NaN
+                if (!core_above(pv, tiny)) {   // too small, or NaN
                     bad = 1;
                     pv = (pv < T(0) ? T(-1) : T(1)) * (tiny > T(0) ? tiny : T(1));
                 }
