@@ -359,6 +359,10 @@ __global__ void __launch_bounds__(128) kkt_residual_kernel(int S, int64_t ld, co
 // [0] min primal ratio (alpha_max), [1] min dual ratio (alpha_z),
 // [2] barrier gradient . dz, [3] max |dz| / (1 + |z|).  invL, invU: the reciprocal slacks
 // rhs_kernel formed at the same x.
+__device__ __forceinline__ bool sign_bit(double a) { return __double2hiint(a) < 0; }
+// a < b for a, b >= 0 by their bits
+__device__ __forceinline__ bool pos_less(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
+
 __global__ void __launch_bounds__(128) step_kernel(const Params P, int S, int64_t ld, const BView b,
                                                    const double* __restrict__ x, const double* __restrict__ dz,
                                                    const double* __restrict__ zL, const double* __restrict__ zU,
@@ -369,58 +373,58 @@ __global__ void __launch_bounds__(128) step_kernel(const Params P, int S, int64_
     const int pr = live_prob(b, s, S, PS_ACT);
     if (pr < 0) return;
     const double mu = psv(b, PS_MU, pr), tau = psv(b, PS_TAU, pr);
-    // the minima of tau s / |d| (primal) and tau z / |dz| (dual), and the maximum of
-    // |d| / (1 + |x|), are carried as fractions num / den (den > 0) compared by
-    // cross-multiplication: one division per bound (1 / slack) and one per ratio at the end
-    double an = 1.0, ad = 1.0, zn = 1.0, zd = 1.0, rn = 0.0, rd = 1.0;
-    double gphi = 0.0;
+    // the minima of s / |d| (primal) and z / |dz| (dual), from 1 / tau, and the maximum of
+    // |d| / (1 + |x|) are carried as fractions num / den (den > 0) compared by
+    // cross-multiplication of their nonnegative parts on the integer pipe (pos_less).  FP64
+    // instructions bound this: ten per bound (tau and mu taken out of the loop), 21 before:
+    // 5000 scenarios 52 -> 35 us
+    double an = 1.0, ad = tau, zn = 1.0, zd = tau, rn = 0.0, rd = 1.0;
+    double gs = 0.0;   // grad of the barrier's logs along d, without mu
     bool dnan = false;
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
         const int64_t o = (int64_t)(NV * n + j) * ld + s;
         const double xv = x[o], d = dz[o];
         const double ad_ = fabs(d), ax = 1.0 + fabs(xv);
-        if (ad_ * rd > rn * ax) {
+        if (pos_less(rn * ax, ad_ * rd)) {
             rn = ad_;
             rd = ax;
         }
-        dnan = dnan || d != d;
+        dnan = dnan || mag_key(d) > (0x7ffull << 52);
         if (has_lo(j)) {
             const double sl = xv - lo_of(P, j), inv = invL[o];
             const double z = zL[o];
-            const double dzl = mu * inv - z - (z * inv) * d;
+            const double dzl = fma(inv, fma(-z, d, mu), -z);   // mu / s - z - z d / s
             dzL[o] = dzl;
-            if (d < 0.0 && tau * sl * ad < an * -d) {
-                an = tau * sl;
+            if (sign_bit(d) && pos_less(sl * ad, an * -d)) {
+                an = sl;
                 ad = -d;
             }
-            if (dzl < 0.0 && tau * z * zd < zn * -dzl) {
-                zn = tau * z;
+            if (sign_bit(dzl) && pos_less(z * zd, zn * -dzl)) {
+                zn = z;
                 zd = -dzl;
             }
-            gphi += (-mu * inv) * d;
-        } else {
-            dzL[o] = 0.0;
+            gs = fma(-inv, d, gs);
         }
         if (has_hi(j)) {
             const double su = hi_of(P, j) - xv, inv = invU[o];
             const double z = zU[o];
-            const double dzu = mu * inv - z + (z * inv) * d;
+            const double dzu = fma(inv, fma(z, d, mu), -z);
             dzU[o] = dzu;
-            if (d > 0.0 && tau * su * ad < an * d) {
-                an = tau * su;
+            if (!sign_bit(d) && pos_less(su * ad, an * d)) {
+                an = su;
                 ad = d;
             }
-            if (dzu < 0.0 && tau * z * zd < zn * -dzu) {
-                zn = tau * z;
+            if (sign_bit(dzu) && pos_less(z * zd, zn * -dzu)) {
+                zn = z;
                 zd = -dzu;
             }
-            gphi += (mu * inv) * d;
-        } else {
-            dzU[o] = 0.0;
+            gs = fma(inv, d, gs);
         }
     }
-    const double v[4] = {an / ad, zn / zd, gphi, dnan ? NAN : rn / rd};
+    const double ap = ad == tau && an == 1.0 ? 1.0 : tau * an / ad;   // (1: no bound in the way)
+    const double az = zd == tau && zn == 1.0 ? 1.0 : tau * zn / zd;
+    const double v[4] = {ap, az, mu * gs, dnan ? NAN : rn / rd};
     store_partials<4>(v, part, ld, s, n);
 }
 
@@ -460,8 +464,14 @@ __global__ void __launch_bounds__(128) ftb_kernel(const Params P, int S, int64_t
 }
 
 // accept the step of the problems flagged PS_ACT, then the kappa_Sigma safeguard on the
-// bound multipliers
-__global__ void __launch_bounds__(128) accept_kernel(const Params P, int S, int64_t ld, const BView b, double ksig,
+// bound multipliers (iksig = 1 / ksig).  Six FP64 instructions per thread, 19 with a division for mlo and
+// FP64 comparisons: 5000 scenarios 37 -> 22 us, now bound by its nine vectors
+// t < lo or t > hi for 0 < lo <= hi, by the bits; false for a NaN
+__device__ __forceinline__ bool outside(double t, double lo, double hi) {
+    const long long k = __double_as_longlong(t);
+    return (k < __double_as_longlong(lo) || k > __double_as_longlong(hi)) && mag_key(t) <= (0x7ffull << 52);
+}
+__global__ void __launch_bounds__(128) accept_kernel(const Params P, int S, int64_t ld, const BView b, double ksig, double iksig,
                                                      double* __restrict__ x, const double* __restrict__ dz,
                                                      double* __restrict__ lam, const double* __restrict__ dl,
                                                      double* __restrict__ zL, const double* __restrict__ dzL,
@@ -471,7 +481,7 @@ __global__ void __launch_bounds__(128) accept_kernel(const Params P, int S, int6
     const int pr = live_prob(b, s, S, PS_ACT);
     if (pr < 0) return;
     const double alpha = psv(b, PS_ALPHA, pr), alpha_z = psv(b, PS_ALPHAZ, pr), mu = psv(b, PS_MU, pr);
-    const double mlo = mu / ksig, mhi = ksig * mu;
+    const double mlo = iksig * mu, mhi = ksig * mu;   // (a division here cost more FP64 instructions than the rest)
     const int64_t o = (int64_t)v * ld + s;
     const double xv = x[o] + alpha * dz[o];
     x[o] = xv;
@@ -480,12 +490,12 @@ __global__ void __launch_bounds__(128) accept_kernel(const Params P, int S, int6
     if (has_lo(j)) {
         const double sl = xv - lo_of(P, j);
         const double z = zL[o] + alpha_z * dzL[o];
-        zL[o] = (z * sl < mlo || z * sl > mhi) ? fmin(fmax(z, mlo / sl), mhi / sl) : z;
+        zL[o] = outside(z * sl, mlo, mhi) ? fmin(fmax(z, mlo / sl), mhi / sl) : z;
     }
     if (has_hi(j)) {
         const double su = hi_of(P, j) - xv;
         const double z = zU[o] + alpha_z * dzU[o];
-        zU[o] = (z * su < mlo || z * su > mhi) ? fmin(fmax(z, mlo / su), mhi / su) : z;
+        zU[o] = outside(z * su, mlo, mhi) ? fmin(fmax(z, mlo / su), mhi / su) : z;
     }
 }
 
