@@ -42,10 +42,7 @@ struct PatternTables {
     short slotH[NV][NV];
     Ent own[3][MAXOWN], abv[3][MAXABV], blw[3][MAXBLW], hes[NHS];
     int nown[3], nabv[3], nblw[3], dslot[3];
-    // the same entries grouped by destination (see kernels.cuh)
-    short ownRp[3][NV + 1], abvRp[3][NV + 1], blwRp[3][NV + 1];
-    Ent ownC[3][MAXOWN], abvC[3][MAXABV], blwC[3][MAXBLW];
-    short ownCp[3][NV + 1], abvCp[3][NV + 1], blwCp[3][NV + 1];
+    short blwRp[3][NV + 1];   // row pointers of blw
     Ent hesF[2 * NHS];
     short hesFp[NV + 1];
     std::vector<int> jrow, jcol, hrow, hcol;
@@ -204,24 +201,12 @@ bool build_pattern(PatternTables& T, std::string& err) {
         }
     T.hrow.push_back(NSC);
     T.hcol.push_back(NSC);
-    // destination-grouped copies: row pointers of the (row-ordered) tables, and copies
-    // ordered by the unknown they feed in J^T y (own column, abv_var, blw_var)
     auto rowptr = [](const Ent* tab, int cnt, short* ptr) {
         for (int r = 0; r <= NV; ++r) {
             int k = 0;
             while (k < cnt && tab[k].r < r) ++k;
             ptr[r] = (short)k;
         }
-    };
-    auto bydest = [](const Ent* tab, int cnt, int kind, Ent* out, short* ptr) {
-        auto dest = [kind](const Ent& e) { return kind == 0 ? (int)e.c : (kind == 1 ? abv_var(e.c) : blw_var(e.c)); };
-        int m = 0;
-        for (int j = 0; j < NV; ++j) {
-            ptr[j] = (short)m;
-            for (int k = 0; k < cnt; ++k)
-                if (dest(tab[k]) == j) out[m++] = tab[k];
-        }
-        ptr[NV] = (short)m;
     };
     for (int t = 0; t < 3; ++t) {
         auto rowsorted = [](const Ent* tab, int cnt) {
@@ -233,8 +218,6 @@ bool build_pattern(PatternTables& T, std::string& err) {
             err = "stage table not in row order";
             return false;
         }
-        rowptr(T.own[t], T.nown[t], T.ownRp[t]);
-        rowptr(T.abv[t], T.nabv[t], T.abvRp[t]);
         rowptr(T.blw[t], T.nblw[t], T.blwRp[t]);
         for (int r = 0; r < NV; ++r)
             if (T.blwRp[t][r + 1] - T.blwRp[t][r] > 6) {   // one entry per unknown of the stage below
@@ -249,9 +232,6 @@ bool build_pattern(PatternTables& T, std::string& err) {
                 return false;
             }
         }
-        bydest(T.own[t], T.nown[t], 0, T.ownC[t], T.ownCp[t]);
-        bydest(T.abv[t], T.nabv[t], 1, T.abvC[t], T.abvCp[t]);
-        bydest(T.blw[t], T.nblw[t], 2, T.blwC[t], T.blwCp[t]);
     }
     // the symmetric Hessian block expanded to both triangles, grouped by row
     {
@@ -302,22 +282,11 @@ cudaError_t upload_tables(int dev) {
     UP(c_segJ, T.segJ);
     UP(c_slotH, T.slotH);
     UP(c_own, T.own);
-    UP(c_abv, T.abv);
-    UP(c_blw, T.blw);
     UP(c_hes, T.hes);
     UP(c_nown, T.nown);
     UP(c_nabv, T.nabv);
     UP(c_nblw, T.nblw);
     UP(c_dslot, T.dslot);
-    UP(c_ownRp, T.ownRp);
-    UP(c_abvRp, T.abvRp);
-    UP(c_blwRp, T.blwRp);
-    UP(c_ownC, T.ownC);
-    UP(c_abvC, T.abvC);
-    UP(c_blwC, T.blwC);
-    UP(c_ownCp, T.ownCp);
-    UP(c_abvCp, T.abvCp);
-    UP(c_blwCp, T.blwCp);
     UP(c_hesF, T.hesF);
     UP(c_hesFp, T.hesFp);
     {

@@ -35,8 +35,6 @@ __constant__ short c_slotJ[3][NR][NLOC];
 __constant__ int c_segJ[N_STAGES + 1];
 __constant__ short c_slotH[NV][NV];
 __constant__ Ent c_own[3][MAXOWN];
-__constant__ Ent c_abv[3][MAXABV];
-__constant__ Ent c_blw[3][MAXBLW];
 __constant__ Ent c_hes[NHS];
 __constant__ int c_nown[3], c_nabv[3], c_nblw[3];
 __constant__ int c_dslot[3];           // the d entry of the stage's hydraulic row
@@ -53,13 +51,7 @@ struct __align__(16) LaneTables {
 };
 static_assert(sizeof(LaneTables) % 16 == 0, "LaneTables is copied as 16-byte words");
 __device__ LaneTables g_lt;
-// The same entries grouped by destination, so that the sparse products below accumulate
-// into statically indexed registers (table-indexed register arrays would live in local
-// memory): row pointers of the row-ordered tables (J v), copies ordered by the unknown
-// they feed (J^T y), and the Hessian block expanded to both triangles by row (H v).
-__constant__ short c_ownRp[3][NV + 1], c_abvRp[3][NV + 1], c_blwRp[3][NV + 1];
-__constant__ Ent c_ownC[3][MAXOWN], c_abvC[3][MAXABV], c_blwC[3][MAXBLW];
-__constant__ short c_ownCp[3][NV + 1], c_abvCp[3][NV + 1], c_blwCp[3][NV + 1];
+// the Hessian block expanded to both triangles by row (H v)
 __constant__ Ent c_hesF[2 * NHS];
 __constant__ short c_hesFp[NV + 1];
 

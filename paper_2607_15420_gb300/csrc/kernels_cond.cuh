@@ -594,7 +594,8 @@ __host__ __device__ constexpr size_t chain_smem(size_t es, int spb, int cg) {
 // core's columns g, g + CG, ... in registers; a step's pivot column travels through shared
 // memory (one barrier per step, two buffers).  The chain is ten dependent inverses of seven
 // dependent steps: latency bounds it, FP64's (64 cycles per multiply-add and warp) most of all, so a
-// scenario's columns are spread over lanes and small blocks over all SMs.
+// scenario's columns are spread over lanes and small blocks over all SMs.  FP64 82 us up to 500 scenarios
+// (a warp's block LU of 22 x 22 blocks: 400), 560 at 20000 (8900); FP32 28 us at 5000 (252).
 template <class T, int SPB, int CG>
 __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, const BView b, T* F, int* __restrict__ sing,
                                                          double pivtol, const int* __restrict__ mask,
@@ -819,7 +820,10 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
 // exchange through shared memory; the chains run on the 30 first lanes of the first warp, a lane
 // per scenario and link quantity.  Small blocks because FP64 instructions bound these kernels and
 // 5000 scenarios are few: 834 blocks share out evenly over 152 SMs (32 scenarios x 10 stages per
-// block left five SMs with twice the others' work), and ten scenarios already use two SMs.
+// block left five SMs with twice the others' work), and ten scenarios already use two SMs.  More per
+// block coalesce better, but their chains take longer: a solve, direction and residual of 35000 scenarios
+// with 6 / 8 / 16 / 32 take 784 / 791 / 781 / 920 us in FP32, 1070 / 1185 / 1336 / 1566 in FP64; of 5000
+// 182 / 210 / 209 / 243 in FP32.  Six blocks of 168 registers per SM (eight of 128: 843 us at 35000).
 constexpr int CS_N = 6;
 constexpr int CS_T = 64;
 constexpr int CS_LINK = NLINK * NLINK * CS_N;    // link map of a stage
@@ -1166,7 +1170,8 @@ __device__ __forceinline__ void cond_solve_t_prec(const CondFac& K, int64_t ld, 
 // p = J^-1 r_c, and with planes the Schur sums of the right-hand side (r_z, r_c): 1 -- planes [2]
 // q^T (r_z - H p), [3] q^T p of the first section, [0], [1] of the second; 2 (one section) -- the
 // factorization's sums with them (store_schur).  q has slack entries only, H none but Sigma
-// there: no product with H.  Grid ceil(S / CS_N), CS_T threads.
+// there: no product with H.  Grid ceil(S / CS_N), CS_T threads.  Latencies and the load / store units
+// bound it: 5000 scenarios FP32 26 us (warp-per-scenario 22 x 22 solves: 58), FP64 10 scenarios 23 us.
 template <int PREC>
 __global__ void __launch_bounds__(CS_T, 6) cond_solve_kernel(const Params P, int S, int64_t ld, const BView b,
                                                           const CondFac K, const double* x,
@@ -1204,7 +1209,8 @@ __global__ void __launch_bounds__(CS_T, 6) cond_solve_kernel(const Params P, int
 // One block-elimination solve after its J^-1 r_c (pv) and Schur step (the steps of the design
 // entries in dz's slots): dz = p - q dtheta, g = r_z - (W + Sigma + dw I) dz, dl = J^-T g.  With az,
 // al (a correction) they are added to that direction.  g0 (optional): g, for the residual.  Grid
-// ceil(S / CS_N), CS_T threads.
+// ceil(S / CS_N), CS_T threads.  5000 scenarios FP32 44-57 us (dz and g, and the
+// transposed solve were 13 + 52), the FP64 pipe 42 % busy with the products with H.
 template <int PREC>
 __global__ void __launch_bounds__(CS_T, 6) cond_direction_kernel(
     const Params P, int S, int64_t ld, const BView b, const CondFac K, const double* __restrict__ hes,

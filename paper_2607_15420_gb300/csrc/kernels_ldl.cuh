@@ -25,7 +25,8 @@
 // Unlike the block LU of J_s this needs no square nonsingular J_s: it is the
 // factorization for dc > 0 (Algorithm IC's branch for a singular Jacobian) and for
 // solves that must count the inertia of every scenario block.  Two warps per scenario, FP64, the
-// block in shared memory.
+// block in shared memory.  The FP64 pipe and the pivots' dependent steps bound it: 500 scenarios 1.18 ms
+// (13.9 with dense couplings and a triangular factorization on one warp), a solve 67 us.
 #pragma once
 
 #include "kernels.cuh"

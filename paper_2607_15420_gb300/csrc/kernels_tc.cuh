@@ -1,14 +1,14 @@
 // kernels_tc.cuh -- FP32 stage-block inverses by blocked Gauss-Jordan exchange with the
 // dense trailing updates on the tensor cores (warp-level mma.sync, TF32 operands split in
-// three products for FP32-level accuracy).  Same input and output as factor_gj_kernel:
+// three products for FP32-level accuracy).  Stored per block:
 // the inverse rows of every stage block in position order, -G_n, the row order, the
 // singular flag.
 //
 // One warp per scenario; the augmented block M = [A_n | B_n] (22 x 33) stays in shared
 // memory.  The 22 pivot columns are taken in panels K of 8 (8, 8, 6).  Inside a panel the
 // exchanges run on the panel's columns only, lane i holding row i's panel entries: the
-// pivot search (one warp maximum of position-tagged keys, ties to the lowest position, the
-// rule of factor_gj_kernel), the pivot row's scaling and the rank-1 updates of the other
+// pivot search (one warp maximum of position-tagged keys, ties to the lowest position:
+// pivot_key32), the pivot row's scaling and the rank-1 updates of the other
 // rows.  With R the panel's pivot rows in step order, the panel's exchanges turn
 // [A_RK B_RN; C_OK D_ON] into [A_RK^-1, -A_RK^-1 B_RN; C_OK A_RK^-1, D_ON - C_OK A_RK^-1 B_RN]
 // (the principal pivot transform), so with the new panel columns M'_K (22 x 8) the other
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(32 * WPB, WPB >= 8 ? 3 : 24 / WPB) factor_gj_t
     for (int n = 0; n < N_STAGES; ++n) {
         const int t = stage_type(n);
         const int base = c_segJ[n];
-        // assemble as factor_gj_kernel: every Jacobian load of the lane first, rows zeroed,
+        // assemble: every Jacobian load of the lane first, rows zeroed,
         // entries scattered, then the Schur update A_n -= C_n G_{n-1} on the lane's row
         StageLoads L;
         L.fetch(lt, n, ld, s, lane, jac);

@@ -499,18 +499,6 @@ __global__ void __launch_bounds__(128) accept_kernel(const Params P, int S, int6
     }
 }
 
-// the problems' own step of their design entries: x[d_p] += alpha_p dz[d_p]   (one thread
-// per problem)
-__global__ void dstep_kernel(int64_t ld, const BView b, double* __restrict__ x, const double* __restrict__ dz,
-                             int nsec = 1) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= b.NP || psv(b, PS_ACT, p) == 0.0) return;
-    for (int k = 0; k < nsec; ++k) {
-        const int64_t o = (int64_t)NSC * ld + (int64_t)k * b.NP + p;
-        x[o] += psv(b, PS_ALPHA, p) * dz[o];
-    }
-}
-
 // starting point: every stage copies the inlet streams (or, with base and the problem's
 // PS_BASE set, the stage states of problem p's expected-value solution at
 // base[v * ldb + p], or of the one shared solution at base[v * ldb]), the slack from the hydraulic row at the problem's d (already in
