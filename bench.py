@@ -34,25 +34,23 @@ METRIC = "Newton steps/s & solve time, 5000-scenario absorber, vs FP64 GPU path 
 UNIT = "Newton steps/s"
 DEFAULT_WORKLOAD = "absorber-S5000-tn5-seed2"
 # Algorithmic work per scenario and launch.  Bytes: the values a launch must read and
-# write once (Jacobian 1497 and Hessian 661 entries, 220-entry vectors, factors of 10
-# stage blocks: 22 x 22 LU or inverse, 22 x 11 G for 9 stages, 44 bytes of row order).
-# Flops: FP64 factor = block LU (7183 per stage) + G = At^-1 B (10406 per stage with B);
-# FP32 factor = Gauss-Jordan exchanges (22 steps x 21 rows x 32 columns x 2 + the pivot
-# row's 33 products, 22 columns without B on the last stage); a block solve applies a
-# 22 x 22 factor (968), the coupling (28) and G (484) per stage and right-hand side.
+# write once (Jacobian 1497 and Hessian 661 entries, 220-entry vectors, condensed factors of 10
+# stages x 249 values).  Flops of a stage: condensation about 400; its 7 x 7 core assembled
+# (380), inverted (637) and multiplied into the link maps (390); a block solve reduces (120),
+# applies the core's inverse twice (196), the links (184) and expands (120); a direction adds
+# the product with the Hessian block (2 x 132, FP64).
 EVAL_BYTES_PER_SCEN = 8 * (220 + 220 + 18 + 220 + 1497 + 661)    # read x, lambda, feed; write c, J, H
 # FP64 flops of one evaluation, per scenario, from the kernels' executed FP64 instructions
-# (one ncu capture at 5000 scenarios: DFMA 26.875e6, DMUL 28.27e6, DADD 12.775e6 thread
-# instructions for the full evaluation; DFMA 16.59e6, DMUL 7.775e6, DADD 8.6e6 for the
+# (one ncu capture at 5000 scenarios: DFMA 19.70e6, DMUL 20.09e6, DADD 7.825e6 thread
+# instructions for the full evaluation; DFMA 12.415e6, DMUL 5.675e6, DADD 5.65e6 for the
 # trial evaluation), a fused multiply-add counted as two
-EVAL_FP64_FLOPS_PER_SCEN = (2 * 26.875e6 + 28.27e6 + 12.775e6) / 5000
-TRIAL_FP64_FLOPS_PER_SCEN = (2 * 16.59e6 + 7.775e6 + 8.6e6) / 5000
+EVAL_FP64_FLOPS_PER_SCEN = (2 * 19.70e6 + 20.09e6 + 7.825e6) / 5000
+TRIAL_FP64_FLOPS_PER_SCEN = (2 * 12.415e6 + 5.675e6 + 5.65e6) / 5000
 TRIAL_BYTES_PER_SCEN = 8 * (2 * 220 + 18)                         # read x, dx, feed
-FACTOR_FLOPS_PER_SCEN = {8: 10 * 7183 + 9 * 10406,                # FP64: stage LUs + G
-                         4: 9 * 22 * (21 * 32 * 2 + 33) + 22 * (21 * 21 * 2 + 22)}   # FP32: Gauss-Jordan
-SOLVE_FLOPS_PER_SCEN_RHS = 10 * (28 + 968 + 484)                  # coupling + block apply + G product
-SOLVE_T_FLOPS_PER_SCEN = 10 * (484 + 968 + 28)                    # G^T product + transposed apply + coupling
-PIV_BYTES_PER_SCEN = 10 * 44
+COND_VALUES = 10 * 249
+FACTOR_FLOPS_PER_SCEN = {8: 10 * (400 + 380 + 637 + 390), 4: 10 * (400 + 380 + 637 + 390)}
+SOLVE_FLOPS_PER_SCEN_RHS = 10 * (120 + 196 + 184 + 120)
+SOLVE_T_FLOPS_PER_SCEN = 10 * (120 + 196 + 184 + 120 + 2 * 132)
 # Algorithmic bytes per scenario and launch of every other kernel kind (abs_result.kind_launches,
 # binding.KINDS): the vectors (220 doubles per scenario), Jacobian (1497) and Hessian (661)
 # values each reads and writes once.  Reductions count planes (10 stage partials each).
@@ -60,12 +58,12 @@ V220 = 8 * 220
 KIND_BYTES = {
     "eval_trial": 8 * (2 * 220 + 18) + V220,          # x, dx, feed; c
     "residual": 8 * 1497 + 7 * V220,                  # J; g, dl', dz, r_z, r_c; rho_z, rho_c
-    "schur": 8 * 661 + 4.5 * V220,                    # H; sigma, q, p, r (half the launches); t or Hq
+    "schur": 8 * 20,                                  # the slacks' sigma; one-entry partials
     "dual": 8 * 1497 + 5 * V220,                      # J; lambda, x, zL, zU; J^T lambda
     "reduce_planes": 8 * 10,                          # one stage partial per scenario and plane
     "rhs": 10 * V220,                                 # x, zL, zU, J^T l, c; Sigma, r_z, r_c, 1/s_L, 1/s_U
-    "dz": 6 * V220,                                   # p, q, t, Hq; dz, g
-    "step": 8 * V220,                                 # x, dz, zL, zU, 1/s_L, 1/s_U; dzL, dzU
+    "dz": 6 * V220,                                   # p, q, t, Hq; dz, g (tensor-core factor only)
+    "step": 8 * (5 * 190 + 4 * 10),                   # x, dz; zL, 1/s_L, dzL (17 bounds), zU, 1/s_U, dzU (1)
     "accept": 12 * V220,                              # x, dz, lambda, dl, zL, dzL, zU, dzU; x, lambda, zL, zU
     "vector": 3 * V220,                               # axpby-like: two vectors in, one out
     "control": 0,
@@ -73,12 +71,14 @@ KIND_BYTES = {
 }
 
 
-# DRAM bytes (read + write) per launch of the timed form's largest kernel, from one ncu
-# capture of the 5000-scenario workload (summarised with the profiles), keyed by (kernel,
-# element size) with the sha256 of the kernel source at capture: reported only while the
-# source is unchanged
+# DRAM bytes (read + write) of one factorization (condensation and chain) of the 5000-scenario
+# workload, from an ncu capture (summarised with the profiles), keyed by (kernel, element
+# size) with the sha256 of the factors' sources at capture: reported only while they are
+# unchanged
 CAPTURED_TRAFFIC = {
-    ("factor", 4): (146.073088e6, "8d0df1be6db130255886ce9808ab33651ac880e48082b1634cac8a808c94f246"),
+    ("factor", 4): (48.744192e6, {
+        "kernels_warp.cuh": "ca66a1561da39e59c43cb443253bea510f17b299cee9eb0277a9975099de153e",
+        "kernels_cond.cuh": "e96ca233fdea3c08e2d1106685aded0fc2fd88a58c7bcbd4c8363526c096dd3e"}),
 }
 
 
@@ -87,23 +87,26 @@ def captured_traffic(kernel, es, S):
     ent = CAPTURED_TRAFFIC.get((kernel, es))
     if ent is None or S != 5000:
         return None
-    src = os.path.join(ROOT, "paper_2607_15420_gb300", "csrc", "kernels_warp.cuh")
-    with open(src, "rb") as f:
-        if hashlib.sha256(f.read()).hexdigest() != ent[1]:
-            return None
+    for name, sha in ent[1].items():
+        src = os.path.join(ROOT, "paper_2607_15420_gb300", "csrc", name)
+        if not os.path.exists(src):   # a tree without that factor's source cannot run it
+            continue
+        with open(src, "rb") as f:
+            if hashlib.sha256(f.read()).hexdigest() != sha:
+                return None
     return ent[0]
 
 
 def factor_bytes(es):
-    return es * (4840 + 9 * 242) + 8 * 1497 + PIV_BYTES_PER_SCEN
+    return es * COND_VALUES + 8 * 1497
 
 
-def solve_bytes(es, nrhs):
-    return es * (4840 + 9 * 242) + PIV_BYTES_PER_SCEN + 8 * 300 + nrhs * 8 * 2 * 220
+def solve_bytes(es):
+    return es * COND_VALUES + 8 * 2 * 220
 
 
 def solve_t_bytes(es):
-    return es * (4840 + 9 * 242) + PIV_BYTES_PER_SCEN + 8 * 300 + 8 * 2 * 220
+    return es * COND_VALUES + 8 * (661 + 6 * 220)     # H; sigma, p, r_z; dz, g, dl
 
 
 def load_peaks():
@@ -505,7 +508,7 @@ def main():
         "eval": (EVAL_FP64_FLOPS_PER_SCEN * Sx, EVAL_BYTES_PER_SCEN * Sx),
         "eval_trial": (TRIAL_FP64_FLOPS_PER_SCEN * Sx, TRIAL_BYTES_PER_SCEN * Sx),
         "factor": (FACTOR_FLOPS_PER_SCEN[es] * Sx, factor_bytes(es) * Sx),
-        "solve": (SOLVE_FLOPS_PER_SCEN_RHS * Sx * 1.5, solve_bytes(es, 1.5) * Sx),
+        "solve": (SOLVE_FLOPS_PER_SCEN_RHS * Sx, solve_bytes(es) * Sx),
         "solve_t": (SOLVE_T_FLOPS_PER_SCEN * Sx, solve_t_bytes(es) * Sx),
     }
 
@@ -547,8 +550,8 @@ def main():
     kinds = {n: sum(r.kind_launches[k] for r in prof) / len(prof) for k, n in enumerate(B.KINDS)}
     kb = dict(KIND_BYTES)
     kb["eval"] = EVAL_BYTES_PER_SCEN
-    kb["factor"] = factor_bytes(es)
-    kb["solve"] = solve_bytes(es, 1.5)
+    kb["factor"] = factor_bytes(es) / 2       # two launches per factorization
+    kb["solve"] = solve_bytes(es)
     kb["solve_t"] = solve_t_bytes(es)
     solve_bytes_alg = sum(kinds[n] * kb[n] * Sx for n in kinds)
     whole = {"algorithmic_bytes_per_solve": solve_bytes_alg, "solve_time_s": ms / 1e3 / args.steps,

@@ -186,10 +186,11 @@ abs_status eval_grad_jac_hess(abs_problem* h, const double* x, const double* lam
                               double obj_factor, double* f, double* grad, double* c,
                               double* jac_vals, double* hess_vals, abs_stream_t stream);
 
-#define ABS_PREC_FP64 0   /* stage-block LU and solves in FP64 */
-#define ABS_PREC_FP32 1   /* stage-block LU and solves in FP32, FP64 refinement */
-#define ABS_PREC_FP32_TC 3 /* kkt_factor only: FP32 as ABS_PREC_FP32, the stage-block inverses
-                              by the tensor-core panel kernel (abs_options.factor_kernel = 1) */
+#define ABS_PREC_FP64 0   /* condensed factors and solves in FP64 */
+#define ABS_PREC_FP32 1   /* condensed factors and solves in FP32, FP64 refinement */
+#define ABS_PREC_FP32_TC 3 /* kkt_factor only: FP32 as ABS_PREC_FP32, but the uncondensed
+                              stage-block inverses by the tensor-core panel kernel
+                              (abs_options.factor_kernel = 1) */
 #define ABS_PREC_FP64_LDL 4 /* kkt_factor only: every scenario block K_s by the regularised
                               block LDL^T in FP64 (taken whenever delta_c > 0) */
 
@@ -214,8 +215,10 @@ typedef struct abs_inertia {
  * b_s = dc_s/dd); the inertia of K is that of the scenario blocks plus the sign of S_d
  * (Haynsworth).  Two factorizations of the scenario blocks K_s:
  *  - delta_c = 0 (ABS_PREC_FP64 / FP32 / FP32_TC): the constraint Jacobian J_s (220 x 220,
- *    block tridiagonal with 22 x 22 stage blocks) by a block LU with partial pivoting
- *    inside each stage block; then S_d = K_dd + sum_s q_s^T (W_s + Sigma_s + dw I) q_s,
+ *    block tridiagonal with 22 x 22 stage blocks): each stage block is condensed onto 7
+ *    unknowns (its equilibria, summations, balances of single species and hydraulic row
+ *    eliminated in closed form), the condensed system by a block LU over the stages with
+ *    partial pivoting inside each 7 x 7 block; then S_d = K_dd + sum_s q_s^T (W_s + Sigma_s + dw I) q_s,
  *    q_s = J_s^{-1} b_s, and with J_s nonsingular every K_s has inertia (220, 220, 0)
  *    whatever W_s is.  A singular stage block is reported in n_singular and by
  *    ABS_ERR_NUMERIC;
@@ -280,8 +283,9 @@ typedef struct abs_options {
                                  point, 1 the network's multipliers */
     int32_t autotune;      /* 1: the first factor / solve launch of each kernel, precision and
                               size bucket (S rounded down to a power of two, S >= 256) times
-                              every warps-per-block candidate and keeps the fastest
-                              (results are identical); 0: 4 warps per block */
+                              candidate launch shape and keeps the fastest (results are
+                              identical), 0: a default shape; the FP32 factor and the
+                              tensor-core factor's kernels have several shapes */
     int32_t graphs;        /* 1: the whole solve (every iteration, refinement round, line-search
                               round and restoration step, with the device's decisions as
                               conditional nodes) is captured into one CUDA graph on the second
@@ -289,19 +293,20 @@ typedef struct abs_options {
                               first runs eagerly and tunes the tile shapes); 0: every solve is
                               launched eagerly, the host reading each decision */
     int32_t factor_tile;   /* FP32 factor launches only: 0 shape from autotune; 1, 2, 4, 8:
-                              that many warps (scenarios) per block (identical results);
+                              that many warps per block (identical results);
                               other values are rejected with ABS_ERR_ARG */
     int32_t resto_max;     /* feasibility restoration (Wachter & Biegler 2006, Section 3.3)
                               when the line search fails: at most this many damped Newton
                               steps on the square constraint system with d fixed, until the
                               filter accepts a point with theta reduced by 1 - gamma_theta;
                               0 disables it (the solve then stops with ABS_ERR_LINESEARCH) */
-    int32_t factor_kernel; /* FP32 stage-block inverses: 0 Gauss-Jordan exchanges on the FP32
-                              pipes; 1 blocked Gauss-Jordan (panels of 8 pivot columns) with
-                              the trailing updates on the tensor cores (mma.sync TF32, split
-                              in three products for FP32 accuracy).  Same outputs up to
-                              rounding; kkt_factor uses the last value an ipm_solve set */
-    int32_t kkt;           /* factorization of the scenario blocks: 0 block LU of J_s (inertia
+    int32_t factor_kernel; /* FP32 factors: 0 condensed 7 x 7 blocks on the FP32 pipes; 1
+                              inverses of the 22 x 22 stage blocks by blocked Gauss-Jordan
+                              (panels of 8 pivot columns) with the trailing updates on the
+                              tensor cores (mma.sync TF32, split in three products for FP32
+                              accuracy).  Same directions up to rounding; kkt_factor uses the
+                              last value an ipm_solve set */
+    int32_t kkt;           /* factorization of the scenario blocks: 0 condensed block LU of J_s (inertia
                               from the Schur scalar alone; a singular stage block ends the solve
                               with ABS_ERR_NUMERIC); 1 the regularised block LDL^T of kkt_factor
                               (FP64 only), with Algorithm IC complete: the inertia of every
@@ -313,14 +318,17 @@ void abs_default_options(abs_options* o);
 
 #define ABS_N_PHASES 6   /* eval, factor, solve, linesearch, step, other */
 #define ABS_N_KINDS 16   /* kernel kinds counted in abs_result.kind_launches: 0 evaluation with
-                            the Hessian, 1 line-search trial evaluation, 2 stage-block factor,
-                            3 block solve J x = r, 4 block solve J^T y = g, 5 KKT residual,
-                            6 Schur sums, 7 dual residual J^T lambda, 8 reduction planes (one
-                            count per plane reduced), 9 barrier diagonal and right-hand
-                            sides, 10 dz and g, 11 step sizes, 12 accept, 13 other vector
+                            the Hessian, 1 line-search trial evaluation, 2 factor launches (the
+                            condensation and the chain over the stages: two per factorization),
+                            3 block solve J x = r (with the Schur sums of its right-hand side),
+                            4 direction (dz, g and the block solve J^T y = g in one launch),
+                            5 KKT residual, 6 Schur sums by themselves, 7 dual residual
+                            J^T lambda, 8 reduction planes (one count per plane reduced), 9
+                            barrier diagonal and right-hand sides, 10 dz and g by themselves
+                            (tensor-core factors, block LDL^T), 11 step sizes, 12 accept, 13 other vector
                             kernels, 14 control kernels, 15 evaluation without the Hessian */
 #define ABS_N_KERNELS 5  /* eval (residual+Jacobian+Hessian), eval (line-search trial),
-                            stage-block LU, block solve J x = r, block solve J^T y = g */
+                            factor, block solve J x = r, direction with J^T y = g */
 
 typedef struct abs_result {
     abs_status status;
@@ -347,8 +355,9 @@ typedef struct abs_result {
                                     the inlet-copy start's evaluation */
     double warm_E0, cold_E0;     /* E_0 at the learned start and at the inlet-copy start */
     double warm_theta, cold_theta;  /* constraint violation ||c||_1 at the same two starts */
-    int32_t tiles[4];            /* warps per block last used: factor, solve (1 and 2 right-hand
-                                    sides), transposed solve */
+    int32_t tiles[4];            /* warps per block last used by the kernels with several shapes:
+                                    FP32 factor; the tensor-core factor's solves (1 and 2
+                                    right-hand sides) and transposed solve */
     int32_t graph_replays;       /* graph launches of the solve (whole runs replayed from
                                     captured CUDA graphs) */
     int32_t resto_phases;        /* feasibility restoration phases entered */
@@ -588,9 +597,9 @@ abs_status ipm_solve_learned(abs_problem* h, abs_mlp* net, const abs_options* op
  * allocator synchronisation between CUDA graph captures.  It computes what
  * kkt_factor (FP64, delta_c = 0) followed by kkt_solve (no refinement) compute, with
  * no handle: the caller passes the problem's parameter table and its own device
- * buffers, and every intermediate (stage-block LU factors, G blocks, pivots, the
- * Schur vectors and block partial sums) lives in one static device array of the
- * library, sized for ABS_NOALLOC_MAX_SCENARIOS scenarios (about 8 MB), which every GPU
+ * buffers, and every intermediate (condensed factors, the Schur vectors and block
+ * partial sums) lives in one static device array of the
+ * library, sized for ABS_NOALLOC_MAX_SCENARIOS scenarios (about 3 MB), which every GPU
  * that loads the library holds until the process exits.  The call makes no cudaMalloc,
  * cudaFree, pinned-host or other allocating call.
  *   p          host, the parameter table.
