@@ -847,9 +847,11 @@ abs_status tuned_launch(abs_problem* h, int kind, int es, std::initializer_list<
     return launch(w);
 }
 
-// the FP64 chain's launch shape: one-warp blocks of 4 scenarios x 8 threads while they leave a
-// scheduler each (the shorter chain), of 8 x 4 above (fewer instructions per scenario)
-constexpr int CHAIN_WIDE_S = 4 * 4 * 152;
+// the FP64 chain's launch shape: one-warp blocks of 4 scenarios x 8 threads while an SM holds up to
+// seven (the shorter chain), of 8 x 4 above (fewer instructions per scenario).  A factorization with
+// 4 x 8 / 8 x 4, us: 500 scenarios 135 / 186, 2432 143 / 192, 3648 173 / 200, 4256 191 / 208,
+// 4600 206 / 209, 5000 282 / 231.
+constexpr int CHAIN_WIDE_S = 4 * 7 * 152;
 
 template <class T, int SPB, int CG>
 abs_status chain_go(abs_problem* h, T* F, double pivtol, const int* mask, cudaStream_t st, const int* skip) {

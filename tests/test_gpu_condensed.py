@@ -1,6 +1,6 @@
 """The condensed factors (kernels_cond.cuh) at the edges of their launch shapes: one scenario,
 blocks of 4, 6, 8 and 32 scenarios full and ragged, both sides of the size at which the FP64 chain
-changes its blocks (2432 scenarios), and singular blocks.
+changes its blocks (4256 scenarios), and singular blocks.
 
 The direction is put back into the dense KKT system of sampled scenarios.  Tolerance: the
 elimination's multipliers are at most 7 and its cores have condition below 1e5, so the backward
@@ -47,7 +47,7 @@ def _system(B, S):
 
 
 @pytest.mark.parametrize("prec", [0, 1])
-@pytest.mark.parametrize("S", [1, 3, 4, 5, 6, 7, 32, 33, 2431, 2432, 2437, 4867])
+@pytest.mark.parametrize("S", [1, 3, 4, 5, 6, 7, 32, 33, 2437, 4255, 4256, 4867])
 def test_direction_solves_the_system(B, S, prec):
     import torch
     dw = 1e-3
