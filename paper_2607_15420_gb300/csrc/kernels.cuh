@@ -140,7 +140,8 @@ __host__ __device__ constexpr int hes_part(int i, int j) {
     return i < 7 ? 0 : (i < LT ? 1 : (j < 9 ? 2 : 3));
 }
 
-// PSUM: also the partials |c| summed and maximal (as a key, off the FP64 pipe)
+// PSUM: also the partials |c| summed (by part, added in their order) and maximal (as a key, off the
+// FP64 pipe)
 template <bool WR, bool WJ, bool WH, bool PSUM, int PART>
 struct DevEmit {
     static constexpr bool want_res = WR, want_jac = WJ, want_hes = WH;
@@ -149,13 +150,13 @@ struct DevEmit {
     double* hv;
     int64_t ld;
     int s, n, t;
-    double asum;
+    double asum[EVAL_PARTS];
     unsigned long long amax;
     __device__ __forceinline__ void res(int r, double v) {
         if (PART >= 0 && res_part(r) != PART) return;
         if (cv) cv[(int64_t)(NR * n + r) * ld + s] = v;
         if (PSUM) {
-            asum += fabs(v);
+            asum[res_part(r)] += fabs(v);
             amax = key_max(amax, mag_key(v));
         }
     }
@@ -187,7 +188,7 @@ __device__ inline void load_stage(const Params& P, int S, int64_t ld, const doub
             const int64_t o = (int64_t)(NV * (n + 1) + abv_var(a)) * ld + s;
             double v = x[o];
             if (dx) v += alpha * dx[o];
-            in.qa[a] = a < 9 ? P.sx[a] * v : (a == 9 ? v : P.sT * v);
+            in.qa[a] = a < 9 ? mul_rn(P.sx[a], v) : (a == 9 ? v : mul_rn(P.sT, v));
         }
     } else {
 #pragma unroll
@@ -201,7 +202,7 @@ __device__ inline void load_stage(const Params& P, int S, int64_t ld, const doub
             const int64_t o = (int64_t)(NV * (n - 1) + blw_var(b)) * ld + s;
             double v = x[o];
             if (dx) v += alpha * dx[o];
-            in.qb[b] = b < 4 ? P.sy[b] * v : (b == 4 ? v : P.sT * v);
+            in.qb[b] = b < 4 ? mul_rn(P.sy[b], v) : (b == 4 ? v : mul_rn(P.sT, v));
         }
     } else {
 #pragma unroll
@@ -241,7 +242,8 @@ __device__ __forceinline__ bool eval_body(const Params& P, const EvalArgs& A, in
     em.s = s;
     em.n = n;
     em.t = stage_type(n);
-    em.asum = 0.0;
+#pragma unroll
+    for (int k = 0; k < EVAL_PARTS; ++k) em.asum[k] = 0.0;
     em.amax = 0;
     StageIn in;
     const double* dx = nullptr;
@@ -280,7 +282,7 @@ __device__ __forceinline__ bool eval_body(const Params& P, const EvalArgs& A, in
         }
     }
     if (PSUM) {
-        v[0] = em.asum;
+        v[0] = PART >= 0 ? em.asum[PART < 0 ? 0 : PART] : ((em.asum[0] + em.asum[1]) + em.asum[2]) + em.asum[3];
         v[1] = key_double(em.amax);
         v[2] = 0.0;
     }
@@ -339,8 +341,8 @@ __device__ __forceinline__ bool eval_part(const Params& P, const EvalArgs& A, in
 // residuals, the Jacobian and the Hessian -- what: 0, 1, 2, a digit per blockIdx.z -- for sizes at which
 // the threads of eval_kernel leave schedulers idle: a warp alone on its scheduler issues an FP64
 // instruction per 64 cycles whatever else the SM does, so twelve short threads finish sooner though
-// together they compute more.  Values agree with eval_kernel's to rounding (the compiler contracts sums
-// differently).
+// together they compute more.  Values and partials are eval_kernel's bit for bit (model.cuh), so a
+// problem's do not depend on the batch it runs in.
 template <bool PSUM>
 __global__ void __launch_bounds__(EVAL_PARTS * EVAL_T) eval_split_kernel(const Params P, const EvalArgs A, int what) {
     __shared__ double sh[3][EVAL_PARTS][EVAL_T];
@@ -360,10 +362,9 @@ __global__ void __launch_bounds__(EVAL_PARTS * EVAL_T) eval_split_kernel(const P
             __syncthreads();
             if (part == 0 && live) {
                 unsigned long long mx = 0;
-                v[0] = 0.0;
+                v[0] = ((sh[0][0][lane] + sh[0][1][lane]) + sh[0][2][lane]) + sh[0][3][lane];
 #pragma unroll
                 for (int q = 0; q < EVAL_PARTS; ++q) {
-                    v[0] += sh[0][q][lane];
                     mx = key_max(mx, mag_key(sh[1][q][lane]));
                 }
                 v[1] = key_double(mx);

@@ -140,7 +140,9 @@ struct StageLam {
 // SM), so the terms are arranged for few of them: products by structural zeros and ones are left
 // out by hand (the compiler may not drop 0 x), Henry's second derivatives are formed per class of
 // species instead of per pair, one division serves several reciprocals.  Every loop unrolls, so
-// an emitter that keeps only some rows or entries leaves out what only the others need.
+// an emitter that keeps only some rows or entries leaves out what only the others need.  Every
+// product that is added to something is an explicit fma or a rounded product (mul_rn), so a value
+// comes out the same whatever else an instance computes.
 #ifdef __CUDACC__
 // ln(x) for the residuals: x = 2^e m, m in [1, 2); 1 / c from a table at the centre c of m's
 // 128th, r = m / c - 1 (|r| < 2^-8, one fma), ln x = e ln 2 + ln c + (r - r^2 / 2 + ... + r^7 / 7)
@@ -171,6 +173,15 @@ __host__ __device__ inline double ln_tab(double x) {
 #endif
 }
 
+// a b rounded, never contracted into a following sum
+__host__ __device__ inline double mul_rn(double a, double b) {
+#ifdef __CUDA_ARCH__
+    return __dmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
+
 #ifdef __CUDACC__
 #pragma nv_exec_check_disable
 #endif
@@ -181,10 +192,10 @@ __host__ __device__ inline void stage_eval(const Params& P, const StageIn& in, c
     const double sT = P.sT;
     double x[9], y[4];
 #pragma unroll
-    for (int l = 0; l < 9; ++l) x[l] = P.sx[l] * in.q[LX + l];
+    for (int l = 0; l < 9; ++l) x[l] = mul_rn(P.sx[l], in.q[LX + l]);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) y[j] = P.sy[j] * in.q[LY + j];
-    const double L = in.q[LL], V = in.q[LV], T = sT * in.q[LT];
+    for (int j = 0; j < 4; ++j) y[j] = mul_rn(P.sy[j], in.q[LY + j]);
+    const double L = in.q[LL], V = in.q[LV], T = mul_rn(sT, in.q[LT]);
     double xa[9], yb[4];
 #pragma unroll
     for (int l = 0; l < 9; ++l) xa[l] = in.qa[l];
@@ -444,13 +455,13 @@ __host__ __device__ inline void stage_eval(const Params& P, const StageIn& in, c
             const double a = cls_a(c) == 1 ? P.henry_m : (cls_a(c) == 2 ? P.henry_w : 0.0);
             const double tp = cls_t(c) == 2 ? 2.0 * p1 : p1;
             bc[c] = cls_a(c) ? a - tp : -tp;
-            g0[c] = c0 * gc[c];
+            g0[c] = mul_rn(c0, gc[c]);
         }
 #pragma unroll
         for (int c = 0; c < 5; ++c)
 #pragma unroll
             for (int d = 0; d <= c; ++d) {
-                double v = c7 * fma(bc[c], bc[d], -(double)(cls_t(c) * cls_t(d)));
+                double v = mul_rn(c7, fma(bc[c], bc[d], -(double)(cls_t(c) * cls_t(d))));
                 if (c == 4) v += d == 4 ? 2.0 * g0[4] : g0[d];   // the factor x7 itself
                 pc[c * (c + 1) / 2 + d] = v;
             }
