@@ -250,7 +250,9 @@ typedef struct abs_solve_info {
  * is <= refine_tol or max_refine steps were taken.
  *   rhs_x, sol_x  device primal vectors (220*ld + 1).
  *   rhs_c, sol_c  device row vectors (220*ld).
- *   info          host or NULL (if non-NULL the call synchronises).          */
+ *   info          host or NULL (if non-NULL the call synchronises).
+ * A NaN in the system, the right-hand side or the solution: info->residual is NaN, and with
+ * max_refine > 0 the call returns ABS_ERR_NUMERIC.                          */
 abs_status kkt_solve(abs_problem* h, const double* rhs_x, const double* rhs_c,
                      double* sol_x, double* sol_c, int max_refine, double refine_tol,
                      abs_solve_info* info, abs_stream_t stream);
