@@ -306,8 +306,10 @@ typedef struct abs_options {
                               inverses of the 22 x 22 stage blocks by blocked Gauss-Jordan
                               (panels of 8 pivot columns) with the trailing updates on the
                               tensor cores (mma.sync TF32, split in three products for FP32
-                              accuracy).  Same directions up to rounding; kkt_factor uses the
-                              last value an ipm_solve set */
+                              accuracy).  Same directions up to rounding.  With 1 the second-
+                              order corrections and FP64 escalations of a solve form condensed
+                              factors besides, in the iterations that have any.  kkt_factor
+                              takes its precision argument instead */
     int32_t kkt;           /* factorization of the scenario blocks: 0 condensed block LU of J_s (inertia
                               from the Schur scalar alone; a singular stage block ends the solve
                               with ABS_ERR_NUMERIC); 1 the regularised block LDL^T of kkt_factor

@@ -434,12 +434,13 @@ struct abs_problem {
         const double* sig = nullptr;
         double d = 0.0, dw = 0.0, dc = 0.0, Kdd = 0.0, A0 = 0.0, Q2 = 0.0, Sd = 0.0;
         bool ldl = false;            // factored by the block LDL^T (kernels_ldl.cuh)
+        bool blocks = false;         // by stage-block inverses (kernels_tc.cuh)
     } fac;
     double* ldl_inv = nullptr;       // [S][N_STAGES][990] inverses of the block LDL^T pivot blocks, packed
     Prof prof;
     int autotune = 1;                // tile autotuner on (options.autotune)
     int factor_tile = 0;             // forced FP32 factor shape (options.factor_tile; 0: none)
-    int factor_kernel = 0;           // FP32 factor: 0 Gauss-Jordan on the FP32 pipes, 1 tensor-core panels
+    int factor_kernel = 0;           // a solve's FP32 factor: 0 condensed, 1 tensor-core panels
     // the engine's own stream (stream capture needs a non-default stream) and the event
     // that orders it after the caller's stream
     cudaStream_t stream = nullptr;
@@ -663,13 +664,18 @@ abs_status ensure_stream(abs_problem* h) {
     return ABS_OK;
 }
 
-// factor storage of a precision (FP32: with the tensor-core factor's own when it is selected)
+// condensed factor storage of a precision
 abs_status ensure_factor(abs_problem* h, int prec) {
     if (!h->cond[prec]) {
         const size_t es = prec == ABS_PREC_FP32 ? sizeof(float) : sizeof(double);
         CK(cudaMalloc(&h->cond[prec], es * (size_t)N_STAGES * CF_COUNT * h->ld));
     }
-    if (prec == ABS_PREC_FP32 && h->factor_kernel == 1 && !h->tcAI) {
+    return ABS_OK;
+}
+
+// the tensor-core FP32 factor's
+abs_status ensure_tc(abs_problem* h) {
+    if (!h->tcAI) {
         CK(cudaMalloc(&h->tcG, sizeof(float) * (size_t)N_STAGES * NV * NABV * h->ld));
         CK(cudaMalloc(&h->piv, (size_t)N_STAGES * PIV_BYTES * h->ld));
         CK(cudaMalloc(&h->tcAI, sizeof(float) * (size_t)N_STAGES * NV * NV * h->ld));
@@ -762,6 +768,8 @@ struct KKTSys {
     // block LDL^T of every scenario block (FP64, dw = PS_DW, dc = PS_DC) instead of the
     // block LU of J_s
     bool ldl = false;
+    // FP32: the uncondensed stage-block inverses of the tensor-core factor
+    bool blocks = false;
     // set before kkt_factor_core: the factorization also solves p = J^-1 rc and (one design
     // entry) forms the first solve's right-hand-side sums with this rz (q^T (rz - H p), q^T p;
     // they do not depend on dw), so that the first KKT solve with them starts from both
@@ -854,19 +862,20 @@ abs_status tuned_launch(abs_problem* h, int kind, int es, std::initializer_list<
 constexpr int CHAIN_WIDE_S = 4 * 7 * 152;
 
 template <class T, int SPB, int CG>
-abs_status chain_go(abs_problem* h, T* F, double pivtol, const int* mask, cudaStream_t st, const int* skip) {
+abs_status chain_go(abs_problem* h, T* F, double pivtol, const int* mask, cudaStream_t st, const int* skip, int* sing) {
     chain_kernel<T, SPB, CG><<<(unsigned)((h->S + SPB - 1) / SPB), SPB * CG, chain_smem(sizeof(T), SPB, CG), st>>>(
-        (int)h->S, h->ld, view(h), F, h->sing, pivtol, mask, skip);
+        (int)h->S, h->ld, view(h), F, sing, pivtol, mask, skip);
     return launch_check(h, KD_FACTOR);
 }
 
 // condensed factors of J_s (kernels_cond.cuh) in T, of the scenarios with mask[s] != 0 only when
 // mask is given.  skip (device flag, optional): when set at run time the launches leave the stored
-// factors as they are (they are those of this Jacobian).  The FP32 chain has four threads
-// per scenario: W warps per block.
+// factors as they are (they are those of this Jacobian).  flags = false: the scenarios' singular
+// flags stay as they are.  The FP32 chain has four threads per scenario: W warps per block.
 template <class T>
 abs_status factor_launch(abs_problem* h, const double* jac, double pivtol, cudaStream_t st,
-                         const int* mask = nullptr, const int* skip = nullptr) {
+                         const int* mask = nullptr, const int* skip = nullptr, bool flags = true) {
+    int* sing = flags ? h->sing : nullptr;
     constexpr bool f32 = std::is_same<T, float>::value;
     T* F = (T*)h->cond[f32 ? ABS_PREC_FP32 : ABS_PREC_FP64];
     prof_begin(h, K_FACTOR, st);
@@ -877,10 +886,10 @@ abs_status factor_launch(abs_problem* h, const double* jac, double pivtol, cudaS
     if constexpr (f32) {
         auto go = [&](int w) {
             switch (w) {
-                case 1: return chain_go<float, 8, 4>(h, F, pivtol, mask, st, skip);
-                case 2: return chain_go<float, 16, 4>(h, F, pivtol, mask, st, skip);
-                case 8: return chain_go<float, 64, 4>(h, F, pivtol, mask, st, skip);
-                default: return chain_go<float, 32, 4>(h, F, pivtol, mask, st, skip);
+                case 1: return chain_go<float, 8, 4>(h, F, pivtol, mask, st, skip, sing);
+                case 2: return chain_go<float, 16, 4>(h, F, pivtol, mask, st, skip, sing);
+                case 8: return chain_go<float, 64, 4>(h, F, pivtol, mask, st, skip, sing);
+                default: return chain_go<float, 32, 4>(h, F, pivtol, mask, st, skip, sing);
             }
         };
         if (h->factor_tile != 0) {
@@ -890,8 +899,8 @@ abs_status factor_launch(abs_problem* h, const double* jac, double pivtol, cudaS
             r = tuned_launch(h, TK_FACTOR, sizeof(T), {1, 2, 4, 8}, WPB_F, go, st);
         }
     } else {
-        r = h->S >= CHAIN_WIDE_S ? chain_go<double, 8, 4>(h, F, pivtol, mask, st, skip)
-                                 : chain_go<double, 4, 8>(h, F, pivtol, mask, st, skip);
+        r = h->S >= CHAIN_WIDE_S ? chain_go<double, 8, 4>(h, F, pivtol, mask, st, skip, sing)
+                                 : chain_go<double, 4, 8>(h, F, pivtol, mask, st, skip, sing);
     }
     prof_end(h, st);
     return r;
@@ -1014,8 +1023,12 @@ abs_status tc_solve_t(abs_problem* h, const double* jac, const double* g, double
     return r;
 }
 
-// the tensor-core factor serves plain FP32 systems; mixed ones take the condensed factors
-bool is_tc(const abs_problem* h, const KKTSys& K) { return K.prec == ABS_PREC_FP32 && h->factor_kernel == 1; }
+// where the tensor-core factor is selected, a mixed system (an escalation, a second-order correction)
+// starts with the FP32 condensed factors that the iteration's own factorization left out: a
+// few of a solve's iterations pay for them instead of every one
+abs_status condense_for_mixed(abs_problem* h, const double* jac, cudaStream_t st) {
+    return h->factor_kernel == 1 ? factor_launch<float>(h, jac, 1e-30, st, nullptr, nullptr, false) : ABS_OK;
+}
 
 abs_status tc_schur(abs_problem* h, const KKTSys& K, const double* p, const double* rz, const int* sing, int terms,
                     cudaStream_t st) {
@@ -1062,15 +1075,18 @@ abs_status kkt_factor_core(abs_problem* h, const KKTSys& K, const double* x, cud
     // FP64 escalation where it stalls
     if (K.prec == ABS_PREC_MIXED) {
         if ((r = ensure_factor(h, ABS_PREC_FP64)) != ABS_OK) return r;
+        if ((r = condense_for_mixed(h, K.jac, st)) != ABS_OK) return r;
         r = factor_launch<double>(h, K.jac, 1e-14, st, h->esc);
+    } else if (K.blocks) {
+        if ((r = ensure_tc(h)) != ABS_OK) return r;
+        r = tc_factor(h, K.jac, 1e-30, st);
     } else {
         if ((r = ensure_factor(h, K.prec)) != ABS_OK) return r;
         if (K.prec == ABS_PREC_FP32) r = factor_launch<float>(h, K.jac, 1e-30, st, nullptr, K.skip);
         else r = factor_launch<double>(h, K.jac, 1e-14, st, nullptr, K.skip);
     }
     if (r != ABS_OK) return r;
-    if (is_tc(h, K)) {
-        if ((r = tc_factor(h, K.jac, 1e-30, st)) != ABS_OK) return r;
+    if (K.blocks) {
         r = K.pre_rc ? tc_solve<2>(h, K.jac, x, K.pre_rc, nullptr, V(h, V_P), V(h, V_Q), st)
                      : tc_solve<1>(h, K.jac, x, nullptr, nullptr, V(h, V_Q), nullptr, st);
         if (r != ABS_OK) return r;
@@ -1102,7 +1118,7 @@ abs_status kkt_solve_launches(abs_problem* h, const KKTSys& K, const double* x, 
                               const double* rc0 = nullptr) {
     abs_status r;
     const int nsec = h->P.nsec;
-    const bool two = nsec == 2, tc = is_tc(h, K);
+    const bool two = nsec == 2, tc = K.blocks;
     const double* dlast = dl;
     if (K.ldl) {
         // v = K_s^-1 [rz; rc] into dz, dl with [2] b^T v_l ([3] zero), dd, then x = v - u dd

@@ -811,7 +811,7 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
         __syncthreads();
         for (int q = 0; q < CG; ++q) bad |= (int)sK[q * SPB + i];
     }
-    if (live && g == 0) sing[s] = bad;
+    if (live && g == 0 && sing) sing[s] = bad;
 }
 
 // ---- block solves ----------------------------------------------------------------------------
