@@ -218,7 +218,12 @@ typedef struct abs_inertia {
  *    block tridiagonal with 22 x 22 stage blocks): each stage block is condensed onto 7
  *    unknowns (its equilibria, summations, balances of single species and hydraulic row
  *    eliminated in closed form), the condensed system by a block LU over the stages with
- *    partial pivoting inside each 7 x 7 block; then S_d = K_dd + sum_s q_s^T (W_s + Sigma_s + dw I) q_s,
+ *    partial pivoting inside each 7 x 7 block (that rests on values the evaluation gives: the
+ *    extents' coefficients -nu, the slack's 1, the entries of a stage's streams in its
+ *    neighbours' rows the negatives of those in its own; where the given jac_vals differ by
+ *    more than 2^12 units in the last place, as after a scaling of rows, or a pivot of the
+ *    condensation cancels, all scenarios take a block LU with partial pivoting over their 22 x
+ *    22 stage blocks as given, several times as long); then S_d = K_dd + sum_s q_s^T (W_s + Sigma_s + dw I) q_s,
  *    q_s = J_s^{-1} b_s, and with J_s nonsingular every K_s has inertia (220, 220, 0)
  *    whatever W_s is.  A singular stage block is reported in n_singular and by
  *    ABS_ERR_NUMERIC;
@@ -226,7 +231,9 @@ typedef struct abs_inertia {
  *    blocks (unknowns and rows of a stage together) with Bunch-Kaufman pivoting inside
  *    each, in FP64; its inertia counted from the pivots.  A zero pivot is reported in
  *    n_zero and n_singular and by ABS_ERR_NUMERIC.
- *   x, jac_vals, hess_vals  device, as produced by eval_grad_jac_hess at the iterate.
+ *   x, jac_vals, hess_vals  device, as produced by eval_grad_jac_hess at the iterate (or edited
+ *              since: see above; the column of d in J is -u_max pi d / 2 from x wherever
+ *              it is solved with, whatever jac_vals say).
  *   diag       host struct (delta_w, delta_c >= 0, else ABS_ERR_ARG).
  *   precision  ABS_PREC_FP64, ABS_PREC_FP32, ABS_PREC_FP32_TC or ABS_PREC_FP64_LDL;
  *              delta_c > 0 needs ABS_PREC_FP64 or ABS_PREC_FP64_LDL (else ABS_ERR_ARG).
@@ -603,14 +610,15 @@ abs_status ipm_solve_learned(abs_problem* h, abs_mlp* net, const abs_options* op
  * no handle: the caller passes the problem's parameter table and its own device
  * buffers, and every intermediate (condensed factors, the Schur vectors and block
  * partial sums) lives in one static device array of the
- * library, sized for ABS_NOALLOC_MAX_SCENARIOS scenarios (about 3 MB), which every GPU
+ * library, sized for ABS_NOALLOC_MAX_SCENARIOS scenarios (about 9 MB), which every GPU
  * that loads the library holds until the process exits.  The call makes no cudaMalloc,
  * cudaFree, pinned-host or other allocating call.
  *   p          host, the parameter table.
  *   S, ld      scenarios (1 <= S <= ABS_NOALLOC_MAX_SCENARIOS; larger S is rejected
  *              with ABS_ERR_ARG) and the leading dimension (S rounded up to 32).
  *   x          device primal vector (only d, its last entry, is read).
- *   jac_vals, hess_vals  device, as eval_grad_jac_hess writes them at the iterate.
+ *   jac_vals, hess_vals  device, as eval_grad_jac_hess writes them at the iterate, or edited
+ *              since (as for kkt_factor).
  *   sigma      device primal vector, the barrier diagonal (d last); delta_w >= 0.
  *   rhs_x, rhs_c, sol_x, sol_c  device primal / row vectors, as for kkt_solve.
  *   schur_d    host or NULL: receives the Schur complement on d.

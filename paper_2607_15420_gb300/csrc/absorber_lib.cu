@@ -404,9 +404,9 @@ struct abs_problem {
     double* vec = nullptr;       // pool of primal-size vectors
     // condensed factors per precision [ABS_PREC_FP64], [ABS_PREC_FP32] (kernels_cond.cuh)
     void* cond[2] = {nullptr, nullptr};
-    // tensor-core FP32 factor: stage-block inverses, G blocks, row order
-    float* tcAI = nullptr;
-    float* tcG = nullptr;
+    // stage-block factors: FP32 inverses or FP64 LU, G blocks, row order (kernels_warp.cuh)
+    void* blk[2] = {nullptr, nullptr};
+    void* blkG[2] = {nullptr, nullptr};
     unsigned char* piv = nullptr;
     int* sing = nullptr;
     double* part = nullptr;      // per-thread partials [KMAX][N_STAGES][ld]
@@ -417,7 +417,7 @@ struct abs_problem {
     int* rcnt = nullptr;         // [NP] chunk arrivals of the running reduction (zero between launches)
     double* red = nullptr;       // [KMAX][NP]
     double* hred = nullptr;      // pinned [KMAX + 2][NP] staging for scalar copies
-    double* hmap = nullptr;      // pinned, device-mapped [RED_HOUT][NP]: fetched reductions
+    double* hmap = nullptr;      // pinned, device-mapped [RED_HOUT][NP]: fetched reductions; then kkt_factor's flag
     double* hmap_dev = nullptr;  // (the reduction kernel writes them straight to host memory)
     double* ps = nullptr;        // device per-problem scalars [PS_NFIELDS][NP]
     double* hps = nullptr;       // host values of ps
@@ -434,7 +434,7 @@ struct abs_problem {
         const double* sig = nullptr;
         double d = 0.0, dw = 0.0, dc = 0.0, Kdd = 0.0, A0 = 0.0, Q2 = 0.0, Sd = 0.0;
         bool ldl = false;            // factored by the block LDL^T (kernels_ldl.cuh)
-        bool blocks = false;         // by stage-block inverses (kernels_tc.cuh)
+        bool blocks = false;         // by the uncondensed stage blocks (kernels_warp.cuh)
     } fac;
     double* ldl_inv = nullptr;       // [S][N_STAGES][990] inverses of the block LDL^T pivot blocks, packed
     Prof prof;
@@ -642,7 +642,7 @@ abs_status ensure_buffers(abs_problem* h) {
     CK(cudaMemset(h->rcnt, 0, sizeof(int) * (size_t)h->NP));
     CK(cudaMalloc(&h->red, sizeof(double) * (size_t)KMAX * h->NP));
     CK(cudaMallocHost(&h->hred, sizeof(double) * (size_t)(KMAX + 2) * h->NP));
-    CK(cudaHostAlloc(&h->hmap, sizeof(double) * (size_t)RED_HOUT * h->NP, cudaHostAllocMapped));
+    CK(cudaHostAlloc(&h->hmap, sizeof(double) * ((size_t)RED_HOUT * h->NP + 1), cudaHostAllocMapped));
     CK(cudaHostGetDevicePointer(&h->hmap_dev, h->hmap, 0));
     CK(cudaMalloc(&h->ps, sizeof(double) * (size_t)PS_NFIELDS * h->NP));
     h->hps = new double[(size_t)PS_NFIELDS * h->NP]();
@@ -673,13 +673,12 @@ abs_status ensure_factor(abs_problem* h, int prec) {
     return ABS_OK;
 }
 
-// the tensor-core FP32 factor's
-abs_status ensure_tc(abs_problem* h) {
-    if (!h->tcAI) {
-        CK(cudaMalloc(&h->tcG, sizeof(float) * (size_t)N_STAGES * NV * NABV * h->ld));
-        CK(cudaMalloc(&h->piv, (size_t)N_STAGES * PIV_BYTES * h->ld));
-        CK(cudaMalloc(&h->tcAI, sizeof(float) * (size_t)N_STAGES * NV * NV * h->ld));
-    }
+// stage-block factor storage of a precision
+abs_status ensure_blocks(abs_problem* h, int prec) {
+    const size_t es = prec == ABS_PREC_FP32 ? sizeof(float) : sizeof(double);
+    if (!h->piv) CK(cudaMalloc(&h->piv, (size_t)N_STAGES * PIV_BYTES * h->ld));
+    if (!h->blkG[prec]) CK(cudaMalloc(&h->blkG[prec], es * (size_t)N_STAGES * NV * NABV * h->ld));
+    if (!h->blk[prec]) CK(cudaMalloc(&h->blk[prec], es * (size_t)N_STAGES * NV * NV * h->ld));
     return ABS_OK;
 }
 
@@ -768,8 +767,11 @@ struct KKTSys {
     // block LDL^T of every scenario block (FP64, dw = PS_DW, dc = PS_DC) instead of the
     // block LU of J_s
     bool ldl = false;
-    // FP32: the uncondensed stage-block inverses of the tensor-core factor
+    // the uncondensed stage blocks: FP32 inverses by the tensor-core factor, FP64 LU
     bool blocks = false;
+    // kkt_factor's Jacobian comes from outside: the condensation checks it and sets this flag
+    // (mapped host memory) where it does not hold
+    int* odd = nullptr;
     // set before kkt_factor_core: the factorization also solves p = J^-1 rc and (one design
     // entry) forms the first solve's right-hand-side sums with this rz (q^T (rz - H p), q^T p;
     // they do not depend on dw), so that the first KKT solve with them starts from both
@@ -871,16 +873,17 @@ abs_status chain_go(abs_problem* h, T* F, double pivtol, const int* mask, cudaSt
 // condensed factors of J_s (kernels_cond.cuh) in T, of the scenarios with mask[s] != 0 only when
 // mask is given.  skip (device flag, optional): when set at run time the launches leave the stored
 // factors as they are (they are those of this Jacobian).  flags = false: the scenarios' singular
-// flags stay as they are.  The FP32 chain has four threads per scenario: W warps per block.
+// flags stay as they are.  odd: see KKTSys.  The FP32 chain has four threads per scenario: W warps per block.
 template <class T>
 abs_status factor_launch(abs_problem* h, const double* jac, double pivtol, cudaStream_t st,
-                         const int* mask = nullptr, const int* skip = nullptr, bool flags = true) {
+                         const int* mask = nullptr, const int* skip = nullptr, bool flags = true, int* odd = nullptr) {
     int* sing = flags ? h->sing : nullptr;
     constexpr bool f32 = std::is_same<T, float>::value;
     T* F = (T*)h->cond[f32 ? ABS_PREC_FP32 : ABS_PREC_FP64];
     prof_begin(h, K_FACTOR, st);
-    condense_kernel<T><<<dim3((unsigned)((h->S + 63) / 64), N_STAGES), 64, 0, st>>>((int)h->S, h->ld, view(h), jac, F,
-                                                                                    mask, skip);
+    const dim3 g((unsigned)((h->S + 63) / 64), N_STAGES);
+    if (odd) condense_kernel<T, true><<<dim3(g.x, 2 * N_STAGES), 64, 0, st>>>((int)h->S, h->ld, view(h), jac, F, mask, skip, odd);
+    else condense_kernel<T, false><<<g, 64, 0, st>>>((int)h->S, h->ld, view(h), jac, F, mask, skip, nullptr);
     abs_status r = launch_check(h, KD_FACTOR);
     if (r != ABS_OK) return r;
     if constexpr (f32) {
@@ -951,23 +954,24 @@ abs_status solve_direction(abs_problem* h, const KKTSys& K, const double* x, con
     return launch_check(h, KD_SOLVE_T);
 }
 
-// ---- the tensor-core FP32 factor (options.factor_kernel = 1): stage-block inverses and their
-// block solves, W warps (scenarios) per block
+// ---- the uncondensed stage blocks: FP32 inverses by the tensor-core factor
+// (options.factor_kernel = 1), FP64 LU; W warps (scenarios) per block
 abs_status tc_factor(abs_problem* h, const double* jac, double pivtol, cudaStream_t st) {
     prof_begin(h, K_FACTOR, st);
-#define TC_GO(W)                                                                                                     \
-    factor_gj_tc_kernel<W><<<gridw(h, W), 32 * W, 0, st>>>((int)h->S, h->ld, view(h), jac, h->tcAI, h->piv, h->tcG, \
-                                                           h->sing, pivtol)
+#define BLK_GO(W)                                                                                                     \
+    factor_gj_tc_kernel<W><<<gridw(h, W), 32 * W, 0, st>>>((int)h->S, h->ld, view(h), jac,                          \
+                                                           (float*)h->blk[ABS_PREC_FP32], h->piv,                   \
+                                                           (float*)h->blkG[ABS_PREC_FP32], h->sing, pivtol)
     auto go = [&](int w) {
         switch (w) {
-            case 1: TC_GO(1); break;
-            case 2: TC_GO(2); break;
-            case 8: TC_GO(8); break;
-            default: TC_GO(4); break;
+            case 1: BLK_GO(1); break;
+            case 2: BLK_GO(2); break;
+            case 8: BLK_GO(8); break;
+            default: BLK_GO(4); break;
         }
         return launch_check(h, KD_FACTOR);
     };
-#undef TC_GO
+#undef BLK_GO
     abs_status r;
     if (h->factor_tile != 0) {
         h->tile[TK_FACTOR] = h->factor_tile;
@@ -979,48 +983,83 @@ abs_status tc_factor(abs_problem* h, const double* jac, double pivtol, cudaStrea
     return r;
 }
 
+abs_status lu_factor(abs_problem* h, const double* jac, double pivtol, cudaStream_t st) {
+    prof_begin(h, K_FACTOR, st);
+    factor_lu_kernel<<<gridw(h, WPB_F), 32 * WPB_F, 0, st>>>((int)h->S, h->ld, view(h), jac,
+                                                             (double*)h->blk[ABS_PREC_FP64], h->piv,
+                                                             (double*)h->blkG[ABS_PREC_FP64], h->sing, pivtol);
+    prof_end(h, st);
+    return launch_check(h, KD_FACTOR);
+}
+
 // J x = r with them (NR_ right-hand sides; a null one means b = dc/dtheta of design entry bsec)
-template <int NR_>
-abs_status tc_solve(abs_problem* h, const double* jac, const double* x, const double* r0, const double* r1, double* o0,
-                    double* o1, cudaStream_t st, int bsec = 0) {
+template <class T, int NR_>
+abs_status blk_solve(abs_problem* h, const double* jac, const double* x, const double* r0, const double* r1, double* o0,
+                     double* o1, cudaStream_t st, int bsec) {
+    constexpr int pi = std::is_same<T, float>::value ? ABS_PREC_FP32 : ABS_PREC_FP64;
     prof_begin(h, K_SOLVE, st);
-#define TC_GO(W)                                                                                                  \
-    solve_warp_kernel<NR_, W><<<gridw(h, W), 32 * W, 0, st>>>(h->P, (int)h->S, h->ld, view(h), jac, h->tcAI, h->piv, \
-                                                              h->tcG, x, r0, r1, o0, o1, bsec)
+#define BLK_GO(W)                                                                                                  \
+    solve_warp_kernel<T, NR_, W><<<gridw(h, W), 32 * W, 0, st>>>(h->P, (int)h->S, h->ld, view(h), jac,            \
+                                                                 (const T*)h->blk[pi], h->piv,                   \
+                                                                 (const T*)h->blkG[pi], x, r0, r1, o0, o1, bsec)
     auto go = [&](int w) {
-        switch (w) {
-            case 1: TC_GO(1); break;
-            case 2: TC_GO(2); break;
-            case 8: TC_GO(8); break;
-            default: TC_GO(4); break;
+        if constexpr (pi == ABS_PREC_FP32) {
+            switch (w) {
+                case 1: BLK_GO(1); break;
+                case 2: BLK_GO(2); break;
+                case 8: BLK_GO(8); break;
+                default: BLK_GO(4); break;
+            }
+        } else {
+            BLK_GO(WPB_S);
         }
         return launch_check(h, KD_SOLVE);
     };
-#undef TC_GO
-    abs_status r = tuned_launch(h, NR_ == 1 ? TK_SOLVE1 : TK_SOLVE2, 4, {1, 2, 4, 8}, WPB_S, go, st);
+#undef BLK_GO
+    abs_status r;
+    if constexpr (pi == ABS_PREC_FP32)
+        r = tuned_launch(h, NR_ == 1 ? TK_SOLVE1 : TK_SOLVE2, sizeof(T), {1, 2, 4, 8}, WPB_S, go, st);
+    else r = go(WPB_S);
     prof_end(h, st);
     return r;
 }
+template <int NR_>
+abs_status blocks_solve(abs_problem* h, int prec, const double* jac, const double* x, const double* r0, const double* r1,
+                    double* o0, double* o1, cudaStream_t st, int bsec = 0) {
+    return prec == ABS_PREC_FP32 ? blk_solve<float, NR_>(h, jac, x, r0, r1, o0, o1, st, bsec)
+                                 : blk_solve<double, NR_>(h, jac, x, r0, r1, o0, o1, st, bsec);
+}
 
 // J^T v = g with them
-abs_status tc_solve_t(abs_problem* h, const double* jac, const double* g, double* out, cudaStream_t st) {
+template <class T>
+abs_status blk_solve_t(abs_problem* h, const double* jac, const double* g, double* out, cudaStream_t st) {
+    constexpr int pi = std::is_same<T, float>::value ? ABS_PREC_FP32 : ABS_PREC_FP64;
     prof_begin(h, K_SOLVE_T, st);
-#define TC_GO(W)                                                                                             \
-    solve_t_warp_kernel<W><<<gridw(h, W), 32 * W, 0, st>>>((int)h->S, h->ld, view(h), jac, h->tcAI, h->piv, \
-                                                           h->tcG, g, out)
+#define BLK_GO(W)                                                                                                  \
+    solve_t_warp_kernel<T, W><<<gridw(h, W), 32 * W, 0, st>>>((int)h->S, h->ld, view(h), jac, (const T*)h->blk[pi], \
+                                                              h->piv, (const T*)h->blkG[pi], g, out)
     auto go = [&](int w) {
-        switch (w) {
-            case 1: TC_GO(1); break;
-            case 2: TC_GO(2); break;
-            case 8: TC_GO(8); break;
-            default: TC_GO(4); break;
+        if constexpr (pi == ABS_PREC_FP32) {
+            switch (w) {
+                case 1: BLK_GO(1); break;
+                case 2: BLK_GO(2); break;
+                case 8: BLK_GO(8); break;
+                default: BLK_GO(4); break;
+            }
+        } else {
+            BLK_GO(WPB_S);
         }
         return launch_check(h, KD_SOLVE_T);
     };
-#undef TC_GO
-    abs_status r = tuned_launch(h, TK_SOLVE_T, 4, {1, 2, 4, 8}, WPB_S, go, st);
+#undef BLK_GO
+    abs_status r;
+    if constexpr (pi == ABS_PREC_FP32) r = tuned_launch(h, TK_SOLVE_T, sizeof(T), {1, 2, 4, 8}, WPB_S, go, st);
+    else r = go(WPB_S);
     prof_end(h, st);
     return r;
+}
+abs_status blocks_solve_t(abs_problem* h, int prec, const double* jac, const double* g, double* out, cudaStream_t st) {
+    return prec == ABS_PREC_FP32 ? blk_solve_t<float>(h, jac, g, out, st) : blk_solve_t<double>(h, jac, g, out, st);
 }
 
 // where the tensor-core factor is selected, a mixed system (an escalation, a second-order correction)
@@ -1030,7 +1069,7 @@ abs_status condense_for_mixed(abs_problem* h, const double* jac, cudaStream_t st
     return h->factor_kernel == 1 ? factor_launch<float>(h, jac, 1e-30, st, nullptr, nullptr, false) : ABS_OK;
 }
 
-abs_status tc_schur(abs_problem* h, const KKTSys& K, const double* p, const double* rz, const int* sing, int terms,
+abs_status blocks_schur(abs_problem* h, const KKTSys& K, const double* p, const double* rz, const int* sing, int terms,
                     cudaStream_t st) {
     double* hq = (terms & SCHUR_DD) ? V(h, V_HQ) : nullptr;
     double* t = (terms & SCHUR_RHS) ? V(h, V_T) : nullptr;
@@ -1078,22 +1117,22 @@ abs_status kkt_factor_core(abs_problem* h, const KKTSys& K, const double* x, cud
         if ((r = condense_for_mixed(h, K.jac, st)) != ABS_OK) return r;
         r = factor_launch<double>(h, K.jac, 1e-14, st, h->esc);
     } else if (K.blocks) {
-        if ((r = ensure_tc(h)) != ABS_OK) return r;
-        r = tc_factor(h, K.jac, 1e-30, st);
+        if ((r = ensure_blocks(h, K.prec)) != ABS_OK) return r;
+        r = K.prec == ABS_PREC_FP32 ? tc_factor(h, K.jac, 1e-30, st) : lu_factor(h, K.jac, 1e-14, st);
     } else {
         if ((r = ensure_factor(h, K.prec)) != ABS_OK) return r;
-        if (K.prec == ABS_PREC_FP32) r = factor_launch<float>(h, K.jac, 1e-30, st, nullptr, K.skip);
-        else r = factor_launch<double>(h, K.jac, 1e-14, st, nullptr, K.skip);
+        if (K.prec == ABS_PREC_FP32) r = factor_launch<float>(h, K.jac, 1e-30, st, nullptr, K.skip, true, K.odd);
+        else r = factor_launch<double>(h, K.jac, 1e-14, st, nullptr, K.skip, true, K.odd);
     }
     if (r != ABS_OK) return r;
     if (K.blocks) {
-        r = K.pre_rc ? tc_solve<2>(h, K.jac, x, K.pre_rc, nullptr, V(h, V_P), V(h, V_Q), st)
-                     : tc_solve<1>(h, K.jac, x, nullptr, nullptr, V(h, V_Q), nullptr, st);
+        r = K.pre_rc ? blocks_solve<2>(h, K.prec, K.jac, x, K.pre_rc, nullptr, V(h, V_P), V(h, V_Q), st)
+                     : blocks_solve<1>(h, K.prec, K.jac, x, nullptr, nullptr, V(h, V_Q), nullptr, st);
         if (r != ABS_OK) return r;
         // a second design entry: q1 = J^-1 b1, b1 the border column of the second section
-        if (two && (r = tc_solve<1>(h, K.jac, x, nullptr, nullptr, V(h, V_Q1), nullptr, st, 1)) != ABS_OK) return r;
+        if (two && (r = blocks_solve<1>(h, K.prec, K.jac, x, nullptr, nullptr, V(h, V_Q1), nullptr, st, 1)) != ABS_OK) return r;
         const bool rhs = K.pre_rc && K.pre_rz && !two;
-        r = tc_schur(h, K, rhs ? V(h, V_P) : nullptr, rhs ? K.pre_rz : nullptr, h->sing,
+        r = blocks_schur(h, K, rhs ? V(h, V_P) : nullptr, rhs ? K.pre_rz : nullptr, h->sing,
                      SCHUR_DD | (rhs ? SCHUR_RHS : 0), st);
     } else if (K.pre_rc && K.pre_rz && !two) {
         r = solve_p(h, K.prec, &K, x, K.pre_rc, K.pre_rz, V(h, V_P), 2, st);
@@ -1135,8 +1174,8 @@ abs_status kkt_solve_launches(abs_problem* h, const KKTSys& K, const double* x, 
         const bool sums_ready = have_p && !two && K.pre_rc == rc && K.pre_rz == rz;
         if (!sums_ready) {
             if (tc) {
-                if (!have_p && (r = tc_solve<1>(h, K.jac, x, rc, nullptr, V(h, V_P), nullptr, st)) != ABS_OK) return r;
-                r = tc_schur(h, K, V(h, V_P), rz, nullptr, SCHUR_RHS, st);
+                if (!have_p && (r = blocks_solve<1>(h, K.prec, K.jac, x, rc, nullptr, V(h, V_P), nullptr, st)) != ABS_OK) return r;
+                r = blocks_schur(h, K, V(h, V_P), rz, nullptr, SCHUR_RHS, st);
             } else {
                 r = solve_p(h, K.prec, &K, x, rc, rz, V(h, V_P), 1, st);
             }
@@ -1153,7 +1192,7 @@ abs_status kkt_solve_launches(abs_problem* h, const KKTSys& K, const double* x, 
                                                       V(h, V_HQ), dz, V(h, V_G), two ? V(h, V_Q1) : nullptr,
                                                       two ? V(h, V_HQ1) : nullptr);
             if ((r = launch_check(h, KD_DZ)) != ABS_OK) return r;
-            if ((r = tc_solve_t(h, K.jac, V(h, V_G), dl, st)) != ABS_OK) return r;
+            if ((r = blocks_solve_t(h, K.prec, K.jac, V(h, V_G), dl, st)) != ABS_OK) return r;
         }
     }
     if (az && (K.ldl || tc)) {   // (ctl_refine adds the design entries' steps)
@@ -1394,8 +1433,10 @@ void absorber_destroy(abs_problem* h) {
     cudaFree(h->vec);
     cudaFree(h->ldl_inv);
     for (int k = 0; k < 2; ++k) cudaFree(h->cond[k]);
-    cudaFree(h->tcAI);
-    cudaFree(h->tcG);
+    for (int k = 0; k < 2; ++k) {
+        cudaFree(h->blk[k]);
+        cudaFree(h->blkG[k]);
+    }
     cudaFree(h->piv);
     cudaFree(h->sing);
     cudaFree(h->part);
@@ -1578,21 +1619,25 @@ extern "C" abs_status abs_measure_fma_peak(int kind, double* gflops) {
 // For callers that cannot allocate device memory after start-up -- code running under
 // a fixed memory budget, inside another runtime's allocator, or between graph
 // captures -- this entry runs the FP64 condensed factorization, the Schur step on d and the
-// block solves with every intermediate in one file-scope device array.  Nothing in the
-// array has to start at zero: every word a call reads was written earlier in that call
-// (the factor kernel writes every scenario's singular flag; every live (scenario,
+// block solves with every intermediate in one file-scope device array (the stage-block LU's,
+// for a Jacobian that the condensed factors do not cover, in the same place).  Nothing in the
+// array has to start at zero: every word that a result depends on was written earlier in that
+// call (the factor kernel writes every scenario's singular flag; every live (scenario,
 // stage) thread writes its partial sums; the per-problem scalars are copied in first).
 namespace {
 
 constexpr int64_t NA_MAX_S = ABS_NOALLOC_MAX_SCENARIOS;    // scenarios per call, at most
 constexpr int64_t NA_LD = NA_MAX_S;                         // a multiple of 32
-constexpr size_t NA_FAC = (size_t)N_STAGES * CF_COUNT * NA_LD;
+constexpr size_t NA_LU = (size_t)N_STAGES * NV * NV * NA_LD, NA_G = (size_t)N_STAGES * NV * NABV * NA_LD;
+constexpr size_t NA_FAC = NA_LU + NA_G;                     // stage-block LU and G, or the condensed factors
+static_assert(NA_FAC >= (size_t)N_STAGES * CF_COUNT * NA_LD, "both fit");
+constexpr size_t NA_PIV = ((size_t)N_STAGES * PIV_BYTES * NA_LD + 7) / 8;   // bytes as doubles
 constexpr size_t NA_VEC = (size_t)NSC * NA_LD + NA_LD;
 constexpr int NA_K = 6;                                     // Schur partial planes
 constexpr size_t NA_PART = (size_t)NA_K * N_STAGES * NA_LD;
-constexpr size_t NA_SING = (NA_LD + 1) / 2;                         // ints as doubles
+constexpr size_t NA_SING = (NA_LD + 1) / 2 + 1;                     // ints as doubles: flags, then the check's
 constexpr size_t NA_PS = PS_NFIELDS;                                // one problem's scalars
-constexpr size_t NA_TOTAL = NA_FAC + NA_VEC + NA_PART + NA_SING + NA_PS;
+constexpr size_t NA_TOTAL = NA_FAC + 5 * NA_VEC + NA_PART + NA_PIV + NA_SING + NA_PS;
 
 // the scratch: every device that loads the library holds it until the process exits
 static __device__ __align__(256) double g_noalloc_scratch[NA_TOTAL];
@@ -1632,8 +1677,11 @@ extern "C" abs_status kkt_newton_noalloc(const abs_params* p, int64_t S, int64_t
     }
     double* F = g_na_base[dev];
     double* pv = F + NA_FAC;
-    double* part = pv + NA_VEC;
-    int* sing = (int*)(part + NA_PART);
+    double *qv = pv + NA_VEC, *gv = qv + NA_VEC, *tv = gv + NA_VEC, *hq = tv + NA_VEC;   // stage-block LU only
+    double* part = hq + NA_VEC;
+    unsigned char* piv = (unsigned char*)(part + NA_PART);
+    int* sing = (int*)((double*)piv + NA_PIV);
+    int* odd = sing + 2 * (NA_SING - 1);
     double* psd = (double*)sing + NA_SING;
     // the problem's constants (derived fields as absorber_create computes them)
     Params P;
@@ -1653,8 +1701,9 @@ extern "C" abs_status kkt_newton_noalloc(const abs_params* p, int64_t S, int64_t
     const BView bv{nullptr, psd, 1};
     const dim3 gs((unsigned)((S + CS_N - 1) / CS_N));
     const CondFac fac{nullptr, F, nullptr};
-    condense_kernel<double><<<dim3((unsigned)((S + 63) / 64), N_STAGES), 64, 0, st>>>((int)S, ld, bv, jac_vals, F,
-                                                                                      nullptr, nullptr);
+    CK(cudaMemsetAsync(odd, 0, sizeof(int), st));
+    condense_kernel<double, true><<<dim3((unsigned)((S + 63) / 64), 2 * N_STAGES), 64, 0, st>>>((int)S, ld, bv, jac_vals, F,
+                                                                                            nullptr, nullptr, odd);
     NA_LAUNCHED();
     chain_kernel<double, 4, 8><<<(unsigned)((S + 3) / 4), 32, chain_smem(sizeof(double), 4, 8), st>>>(
         (int)S, ld, bv, F, sing, 1e-14, nullptr, nullptr);
@@ -1668,7 +1717,24 @@ extern "C" abs_status kkt_newton_noalloc(const abs_params* p, int64_t S, int64_t
     CK(cudaMemcpyAsync(&hx[0], sigma + od, sizeof(double), cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(&hx[1], rhs_x + od, sizeof(double), cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(g_na_host_part, part, sizeof(double) * NA_K * (size_t)plane, cudaMemcpyDeviceToHost, st));
+    int blocks = 0;   // the Jacobian needs the stage-block LU
+    CK(cudaMemcpyAsync(&blocks, odd, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    const dim3 gf((unsigned)((S + WPB_F - 1) / WPB_F)), gb((unsigned)((S + WPB_S - 1) / WPB_S));
+    if (blocks) {
+        double* G = F + NA_LU;
+        factor_lu_kernel<<<gf, 32 * WPB_F, 0, st>>>((int)S, ld, bv, jac_vals, F, piv, G, sing, 1e-14);
+        NA_LAUNCHED();
+        // p = J^-1 r_c, q = J^-1 b and the Schur sums
+        solve_warp_kernel<double, 2><<<gb, 32 * WPB_S, 0, st>>>(P, (int)S, ld, bv, jac_vals, F, piv, G, x, rhs_c,
+                                                                nullptr, pv, qv);
+        NA_LAUNCHED();
+        schur_kernel<false><<<dim3((unsigned)((S + QS_SCEN - 1) / QS_SCEN), N_STAGES), kThr, 0, st>>>(
+            (int)S, ld, bv, hess_vals, sigma, true, pv, qv, rhs_x, sing, part, SCHUR_DD | SCHUR_RHS, hq, tv);
+        NA_LAUNCHED();
+        CK(cudaMemcpyAsync(g_na_host_part, part, sizeof(double) * NA_K * (size_t)plane, cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+    }
     double red[NA_K];
     for (int k = 0; k < NA_K; ++k) {
         double a = 0.0;
@@ -1685,8 +1751,15 @@ extern "C" abs_status kkt_newton_noalloc(const abs_params* p, int64_t S, int64_t
     const double beta = red[2] - delta_w * red[3];
     const double dd = (hx[1] - beta) / Sd;
     CK(cudaMemcpyAsync(sol_x + od, &dd, sizeof(double), cudaMemcpyHostToDevice, st));
-    cond_direction_kernel<CP_FP64><<<gs, CS_T, cond_smem(sizeof(double)), st>>>(
-        P, (int)S, ld, bv, fac, hess_vals, sigma, true, x, pv, rhs_x, sol_x, sol_c, nullptr, nullptr, nullptr);
+    if (blocks) {
+        dz_fast_kernel<<<dim3((unsigned)((S + kThr - 1) / kThr), NSC), kThr, 0, st>>>((int)S, ld, bv, pv, qv, tv, hq,
+                                                                                    sol_x, gv);
+        NA_LAUNCHED();
+        solve_t_warp_kernel<double><<<gb, 32 * WPB_S, 0, st>>>((int)S, ld, bv, jac_vals, F, piv, F + NA_LU, gv, sol_c);
+    } else {
+        cond_direction_kernel<CP_FP64><<<gs, CS_T, cond_smem(sizeof(double)), st>>>(
+            P, (int)S, ld, bv, fac, hess_vals, sigma, true, x, pv, rhs_x, sol_x, sol_c, nullptr, nullptr, nullptr);
+    }
     NA_LAUNCHED();
 #undef NA_LAUNCHED
     // dd lives on this stack frame until the copy above has completed

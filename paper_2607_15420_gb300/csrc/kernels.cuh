@@ -113,6 +113,14 @@ __device__ __forceinline__ unsigned long long key_max(unsigned long long a, unsi
     return a > b ? a : b;
 }
 __device__ __forceinline__ double key_double(unsigned long long k) { return __longlong_as_double((long long)k); }
+// maximum of magnitude keys over a warp: the high words first, then the low words among the lanes
+// that hold the highest
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long key) {
+    const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    return ((unsigned long long)mh << 32) | ml;
+}
 
 template <int K>
 __device__ inline void store_partials(const double (&v)[K], double* part, int64_t ld, int s, int n) {

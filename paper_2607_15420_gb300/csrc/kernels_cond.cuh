@@ -35,7 +35,9 @@
 // small sizes and FP32.
 //
 // The Jacobian values are those of the evaluation: the extents' coefficients -nu, the
-// slack's 1, and a stage's stream entries in its neighbours' rows the negatives of its own.
+// slack's 1, and a stage's stream entries in its neighbours' rows the negatives of its own.  A
+// Jacobian from outside the library is checked for that (condense_conforms); where it differs
+// the 22 x 22 stage blocks are factored as they are (kernels_warp.cuh).
 #pragma once
 
 #include "kernels.cuh"
@@ -115,10 +117,18 @@ __host__ __device__ inline float cond_recip(float a) {
 __host__ __device__ inline double cond_fma(double a, double b, double c) { return fma(a, b, c); }
 __host__ __device__ inline float cond_fma(float a, float b, float c) { return fmaf(a, b, c); }
 
+// |a| <= lim, false for NaN
+__device__ __forceinline__ bool within(double a, double lim) {
+    return mag_key(a) <= (unsigned long long)__double_as_longlong(lim);
+}
+__device__ __forceinline__ bool within(float a, float lim) { return fabsf(a) <= lim; }
+
 // Condense one stage: A(r, lv) its own Jacobian entries, Lt the energy row's liquid share of
-// dT, Vt its vapour share (Lt + Vt = A(R_E, LT)); into f, all but At^-1, D, T.
+// dT, Vt its vapour share (Lt + Vt = A(R_E, LT)); into f, all but At^-1, D, T.  True where the
+// fixed pivots are safe: x_H2O's, a sum of terms of one sign at interior points, is no less than
+// 1 / 256 of any term, the others are finite.
 template <class T, class Own>
-__host__ __device__ inline void condense_stage(const Own& A, T Lt, T Vt, const CondRef<T>& f) {
+__device__ inline bool condense_stage(const Own& A, T Lt, T Vt, const CondRef<T>& f) {
     // ---- equilibria: x2 (R1), x4 (R4), x5 (R3), x6 (R2), x7 (R5) -----------------------------
     constexpr int R1 = R_RX, R2 = R_RX + 1, R3 = R_RX + 2, R4 = R_RX + 3, R5 = R_RX + 4;
     const T i12 = cond_recip(A(R1, 2)), i44 = cond_recip(A(R4, 4)), i35 = cond_recip(A(R3, 5)),
@@ -312,6 +322,10 @@ __host__ __device__ inline void condense_stage(const Own& A, T Lt, T Vt, const C
     f(CF_VV) = vv;
     f(CF_HV) = A(R_H, LV);
     f(CF_HT) = A(R_H, LT);
+    constexpr T TOP = sizeof(T) == 8 ? T(1.7976931348623157e308) : T(3.4028234663852886e38);   // finite
+    return (int)within(i12, TOP) & within(iy1, TOP) & within(iy0, TOP) & within(iy2, TOP) &
+           within((T)A(R_SX, 8) * i8, T(256)) & within(s4 * X48, T(256)) & within(s5 * X58, T(256)) &
+           within(s6 * X68, T(256)) & within(s7 * X78, T(256));
 }
 
 // The right-hand side of the core: r -> rc; the eliminated fractions' own parts -> rho
@@ -543,17 +557,75 @@ struct OwnEntries {
     __device__ __forceinline__ T operator()(int r, int lv) const { return (T)j[(int64_t)c_slotJ[t][r][lv] * ld]; }
 };
 
+// a = b to 2^12 units in the last place (4.5e-13 to 9e-13 relative: values computed in another order
+// of the same operations agree to a few), or both zero; on the integer pipe
+__device__ __forceinline__ bool alike(double a, double b) {
+    const unsigned long long x = (unsigned long long)__double_as_longlong(a),
+                             y = (unsigned long long)__double_as_longlong(b);
+    return x - y + 4096ull <= 8192ull || ((x | y) << 1) == 0ull;
+}
+__device__ __forceinline__ bool opposite(double a, double b) { return alike(a, -b); }
+// Whether the values that the condensation of a stage assumes instead of reading are there.  Every load
+// is issued at once: no condition skips one.
+__device__ __forceinline__ bool condense_conforms(const double* __restrict__ jac, int64_t ld, int s, int n) {
+    const int t = stage_type(n);
+    const OwnEntries<double> A{jac + (int64_t)c_segJ[n] * ld + s, ld, t};
+    int ok = alike(A(R_H, LS), 1.0);
+    static_for<0, 9>([&](auto C) {
+        constexpr int c = decltype(C)::value;
+        static_for<0, 5>([&](auto K) {
+            constexpr int k = decltype(K)::value;
+            if constexpr (nu(c, k) != 0)
+                ok &= alike(A(c, LE + k), -nu(c, k));
+        });
+    });
+    const int below = n > 0 ? n - 1 : 0, above = n + 1 < N_STAGES ? n + 1 : N_STAGES - 1;
+    const OwnEntries<double> B{jac + (int64_t)c_segJ[below] * ld + s, ld, stage_type(below)},
+        U{jac + (int64_t)c_segJ[above] * ld + s, ld, stage_type(above)};
+    if (n > 0) {   // its liquid in the rows of the stage below
+        static_for<0, 9>([&](auto C) {
+            constexpr int c = decltype(C)::value;
+            ok &= opposite(A(c, c), B(c, AX + c));
+            ok &= opposite(A(c, LL), B(c, AL));
+            ok &= opposite(A(R_E, c), B(R_E, AX + c));
+        });
+        ok &= opposite(A(R_E, LL), B(R_E, AL));
+    }
+    if (n + 1 < N_STAGES) {   // its vapour in the rows of the stage above
+        static_for<0, 4>([&](auto J) {
+            constexpr int j = decltype(J)::value;
+            ok &= opposite(A(7 + j, LY + j), U(7 + j, BY + j));
+            ok &= opposite(A(7 + j, LV), U(7 + j, BV));
+            ok &= opposite(A(R_E, LY + j), U(R_E, BY + j));
+        });
+        ok &= opposite(A(R_E, LV), U(R_E, BV));
+        if (n > 0) {   // the shares of its energy row's dT in the neighbours' rows, and their sum
+            const double a = A(R_E, LT), l = B(R_E, AT), v = U(R_E, BT);
+            ok &= fabs(a + v + l) <= 0x1p-40 * (fabs(v) + fabs(l));
+        }
+    }
+    return ok;
+}
+
 // Every (scenario, stage) condensed, one thread each: about 330 multiply-adds, all stages at
 // once.  mask (optional): only scenarios with mask[s] != 0.  skip (optional, device): the
-// stored values are those of this Jacobian.  Grid (ceil(S / 64), N_STAGES), 64 threads.
-template <class T>
+// stored values are those of this Jacobian.  CHECK (a Jacobian from outside the library): *odd is set
+// where the condensation does not hold, by blocks of their own next to those that condense the same
+// stage (its entries come from L2; on the same threads their loads cost up to twice as much): kkt_factor
+// of 20000 scenarios FP64 700 -> 727 us, FP32 157 -> 173, of up to 500 the same.  Grid (ceil(S / 64),
+// N_STAGES, with CHECK twice that), 64 threads.
+template <class T, bool CHECK>
 __global__ void __launch_bounds__(64) condense_kernel(int S, int64_t ld, const BView b, const double* __restrict__ jac,
                                                       T* __restrict__ F, const int* __restrict__ mask,
-                                                      const int* __restrict__ skip) {
+                                                      const int* __restrict__ skip, int* __restrict__ odd) {
     if (skip && *skip) return;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n = blockIdx.y;
+    const int n = CHECK ? blockIdx.y >> 1 : blockIdx.y;
     if (live_prob(b, s, S, PS_ACT) < 0 || (mask && mask[s] == 0)) return;
+    if (CHECK && (blockIdx.y & 1)) {
+        if (!condense_conforms(jac, ld, s, n)) *odd = 1;
+        return;
+    }
     const int t = stage_type(n);
     const OwnEntries<T> A{jac + (int64_t)c_segJ[n] * ld + s, ld, t};
     // the energy row's dT: the liquid's share from the stage below's row, the vapour's from the
@@ -567,7 +639,8 @@ __global__ void __launch_bounds__(64) condense_kernel(int S, int64_t ld, const B
         Vt = -(T)jac[(int64_t)(c_segJ[1] + c_slotJ[1][R_E][BT]) * ld + s];
         Lt = tot - Vt;
     }
-    condense_stage<T>(A, Lt, Vt, cond_ref(F, ld, n, s));
+    const bool safe = condense_stage<T>(A, Lt, Vt, cond_ref(F, ld, n, s));
+    if (CHECK && !safe) *odd = 1;
 }
 
 // the magnitude order of a pivot candidate: for FP64 by the high word (a relative 2^-20)

@@ -128,15 +128,6 @@ __device__ inline void ldl_assemble_diag(double* W, int64_t ld, int s, int n, co
     }
 }
 
-// maximum of magnitude keys over a warp: the high words first, then the low words among the lanes
-// that hold the highest
-__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long key) {
-    const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
-    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
-    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-    return ((unsigned long long)mh << 32) | ml;
-}
-
 // the largest |entry| of column k over the indices not in done and other than k, and its lowest
 // index (every lane of the warp gets both; each warp of the block for itself)
 __device__ __forceinline__ double ldl_colmax(const double* W, int k, unsigned long long done, int& row) {
