@@ -309,10 +309,7 @@ cudaError_t upload_tables(int dev) {
     }
     {
         static LnEntry ln[LN_TAB];
-        for (int j = 0; j < LN_TAB; ++j) {
-            ln[j].inv = (double)(1.0L / (1.0L + ((long double)j + 0.5L) / LN_TAB));
-            ln[j].ln = (double)-logl((long double)ln[j].inv);
-        }
+        fill_ln_table(ln);
         UP(g_ln, ln);
     }
 #undef UP

@@ -93,8 +93,10 @@ __host__ __device__ inline CondRef<T> cond_ref(T* F, int64_t ld, int n, int64_t 
     return CondRef<T>{F + (int64_t)n * CF_COUNT * ld + s, ld};
 }
 
-// 1 / a: the hardware's approximate reciprocal and one third-order step r (1 + e + e^2),
-// e = 1 - a r, for FP64 (three dependent FP64 operations, against five of a second-order pair)
+// 1 / a: the hardware's approximate reciprocal and one step of the hyperpower iteration (Altman 1960),
+// e = 1 - a r: of third order r (1 + e + e^2) for FP64 (three dependent FP64 operations, against five of a
+// pair of second order), of second for FP32; within a unit in the last place for |a| in 2^-1000 .. 2^1000
+// and 2^-124 .. 2^124, as a division; beyond that (the hardware's takes subnormal numbers as 0) not
 __host__ __device__ inline double cond_recip(double a) {
 #ifdef __CUDA_ARCH__
     double r;

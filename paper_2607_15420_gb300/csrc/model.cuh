@@ -18,6 +18,8 @@
 #pragma once
 
 #include <math.h>
+#include <stdint.h>
+#include <string.h>
 
 #ifndef __CUDACC__
 #define __host__
@@ -144,30 +146,49 @@ struct StageLam {
 // product that is added to something is an explicit fma or a rounded product (mul_rn), so a value
 // comes out the same whatever else an instance computes.
 #ifdef __CUDACC__
-// ln(x) for the residuals: x = 2^e m, m in [1, 2); 1 / c from a table at the centre c of m's
-// 128th, r = m / c - 1 (|r| < 2^-8, one fma), ln x = e ln 2 + ln c + (r - r^2 / 2 + ... + r^7 / 7)
-// (the table-driven method of Tang 1990): 11 FP64 instructions against about 30 of log(), errors
-// of a rounding of the larger terms.  Anything but a positive normal number goes to log().
-struct LnEntry {
-    double inv, ln;   // 1 / c rounded, -ln(inv)
+// ln(x) for the residuals and the barrier: x = 2^e m, m in [1, 2), from 1 / c rounded to 11 bits at the
+// nearest c = 1 + j / 512, r = m / c - 1 (exact, |r| < 2^-9.6), ln x = e ln 2 + ln c + (r - r^2 / 2 + ... -
+// r^6 / 6) (the table-driven method of Tang 1990).  From j = 213 on m / 2 and e + 1 are taken, so that x next
+// to 1 has e = 0, c = 1 and no cancellation; ln 2 and ln c as a multiple of 2^-42 (their sum exact) and
+// a rest.  12 FP64 instructions against about 30 of log(), within a unit in the last place as that.
+// Anything but a positive normal number goes to log().
+struct __align__(16) LnEntry {
+    double hi, lo;   // -ln(1 / c) (of 2 / c from j = 213 on) in two parts; in hi's last 11 bits 2048 / c - 1024
 };
-constexpr int LN_TAB = 128;
+constexpr int LN_TAB = 513, LN_HALF = 213;
 __device__ LnEntry g_ln[LN_TAB];
+
+inline void fill_ln_table(LnEntry* t) {
+    for (int j = 0; j < LN_TAB; ++j) {
+        const long double inv = roundl(2048.0L / (1.0L + (long double)j / 512)) / 2048;
+        const long double v = -logl(j >= LN_HALF ? 2 * inv : inv);
+        double hi = (double)(roundl(v * 0x1p42L) * 0x1p-42L);   // |hi| < 0.36: its last 12 bits are zero
+        t[j].lo = (double)(v - (long double)hi);
+        uint64_t bits;
+        memcpy(&bits, &hi, sizeof(bits));
+        bits |= (uint64_t)(inv * 2048) - 1024;
+        memcpy(&t[j].hi, &bits, sizeof(bits));
+    }
+}
 #endif
 __host__ __device__ inline double ln_tab(double x) {
 #ifdef __CUDA_ARCH__
     const int hi = __double2hiint(x);
     if (!(hi >= 0x00100000 && hi < 0x7ff00000)) return log(x);
     const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(x));
-    const LnEntry t = g_ln[(hi >> 13) & (LN_TAB - 1)];
-    const double e = (double)((hi >> 20) - 1023);
-    const double r = fma(m, t.inv, -1.0);
-    double q = fma(r, 1.0 / 7.0, -1.0 / 6.0);
-    q = fma(r, q, 0.2);
+    const int j = ((hi & 0x000fffff) + 0x400) >> 11;
+    const LnEntry t = g_ln[j];
+    const int code = __double2loint(t.hi);
+    const double inv = __hiloint2double(0x3fe00000 + ((code & 0x7ff) << 10), 0);
+    const double thi = __hiloint2double(__double2hiint(t.hi), code & ~0x7ff);
+    const double e = (double)((hi >> 20) - 1023 + (j >= LN_HALF));
+    const double r = fma(m, inv, -1.0);
+    double q = fma(r, -1.0 / 6.0, 0.2);
     q = fma(r, q, -0.25);
     q = fma(r, q, 1.0 / 3.0);
     q = fma(r, q, -0.5);
-    return fma(e, 0.69314718055994530942, t.ln) + fma(r * r, q, r);
+    const double h = fma(e, 0x1.62e42fefa38p-1, thi), lo = fma(e, 0x1.ef35793c7673p-45, t.lo);   // ln 2 in two parts
+    return h + (r + fma(r * r, q, lo));
 #else
     return log(x);
 #endif
