@@ -1283,14 +1283,16 @@ __global__ void __launch_bounds__(CS_T, 6) cond_solve_kernel(const Params P, int
 
 // One block-elimination solve after its J^-1 r_c (pv) and Schur step (the steps of the design
 // entries in dz's slots): dz = p - q dtheta, g = r_z - (W + Sigma + dw I) dz, dl = J^-T g.  With az,
-// al (a correction) they are added to that direction.  g0 (optional): g, for the residual.  Grid
+// al (a correction) they are added to that direction.  g0 (optional): g, for the residual.  r_z and dz
+// may be one vector: every entry is read, by the repeated places too (of the same warp), before it
+// is written.  Grid
 // ceil(S / CS_N), CS_T threads.  5000 scenarios FP32 44-57 us (dz and g, and the
 // transposed solve were 13 + 52), the FP64 pipe 42 % busy with the products with H.
 template <int PREC>
 __global__ void __launch_bounds__(CS_T, 6) cond_direction_kernel(
     const Params P, int S, int64_t ld, const BView b, const CondFac K, const double* __restrict__ hes,
     const double* __restrict__ sig, bool use_w, const double* x, const double* __restrict__ pv,
-    const double* __restrict__ rz, double* dzo, double* __restrict__ dlo, double* __restrict__ az,
+    const double* rz, double* dzo, double* __restrict__ dlo, double* __restrict__ az,
     double* __restrict__ al, double* __restrict__ g0) {
     extern __shared__ __align__(16) unsigned char cond_sm[];
     const CondPlace at(S, b);
@@ -1324,6 +1326,7 @@ __global__ void __launch_bounds__(CS_T, 6) cond_direction_kernel(
                         if (i != j) g[j] = fma(-v, dz[i], g[j]);
                     }
         }
+        __syncwarp();
         if (live)
 #pragma unroll
             for (int j = 0; j < NV; ++j) {
