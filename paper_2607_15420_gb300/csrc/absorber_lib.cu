@@ -780,12 +780,12 @@ struct KKTSys {
 };
 
 // ---- block-tile autotuner ----------------------------------------------------------------
-// The warp kernels run one scenario per warp; how many warps share a block (and with it
-// the block's static shared memory) sets the resident blocks per SM and the tail of the
-// last wave.  The first launch of a kernel kind, precision and size bucket (powers of
-// two of S) on a device times every candidate (best of two timings) on that launch's own data -- each
-// candidate computes the same values bit for bit, one warp per scenario -- and keeps the
-// fastest for every later launch with that key.  Launches below TUNE_MIN_S scenarios are
+// Of the kernels with several shapes (the FP32 chain, four threads per scenario; the stage blocks'
+// kernels, a warp per scenario) the number of warps in a block, and with it the block's shared
+// memory, sets the resident blocks per SM and the tail of the last wave.  The first launch of a
+// kernel kind, precision and size bucket (powers of two of S) on a device times every
+// candidate (best of two timings) on that launch's own data -- each candidate computes the
+// same values bit for bit -- and keeps the fastest for every later launch with that key.  Launches below TUNE_MIN_S scenarios are
 // latency-bound and use the default shape.
 constexpr int TUNE_MIN_S = 256;
 std::mutex g_tune_mu;

@@ -86,10 +86,10 @@ template <class T>
 struct CondRef {   // the stored values of one stage of one scenario
     T* f;
     int64_t ld;
-    __host__ __device__ T& operator()(int e) const { return f[(int64_t)e * ld]; }
+    __device__ T& operator()(int e) const { return f[(int64_t)e * ld]; }
 };
 template <class T>
-__host__ __device__ inline CondRef<T> cond_ref(T* F, int64_t ld, int n, int64_t s) {
+__device__ inline CondRef<T> cond_ref(T* F, int64_t ld, int n, int64_t s) {
     return CondRef<T>{F + (int64_t)n * CF_COUNT * ld + s, ld};
 }
 
@@ -97,27 +97,19 @@ __host__ __device__ inline CondRef<T> cond_ref(T* F, int64_t ld, int n, int64_t 
 // e = 1 - a r: of third order r (1 + e + e^2) for FP64 (three dependent FP64 operations, against five of a
 // pair of second order), of second for FP32; within a unit in the last place for |a| in 2^-1000 .. 2^1000
 // and 2^-124 .. 2^124, as a division; beyond that (the hardware's takes subnormal numbers as 0) not
-__host__ __device__ inline double cond_recip(double a) {
-#ifdef __CUDA_ARCH__
+__device__ inline double cond_recip(double a) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
     const double e = fma(-a, r, 1.0);
     return fma(r, fma(e, e, e), r);
-#else
-    return 1.0 / a;
-#endif
 }
-__host__ __device__ inline float cond_recip(float a) {
-#ifdef __CUDA_ARCH__
+__device__ inline float cond_recip(float a) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
     return fmaf(r, fmaf(-a, r, 1.0f), r);
-#else
-    return 1.0f / a;
-#endif
 }
-__host__ __device__ inline double cond_fma(double a, double b, double c) { return fma(a, b, c); }
-__host__ __device__ inline float cond_fma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ inline double cond_fma(double a, double b, double c) { return fma(a, b, c); }
+__device__ inline float cond_fma(float a, float b, float c) { return fmaf(a, b, c); }
 
 // |a| <= lim, false for NaN
 __device__ __forceinline__ bool within(double a, double lim) {
@@ -335,7 +327,7 @@ __device__ inline bool condense_stage(const Own& A, T Lt, T Vt, const CondRef<T>
 // neighbours' core rows: lo (liquid, rows b, c, d, E of the stage below) and go (vapour: CO2,
 // H2O, N2, enthalpy, of the stage above), which those stages add to their rc.
 template <class T>
-__host__ __device__ inline void cond_reduce(const CondRef<const T>& f, const T (&r)[NR], T (&rc)[NCORE], T (&rho)[9],
+__device__ inline void cond_reduce(const CondRef<const T>& f, const T (&r)[NR], T (&rc)[NCORE], T (&rho)[9],
                                             T (&lo)[4], T (&go)[4]) {
     const T p2 = r[R_RX] * f(CF_I12);
     T p4 = r[R_RX + 3] * f(CF_I44);
@@ -395,7 +387,7 @@ __host__ __device__ inline void cond_reduce(const CondRef<const T>& f, const T (
 // From the core unknowns c: the stage's fractions, flows and temperature into u, and the flows
 // the extents need: fl = (f1, f3, f5, f6, f7: liquid flows of rows 1, 3, 5, 6, 7; CO2 vapour).
 template <class T>
-__host__ __device__ inline void cond_expand(const CondRef<const T>& f, const T (&c)[NCORE], const T (&rho)[9],
+__device__ inline void cond_expand(const CondRef<const T>& f, const T (&c)[NCORE], const T (&rho)[9],
                                             T (&u)[NV], T (&fl)[6]) {
     u[0] = c[0];
     u[1] = c[1];
@@ -433,7 +425,7 @@ __host__ __device__ inline void cond_expand(const CondRef<const T>& f, const T (
 // The extents and the slack, from the stage's flows fl, the liquid flows of the stage above
 // fa (zero for the top stage) and the CO2 vapour flow of the stage below vb (zero for the bottom).
 template <class T>
-__host__ __device__ inline void cond_extents(const CondRef<const T>& f, const T (&r)[NR], const T (&fl)[6],
+__device__ inline void cond_extents(const CondRef<const T>& f, const T (&r)[NR], const T (&fl)[6],
                                              const T (&fa)[5], T vb, T (&u)[NV]) {
     u[LE + 0] = r[1] - (fl[0] - fa[0]);
     u[LE + 1] = (fl[3] - fa[3]) - r[6];
@@ -447,7 +439,7 @@ __host__ __device__ inline void cond_extents(const CondRef<const T>& f, const T 
 // extents' entries of g of the stage above and below (zero past the ends).  Core right-hand
 // side -> gc, the eliminated fractions' entries -> gam (x2, x4, x5, x6, x7, x8, y1, y0, y2).
 template <class T>
-__host__ __device__ inline void cond_reduce_t(const CondRef<const T>& f, const T (&g)[NV], T ea4, const T (&eb)[5],
+__device__ inline void cond_reduce_t(const CondRef<const T>& f, const T (&g)[NV], T ea4, const T (&eb)[5],
                                               T (&gc)[NCORE], T (&gam)[9]) {
     const T p1 = eb[0] - g[LE + 0], p6 = g[LE + 1] - eb[1], p5 = g[LE + 2] - eb[2], p3 = eb[3] - g[LE + 3],
             p7 = eb[4] - g[LE + 4], pv = ea4 - g[LE + 4];
@@ -491,7 +483,7 @@ __host__ __device__ inline void cond_reduce_t(const CondRef<const T>& f, const T
 // cond_reduce.  dl: the stage's multipliers of rows b, c, d, E less those of the stage below;
 // dg: its multipliers of the vapour links (CO2, H2O, N2, enthalpy) less those of the stage above.
 template <class T>
-__host__ __device__ inline void cond_expand_t(const CondRef<const T>& f, const T (&g)[NV], const T (&w)[NCORE],
+__device__ inline void cond_expand_t(const CondRef<const T>& f, const T (&g)[NV], const T (&w)[NCORE],
                                               const T (&dl)[4], const T (&dg)[4], const T (&gam)[9], T (&v)[NR]) {
     v[0] = w[0];
     v[1] = g[LE + 0] + (w[0] + w[1]);
@@ -659,8 +651,8 @@ __device__ __forceinline__ bool core_above(double a, double tiny) {
 __device__ __forceinline__ bool core_above(float a, float tiny) { return fabsf(a) > tiny; }
 
 __host__ __device__ constexpr size_t chain_smem(size_t es, int spb, int cg) {
-    // N At^-1 (7 x 5); CG > 1: two pivot-column buffers (7 + reciprocal), pivot rows, column maxima
-    return (size_t)spb * (35 * es + (cg > 1 ? 16 * es + (2 + 2 * cg) * sizeof(int) : 0));
+    // N At^-1 (7 x 5), two pivot-column buffers (7 + reciprocal), pivot rows, column maxima
+    return (size_t)spb * (51 * es + (2 + 2 * cg) * sizeof(int));
 }
 
 // The chain over the stages: At_n from the stored M, N and the stage below's K, its inverse by
@@ -685,10 +677,10 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
     const int i = (int)threadIdx.x % SPB, g = (int)threadIdx.x / SPB;
     const int s = blockIdx.x * SPB + i;
     const bool live = live_prob(b, s, S, PS_ACT) >= 0 && !(mask && mask[s] == 0);
-    if (CG == 1 ? !live : !__syncthreads_or(live)) return;
+    if (!__syncthreads_or(live)) return;
     int bad = 0;
     T kc[5][5];   // K of the stage below
-    // the thread's columns of a stage's M and N (CG > 1): loaded a stage ahead, so that the elimination
+    // the thread's columns of a stage's M and N: loaded a stage ahead, so that the elimination
     // does not start with a wait for memory
     T cm[NCOL][5], ce[NCOL][5];
     auto columns = [&](int n) {
@@ -703,7 +695,7 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
             }
         }
     };
-    if constexpr (CG > 1) columns(0);
+    columns(0);
 #pragma unroll 1
     for (int n = 0; n < N_STAGES; ++n) {
         const CondRef<T> f = cond_ref(F, ld, n, (int64_t)s);
@@ -727,18 +719,10 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
         for (int c = 0; c < NCOL; ++c) {
             const int j = g + CG * c;
             T m[5], e[5];
-            if constexpr (CG == 1) {
 #pragma unroll
-                for (int k = 0; k < 5; ++k) {
-                    m[k] = c < 5 ? M[k][c < 5 ? c : 0] : T(0);
-                    e[k] = c < 4 ? N[k][c < 4 ? c : 0] : (c == 5 ? N[k][4] : (c == 6 ? N[k][5] : T(0)));
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < 5; ++k) {
-                    m[k] = cm[c][k];
-                    e[k] = ce[c][k];
-                }
+            for (int k = 0; k < 5; ++k) {
+                m[k] = cm[c][k];
+                e[k] = ce[c][k];
             }
             if (n > 0) {
 #pragma unroll
@@ -757,21 +741,18 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
 #pragma unroll
                 for (int r = 0; r < NCORE; ++r) km = max(km, core_key(a[c][r]));
         }
-        if constexpr (CG > 1) {
-            sK[((n & 1) * CG + g) * SPB + i] = km;
-            __syncthreads();
+        sK[((n & 1) * CG + g) * SPB + i] = km;
+        __syncthreads();
 #pragma unroll
-            for (int q = 0; q < CG; ++q) km = max(km, sK[((n & 1) * CG + q) * SPB + i]);
-        }
-        if constexpr (CG > 1)
-            if (n + 1 < N_STAGES) columns(n + 1);
+        for (int q = 0; q < CG; ++q) km = max(km, sK[((n & 1) * CG + q) * SPB + i]);
+        if (n + 1 < N_STAGES) columns(n + 1);
         const T tiny = (T)pivtol * core_mag(km, T(0));
         unsigned orig = 0x6543210u;   // nibble k: the row now at position k
 #pragma unroll
         for (int k = 0; k < NCORE; ++k) {
             T fc[NCORE], piv = T(0);
             int p = k;
-            const bool own = CG == 1 || g == k % CG;
+            const bool own = g == k % CG;
             if (own) {
                 T(&c)[NCORE] = a[k / CG];
                 unsigned best = core_key(c[k]);
@@ -797,22 +778,20 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
 #pragma unroll
                 for (int r = 0; r < NCORE; ++r) fc[r] = c[r];
             }
-            if constexpr (CG > 1) {
-                T* bp = sP + (k & 1) * 8 * SPB;
-                if (own) {
+            T* bp = sP + (k & 1) * 8 * SPB;
+            if (own) {
 #pragma unroll
-                    for (int r = 0; r < NCORE; ++r)
-                        if (r != k) bp[r * SPB + i] = fc[r];
-                    bp[7 * SPB + i] = piv;
-                    sR[(k & 1) * SPB + i] = p;
-                }
-                __syncthreads();
-                if (!own) {
+                for (int r = 0; r < NCORE; ++r)
+                    if (r != k) bp[r * SPB + i] = fc[r];
+                bp[7 * SPB + i] = piv;
+                sR[(k & 1) * SPB + i] = p;
+            }
+            __syncthreads();
+            if (!own) {
 #pragma unroll
-                    for (int r = 0; r < NCORE; ++r) fc[r] = r != k ? bp[r * SPB + i] : T(0);
-                    piv = bp[7 * SPB + i];
-                    p = sR[(k & 1) * SPB + i];
-                }
+                for (int r = 0; r < NCORE; ++r) fc[r] = r != k ? bp[r * SPB + i] : T(0);
+                piv = bp[7 * SPB + i];
+                p = sR[(k & 1) * SPB + i];
             }
             // rows k and p change places, row k scales by the pivot's reciprocal, the others subtract
             // their multiple of it; the pivot column itself starts from the unit vector (one code
@@ -874,18 +853,16 @@ __global__ void __launch_bounds__(SPB * CG) chain_kernel(int S, int64_t ld, cons
                 }
             }
         }
-        if constexpr (CG > 1) __syncthreads();
+        __syncthreads();
         if (g == CG - 1 && live)
 #pragma unroll
             for (int q = 0; q < 5; ++q)
                 f(CF_D + 5 * q) = (sN[(5 + q) * SPB + i] + sN[(10 + q) * SPB + i]) - sN[(15 + q) * SPB + i];
     }
-    if constexpr (CG > 1) {
-        __syncthreads();
-        sK[g * SPB + i] = (unsigned)bad;
-        __syncthreads();
-        for (int q = 0; q < CG; ++q) bad |= (int)sK[q * SPB + i];
-    }
+    __syncthreads();
+    sK[g * SPB + i] = (unsigned)bad;
+    __syncthreads();
+    for (int q = 0; q < CG; ++q) bad |= (int)sK[q * SPB + i];
     if (live && g == 0 && sing) sing[s] = bad;
 }
 

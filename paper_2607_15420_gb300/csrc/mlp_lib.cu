@@ -46,7 +46,7 @@ struct abs_mlp {
     int dev = 0;
     float* theta = nullptr;          // FP32 master parameters [NPAR]
     __nv_bfloat16* wb = nullptr;     // bfloat16 copies at the same offsets (weights only are read)
-    __nv_bfloat16* wt = nullptr;     // W2..W4's again as 64 x 256 tiles in the tensor cores' layout
+    __nv_bfloat16* wt = nullptr;     // W2..W4's again as 128 x 128 chunks in the tensor cores' layout
     float* grad = nullptr;           // [NPAR]
     float* m = nullptr;              // Adam moments [NPAR]
     float* v = nullptr;
